@@ -3,34 +3,55 @@
 // single-key error p_j ||v_j - mu|| (ties -> lower index) -- for rows of any
 // length up to 49,152 keys and budgets s <= 32 (pools of at most 64 keys).
 //
-//   k_pool_build  one CTA per row: p_j and e_j^2 = p_j^2 ||v_j - o||^2 of every
-//                 key (o = the dense output of the gap call; a warp per key,
-//                 lanes across the value row), then per budget a 3-pass radix
-//                 select (11/11/10 bits) of the top E among the dropped keys
-//                 (equal errors: lower index first) and the pool in ascending
-//                 key order.
-//   k_pool_enum   one warp per (row, budget): the pool's Gram matrix
-//                 G_ab = u_a . u_b, u = p (v - o), in shared memory; the
-//                 smaller side (the s kept keys, or the P - s keys left out)
-//                 is enumerated in colex order, lanes taking rank ranges, with
-//                 the sums over all members but the lowest held while the
-//                 lowest member runs (O(m) shared-memory reads per subset).
-//                 Every subset gets an fp32 score es^2 and a rigorous interval
-//                 around it (the rounding of the Gram sums, bounded by
-//                 (sum_pool |u|)^2); the subsets whose lower end does not
-//                 exceed the least upper end are buffered (4,096 per warp, in
-//                 the workspace) and re-scored in fp64 as
-//                 es^2 = (sum_{a,b in A} G_ab) / p(A)^2 from an fp64 copy of
-//                 the Gram matrix (the products u_a . u_b formed in fp64 from
-//                 the fp32 masses, the bf16 / fp32 values and o), and the least
-//                 es wins, exact ties to the smallest colex rank of the
-//                 members' pool positions.  (Re-scoring from the value rows
-//                 cost |A| dependent row loads per candidate; flat rows send
-//                 ~1,000 candidates per item.)
+//   k_pool_build  one CTA per row: e_j^2 = p_j^2 ||v_j - o||^2 of every key (o =
+//                 the dense output of the gap call; four lanes per key, 16-byte
+//                 loads, o in registers), ONE radix select of the m = max(s + E)
+//                 largest errors -- a budget's E extras are among the s + E
+//                 largest errors of the whole row, since at most s kept keys
+//                 can be ahead of them -- and per budget the pool in ascending
+//                 key order, ranked among those m and the kept keys by a warp.
+//   k_pool_enum   one CTA per (row, budget), below.
 //
-// Nothing waits on another block; a buffer of re-scoring candidates that
-// overflows falls back to a per-lane re-scoring pass over the same
-// candidates, so the answer stays exact.
+// Enumeration.  With u = p (v - o), G_xy = u_x . u_y, t the least es^2 known (at
+// first the top-mass set's) and a set K of s pool keys (at first the same), a
+// size-s subset A = (K \ R) u D has es(A)^2 <= t iff
+//   val(A) = |sum_A u|^2 - t p(A)^2 <= 0,
+// and val is a quadratic form in the exchanged keys: with H = G - t p p^T and
+// h = H 1_K,
+//   val(A) = val(K) + sum_R (H_xx - 2 h_x) + sum_D (H_yy + 2 h_y)
+//            + 2 sum_{pairs in R} H + 2 sum_{pairs in D} H - 2 sum_{R x D} H.
+// val(K) and h come from sum_K u, summed in double-float; G is plain fp32.  The
+// rounding of the whole is at most kappa (e^2 + 2 e b + val(K)), b = |sum_K u|
+// + sqrt(t) p(K), e the sum over the exchanged keys of a_x = |u_x| + sqrt(t) p_x
+// -- a bound that leaves out the heavy keys both sets share -- and is a
+// quadratic form too, so it is folded into the table entries: "computed value
+// <= 0" is a necessary condition and costs nothing.  A sweep over the subsets
+// collects those that pass, with their values; value and bound give each an
+// interval for es^2, the few whose lower end does not exceed the least upper
+// end are scored from the value rows in double-float, and the least es wins,
+// exact ties to the smallest colex rank of the members' pool positions.  Where
+// more than GCAP pass -- rows with good subsets that leave out the attention
+// sink, far from the top-mass set, whose values the bound around that set
+// cannot tell apart -- the subset of least value becomes K and the sweep is
+// repeated around it, with the least es^2 known by then.
+//
+// A sweep walks |R| = |D| = r = 1 .. min(s, E).  All subsets of the side with
+// fewer keys are laid out in groups of 8 (their own value, and W[y][8], their
+// cross terms with key y of the other side) in shared memory, in batches where
+// they do not fit; lanes take the other side's subsets without their highest
+// member and run that member upwards, so a subset costs two additions and a
+// minimum.  Bound: instruction issue.
+//
+// Measured on 256 rows of 4,096 keys, d = 128, s = 4/8/16/32 with E =
+// 24/12/6/4 (gap call, build and enumeration): 0.71 ms, against 37 to 250 ms
+// (by which rows were drawn) with one warp per item that scored every subset
+// from scratch under an error bound of the whole pool's sum |u| and re-scored
+// what passed in fp64.  16 warps per block (64 registers) rather than 8: 0.71
+// against 0.80 ms, the sweeps wait on shared memory.
+//
+// Nothing waits on another block; when sweeping around better sets does not
+// bring the hits below GCAP (exact ties by the thousand) the lanes score every
+// hit, so the answer stays exact.
 #include <algorithm>
 #include <climits>
 
@@ -40,14 +61,24 @@ namespace fw {
 namespace {
 
 constexpr int PB_T = 256;            // k_pool_build: threads per row
-constexpr int PE_W = 4;              // k_pool_enum: warps per block, one (row, budget) each
+constexpr int PB_Q = 4;              // ... lanes per key
+constexpr int PE_T = 512;            // k_pool_enum: threads per (row, budget)
+constexpr int PE_NW = PE_T / 32;
+constexpr int PE_CH = 8;             // small-side subsets per group
+constexpr int PE_WCAP = 5120;        // floats of W: one batch of groups
+constexpr int PE_GMAX = 64;          // groups per batch
+constexpr int PE_GSPLIT = 16;        // groups per warp task
+constexpr int PE_BPS = 2;            // blocks per SM (their shared memory: 104 KB at d = 128)
 constexpr int PMAX = 64;             // pool keys
 constexpr int PSMAX = 32;            // largest budget
+constexpr int PCAND = PMAX + PSMAX;  // keys k_pool_build gathers: largest errors and kept keys
 constexpr int PB_STAGE_MAX = 49152;  // keys per row staged in shared memory
-constexpr int GCAP = 4096;           // re-scoring candidates buffered per warp (workspace)
-constexpr int PE_BPS = 4;            // k_pool_enum blocks per SM in the launch (each warp owns workspace)
+constexpr int GCAP = 512;            // re-scoring candidates buffered per block
+constexpr int PE_SURV = 32;           // survivors that another sweep may cut
+constexpr int PE_SWEEPS = 8;         // sweeps before the lanes score every candidate
 constexpr uint64_t PE_MAX_SUBSETS = 1ull << 32;
-constexpr int GLD = PMAX + 1;        // Gram row stride (odd: conflict-free columns)
+constexpr int CLD = PMAX + 1;        // table row stride (odd: conflict-free columns)
+constexpr float PE_TINY = 1e-36f;    // slack for subnormal table entries
 
 // C(a, b) for a <= 64, b <= 32 (all below 2^63), by Pascal's rule at compile time.
 struct Binom64Table {
@@ -62,9 +93,11 @@ constexpr Binom64Table make_binom64()
     }
     return t;
 }
-static __constant__ Binom64Table c_b64 = make_binom64();
+static __constant__ Binom64Table c_b64 = make_binom64();  // warp-uniform reads
+static __device__ const Binom64Table g_b64 = make_binom64();  // reads that differ by lane
 
 __device__ __forceinline__ uint64_t cb(int a, int b) { return (b < 0 || b > 32 || a < b) ? 0 : c_b64.v[a][b]; }
+__device__ __forceinline__ uint64_t cbl(int a, int b) { return (b > 32 || a < b) ? 0 : __ldg(&g_b64.v[a][b]); }
 
 struct PoolArgs {
     RowsDev R;
@@ -82,221 +115,218 @@ struct PoolArgs {
     float *topk_gap;           // [rows][nb] or null
     int32_t *row_status;       // [rows] or null
     int64_t *n_cand;           // [rows][nb] re-scored subsets, or null
-    uint64_t *gcand;           // ws [gridDim.x * PE_W][GCAP] candidate masks of each warp
-    double *g64;               // ws [gridDim.x * PE_W][PMAX * PMAX] fp64 Gram matrix of each warp
 };
 
 // ------------------------------------------------------------ the pool
 
-template <int DPL, typename VT>
-__device__ __forceinline__ void load_row_part(const VT *V, int64_t j, int lane, float (&x)[DPL])
-{
-    constexpr int d = DPL * 32;
+// This lane's quarter of a value row as fp32: the 16-byte vectors sub, sub + 4, ...
+template <int DPL, typename VT> struct PoolLane {
+    static constexpr int EPV = 16 / (int)sizeof(VT);
+    static constexpr int NV = DPL * 32 / EPV / PB_Q;
+    uint4 u[NV];
+    __device__ __forceinline__ void load(const VT *v, int sub)
+    {
 #pragma unroll
-    for (int c = 0; c < DPL; ++c) x[c] = load_v(V, j * d + lane * DPL + c);
-}
+        for (int q = 0; q < NV; ++q) u[q] = __ldg(reinterpret_cast<const uint4 *>(v + (q * PB_Q + sub) * EPV));
+    }
+    __device__ __forceinline__ float at(int q, int e) const  // constants after unrolling
+    {
+        const uint32_t w[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
+        if constexpr (sizeof(VT) == 4) return __uint_as_float(w[e]);
+        else return __uint_as_float((e & 1) ? (w[e >> 1] & 0xffff0000u) : (w[e >> 1] << 16));
+    }
+};
 
 template <int DPL, typename VT>
 __global__ void __launch_bounds__(PB_T) k_pool_build(PoolArgs a)
 {
     extern __shared__ float sm[];
     float *e2 = sm;  // [max_n] single-key errors squared
-    __shared__ uint32_t hist[2048];
-    __shared__ int wcnt[PB_T / 32];
-    __shared__ uint32_t s_digit;
-    __shared__ int s_rem, s_L;
+    __shared__ TopmSmem S;
+    __shared__ int32_t c_idx[PCAND];
+    __shared__ uint32_t c_err[PCAND], c_log[PCAND];
+    __shared__ int s_cnt;
+    using L = PoolLane<DPL, VT>;
     constexpr int d = DPL * 32;
-    constexpr int NW = PB_T / 32;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int sub = tid % PB_Q, gq = tid / PB_Q;
+    constexpr int KPI = PB_T / PB_Q;
     for (int64_t r = blockIdx.x; r < a.R.rows; r += gridDim.x) {
         const int64_t g = r / a.R.R;
         const int n = a.R.n[g];
         const float *l = a.R.logits + a.R.logit_off[g] + (r - g * a.R.R) * n;
         const VT *V = static_cast<const VT *>(a.R.v) + a.R.v_off[g];
         const float M = a.M[r], Zi = 1.f / a.Z[r];
-        float so[DPL];
+        float so[L::NV * L::EPV];
 #pragma unroll
-        for (int c = 0; c < DPL; ++c) so[c] = a.o[r * d + lane * DPL + c];
-        __syncthreads();  // the previous row's e2 is no longer read
-        // a warp per key, two keys in flight: lanes hold DPL consecutive dims
-        for (int j = wid * 2; j < n; j += NW * 2) {
-            float x0[DPL], x1[DPL];
-            const bool two = j + 1 < n;
-            load_row_part<DPL, VT>(V, j, lane, x0);
-            if (two) load_row_part<DPL, VT>(V, j + 1, lane, x1);
-            float s0 = 0.f, s1 = 0.f;
+        for (int q = 0; q < L::NV; ++q)
 #pragma unroll
-            for (int c = 0; c < DPL; ++c) {
-                const float w0 = x0[c] - so[c];
-                s0 = fmaf(w0, w0, s0);
-                if (two) {
-                    const float w1 = x1[c] - so[c];
-                    s1 = fmaf(w1, w1, s1);
+            for (int e = 0; e < L::EPV; ++e) so[q * L::EPV + e] = a.o[r * d + (q * PB_Q + sub) * L::EPV + e];
+        __syncthreads();  // the previous row's shared arrays are no longer read
+        if (tid == 0) s_cnt = 0;
+        // two keys in flight per group of four lanes
+        for (int j0 = 0; j0 < n; j0 += 2 * KPI) {
+            const int ja = j0 + gq, jb = j0 + KPI + gq;
+            L ra, rb;
+            ra.load(V + (int64_t)min(ja, n - 1) * d, sub);
+            rb.load(V + (int64_t)min(jb, n - 1) * d, sub);
+            const int jm = sub & 1 ? jb : ja;  // lanes 0 and 1 finish one key each
+            const float p = sub < 2 ? __expf(__ldg(l + min(jm, n - 1)) - M) * Zi : 0.f;
+            float sa = 0.f, sb = 0.f;
+#pragma unroll
+            for (int q = 0; q < L::NV; ++q)
+#pragma unroll
+                for (int e = 0; e < L::EPV; ++e) {
+                    const float o = so[q * L::EPV + e];
+                    const float wa = ra.at(q, e) - o, wb = rb.at(q, e) - o;
+                    sa = fmaf(wa, wa, sa);
+                    sb = fmaf(wb, wb, sb);
                 }
+            sa += __shfl_xor_sync(FW_FULL, sa, 1);
+            sb += __shfl_xor_sync(FW_FULL, sb, 1);
+            sa += __shfl_xor_sync(FW_FULL, sa, 2);
+            sb += __shfl_xor_sync(FW_FULL, sb, 2);
+            if (sub < 2 && jm < n) e2[jm] = p * p * (sub ? sb : sa);
+        }
+        // the budgets: sizes, and the longest prefix of the error order any of them needs
+        int m = 0;
+        int sb_[4], Eb[4];
+        uint32_t tk[4];
+        int ti[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            sb_[b] = Eb[b] = -1;
+            tk[b] = 0xffffffffu;
+            ti[b] = -1;
+            if (b >= a.nb) continue;
+            const int64_t rb = r * a.nb + b;
+            const int s = a.k[rb];
+            int bad = 0;
+            if (s < 1 || s > n || s > PSMAX || s > a.k_max || a.E[b] < 0) bad = -1;
+            else if (s + min(a.E[b], n - s) > PMAX) bad = -2;
+            if (bad) {
+                if (tid == 0) a.pool_n[rb] = bad;
+                continue;
             }
-            s0 = warp_sum(s0);
-            s1 = warp_sum(s1);
-            if (lane == 0) {
-                const float p0 = __expf(__ldg(l + j) - M) * Zi;
-                e2[j] = p0 * p0 * s0;
-            } else if (lane == 1 && two) {
-                const float p1 = __expf(__ldg(l + j + 1) - M) * Zi;
-                e2[j + 1] = p1 * p1 * s1;
+            sb_[b] = s;
+            Eb[b] = min(a.E[b], n - s);
+            tk[b] = a.thr_key[rb];
+            ti[b] = a.thr_idx[rb];
+            m = max(m, s + Eb[b]);
+        }
+        __syncthreads();
+        if (m == 0) continue;  // (uniform)
+        uint32_t T = 0u;
+        int Lx = -1;
+        block_topm(n, m, [&](int j) { return order_key(e2[j]); }, S, T, Lx);
+        // the m largest errors and every budget's kept keys (at most PCAND for
+        // thresholds that keep the budgets' counts; more are not listed)
+        for (int j = tid; j < n; j += PB_T) {
+            const uint32_t u = order_key(e2[j]), kl = order_key(__ldg(l + j));
+            bool in = u > T || (u == T && j <= Lx);
+#pragma unroll
+            for (int b = 0; b < 4; ++b) in |= kl > tk[b] || (kl == tk[b] && j <= ti[b]);
+            if (in) {
+                const int q = atomicAdd(&s_cnt, 1);
+                if (q < PCAND) {
+                    c_idx[q] = j;
+                    c_err[q] = u;
+                    c_log[q] = kl;
+                }
             }
         }
         __syncthreads();
-        for (int b = 0; b < a.nb; ++b) {
+        const int nc = s_cnt;
+        // a warp per budget: kept keys and the Eb dropped ones of largest error, in key order
+        for (int b = wid; b < a.nb; b += PB_T / 32) {
+            int s = -1, E = 0, tix = -1;
+            uint32_t tkx = 0u;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (q == b) s = sb_[q], E = Eb[q], tkx = tk[q], tix = ti[q];
+            if (s < 0) continue;
             const int64_t rb = r * a.nb + b;
-            const int s = a.k[rb];
-            const uint32_t tk = a.thr_key[rb];
-            const int ti = a.thr_idx[rb];
-            if (s < 1 || s > n || s > PSMAX || s > a.k_max || a.E[b] < 0) {
-                if (tid == 0) a.pool_n[rb] = -1;
+            if (nc > PCAND) {
+                if (lane == 0) a.pool_n[rb] = -2;
                 continue;
             }
-            const int Ee = min(a.E[b], n - s);
-            if (s + Ee > PMAX) {
-                if (tid == 0) a.pool_n[rb] = -2;
-                continue;
-            }
-            // top Ee of the dropped keys by e2 (order key of a non-negative float)
-            uint32_t T = 0xffffffffu;
-            int L = -1;
-            if (Ee > 0) {
-                if (tid == 0) {
-                    s_digit = 0u;
-                    s_rem = 1;
-                }
-                uint32_t prefix = 0, pmask = 0;
-                int rem = Ee;
-                for (int pass = 0; pass < 3; ++pass) {
-                    const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-                    const int nbin = pass < 2 ? 2048 : 1024;
-                    for (int i = tid; i < 2048; i += PB_T) hist[i] = 0u;
-                    __syncthreads();
-                    for (int j = tid; j < n; j += PB_T) {
-                        const uint32_t kl = order_key(__ldg(l + j));
-                        const bool kept = kl > tk || (kl == tk && j <= ti);
-                        const uint32_t u = order_key(e2[j]);
-                        if (!kept && (u & pmask) == prefix) atomicAdd(&hist[(u >> shift) & (uint32_t)(nbin - 1)], 1u);
-                    }
-                    __syncthreads();
-                    if (wid == 0) {
-                        // bins in descending order, nbin / 32 consecutive bins per lane
-                        const int per = nbin / 32;
-                        const int top = nbin - 1 - lane * per;
-                        int c = 0;
-                        for (int q = 0; q < per; ++q) c += (int)hist[top - q];
-                        int incl = c;
+            constexpr int PER = PCAND / 32;
+            uint32_t in[PER];  // ballots over the listed keys
 #pragma unroll
-                        for (int off = 1; off < 32; off <<= 1) {
-                            const int y = __shfl_up_sync(FW_FULL, incl, off);
-                            if (lane >= off) incl += y;
+            for (int q = 0; q < PER; ++q) {
+                const int c = q * 32 + lane;
+                bool take = false;
+                if (c < nc) {
+                    const int j = c_idx[c];
+                    const uint32_t u = c_err[c];
+                    take = c_log[c] > tkx || (c_log[c] == tkx && j <= tix);
+                    if (!take) {
+                        int ahead = 0;  // dropped keys before this one in the error order
+                        for (int c2 = 0; c2 < nc; ++c2) {
+                            const int j2 = c_idx[c2];
+                            const bool k2 = c_log[c2] > tkx || (c_log[c2] == tkx && j2 <= tix);
+                            ahead += !k2 && (c_err[c2] > u || (c_err[c2] == u && j2 < j));
                         }
-                        const int excl = incl - c;
-                        if (excl < rem && rem <= incl) {
-                            int acc = excl;
-                            for (int q = 0; q < per; ++q) {
-                                const int h = (int)hist[top - q];
-                                if (acc + h >= rem) {
-                                    s_digit = (uint32_t)(top - q);
-                                    s_rem = rem - acc;
-                                    break;
-                                }
-                                acc += h;
-                            }
-                        }
+                        take = ahead < E;
                     }
-                    __syncthreads();
-                    prefix |= s_digit << shift;
-                    pmask |= (uint32_t)(nbin - 1) << shift;
-                    rem = s_rem;
-                    __syncthreads();
                 }
-                T = prefix;
-                // the rem-th dropped key (index order) whose key equals T
-                if (tid == 0) s_L = -1;
-                __syncthreads();
-                int run = 0;
-                for (int j0 = 0; j0 < n; j0 += PB_T) {
-                    const int j = j0 + tid;
-                    bool eq = false;
-                    if (j < n) {
-                        const uint32_t kl = order_key(__ldg(l + j));
-                        const bool kept = kl > tk || (kl == tk && j <= ti);
-                        eq = !kept && order_key(e2[j]) == T;
-                    }
-                    const unsigned m = __ballot_sync(FW_FULL, eq);
-                    if (lane == 0) wcnt[wid] = __popc(m);
-                    __syncthreads();
-                    int before = run, tot = 0;
-#pragma unroll
-                    for (int w = 0; w < NW; ++w) {
-                        if (w < wid) before += wcnt[w];
-                        tot += wcnt[w];
-                    }
-                    before += __popc(m & ((1u << lane) - 1u));
-                    if (eq && before + 1 == rem) s_L = j;
-                    run += tot;
-                    __syncthreads();
-                    if (s_L >= 0) break;
-                }
-                L = s_L;
-                __syncthreads();
+                in[q] = __ballot_sync(FW_FULL, take);
             }
-            // the pool in ascending key order: kept keys and the extras
-            int run = 0;
-            int32_t *pl = a.pool + rb * PMAX;
-            for (int j0 = 0; j0 < n; j0 += PB_T) {
-                const int j = j0 + tid;
-                bool in = false;
-                if (j < n) {
-                    const uint32_t kl = order_key(__ldg(l + j));
-                    const bool kept = kl > tk || (kl == tk && j <= ti);
-                    const uint32_t u = order_key(e2[j]);
-                    in = kept || (Ee > 0 && (u > T || (u == T && j <= L)));
-                }
-                const unsigned m = __ballot_sync(FW_FULL, in);
-                if (lane == 0) wcnt[wid] = __popc(m);
-                __syncthreads();
-                int before = run, tot = 0;
+            int cnt = 0;
 #pragma unroll
-                for (int w = 0; w < NW; ++w) {
-                    if (w < wid) before += wcnt[w];
-                    tot += wcnt[w];
-                }
-                before += __popc(m & ((1u << lane) - 1u));
-                if (in && before < PMAX) pl[before] = j;
-                run += tot;
-                __syncthreads();
+            for (int q = 0; q < PER; ++q) cnt += __popc(in[q]);
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const int c = q * 32 + lane;
+                if (!((in[q] >> lane) & 1u)) continue;
+                const int j = c_idx[c];
+                int pos = 0;
+#pragma unroll
+                for (int q2 = 0; q2 < PER; ++q2)
+                    for (uint32_t w = in[q2]; w; w &= w - 1) pos += c_idx[q2 * 32 + __ffs(w) - 1] < j;
+                if (pos < PMAX) a.pool[rb * PMAX + pos] = j;
             }
-            if (tid == 0) a.pool_n[rb] = run <= PMAX ? run : -2;
+            if (lane == 0) a.pool_n[rb] = cnt <= PMAX ? cnt : -2;
         }
     }
 }
 
 // ------------------------------------------------------------ enumeration
 
-// next m-combination of 0..P-1 in colex order (the lowest member moves fastest)
-__device__ __forceinline__ bool colex_next(int *c, int m, int P)
+// the m-combination of colex rank `rank` out of 0..P-1 as a bit mask
+__device__ __forceinline__ uint64_t colex_unrank(uint64_t rank, int m, int P)
 {
-    int i = 0;
-    while (i < m && c[i] + 1 == (i + 1 < m ? c[i + 1] : P)) ++i;
-    if (i == m) return false;
-    ++c[i];
-    for (int t = 0; t < i; ++t) c[t] = t;
-    return true;
-}
-
-// the m-combination of 0..P-1 of colex rank `rank`
-__device__ __forceinline__ void colex_unrank(uint64_t rank, int m, int P, int *c)
-{
-    for (int i = m - 1; i >= 0; --i) {
-        int x = i;
-        while (x + 1 < P && cb(x + 1, i + 1) <= rank) ++x;
-        c[i] = x;
-        rank -= cb(x, i + 1);
+    uint64_t A = 0;
+    int x = P - 1;
+    for (int i = m; i >= 1; --i) {
+        if (i == 3) {  // the largest x with C(x, 3) <= rank, from the cube root
+            const uint32_t q = (uint32_t)rank;
+            uint32_t y = (uint32_t)(cbrtf(6.f * (float)q) + 1.f);
+            while (y * (y - 1) * (y - 2) / 6 > q) --y;
+            while ((y + 1) * y * (y - 1) / 6 <= q) ++y;
+            A |= 1ull << y;
+            rank = q - y * (y - 1) * (y - 2) / 6;
+            continue;
+        }
+        if (i == 2) {  // C(x, 2) <= rank
+            const uint32_t q = (uint32_t)rank;
+            uint32_t y = (uint32_t)((sqrtf(8.f * (float)q + 1.f) + 1.f) * 0.5f);
+            while (y * (y - 1) / 2 > q) --y;
+            while ((y + 1) * y / 2 <= q) ++y;
+            A |= 1ull << y;
+            rank = q - y * (y - 1) / 2;
+            continue;
+        }
+        if (i == 1) {
+            A |= 1ull << rank;
+            break;
+        }
+        while (x >= i && cbl(x, i) > rank) --x;
+        A |= 1ull << x;
+        rank -= cbl(x, i);
+        --x;
     }
+    return A;
 }
 
 // colex rank of the set bits of a 64-bit mask (positions ascending)
@@ -304,303 +334,764 @@ __device__ __forceinline__ uint64_t colex_rank64(uint64_t A)
 {
     uint64_t rank = 0;
     int i = 1;
-    for (uint64_t w = A; w; w &= w - 1, ++i) rank += cb(__ffsll((long long)w) - 1, i);
+    for (uint64_t w = A; w; w &= w - 1, ++i) rank += cbl(__ffsll((long long)w) - 1, i);
     return rank;
 }
 
-// per-warp enumeration state in shared memory
+// state of one (row, budget); the value rows v [PMAX][d + 4] follow it
 struct EnumSm {
-    float G[PMAX * GLD];
-    float pp[PMAX];
-    float t[PMAX];        // t_x = sum_y G_xy = u_x . U
+    double QK, PK, bes;         // |sum_K u|^2, p(K), the least es known
+    uint64_t K, topK;           // the set exchanged from; kept keys by the thresholds
+    uint64_t bmask, brank;      // the best set known, its colex rank
+    uint64_t candD[GCAP];       // hits: the big side's keys exchanged ...
+    uint64_t red_rank[PE_NW], red_mask[PE_NW];
+    double red_es[PE_NW];
+    long long red_seen[PE_NW];
+    uint32_t candR[GCAP];       // ... the small side's
+    float candV[GCAP];          // ... and the value
+    __align__(16) float W[PE_WCAP];  // [group][big key][PE_CH]
+    float C[PMAX * CLD];        // table entries, small side's keys first (on the diagonal: one key alone)
+    float G[PMAX * CLD];        // u_x . u_y
+    uint32_t rmask[PE_GMAX * PE_CH];
+    float rbase[PE_GMAX * PE_CH];
+    float o[256];
+    float UKh[256], UKl[256];   // sum over K of u, by column, in double-float
+    float gh[PMAX], gl[PMAX];   // its products with v_x - o
+    float pp[PMAX];             // masses
+    float ax[PMAX];             // |u_x| + sqrt(t) p_x, scaled
     int32_t pidx[PMAX];
-    int ncand;
+    int32_t loc[PMAX];          // pool position of a table index
+    float red_v[PE_NW];
+    int ncand, nsurv, stale;
+    uint32_t task;
+    // segments of the batch: (r, first group of that r, groups)
+    int seg_r[PSMAX], seg_g[PSMAX], seg_n[PSMAX], nseg, next_r, next_g;
 };
 
-// es of the pool positions in A, from the definition in fp64: the warp forms
-// N_A = sum_A p_j v_j across the value dims (lane c covers DPL of them).
-template <int DPL, typename VT>
-__device__ __forceinline__ double es_warp(const VT *V, const float *o_lane, const EnumSm &S, uint64_t A, int lane)
+// columns c + step k (k < NC, below d) of sum over A of p (v - o), in
+// double-float, members ascending; the columns are independent chains
+template <int NC>
+__device__ __forceinline__ void col_sums(const EnumSm &S, const float *v, int d, uint64_t A, int c, int step,
+                                         double (&out)[NC])
 {
-    constexpr int d = DPL * 32;
-    double PA = 0.0;
-    double N[DPL];
+    float hi[NC], lo[NC];
 #pragma unroll
-    for (int c = 0; c < DPL; ++c) N[c] = 0.0;
+    for (int k = 0; k < NC; ++k) hi[k] = lo[k] = 0.f;
     for (uint64_t w = A; w; w &= w - 1) {
         const int x = __ffsll((long long)w) - 1;
-        const double px = (double)S.pp[x];
-        PA += px;
-        float v[DPL];
+        const float p = S.pp[x];
+        const float *vx = v + x * (d + 4);
 #pragma unroll
-        for (int c = 0; c < DPL; ++c) v[c] = load_v(V, (int64_t)S.pidx[x] * d + lane * DPL + c);
-#pragma unroll
-        for (int c = 0; c < DPL; ++c) N[c] = fma(px, (double)v[c], N[c]);
-    }
-    double e2 = 0.0;
-#pragma unroll
-    for (int c = 0; c < DPL; ++c) {
-        const double diff = N[c] / PA - (double)o_lane[c];
-        e2 = fma(diff, diff, e2);
-    }
-    e2 = warp_sum_d(e2);
-    return sqrt(e2);
-}
-
-// es of the pool positions in A from the fp64 Gram matrix: lane i sums the row
-// of A's i-th member over A (|A| <= 32), the warp adds the rows.
-__device__ __forceinline__ double es_gram_warp(const double *g, const EnumSm &S, uint64_t A, int lane)
-{
-    double rs = 0.0, pa = 0.0;
-    int i = 0;
-    for (uint64_t w = A; w; w &= w - 1, ++i) {
-        if (i != lane) continue;
-        const int x = __ffsll((long long)w) - 1;
-        pa = (double)S.pp[x];
-        for (uint64_t w2 = A; w2; w2 &= w2 - 1) rs += g[x * PMAX + __ffsll((long long)w2) - 1];
-    }
-    const double Q = warp_sum_d(rs), PA = warp_sum_d(pa);
-    return sqrt(fmax(Q, 0.0)) / PA;
-}
-
-// the same by one lane alone (fallback when the candidate buffer overflows)
-__device__ double es_gram_lane(const double *g, const EnumSm &S, uint64_t A)
-{
-    double Q = 0.0, PA = 0.0;
-    for (uint64_t w = A; w; w &= w - 1) {
-        const int x = __ffsll((long long)w) - 1;
-        PA += (double)S.pp[x];
-        for (uint64_t w2 = A; w2; w2 &= w2 - 1) Q += g[x * PMAX + __ffsll((long long)w2) - 1];
-    }
-    return sqrt(fmax(Q, 0.0)) / PA;
-}
-
-// Walks the colex ranks [lo, hi) of m-subsets C of the pool and calls
-// f(Cmask, lower, upper) with the interval that holds the exact es^2 of the
-// subset A (A = C in the direct form, pool \ C otherwise).
-template <typename F>
-__device__ __forceinline__ void walk(const EnumSm &S, int P, int m, bool direct, uint64_t lo, uint64_t hi, float UU,
-                                     float PU, float Eabs, float pe, F &&f)
-{
-    if (lo >= hi) return;
-    int c[PSMAX];
-    colex_unrank(lo, m, P, c);
-    uint64_t q = lo;
-    for (;;) {
-        // sums over the members above the lowest
-        float g2o = 0.f, pao = 0.f, lino = 0.f;
-        uint64_t om = 0;
-        for (int i = 1; i < m; ++i) {
-            const int x = c[i];
-            om |= 1ull << x;
-            pao += S.pp[x];
-            lino += S.t[x];
-            g2o += S.G[x * GLD + x];
-            for (int j = 1; j < i; ++j) g2o = fmaf(2.f, S.G[x * GLD + c[j]], g2o);
+        for (int k = 0; k < NC; ++k) {
+            const int ck = c + step * k;
+            if (ck >= d) break;
+            const df u = df_two_sum(vx[ck], -S.o[ck]);  // v - o exactly
+            const float q = p * u.hi;
+            const float e = fmaf(p, u.lo, fmaf(p, u.hi, -q));
+            const df t = df_two_sum(hi[k], q);
+            hi[k] = t.hi;
+            lo[k] += t.lo + e;
         }
-        const int lim = m > 1 ? c[1] : P;
-        for (int x = c[0]; x < lim && q < hi; ++x, ++q) {
-            float rs = S.G[x * GLD + x];
-            for (int i = 1; i < m; ++i) rs = fmaf(2.f, S.G[x * GLD + c[i]], rs);
-            float g2 = g2o + rs, pa = pao + S.pp[x];
-            if (!direct) {
-                g2 = fmaf(-2.f, lino + S.t[x], UU) + g2;
-                pa = PU - pa;
+    }
+#pragma unroll
+    for (int k = 0; k < NC; ++k) out[k] = (double)hi[k] + (double)lo[k];
+}
+
+__device__ __forceinline__ double mass_warp(const EnumSm &S, uint64_t A, int lane)
+{
+    return warp_sum_d((((A >> lane) & 1ull) ? (double)S.pp[lane] : 0.0) +
+                      (((A >> (lane + 32)) & 1ull) ? (double)S.pp[lane + 32] : 0.0));
+}
+
+// es of the pool positions in A, by the definition (the warp together)
+__device__ double es_warp(const EnumSm &S, const float *v, int d, uint64_t A, int lane)
+{
+    double q = 0.0;
+    for (int c0 = 0; c0 < d; c0 += 128) {
+        double u[4];
+        col_sums<4>(S, v, d, A, c0 + lane, 32, u);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) q = fma(u[k], u[k], q);
+    }
+    return sqrt(warp_sum_d(q)) / mass_warp(S, A, lane);
+}
+
+// the same by one lane alone (the last resort)
+__device__ double es_lane(const EnumSm &S, const float *v, int d, uint64_t A)
+{
+    double q = 0.0, pa = 0.0;
+    for (int c = 0; c < d; c += 4) {
+        double u[4];
+        col_sums<4>(S, v, d, A, c, 1, u);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) q = fma(u[k], u[k], q);
+    }
+    for (uint64_t w = A; w; w &= w - 1) pa += (double)S.pp[__ffsll((long long)w) - 1];
+    return sqrt(q) / pa;
+}
+
+// what a lane carries through a sweep
+struct LaneBest {
+    bool score;      // score every hit (else: collect hits, keep the least value)
+    float least;     // least value and its subset
+    uint32_t R;
+    uint64_t D;
+    uint64_t mask;   // the subset of least es
+    double es;
+    uint64_t rank;
+    int64_t seen;    // subsets scored
+};
+
+// the subset that exchanges the small side's keys in R and the big side's in D
+__device__ __forceinline__ uint64_t exchanged(const EnumSm &S, int ns, uint32_t R, uint64_t D)
+{
+    uint64_t A = S.K;
+    for (uint32_t w = R; w; w &= w - 1) A ^= 1ull << S.loc[__ffs(w) - 1];
+    for (uint64_t w = D; w; w &= w - 1) A ^= 1ull << S.loc[ns + __ffsll((long long)w) - 1];
+    return A;
+}
+
+// a subset that can reach es^2 = t (rare).  Once the list has overflowed only
+// values below the lane's least are looked at: returns the new limit.
+__device__ __noinline__ float sweep_hit(EnumSm &S, const float *v, int d, LaneBest &lb, int ns, uint32_t R, uint64_t D,
+                                       float val)
+{
+    if (lb.score) {
+        ++lb.seen;
+        const uint64_t A = exchanged(S, ns, R, D);
+        const double es = es_lane(S, v, d, A);
+        const uint64_t rank = colex_rank64(A);
+        if (es < lb.es || (es == lb.es && rank < lb.rank)) {
+            lb.es = es;
+            lb.rank = rank;
+            lb.mask = A;
+        }
+        return PE_TINY;
+    }
+    if (val < lb.least) {
+        lb.least = val;
+        lb.R = R;
+        lb.D = D;
+    }
+    const int q = *(volatile int *)&S.ncand > GCAP ? GCAP : atomicAdd(&S.ncand, 1);
+    if (q < GCAP) {
+        S.candR[q] = R;
+        S.candD[q] = D;
+        S.candV[q] = val;
+        return PE_TINY;
+    }
+    return lb.least;
+}
+
+// The big-side subsets U u {x}, x > max U, against the groups [g0, g1) of a
+// segment (first slot of the segment: slot0), NR subsets each but the last
+// group's.  RM = |U| (RM = -1: any, members by bit loops).  One: the segment
+// has a single group of at most 2 subsets.
+template <int RM, bool One>
+__device__ __forceinline__ void sweep_run(EnumSm &S, const float *v, int d, LaneBest &lb, float &limit, int ns, int nbg,
+                                          uint64_t U, int slot0, int g0, int g1, int nr)
+{
+    const float *C = S.C + ns * CLD + ns;  // the big side's block
+    int um[RM > 0 ? RM : 1];
+    float fU = 0.f;
+    if constexpr (RM >= 0) {
+        uint64_t w = U;
+#pragma unroll
+        for (int i = 0; i < RM; ++i) {
+            um[i] = __ffsll((long long)w) - 1;
+            w &= w - 1;
+            float f = C[um[i] * CLD + um[i]];
+#pragma unroll
+            for (int h = 0; h < i; ++h) f += C[um[i] * CLD + um[h]];
+            fU += f;
+        }
+    } else {
+        for (uint64_t w = U; w; w &= w - 1) {
+            const int y = __ffsll((long long)w) - 1;
+            float f = C[y * CLD + y];
+            for (uint64_t w2 = U & ((1ull << y) - 1ull); w2; w2 &= w2 - 1) f += C[y * CLD + __ffsll((long long)w2) - 1];
+            fU += f;
+        }
+    }
+    const int top = U ? 64 - __clzll((long long)U) : 0;
+    auto pairs = [&](int x) {  // key x alone and with U
+        float lw = C[x * CLD + x];
+        if constexpr (RM >= 0) {
+#pragma unroll
+            for (int i = 0; i < RM; ++i) lw += C[x * CLD + um[i]];
+        } else {
+            for (uint64_t w = U; w; w &= w - 1) lw += C[x * CLD + __ffsll((long long)w) - 1];
+        }
+        return lw;
+    };
+    auto members = [&](auto &&f) {
+        if constexpr (RM >= 0) {
+#pragma unroll
+            for (int i = 0; i < RM; ++i) f(um[i]);
+        } else {
+            for (uint64_t w = U; w; w &= w - 1) f(__ffsll((long long)w) - 1);
+        }
+    };
+    // the key run upwards is taken NX values at a time: independent chains
+    if constexpr (One) {
+        constexpr int NX = 2;
+        for (int c = 0; c < nr; ++c) {
+            const float *W = S.W + (slot0 / PE_CH) * nbg * PE_CH + c;
+            float base = S.rbase[slot0 + c] + fU;
+            members([&](int y) { base += W[y * PE_CH]; });
+            for (int x = top; x < nbg; x += NX) {
+                float val[NX];
+#pragma unroll
+                for (int h = 0; h < NX; ++h) {
+                    const int xh = min(x + h, nbg - 1);
+                    val[h] = base + (pairs(xh) + W[xh * PE_CH]);
+                    if (x + h >= nbg) val[h] = INFINITY;
+                }
+                if (fminf(val[0], val[1]) <= limit) {
+#pragma unroll
+                    for (int h = 0; h < NX; ++h)
+                        if (val[h] <= limit)
+                            limit = sweep_hit(S, v, d, lb, ns, S.rmask[slot0 + c], U | (1ull << (x + h)), val[h]);
+                }
             }
-            const float num_lo = fmaxf(g2 - Eabs, 0.f), num_hi = g2 + Eabs;
-            const float pl = pa + pe, ph = pa - pe;
-            const float lower = num_lo / (pl * pl) * (1.f - 1e-6f);
-            const float upper = ph > 0.f ? num_hi / (ph * ph) * (1.f + 1e-6f) : INFINITY;
-            f(om | (1ull << x), lower, upper);
         }
-        if (q >= hi) return;
-        c[0] = lim - 1;
-        if (!colex_next(c, m, P)) return;
+    } else {
+        constexpr int NX = 1;
+        for (int g = g0; g < g1; ++g) {
+            const int slot = slot0 + g * PE_CH;
+            const float *W = S.W + (slot / PE_CH) * nbg * PE_CH;
+            float base[PE_CH];
+#pragma unroll
+            for (int c = 0; c < PE_CH; ++c) base[c] = S.rbase[slot + c] + fU;
+            members([&](int y) {
+                const float4 wa = *reinterpret_cast<const float4 *>(W + y * PE_CH);
+                const float4 wb = *reinterpret_cast<const float4 *>(W + y * PE_CH + 4);
+                base[0] += wa.x, base[1] += wa.y, base[2] += wa.z, base[3] += wa.w;
+                base[4] += wb.x, base[5] += wb.y, base[6] += wb.z, base[7] += wb.w;
+            });
+            for (int x = top; x < nbg; x += NX) {
+                float val[NX][PE_CH], mn = INFINITY;
+#pragma unroll
+                for (int h = 0; h < NX; ++h) {
+                    const int xh = min(x + h, nbg - 1);
+                    const float lw = x + h < nbg ? pairs(xh) : INFINITY;
+                    const float4 wa = *reinterpret_cast<const float4 *>(W + xh * PE_CH);
+                    const float4 wb = *reinterpret_cast<const float4 *>(W + xh * PE_CH + 4);
+                    val[h][0] = base[0] + (lw + wa.x), val[h][1] = base[1] + (lw + wa.y);
+                    val[h][2] = base[2] + (lw + wa.z), val[h][3] = base[3] + (lw + wa.w);
+                    val[h][4] = base[4] + (lw + wb.x), val[h][5] = base[5] + (lw + wb.y);
+                    val[h][6] = base[6] + (lw + wb.z), val[h][7] = base[7] + (lw + wb.w);
+                    mn = fminf(mn, fminf(fminf(fminf(val[h][0], val[h][1]), fminf(val[h][2], val[h][3])),
+                                         fminf(fminf(val[h][4], val[h][5]), fminf(val[h][6], val[h][7]))));
+                }
+                if (mn <= limit) {
+#pragma unroll
+                    for (int h = 0; h < NX; ++h)
+#pragma unroll
+                        for (int c = 0; c < PE_CH; ++c)
+                            if (val[h][c] <= limit)
+                                limit = sweep_hit(S, v, d, lb, ns, S.rmask[slot + c], U | (1ull << (x + h)), val[h][c]);
+                }
+            }
+        }
     }
 }
 
-template <int DPL, typename VT>
-__global__ void __launch_bounds__(PE_W * 32) k_pool_enum(PoolArgs a)
+template <bool One>
+__device__ __forceinline__ void sweep_u(EnumSm &S, const float *v, int d, LaneBest &lb, float &limit, int ns, int nbg,
+                                        int r, uint64_t U, int slot0, int g0, int g1, int nr)
+{
+    switch (r) {
+    case 1: sweep_run<0, One>(S, v, d, lb, limit, ns, nbg, U, slot0, g0, g1, nr); break;
+    case 2: sweep_run<1, One>(S, v, d, lb, limit, ns, nbg, U, slot0, g0, g1, nr); break;
+    case 3: sweep_run<2, One>(S, v, d, lb, limit, ns, nbg, U, slot0, g0, g1, nr); break;
+    case 4: sweep_run<3, One>(S, v, d, lb, limit, ns, nbg, U, slot0, g0, g1, nr); break;
+    case 5: sweep_run<4, One>(S, v, d, lb, limit, ns, nbg, U, slot0, g0, g1, nr); break;
+    case 6: sweep_run<5, One>(S, v, d, lb, limit, ns, nbg, U, slot0, g0, g1, nr); break;
+    case 7: sweep_run<6, One>(S, v, d, lb, limit, ns, nbg, U, slot0, g0, g1, nr); break;
+    case 8: sweep_run<7, One>(S, v, d, lb, limit, ns, nbg, U, slot0, g0, g1, nr); break;
+    default: sweep_run<-1, One>(S, v, d, lb, limit, ns, nbg, U, slot0, g0, g1, nr); break;
+    }
+}
+
+// every exchange of r = 1 .. ns keys (all threads of the block)
+__device__ __noinline__ void sweep(EnumSm &S, const float *v, int d, LaneBest &lb, int ns, int nbg, float base0)
+{
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    float limit = PE_TINY;  // values up to this are hits
+    const int room = min(PE_GMAX, PE_WCAP / (nbg * PE_CH));
+    if (tid == 0) {
+        S.next_r = 1;
+        S.next_g = 0;
+    }
+    for (;;) {
+        __syncthreads();
+        // ---- the next batch of groups
+        if (tid == 0) {
+            int n = 0, left = room, r = S.next_r, g = S.next_g;
+            while (r <= ns && left > 0) {
+                const int64_t ng = (int64_t)((cb(ns, r) + PE_CH - 1) / PE_CH);
+                const int take = (int)min((int64_t)left, ng - g);
+                S.seg_r[n] = r;
+                S.seg_g[n] = g;
+                S.seg_n[n] = take;
+                ++n;
+                left -= take;
+                g += take;
+                if (g >= ng) {
+                    ++r;
+                    g = 0;
+                }
+            }
+            S.task = 0u;
+            S.nseg = n;
+            S.next_r = r;
+            S.next_g = g;
+        }
+        __syncthreads();
+        const int nseg = S.nseg;
+        if (nseg == 0) return;
+        int slots = 0;
+        for (int i = 0; i < nseg; ++i) slots += S.seg_n[i] * PE_CH;
+        for (int e = tid; e < slots; e += PE_T) {
+            int i = 0, rel = e;
+            while (rel >= S.seg_n[i] * PE_CH) rel -= S.seg_n[i++] * PE_CH;
+            const int r = S.seg_r[i];
+            const uint64_t rank = (uint64_t)S.seg_g[i] * PE_CH + rel;
+            uint32_t Rm = 0;
+            float f = INFINITY;
+            if (rank < cbl(ns, r)) {
+                Rm = (uint32_t)colex_unrank(rank, r, ns);
+                f = base0;
+                for (uint32_t w = Rm; w; w &= w - 1) {
+                    const int x = __ffs(w) - 1;
+                    f += S.C[x * CLD + x];
+                    for (uint32_t w2 = Rm & ((1u << x) - 1u); w2; w2 &= w2 - 1) f += S.C[x * CLD + __ffs(w2) - 1];
+                }
+            }
+            S.rmask[e] = Rm;
+            S.rbase[e] = f;
+        }
+        __syncthreads();
+        for (int e = tid; e < slots * nbg; e += PE_T) {  // e = (group, y, c)
+            const int c = e % PE_CH, gy = e / PE_CH, g = gy / nbg, y = gy - g * nbg;
+            float f = 0.f;
+            for (uint32_t w = S.rmask[g * PE_CH + c]; w; w &= w - 1) f += S.C[(__ffs(w) - 1) * CLD + ns + y];
+            S.W[e] = f;
+        }
+        __syncthreads();
+        // ---- tasks (segment, 32 subsets U, PE_GSPLIT groups), taken by the warps as they finish
+        uint64_t tfirst = 0;
+        uint32_t t = 0;
+        int slot0 = 0;
+        if (lane == 0) t = atomicAdd(&S.task, 1u);
+        t = __shfl_sync(FW_FULL, t, 0);
+        for (int i = 0; i < nseg; ++i) {
+            const int r = S.seg_r[i], ng = S.seg_n[i];
+            const uint64_t NR = cb(ns, r), NU = cb(nbg - 1, r - 1);
+            const bool one = NR <= 2;
+            const int nsp = (ng + PE_GSPLIT - 1) / PE_GSPLIT;
+            const uint64_t nt = (NU + 31) / 32 * nsp;
+            while (t < tfirst + nt) {
+                const uint64_t q = t - tfirst, ub = q / nsp, u = ub * 32 + lane;
+                const int g0 = (int)(q - ub * nsp) * PE_GSPLIT, g1 = min(ng, g0 + PE_GSPLIT);
+                if (u < NU) {
+                    const uint64_t U = r > 1 ? colex_unrank(u, r - 1, nbg - 1) : 0;
+                    if (one) sweep_u<true>(S, v, d, lb, limit, ns, nbg, r, U, slot0, g0, g1, (int)NR);
+                    else sweep_u<false>(S, v, d, lb, limit, ns, nbg, r, U, slot0, g0, g1, 0);
+                }
+                __syncwarp();
+                if (lane == 0) t = atomicAdd(&S.task, 1u);
+                t = __shfl_sync(FW_FULL, t, 0);
+            }
+            tfirst += nt;
+            slot0 += ng * PE_CH;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
-    constexpr int d = DPL * 32;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    EnumSm &S = reinterpret_cast<EnumSm *>(smraw)[wid];
-    const int64_t wslot = (int64_t)blockIdx.x * PE_W + wid;
-    uint64_t *gc = a.gcand + wslot * GCAP;
-    double *g64 = a.g64 + wslot * (PMAX * PMAX);
+    EnumSm &S = *reinterpret_cast<EnumSm *>(smraw);
+    float *v = reinterpret_cast<float *>(smraw + (sizeof(EnumSm) + 15) / 16 * 16);  // [PMAX][d + 4]
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int d = a.R.d, ld = d + 4;
+    const bool bf16 = a.R.v_dtype == FW_BF16;
     const int64_t items = a.R.rows * a.nb;
-    for (int64_t it = (int64_t)blockIdx.x * PE_W + wid; it < items; it += (int64_t)gridDim.x * PE_W) {
+    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
         const int64_t r = it / a.nb;
         const int64_t g = r / a.R.R;
         const int n = a.R.n[g];
         const float *l = a.R.logits + a.R.logit_off[g] + (r - g * a.R.R) * n;
-        const VT *V = static_cast<const VT *>(a.R.v) + a.R.v_off[g];
+        const int64_t voff = a.R.v_off[g];
         const float M = a.M[r], Zi = 1.f / a.Z[r];
         const int s = a.k[it];
         const int P = a.pool_n[it];
         int32_t *bi = a.best_idx + it * a.k_max;
-        const bool direct = s <= P - s;
-        const int m = direct ? s : P - s;
         // refused items: an out-of-range budget (P = -1), a pool over PMAX keys
         // (P = -2), or more subsets than the enumeration takes
         int refuse = P == -1 ? FW_ERR_INVALID_ARG : (P < 0 ? FW_ERR_UNSUPPORTED : 0);
         if (!refuse && P < s) refuse = FW_ERR_INVALID_ARG;  // thresholds that keep fewer than s keys
-        const uint64_t T = refuse ? 0 : cb(P, m);
-        if (!refuse && T > PE_MAX_SUBSETS) refuse = FW_ERR_UNSUPPORTED;
+        if (!refuse && cb(P, min(s, P - s)) > PE_MAX_SUBSETS) refuse = FW_ERR_UNSUPPORTED;
         if (refuse) {
-            if (lane == 0) {
+            if (tid == 0) {
                 if (a.row_status) atomicMax(a.row_status + r, refuse);
                 a.best_gap[it] = __int_as_float(0x7fc00000);
                 if (a.topk_gap) a.topk_gap[it] = __int_as_float(0x7fc00000);
                 if (a.n_cand) a.n_cand[it] = 0;
             }
-            for (int q = lane; q < a.k_max; q += 32) bi[q] = -1;
+            for (int q = tid; q < a.k_max; q += PE_T) bi[q] = -1;
             continue;
         }
-        float ol[DPL];
-#pragma unroll
-        for (int c = 0; c < DPL; ++c) ol[c] = a.o[r * d + lane * DPL + c];
-        for (int q = lane; q < P; q += 32) {
-            const int j = a.pool[it * PMAX + q];
-            S.pidx[q] = j;
-            S.pp[q] = __expf(__ldg(l + j) - M) * Zi;
+        __syncthreads();  // the previous item's state is no longer read
+        if (wid < 2) {  // masses; the kept keys by the thresholds
+            const int x = tid;
+            bool kept = false;
+            float p = 0.f;
+            if (x < P) {
+                const int j = a.pool[it * PMAX + x];
+                const float lj = __ldg(l + j);
+                S.pidx[x] = j;
+                p = __expf(lj - M) * Zi;
+                const uint32_t kl = order_key(lj), tk = a.thr_key[it];
+                kept = kl > tk || (kl == tk && j <= a.thr_idx[it]);
+            }
+            S.pp[x] = p;
+            const uint32_t bal = __ballot_sync(FW_FULL, kept);
+            if (lane == 0) reinterpret_cast<uint32_t *>(&S.topK)[wid] = bal;
         }
-        if (lane == 0) S.ncand = 0;
-        __syncwarp();
-        // Gram matrix of u = p (v - o) in fp64 (the warp forms each product
-        // across d): the fp64 copy for the re-scoring, its fp32 rounding for
-        // the walk
-        for (int x = 0; x < P; ++x) {
-            float vx[DPL];
-            load_row_part<DPL, VT>(V, S.pidx[x], lane, vx);
-            double dx[DPL];
-#pragma unroll
-            for (int c = 0; c < DPL; ++c) dx[c] = (double)vx[c] - (double)ol[c];
-            for (int y = x; y < P; ++y) {
-                float vy[DPL];
-                load_row_part<DPL, VT>(V, S.pidx[y], lane, vy);
-                double acc = 0.0;
-#pragma unroll
-                for (int c = 0; c < DPL; ++c) acc = fma(dx[c], (double)vy[c] - (double)ol[c], acc);
-                acc = warp_sum_d(acc) * (double)S.pp[x] * (double)S.pp[y];
+        for (int c = tid; c < d; c += PE_T) S.o[c] = a.o[r * d + c];
+        __syncthreads();
+        // ---- value rows (zeros past P in the last pair of rows), 4 columns per thread and step
+        for (int e = tid; e < ((P + 1) & ~1) * (d / 4); e += PE_T) {
+            const int x = e / (d / 4), c = (e - x * (d / 4)) * 4;
+            float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (x < P) {
+                const int64_t i = voff + (int64_t)S.pidx[x] * d + c;
+                if (bf16) {
+                    const uint2 h = __ldg(reinterpret_cast<const uint2 *>(static_cast<const uint16_t *>(a.R.v) + i));
+                    u = make_float4(__uint_as_float(h.x << 16), __uint_as_float(h.x & 0xffff0000u),
+                                    __uint_as_float(h.y << 16), __uint_as_float(h.y & 0xffff0000u));
+                } else {
+                    u = __ldg(reinterpret_cast<const float4 *>(static_cast<const float *>(a.R.v) + i));
+                }
+            }
+            *reinterpret_cast<float4 *>(v + x * ld + c) = u;
+        }
+        __syncthreads();
+        // ---- G in fp32: 2 x 2 keys per thread and step, four partial sums per entry
+        {
+            const int P2 = (P + 1) / 2, nt = P2 * (P2 + 1) / 2;
+            for (int i = tid; i < nt; i += PE_T) {
+                int x = (int)((sqrtf(8.f * (float)i + 1.f) - 1.f) * 0.5f);
+                while (x * (x + 1) / 2 > i) --x;
+                while ((x + 1) * (x + 2) / 2 <= i) ++x;
+                const int y = i - x * (x + 1) / 2;
+                const float *x0 = v + 2 * x * ld, *y0 = v + 2 * y * ld;
+                float4 s00{}, s01{}, s10{}, s11{};
+                for (int c = 0; c < d; c += 4) {
+                    const float4 o4 = *reinterpret_cast<const float4 *>(S.o + c);
+                    auto diff = [&](const float *q) {
+                        const float4 u = *reinterpret_cast<const float4 *>(q);
+                        return make_float4(u.x - o4.x, u.y - o4.y, u.z - o4.z, u.w - o4.w);
+                    };
+                    const float4 xa = diff(x0 + c), xb = diff(x0 + ld + c), ya = diff(y0 + c), yb = diff(y0 + ld + c);
+                    auto mac = [](float4 &s, const float4 &p, const float4 &q) {
+                        s.x = fmaf(p.x, q.x, s.x), s.y = fmaf(p.y, q.y, s.y);
+                        s.z = fmaf(p.z, q.z, s.z), s.w = fmaf(p.w, q.w, s.w);
+                    };
+                    mac(s00, xa, ya), mac(s01, xa, yb), mac(s10, xb, ya), mac(s11, xb, yb);
+                }
+                auto put = [&](int p, int q, const float4 &s4) {
+                    if (p >= P || q >= P) return;
+                    const float w = ((s4.x + s4.y) + (s4.z + s4.w)) * (S.pp[p] * S.pp[q]);
+                    S.G[p * CLD + q] = S.G[q * CLD + p] = w;
+                };
+                put(2 * x, 2 * y, s00), put(2 * x + 1, 2 * y, s10), put(2 * x + 1, 2 * y + 1, s11);
+                if (x != y) put(2 * x, 2 * y + 1, s01);
+            }
+        }
+        const uint64_t topK = S.topK;
+        // the set exchanged from: the top-mass set (s keys also where the
+        // caller's thresholds keep another count)
+        uint64_t K = __popcll(topK) == s ? topK : (1ull << s) - 1ull;
+        const bool ksmall = s <= P - s;  // the smaller side: K or the keys outside it
+        const int ns = ksmall ? s : P - s, nbg = P - ns;
+        // roundings: the table sums' chains, and the entries' own (fp32 G)
+        const float kappa = (float)(ns * (ns + 1) / 2 + 2 * ns + 10 + d / 4 + 12) * 1.5f * 5.9604645e-8f;
+        int64_t ncand = 1;
+        // the block's subset of least value (every thread)
+        auto least_of = [&](LaneBest &lb) -> uint64_t {
+            uint64_t mk = lb.least < INFINITY ? exchanged(S, ns, lb.R, lb.D) : ~0ull;
+            for (int o = 16; o; o >>= 1) {
+                const float v2 = __shfl_xor_sync(FW_FULL, lb.least, o);
+                const uint64_t om = __shfl_xor_sync(FW_FULL, mk, o);
+                if (v2 < lb.least || (v2 == lb.least && om < mk)) {
+                    lb.least = v2;
+                    mk = om;
+                }
+            }
+            __syncthreads();
+            if (lane == 0) {
+                S.red_v[wid] = lb.least;
+                S.red_mask[wid] = mk;
+            }
+            __syncthreads();
+            for (int w = 0; w < PE_NW; ++w)
+                if (S.red_v[w] < lb.least || (S.red_v[w] == lb.least && S.red_mask[w] < mk)) {
+                    lb.least = S.red_v[w];
+                    mk = S.red_mask[w];
+                }
+            return mk;
+        };
+        // (fp64 runs at 1/60 of fp32's rate here: scalars in fp64 are one thread's work)
+        for (int round = 0;; ++round) {
+            // ---- sum_K u
+            for (int c = tid; c < d; c += PE_T) {
+                double uc[1];
+                col_sums<1>(S, v, d, K, c, 1, uc);
+                const df u = df_from_double(uc[0]);
+                S.UKh[c] = u.hi;
+                S.UKl[c] = u.lo;
+            }
+            if (tid < P) {  // table order: the smaller side's keys first
+                const bool kept = (K >> tid) & 1ull;
+                const int i = __popcll((kept ? K : ~K) & ((1ull << tid) - 1ull));
+                S.loc[kept == ksmall ? i : ns + i] = tid;
+            }
+            __syncthreads();
+            if (wid == 0) {  // es(K), and the best set so far
+                double q = 0.0;
+                for (int c = lane; c < d; c += 32) {  // (es_warp's order)
+                    const double u = (double)S.UKh[c] + (double)S.UKl[c];
+                    q = fma(u, u, q);
+                }
+                q = warp_sum_d(q);
+                const double pk = mass_warp(S, K, lane);
                 if (lane == 0) {
-                    S.G[x * GLD + y] = S.G[y * GLD + x] = (float)acc;
-                    g64[x * PMAX + y] = g64[y * PMAX + x] = acc;
+                    const double ek = sqrt(q) / pk;
+                    const uint64_t krank = colex_rank64(K);
+                    if (round == 0) S.stale = 0;
+                    else S.stale = ek < S.bes ? 0 : S.stale + 1;
+                    if (round == 0 || ek < S.bes || (ek == S.bes && krank < S.brank)) {
+                        S.bes = ek;
+                        S.bmask = K;
+                        S.brank = krank;
+                    }
+                    S.QK = q;
+                    S.PK = pk;
+                    S.K = K;
+                    S.ncand = S.nsurv = 0;
+                    if (round == 0 && a.topk_gap && topK == K) a.topk_gap[it] = (float)ek;
                 }
             }
-        }
-        __syncwarp();
-        float S1 = 0.f;
-        for (int x = lane; x < P; x += 32) {
-            float sx = 0.f;
-            for (int y = 0; y < P; ++y) sx += S.G[x * GLD + y];
-            S.t[x] = sx;
-            S1 += sqrtf(fmaxf(S.G[x * GLD + x], 0.f));
-        }
-        __syncwarp();
-        float UU = 0.f, PU = 0.f;
-        for (int x = lane; x < P; x += 32) {
-            UU += S.t[x];
-            PU += S.pp[x];
-        }
-        UU = warp_sum(UU);
-        PU = warp_sum(PU);
-        S1 = warp_sum(S1) * 1.0001f;
-        // Rounding bound: every Gram entry, partial sum and t_x is bounded by
-        // S1^2 (|G_xy| <= |u_x||u_y|); the products carry <= DPL + 8 roundings,
-        // the score's chains <= 2P + m^2 + 2m more; twice that for safety.
-        const float Eabs = (float)(2 * DPL + 32 + 4 * P + 2 * m * m + 4 * m) * 5.9604645e-8f * S1 * S1;
-        const float pe = (float)(2 * P + 2 * m + 8) * 5.9604645e-8f * PU;
-        // lane ranges of colex ranks
-        const uint64_t qn = T / 32, rm = T % 32;
-        uint64_t lo = qn * lane + min((uint64_t)lane, rm);
-        const uint64_t hi = lo + qn + ((uint64_t)lane < rm ? 1 : 0);
-        const uint64_t all = P == 64 ? ~0ull : ((1ull << P) - 1ull);
-        // pass 1: the least upper end (m = 0: the pool itself is the only subset)
-        float U = INFINITY;
-        if (m == 0) lo = hi;
-        walk(S, P, m, direct, lo, hi, UU, PU, Eabs, pe, [&](uint64_t, float, float up) { U = fminf(U, up); });
-        U = warp_min(U);
-        // pass 2: buffer every subset whose interval reaches down to U
-        int over = 0;
-        int64_t ncand = 0;
-        walk(S, P, m, direct, lo, hi, UU, PU, Eabs, pe, [&](uint64_t Cm, float low, float) {
-            if (low <= U) {
-                ++ncand;
-                const int slot = atomicAdd(&S.ncand, 1);
-                if (slot < GCAP) gc[slot] = direct ? Cm : (all & ~Cm);
-                else over = 1;
-            }
-        });
-        __syncwarp();
-        over = __any_sync(FW_FULL, over);
-        double bes = INFINITY;
-        uint64_t brank = ~0ull, bmask = 0;
-        if (m == 0) {
-            // the pool is the kept set itself: one subset
-            bmask = all;
-            bes = es_warp<DPL, VT>(V, ol, S, all, lane);
-        } else if (!over) {
-            const int nc = S.ncand;
-            for (int q = 0; q < nc; ++q) {
-                const uint64_t A = gc[q];
-                const double es = es_gram_warp(g64, S, A, lane);
-                const uint64_t rank = colex_rank64(A);
-                if (es < bes || (es == bes && rank < brank)) {
-                    bes = es;
-                    brank = rank;
-                    bmask = A;
+            // its products with the pool: four lanes per key
+            for (int x = tid >> 2; x < P; x += PE_T / 4) {
+                float hi = 0.f, lo = 0.f;
+                for (int c = tid & 3; c < d; c += 4) {
+                    const df u = df_two_sum(v[x * ld + c], -S.o[c]);
+                    const float kh = S.UKh[c], kl = S.UKl[c];
+                    const float q = u.hi * kh;
+                    const float e = fmaf(u.lo, kh, fmaf(u.hi, kl, fmaf(u.hi, kh, -q)));
+                    const df t = df_two_sum(hi, q);
+                    hi = t.hi;
+                    lo += t.lo + e;
+                }
+                df q{hi, lo};
+                const uint32_t quad = 0xfu << (lane & 28);
+#pragma unroll
+                for (int o = 1; o < 4; o <<= 1) {
+                    const df q2{__shfl_xor_sync(quad, q.hi, o), __shfl_xor_sync(quad, q.lo, o)};
+                    q = df_add(q, q2);
+                }
+                if ((tid & 3) == 0) {
+                    S.gh[x] = q.hi;
+                    S.gl[x] = q.lo;
                 }
             }
-        } else {
-            // every lane re-scores its own candidates alone
-            walk(S, P, m, direct, lo, hi, UU, PU, Eabs, pe, [&](uint64_t Cm, float low, float) {
-                if (low <= U) {
-                    const uint64_t A = direct ? Cm : (all & ~Cm);
-                    const double es = es_gram_lane(g64, S, A);
-                    const uint64_t rank = colex_rank64(A);
-                    if (es < bes || (es == bes && rank < brank)) {
-                        bes = es;
-                        brank = rank;
-                        bmask = A;
+            __syncthreads();
+            if (round == 0 && a.topk_gap && topK != K && wid == 0) {
+                const double te = es_warp(S, v, d, topK, lane);
+                if (lane == 0) a.topk_gap[it] = (float)te;
+            }
+            if (ns == 0) break;
+            // ---- the tables, scaled by a power of two that brings the largest a_x^2 near 1
+            const float tf = (float)S.bes * (float)S.bes;
+            float amax = 0.f;
+            for (int x = lane; x < P; x += 32) amax = fmaxf(amax, S.G[x * CLD + x] + tf * S.pp[x] * S.pp[x]);
+            amax = warp_max(amax);
+            // (vectors that are all zero, subnormal or beyond fp32's range: no
+            // value decides anything, every subset is a hit)
+            const bool blind = !(amax > 1e-30f && amax < 1e30f);
+            const float sc = blind ? 1.f : scalbnf(1.f, -ilogbf(amax));
+            if (tid < P) {
+                const float st = sqrtf(tf * sc) * 1.00001f;
+                S.ax[tid] = sqrtf(S.G[tid * CLD + tid] * sc) * 1.00001f + st * S.pp[tid];
+                // h_x = u_x . sum_K u - t p_x p(K), kept in the slot of the double-float product
+                const double t = S.bes * S.bes;
+                S.gh[tid] = (float)(((double)S.gh[tid] + (double)S.gl[tid] - t * S.PK) * (double)S.pp[tid] * (double)sc);
+                if (tid == 0) {
+                    S.red_v[0] = (float)((S.QK - t * S.PK * S.PK) * (double)sc);
+                    S.red_v[1] = (sqrtf((float)(S.QK * (double)sc)) + st * (float)S.PK) * 1.00001f;
+                    S.red_v[2] = (float)(t * (double)sc);
+                }
+            }
+            __syncthreads();
+            const float c0 = S.red_v[0], b0 = S.red_v[1], ts = S.red_v[2];
+            const float base0 = blind ? -1.f : c0 - kappa * fabsf(c0);
+            for (int i = wid; i < P; i += PE_NW) {
+                const int x = S.loc[i];
+                const float ax = S.ax[x], px = S.pp[x];
+                for (int j = lane; j <= i; j += 32) {
+                    const int y = S.loc[j];
+                    const float H = S.G[x * CLD + y] * sc - ts * px * S.pp[y];
+                    float w;
+                    if (i == j) w = H + ((i < ns) == ksmall ? -2.f : 2.f) * S.gh[x] - kappa * ax * (ax + 2.f * b0);
+                    else w = ((i < ns) == (j < ns) ? 2.f : -2.f) * H - 2.f * kappa * ax * S.ax[y];
+                    S.C[i * CLD + j] = S.C[j * CLD + i] = blind ? 0.f : w;
+                }
+            }
+            const bool score = round >= PE_SWEEPS;
+            LaneBest lb;
+            lb.score = score;
+            lb.least = INFINITY;
+            lb.R = 0;
+            lb.D = 0;
+            lb.mask = S.bmask;
+            lb.rank = S.brank;
+            lb.es = INFINITY;
+            lb.seen = 0;
+            if (score) lb.es = es_lane(S, v, d, lb.mask);  // (by the operations the lanes use)
+            sweep(S, v, d, lb, ns, nbg, base0);  // (begins and ends with block barriers)
+            if (score) {
+                int64_t seen = lb.seen;
+                for (int o = 16; o; o >>= 1) {
+                    seen += __shfl_xor_sync(FW_FULL, seen, o);
+                    const double oe = __shfl_xor_sync(FW_FULL, lb.es, o);
+                    const uint64_t orank = __shfl_xor_sync(FW_FULL, lb.rank, o);
+                    const uint64_t om = __shfl_xor_sync(FW_FULL, lb.mask, o);
+                    if (oe < lb.es || (oe == lb.es && orank < lb.rank)) {
+                        lb.es = oe;
+                        lb.rank = orank;
+                        lb.mask = om;
                     }
                 }
-            });
-            for (int off = 16; off; off >>= 1) {
-                const double oe = __shfl_xor_sync(FW_FULL, bes, off);
-                const uint64_t orank = __shfl_xor_sync(FW_FULL, brank, off);
-                const uint64_t omask = __shfl_xor_sync(FW_FULL, bmask, off);
-                if (oe < bes || (oe == bes && orank < brank)) {
-                    bes = oe;
-                    brank = orank;
-                    bmask = omask;
+                if (lane == 0) {
+                    S.red_es[wid] = lb.es;
+                    S.red_rank[wid] = lb.rank;
+                    S.red_mask[wid] = lb.mask;
+                    S.red_seen[wid] = seen;
+                }
+                __syncthreads();
+                ncand = 1;
+                for (int w = 0; w < PE_NW; ++w) ncand += S.red_seen[w];
+                if (tid == 0) S.bes = INFINITY;  // (the warps' include it)
+                break;
+            }
+            if (S.ncand > GCAP) {  // (uniform)
+                // again around the subset of least value; when three rounds brought
+                // no better es the values decide nothing more
+                const uint64_t mk = least_of(lb);
+                if (S.stale >= 3 || mk == K) round = PE_SWEEPS - 1;
+                K = mk;
+                __syncthreads();  // the state above is no longer read
+                continue;
+            }
+            // ---- each hit's interval of es^2 - t: [v, v + 2 bound] / p(A)^2
+            const int seen = S.ncand;
+            constexpr int PER = (GCAP + PE_T - 1) / PE_T;
+            float up = 0.f;
+            float myl[PER];
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const int i = tid + q * PE_T;
+                myl[q] = INFINITY;
+                if (i >= seen) continue;
+                double pr = 0.0, pd = 0.0;
+                float e = 0.f;
+                for (uint32_t w = S.candR[i]; w; w &= w - 1) {
+                    const int x = S.loc[__ffs(w) - 1];
+                    pr += (double)S.pp[x];
+                    e += S.ax[x];
+                }
+                for (uint64_t w = S.candD[i]; w; w &= w - 1) {
+                    const int x = S.loc[ns + __ffsll((long long)w) - 1];
+                    pd += (double)S.pp[x];
+                    e += S.ax[x];
+                }
+                const double pa = S.PK + (ksmall ? pd - pr : pr - pd);
+                // masses that cancel to nothing leave the hit to the exact score
+                const float p2 = !blind && pa > 1e-9 * (pr + pd) ? (float)(pa * pa) : 0.f;
+                const float lov = S.candV[i];
+                const float upv = lov + 2.f * kappa * (e * (e + 2.f * b0) + fabsf(c0)) * 1.001f + 2.f * PE_TINY;
+                myl[q] = p2 > 0.f ? (lov - 1e-5f * fabsf(lov)) / p2 : -INFINITY;
+                if (p2 > 0.f) up = fminf(up, (upv + 1e-5f * fabsf(upv)) / p2);
+            }
+            up = warp_min(up);
+            if (lane == 0) S.red_v[wid] = up;
+            __syncthreads();
+            for (int w = 0; w < PE_NW; ++w) up = fminf(up, S.red_v[w]);
+            // the survivors' subsets in place of their hits, then a list of them
+            uint32_t keep = 0;
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const int i = tid + q * PE_T;
+                if (i < seen && myl[q] <= up) {
+                    S.candD[i] = exchanged(S, ns, S.candR[i], S.candD[i]);
+                    keep |= 1u << q;
                 }
             }
-        }
-        // the top-mass set: the pool's kept keys
-        uint64_t K = 0;
-        {
-            const uint32_t tk = a.thr_key[it];
-            const int ti = a.thr_idx[it];
-            for (int x = lane; x < P; x += 32) {
-                const uint32_t kl = order_key(__ldg(l + S.pidx[x]));
-                if (kl > tk || (kl == tk && S.pidx[x] <= ti)) K |= 1ull << x;
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < PER; ++q)
+                if ((keep >> q) & 1u) S.candR[atomicAdd(&S.nsurv, 1)] = (uint32_t)(tid + q * PE_T);
+            __syncthreads();
+            const int nsv = S.nsurv;
+            if (nsv > PE_SURV && round < 2 && !blind) {  // the values around K do not tell them apart
+                const uint64_t mk = least_of(lb);
+                if (mk != K) {
+                    K = mk;
+                    __syncthreads();
+                    continue;
+                }
             }
-            for (int off = 16; off; off >>= 1) K |= __shfl_xor_sync(FW_FULL, K, off);
+            ncand = nsv + 1;
+            double wes = INFINITY;
+            uint64_t wrank = ~0ull, wmask = 0;
+            for (int q = wid; q < nsv; q += PE_NW) {
+                const uint64_t A = S.candD[S.candR[q]];
+                const double es = es_warp(S, v, d, A, lane);
+                const uint64_t rank = colex_rank64(A);
+                if (es < wes || (es == wes && rank < wrank)) {
+                    wes = es;
+                    wrank = rank;
+                    wmask = A;
+                }
+            }
+            if (lane == 0) {
+                S.red_es[wid] = wes;
+                S.red_rank[wid] = wrank;
+                S.red_mask[wid] = wmask;
+            }
+            break;
         }
-        const double tes = a.topk_gap ? es_warp<DPL, VT>(V, ol, S, K, lane) : 0.0;
-        ncand = (int64_t)warp_sum_d((double)ncand);
-        if (lane == 0) {
-            a.best_gap[it] = (float)bes;
-            if (a.topk_gap) a.topk_gap[it] = (float)tes;
+        __syncthreads();
+        if (tid == 0) {
+            if (ns > 0)
+                for (int w = 0; w < PE_NW; ++w)
+                    if (S.red_es[w] < S.bes || (S.red_es[w] == S.bes && S.red_rank[w] < S.brank)) {
+                        S.bes = S.red_es[w];
+                        S.brank = S.red_rank[w];
+                        S.bmask = S.red_mask[w];
+                    }
+            a.best_gap[it] = (float)S.bes;
             if (a.n_cand) a.n_cand[it] = ncand;
         }
-        bmask = __shfl_sync(FW_FULL, bmask, 0);
-        for (int x = lane; x < P; x += 32)
-            if ((bmask >> x) & 1ull) bi[__popcll(bmask & ((1ull << x) - 1ull))] = S.pidx[x];
-        for (int q = s + lane; q < a.k_max; q += 32) bi[q] = -1;
-        __syncwarp();
+        __syncthreads();
+        const uint64_t bmask = S.bmask;
+        if (tid < P && ((bmask >> tid) & 1ull)) bi[__popcll(bmask & ((1ull << tid) - 1ull))] = S.pidx[tid];
+        for (int q = s + tid; q < a.k_max; q += PE_T) bi[q] = -1;
     }
 }
 
@@ -608,24 +1099,9 @@ __global__ void __launch_bounds__(PE_W * 32) k_pool_enum(PoolArgs a)
 
 static size_t pool_bytes(const RowsDev &R, int nb) { return align256((size_t)R.rows * nb * PMAX * 4); }
 
-// blocks of the enumeration launch: PE_BPS per SM, fewer when there are fewer items
-static int64_t pool_enum_blocks(const RowsDev &R, int nb)
-{
-    int sms = 0;
-    if (device_sms(&sms) != FW_OK) sms = 152;  // no device: the size query still answers
-    const int64_t items = R.rows * nb;
-    return std::max<int64_t>(1, std::min<int64_t>((items + PE_W - 1) / PE_W, (int64_t)sms * PE_BPS));
-}
-
-// per warp of the enumeration launch: the candidate buffer and the fp64 Gram matrix
-static size_t warp_ws_bytes(const RowsDev &R, int nb)
-{
-    return align256((size_t)pool_enum_blocks(R, nb) * PE_W * (GCAP + PMAX * PMAX) * 8);
-}
-
 size_t pool_best_subset_workspace(const RowsDev &R, int nb)
 {
-    return pool_bytes(R, nb) + align256((size_t)R.rows * nb * 4) + warp_ws_bytes(R, nb);
+    return pool_bytes(R, nb) + align256((size_t)R.rows * nb * 4);
 }
 
 fw_status pool_best_subset(const RowsDev &R, const int32_t *k, int nb, const int32_t *E, const fw_gap_out &topk,
@@ -645,11 +1121,6 @@ fw_status pool_best_subset(const RowsDev &R, const int32_t *k, int nb, const int
     a.Z = topk.row_sum;
     a.pool = (int32_t *)ws;
     a.pool_n = (int32_t *)((char *)ws + pool_bytes(R, nb));
-    {
-        char *w = (char *)ws + pool_bytes(R, nb) + align256((size_t)R.rows * nb * 4);
-        a.gcand = (uint64_t *)w;
-        a.g64 = (double *)(w + (size_t)pool_enum_blocks(R, nb) * PE_W * GCAP * 8);
-    }
     a.best_gap = best_gap;
     a.best_idx = best_idx;
     a.k_max = k_max;
@@ -662,11 +1133,11 @@ fw_status pool_best_subset(const RowsDev &R, const int32_t *k, int nb, const int
     FW_DISPATCH(R.d, R.v_dtype, {
         const size_t sb = (size_t)R.max_n * 4;
         FW_CUDA_CHECK(cudaFuncSetAttribute(k_pool_build<DPL, VT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb));
-        FW_LAUNCH((k_pool_build<DPL, VT>), (unsigned)std::min<int64_t>(R.rows, (int64_t)sms * 4), PB_T, sb, st, a);
-        const size_t se = (size_t)PE_W * sizeof(EnumSm);
-        FW_CUDA_CHECK(cudaFuncSetAttribute(k_pool_enum<DPL, VT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)se));
-        FW_LAUNCH((k_pool_enum<DPL, VT>), (unsigned)pool_enum_blocks(R, nb), PE_W * 32, se, st, a);
+        FW_LAUNCH((k_pool_build<DPL, VT>), (unsigned)std::min<int64_t>(R.rows, (int64_t)sms * 8), PB_T, sb, st, a);
     });
+    const size_t se = (sizeof(EnumSm) + 15) / 16 * 16 + (size_t)PMAX * (R.d + 4) * 4;
+    FW_CUDA_CHECK(cudaFuncSetAttribute(k_pool_enum, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)se));
+    FW_LAUNCH(k_pool_enum, (unsigned)std::min<int64_t>(R.rows * nb, 1 << 20), PE_T, se, st, a);
     return FW_OK;
 }
 
