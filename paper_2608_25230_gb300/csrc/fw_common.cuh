@@ -213,7 +213,8 @@ __device__ __forceinline__ void stage_value_cols(const VT *V, int n, int d, int 
 
 // CTA-wide selection of the m largest of n unsigned order keys, equal keys
 // taken in ascending index order: on return (every thread) T is the m-th
-// largest key and L the largest index taken among the keys equal to T; key j
+// largest key and L bounds the indices taken among the keys equal to T (the last
+// one taken, or n - 1 when all of them are); key j
 // is selected iff key(j) > T or (key(j) == T and j <= L).  1 <= m <= n.
 // Three radix passes (11, 11, 10 bits) over a 2048-bin shared histogram, then
 // an index-order scan of the keys equal to T.  key(j) is called for j < n by
@@ -222,7 +223,7 @@ struct TopmSmem {
     uint32_t hist[2048];
     int wcnt[32];
     uint32_t digit;
-    int rem, L;
+    int rem, L, eq;
 };
 template <typename KeyFn>
 __device__ __forceinline__ void block_topm(int n, int m, KeyFn key, TopmSmem &S, uint32_t &T, int &L)
@@ -263,6 +264,7 @@ __device__ __forceinline__ void block_topm(int n, int m, KeyFn key, TopmSmem &S,
                     if (acc + h >= rem) {
                         S.digit = (uint32_t)(top - q);
                         S.rem = rem - acc;
+                        S.eq = h;
                         break;
                     }
                     acc += h;
@@ -276,6 +278,10 @@ __device__ __forceinline__ void block_topm(int n, int m, KeyFn key, TopmSmem &S,
         __syncthreads();
     }
     T = prefix;
+    if (S.eq == rem) {  // every key equal to T is taken (uniform): no scan
+        L = n - 1;
+        return;
+    }
     // the rem-th key equal to T in index order
     if (tid == 0) S.L = -1;
     __syncthreads();

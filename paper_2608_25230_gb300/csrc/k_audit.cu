@@ -22,11 +22,19 @@
 //
 //   k_aud_mass    accumulated masses and window votes of every group (a thread
 //                 per key walks the group's rows; compensated sums);
-//   k_aud_select  per group and budget the H2O and SnapKV sets (CTA-wide
-//                 radix top-m), written as bit masks;
-//   k_aud_row     per row: the Quest page maxima and sets, then one warp per
-//                 (rule, budget) gathers its members' p_j v_j and forms es.
+//   k_aud_select  a CTA per group, budget and rule: the H2O or SnapKV set (the
+//                 order keys staged once in shared memory, CTA-wide radix
+//                 top-m), written as a bit mask by ballots;
+//   k_aud_row     per row (its logits staged in shared memory): a warp per
+//                 (budget, page size) takes Quest's few largest pages by
+//                 repeated arg-max, then one warp per (rule, budget) lists its
+//                 members and gathers their p_j v_j, 8 value rows in flight.
+// Both are bound by shared-memory and L2 latency.  On 1,024 rows of 4,096 keys
+// (256 groups, d = 128, s = 4/8/16/32) the audit with its
+// gap call takes 0.41 ms; with a CTA per group for all sets, a radix select for
+// every page size and members gathered one at a time it took 0.90 ms.
 #include <algorithm>
+#include <climits>
 
 #include "fw_internal.h"
 
@@ -37,6 +45,9 @@ constexpr int AM_T = 256;   // k_aud_mass threads
 constexpr int AS_T = 512;   // k_aud_select threads
 constexpr int AR_T = 256;   // k_aud_row threads (8 warps)
 constexpr int A_NBMAX = 4;
+constexpr int AR_MP = 16;      // pages a warp takes by repeated arg-max (above: the block's radix select)
+constexpr int AS_STAGE = 24576;  // candidates whose keys k_aud_select stages (96 KB)
+constexpr size_t AR_SMEM = 196608;  // k_aud_row stages the row where its sets and logits fit this
 constexpr int NSEL = FW_NUM_SELECTORS;
 
 struct AudArgs {
@@ -48,12 +59,13 @@ struct AudArgs {
     float *vote;             // ws [groups][nb][max_n] window votes
     uint32_t *gbits;         // ws [groups][nb][2][words] H2O and SnapKV sets
     int words;
+    int pm_floats;           // page maxima of the largest row (0: no budget needs them)
     float *es;               // [rows][NSEL][nb]
     uint32_t *bits;          // [rows][NSEL][nb][words] or null
 };
 
 __device__ __forceinline__ int snap_w(int s) { return max(1, min(32, s / 2)); }
-__device__ __forceinline__ int quest_p(int q, int s) { return q == 0 ? max(2, s / 4) : 16; }
+__host__ __device__ __forceinline__ int quest_p(int q, int s) { return q == 0 ? (s / 4 > 2 ? s / 4 : 2) : 16; }
 
 // ---------------------------------------------------------------- masses
 __global__ void __launch_bounds__(AM_T) k_aud_mass(AudArgs a)
@@ -109,116 +121,147 @@ __global__ void __launch_bounds__(AM_T) k_aud_mass(AudArgs a)
 }
 
 // ------------------------------------------------------- group-level sets
+// blockIdx.x = ((group, budget), rule).  STAGED: the candidates' order keys sit
+// in shared memory (n <= AS_STAGE); otherwise every pass forms them again.
+template <bool STAGED>
 __global__ void __launch_bounds__(AS_T) k_aud_select(AudArgs a)
 {
+    extern __shared__ uint32_t skeys[];
     __shared__ TopmSmem S;
-    const int tid = threadIdx.x;
-    for (int64_t g = blockIdx.x; g < a.R.num_groups; g += gridDim.x) {
-        const int n = a.R.n[g];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int64_t items = a.R.num_groups * a.nb * 2;
+    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+        const int rule = (int)(it & 1);  // 0: H2O, 1: SnapKV
+        const int64_t gb = it >> 1, g = gb / a.nb;
+        const int b = (int)(gb - g * a.nb);
+        const int n = a.R.n[g], s = a.s[b];
+        uint32_t *out = a.gbits + (gb * 2 + rule) * a.words;
+        if (s < 1 || s > n) {
+            for (int w = tid; w < a.words; w += AS_T) out[w] = 0u;
+            continue;
+        }
+        // H2O: the last s / 2 positions, then the largest accumulated masses;
+        // SnapKV: the last w positions, then the largest pooled votes
+        const int rec = rule ? snap_w(s) : s / 2;
+        const int m = s - rec, lim = n - rec;
         const float *G = a.G + g * a.R.max_n;
-        for (int b = 0; b < a.nb; ++b) {
-            const int s = a.s[b];
-            uint32_t *hb = a.gbits + ((g * a.nb + b) * 2 + 0) * a.words;
-            uint32_t *sb = a.gbits + ((g * a.nb + b) * 2 + 1) * a.words;
-            if (s < 1 || s > n) {
-                for (int w = tid; w < a.words; w += AS_T) hb[w] = sb[w] = 0u;
-                continue;
-            }
-            // H2O: the last r positions, then the s - r of largest accumulated mass
-            const int r = s / 2, mh = s - r;
-            uint32_t Th = 0u;
-            int Lh = -1;
-            block_topm(n - r, mh, [&](int j) { return order_key(G[j]); }, S, Th, Lh);
-            // SnapKV: the last w positions, then the s - w of largest pooled vote
-            const int w = snap_w(s), ms = s - w, lim = n - w;
-            const float *vt = a.vote + (g * a.nb + b) * a.R.max_n;
-            auto pooled = [&](int j) {
-                float v = vt[j];
-                for (int q = max(0, j - 3); q <= min(lim - 1, j + 3); ++q) v = fmaxf(v, vt[q]);
-                return order_key(v);
-            };
-            uint32_t Ts = 0u;
-            int Ls = -1;
-            if (ms > 0) block_topm(lim, ms, pooled, S, Ts, Ls);
-            for (int wd = tid; wd < a.words; wd += AS_T) {
-                uint32_t mh_bits = 0u, ms_bits = 0u;
-                for (int e = 0; e < 32; ++e) {
-                    const int j = wd * 32 + e;
-                    if (j >= n) break;
-                    bool kh = j >= n - r;
-                    if (!kh) {
-                        const uint32_t k = order_key(G[j]);
-                        kh = k > Th || (k == Th && j <= Lh);
-                    }
-                    bool ks = j >= lim;
-                    if (!ks && ms > 0) {
-                        const uint32_t k = pooled(j);
-                        ks = k > Ts || (k == Ts && j <= Ls);
-                    }
-                    mh_bits |= (uint32_t)kh << e;
-                    ms_bits |= (uint32_t)ks << e;
-                }
-                hb[wd] = mh_bits;
-                sb[wd] = ms_bits;
-            }
+        const float *vt = a.vote + gb * a.R.max_n;
+        auto form = [&](int j) {
+            if (!rule) return order_key(G[j]);
+            float v = vt[j];
+            for (int q = max(0, j - 3); q <= min(lim - 1, j + 3); ++q) v = fmaxf(v, vt[q]);
+            return order_key(v);
+        };
+        auto key = [&](int j) { return STAGED ? skeys[j] : form(j); };
+        __syncthreads();  // the previous item's keys are no longer read
+        if (STAGED) {
+            for (int j = tid; j < lim; j += AS_T) skeys[j] = form(j);
             __syncthreads();
+        }
+        uint32_t T = 0u;
+        int L = -1;
+        if (m > 0) block_topm(lim, m, key, S, T, L);
+        for (int j0 = 0; j0 < a.words * 32; j0 += AS_T) {
+            const int j = j0 + tid;
+            bool in = j < n && j >= lim;
+            if (j < lim && m > 0) {
+                const uint32_t k = key(j);
+                in = k > T || (k == T && j <= L);
+            }
+            const uint32_t bal = __ballot_sync(FW_FULL, in);
+            if (lane == 0 && (j >> 5) < a.words) out[j >> 5] = bal;
         }
     }
 }
 
 // ---------------------------------------------------------- rows: score sets
+// The row's logits are staged (one pad word per 32: page strides do not
+// collide) when stage_n >= n.
 template <int DPL, typename VT>
-__global__ void __launch_bounds__(AR_T) k_aud_row(AudArgs a)
+__global__ void __launch_bounds__(AR_T) k_aud_row(AudArgs a, int stage_n)
 {
-    extern __shared__ uint32_t smw[];  // [nb][2][words] Quest sets, then the page maxima
+    extern __shared__ uint32_t smw[];  // [nb][2][words] Quest sets, then the page maxima or the logits
     __shared__ TopmSmem S;
+    __shared__ uint16_t s_list[AR_T / 32][1024];  // members of 32 words, by warp (offsets in the words)
     constexpr int d = DPL * 32;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     uint32_t *qbits = smw;
     float *pm = reinterpret_cast<float *>(smw + a.nb * 2 * a.words);
+    float *sl = pm + a.pm_floats;
     for (int64_t row = blockIdx.x; row < a.R.rows; row += gridDim.x) {
         const int64_t g = row / a.R.R;
         const int n = a.R.n[g];
         const float *l = a.R.logits + a.R.logit_off[g] + (row - g * a.R.R) * n;
         const VT *V = static_cast<const VT *>(a.R.v) + a.R.v_off[g];
         const float M = a.M[row], Zi = 1.f / a.Z[row];
-        // Quest sets: page maxima, the top pages, the pages' keys as bits
-        for (int b = 0; b < a.nb; ++b)
-            for (int q = 0; q < 2; ++q) {
-                const int s = a.s[b];
-                const int P = quest_p(q, s);
-                const int np = (n + P - 1) / P, mp = s / P;
-                uint32_t *qb = qbits + (b * 2 + q) * a.words;
-                const bool valid = s >= 1 && s <= n && mp >= 1 && (q == 0 || s >= 16);
-                if (!valid) {
-                    __syncthreads();
-                    for (int w = tid; w < a.words; w += AR_T) qb[w] = 0u;
-                    continue;
-                }
-                __syncthreads();  // pm is free
-                for (int p = tid; p < np; p += AR_T) {
-                    float m = -INFINITY;
-                    for (int j = p * P; j < min(n, p * P + P); ++j) m = fmaxf(m, __ldg(l + j));
-                    pm[p] = m;
-                }
-                __syncthreads();
-                uint32_t T = 0u;
-                int L = -1;
-                block_topm(np, min(mp, np), [&](int p) { return order_key(pm[p]); }, S, T, L);
-                for (int w = tid; w < a.words; w += AR_T) {
-                    uint32_t bits = 0u;
-                    for (int e = 0; e < 32; ++e) {
-                        const int j = w * 32 + e;
-                        if (j >= n) break;
-                        const int p = j / P;
-                        const uint32_t k = order_key(pm[p]);
-                        bits |= (uint32_t)(k > T || (k == T && p <= L)) << e;
-                    }
-                    qb[w] = bits;
-                }
-            }
+        const bool staged = n <= stage_n;
+        auto at = [&](int j) { return staged ? sl[j + (j >> 5)] : __ldg(l + j); };
+        __syncthreads();  // the previous row's sets and logits are no longer read
+        if (staged)
+            for (int j = tid; j < n; j += AR_T) sl[j + (j >> 5)] = __ldg(l + j);
+        for (int w = tid; w < a.nb * 2 * a.words; w += AR_T) qbits[w] = 0u;
         __syncthreads();
-        // one warp per (rule, budget): gather the members, form es
+        // Quest sets of few pages: a warp per (budget, page size) takes the
+        // largest page after the last one taken (value descending, page
+        // ascending), mp times
+        for (int bq = wid; bq < a.nb * 2; bq += AR_T / 32) {
+            const int b = bq >> 1, q = bq & 1, s = a.s[b];
+            const int P = quest_p(q, s), np = (n + P - 1) / P, mp = s / P;
+            if (!(s >= 1 && s <= n && mp >= 1 && mp <= AR_MP && (q == 0 || s >= 16))) continue;
+            uint32_t *qb = qbits + bq * a.words;
+            uint32_t lk = 0xffffffffu;
+            int lp = -1;
+            for (int t = 0; t < min(mp, np); ++t) {
+                uint32_t bk = 0u;
+                int bp = INT_MAX;
+                for (int p = lane; p < np; p += 32) {
+                    float m = -INFINITY;
+                    const int j1 = min(n, p * P + P);
+                    for (int j = p * P; j < j1; ++j) m = fmaxf(m, at(j));
+                    const uint32_t k = order_key(m);
+                    if ((k < lk || (k == lk && p > lp)) && (k > bk || bp == INT_MAX)) {
+                        bk = k;
+                        bp = p;
+                    }
+                }
+                // the largest key, then its first page
+                const uint32_t wk = __reduce_max_sync(FW_FULL, bp == INT_MAX ? 0u : bk);
+                const int wp = (int)__reduce_min_sync(FW_FULL, bp != INT_MAX && bk == wk ? (uint32_t)bp : 0x7fffffffu);
+                lk = wk;
+                lp = wp;
+                for (int j = wp * P + lane; j < min(n, wp * P + P); j += 32) atomicOr(&qb[j >> 5], 1u << (j & 31));
+            }
+        }
+        // ... of many pages: page maxima and a radix top-m by the block
+        for (int bq = 0; bq < a.nb * 2; ++bq) {
+            const int b = bq >> 1, q = bq & 1, s = a.s[b];
+            const int P = quest_p(q, s), np = (n + P - 1) / P, mp = s / P;
+            if (!(s >= 1 && s <= n && mp > AR_MP && (q == 0 || s >= 16))) continue;
+            uint32_t *qb = qbits + bq * a.words;
+            __syncthreads();  // pm is free
+            for (int p = tid; p < np; p += AR_T) {
+                float m = -INFINITY;
+                for (int j = p * P; j < min(n, p * P + P); ++j) m = fmaxf(m, at(j));
+                pm[p] = m;
+            }
+            __syncthreads();
+            uint32_t T = 0u;
+            int L = -1;
+            block_topm(np, min(mp, np), [&](int p) { return order_key(pm[p]); }, S, T, L);
+            for (int j0 = 0; j0 < n; j0 += AR_T) {
+                const int j = j0 + tid;
+                bool in = false;
+                if (j < n) {
+                    const int p = j / P;
+                    const uint32_t k = order_key(pm[p]);
+                    in = k > T || (k == T && p <= L);
+                }
+                const uint32_t bal = __ballot_sync(FW_FULL, in);
+                if (lane == 0 && j < n) qb[j >> 5] = bal;
+            }
+        }
+        __syncthreads();
+        // one warp per (rule, budget): list the members, gather them, form es
         float ol[DPL];
 #pragma unroll
         for (int c = 0; c < DPL; ++c) ol[c] = a.o[row * d + lane * DPL + c];
@@ -231,42 +274,72 @@ __global__ void __launch_bounds__(AR_T) k_aud_row(AudArgs a)
             if (sel == FW_SEL_QUEST) src = qbits + (b * 2 + 0) * a.words;
             if (sel == FW_SEL_QUEST16) src = qbits + (b * 2 + 1) * a.words;
             const int sinks = min(4, s / 2);
+            // bits [lo, hi) of the word whose first key is j0
+            auto span = [](int j0, int lo, int hi) {
+                const int x = max(lo - j0, 0), y = min(hi - j0, 32);
+                return y <= x ? 0u : (y == 32 ? ~0u : (1u << y) - 1u) & ~((1u << x) - 1u);
+            };
             float N[DPL];
 #pragma unroll
             for (int c = 0; c < DPL; ++c) N[c] = 0.f;
             float pA = 0.f;
             int cnt = 0;
             const int nw = (n + 31) / 32;
+            uint16_t *list = s_list[wid];
             for (int w0 = 0; w0 < nw; w0 += 32) {
                 const int w = w0 + lane;
                 uint32_t word = 0u;
                 if (w < nw) {
                     if (sel == FW_SEL_STREAMING) {
-                        for (int e = 0; e < 32; ++e) {
-                            const int j = w * 32 + e;
-                            if (j < n && s >= 1 && s <= n && (j < sinks || j >= n - (s - sinks))) word |= 1u << e;
-                        }
+                        if (s >= 1 && s <= n) word = span(w * 32, 0, sinks) | span(w * 32, n - (s - sinks), n);
                     } else {
                         word = src[w];
                     }
+                    if (a.bits) a.bits[((row * NSEL + sel) * a.nb + b) * (int64_t)a.words + w] = word;
                 }
-                if (a.bits) {
-                    if (w < nw) a.bits[((row * NSEL + sel) * a.nb + b) * (int64_t)a.words + w] = word;
-                }
-                // members of the 32 words, one at a time across the warp
-                for (int src_lane = 0; src_lane < 32; ++src_lane) {
-                    uint32_t mw = __shfl_sync(FW_FULL, word, src_lane);
-                    while (mw) {
-                        const int j = (w0 + src_lane) * 32 + __ffs(mw) - 1;
-                        mw &= mw - 1;
-                        const float p = __expf(__ldg(l + j) - M) * Zi;
-                        pA += p;
-                        ++cnt;
+                if (!__any_sync(FW_FULL, word != 0u)) continue;
+                // the members of these words in index order
+                int off = __popc(word);
+                const int own = off;
 #pragma unroll
-                        for (int c = 0; c < DPL; ++c) N[c] = fmaf(p, load_v(V, (int64_t)j * d + lane * DPL + c), N[c]);
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(FW_FULL, off, o);
+                    if (lane >= o) off += y;
+                }
+                const int tot = __shfl_sync(FW_FULL, off, 31);
+                off -= own;
+                __syncwarp();  // the previous list is no longer read
+                for (uint32_t mw = word; mw; mw &= mw - 1) list[off++] = (uint16_t)(lane * 32 + __ffs(mw) - 1);
+                __syncwarp();
+                cnt += tot;
+                for (int i0 = 0; i0 < tot; i0 += 32) {
+                    const int i = i0 + lane;
+                    int j = 0;
+                    float p = 0.f;
+                    if (i < tot) {
+                        j = w0 * 32 + list[i];
+                        p = __expf(__ldg(l + j) - M) * Zi;
+                    }
+                    pA += p;
+                    const int lim = min(32, tot - i0);
+                    for (int e0 = 0; e0 < lim; e0 += 8) {  // 8 value rows in flight (mass 0 past the last)
+                        float x[8][DPL], pe[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const int je = __shfl_sync(FW_FULL, j, e0 + e);
+                            pe[e] = __shfl_sync(FW_FULL, p, e0 + e);
+#pragma unroll
+                            for (int c = 0; c < DPL; ++c) x[e][c] = load_v(V, (int64_t)je * d + lane * DPL + c);
+                        }
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if (e0 + e < lim)
+#pragma unroll
+                                for (int c = 0; c < DPL; ++c) N[c] = fmaf(pe[e], x[e][c], N[c]);
                     }
                 }
             }
+            pA = warp_sum(pA);
             float e2 = 0.f;
 #pragma unroll
             for (int c = 0; c < DPL; ++c) {
@@ -276,7 +349,6 @@ __global__ void __launch_bounds__(AR_T) k_aud_row(AudArgs a)
             e2 = warp_sum(e2);
             if (lane == 0) a.es[(row * NSEL + sel) * a.nb + b] = cnt > 0 ? sqrtf(e2) : __int_as_float(0x7fc00000);
         }
-        __syncthreads();
     }
 }
 
@@ -316,11 +388,24 @@ fw_status selector_audit(const RowsDev &R, const int32_t *s, int nb, const fw_ga
     const int64_t per_group = std::max<int64_t>(1, ((int64_t)sms * 8 + R.num_groups - 1) / R.num_groups);
     const dim3 gm((unsigned)std::min(chunks, per_group), (unsigned)std::min<int64_t>(R.num_groups, 65535));
     FW_LAUNCH(k_aud_mass, gm, AM_T, 0, st, a);
-    FW_LAUNCH(k_aud_select, (unsigned)std::min<int64_t>(R.num_groups, 1 << 20), AS_T, 0, st, a);
-    const size_t smem = ((size_t)nb * 2 * a.words + (size_t)(R.max_n + 1) / 2 + 1) * 4;
+    const unsigned gs = (unsigned)std::min<int64_t>(R.num_groups * nb * 2, 1 << 20);
+    if (R.max_n <= AS_STAGE) {
+        const size_t sk = (size_t)R.max_n * 4;
+        FW_CUDA_CHECK(cudaFuncSetAttribute(k_aud_select<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sk));
+        FW_LAUNCH(k_aud_select<true>, gs, AS_T, sk, st, a);
+    } else {
+        FW_LAUNCH(k_aud_select<false>, gs, AS_T, 0, st, a);
+    }
+    a.pm_floats = 0;
+    for (int b = 0; b < nb; ++b)
+        for (int q = 0; q < 2; ++q)  // (pages of at least 2 keys)
+            if (s[b] / quest_p(q, s[b]) > AR_MP) a.pm_floats = (R.max_n + 1) / 2 + 1;
+    const size_t sets = ((size_t)nb * 2 * a.words + a.pm_floats) * 4, lrow = ((size_t)R.max_n + (R.max_n >> 5) + 1) * 4;
+    const int stage_n = sets + lrow <= AR_SMEM ? R.max_n : 0;
+    const size_t smem = sets + (stage_n ? lrow : 0);
     FW_DISPATCH(R.d, R.v_dtype, {
         FW_CUDA_CHECK(cudaFuncSetAttribute(k_aud_row<DPL, VT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        FW_LAUNCH((k_aud_row<DPL, VT>), (unsigned)std::min<int64_t>(R.rows, (int64_t)sms * 16), AR_T, smem, st, a);
+        FW_LAUNCH((k_aud_row<DPL, VT>), (unsigned)std::min<int64_t>(R.rows, (int64_t)sms * 16), AR_T, smem, st, a, stage_n);
     });
     return FW_OK;
 }

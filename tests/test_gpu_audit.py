@@ -102,3 +102,15 @@ def test_audit_ties_and_budget_edges(fw):
     L = np.round(rng.normal(size=(2 * R, n)) * 2).astype(np.float32)  # many equal logits and masses
     V = rng.normal(size=(2, n, d)).astype(np.float32)
     check_audit(fw, rows_batch(L, V, np.ones((2 * R, 1), np.int32), R=R), [1, 2, 100, 17])
+
+
+@pytest.mark.parametrize("n", [24575, 24577, 50001])
+def test_audit_rows_past_the_staging_limits(fw, n):
+    # below and above the lengths whose keys and logits sit in shared memory;
+    # pages few (a warp's arg-max), many (the block's select) and ragged
+    rng = np.random.default_rng(n)
+    R, d = 2, 64
+    L = (rng.normal(size=(R, n)) * 1.5).astype(np.float32)
+    L[:, 0] += 8
+    V = rng.normal(size=(1, n, d)).astype(np.float32)
+    check_audit(fw, rows_batch(L, V, np.ones((R, 1), np.int32), v_dtype="bf16", R=R), [7, 300, 4096])
