@@ -8,19 +8,27 @@
 //   r_j    = max of vote over [j - h, j + h] clipped to the prefix [0, T - w)
 //            for prefix positions (h = pool / 2), r_j = vote_j in the window.
 //
-// One CTA per cell, two passes over its keys (per-query softmax statistics,
-// then the votes); each pass is a GEMM of 128-key tiles against the window:
+// A cell's keys are split over S slices, a CTA each, and two launches read them:
+// k_wscore<1> keeps every query's softmax statistics over the slice, k_wscore<2>
+// merges the slices' statistics and writes the votes; k_wpool takes the window
+// maxima of the votes.  Each is a GEMM of 128-key tiles against the window:
 // D[128 keys][32 queries] = K_tile (128 x d, K-major) x Q^T (d x 32, K-major)
 // on tcgen05 (bf16 x bf16 -> fp32 in TMEM), the K tiles brought in by TMA
-// (128-byte swizzle, three stages), the window queries by TMA once per cell.
-// Warp 0 issues the TMA loads, warp 1 the MMAs (and owns the TMEM: two
-// accumulators of 32 columns), warps 2-5 read the accumulators (one TMEM lane
-// quarter each: 32 keys x 32 queries per thread row) and keep per-query
-// running max / sum (pass 1) or add up the votes (pass 2).  Every wait is
-// bounded; a wait that gives up marks the cell FW_ERR_TIMEOUT, the warps keep
-// their loop shape (so named barriers still meet), in-flight copies are waited
-// for, and the TMEM is freed.
+// (128-byte swizzle, three stages), the window queries by TMA once per CTA.
+// Warp 0 issues the TMA loads, warp 1 the MMAs (and owns the TMEM: four
+// accumulators of 32 columns), warps 2-9 read the accumulators, two warps per
+// TMEM lane quarter: in the first launch each takes half of the queries, in the
+// second every other tile.  Every wait is bounded; a wait that gives up marks
+// the cell FW_ERR_TIMEOUT, the warps keep their loop shape, in-flight copies
+// are waited for, and the TMEM is freed.
+//
+// Bound: HBM, the keys read twice.  256 cells x 32,768 keys, d = 128: 0.65 ms,
+// 6.6 TB/s; one CTA per cell with four epilogue warps, a true running maximum
+// (nine operations per element in the first pass instead of four) and both
+// passes in one launch took 2.02 ms, and 0.89 ms for 8 cells (now 0.06).
 #include <cuda.h>  // CUtensorMap and its enums (the encoder comes from the driver at run time)
+
+#include <algorithm>
 
 #include "fw_internal.h"
 #include "tc_sm100.cuh"
@@ -30,19 +38,25 @@ namespace {
 
 constexpr int WS_KT = 128;                 // keys per tile: the MMA's M
 constexpr int WS_N = 32;                   // window queries per tile: the MMA's N (w <= 32, padded)
+constexpr int WS_H = WS_N / 2;             // queries per warp in the statistics launch
 constexpr int WS_STAGES = 3;               // K tiles in flight
-constexpr int WS_THREADS = 192;            // TMA warp, MMA warp, four epilogue warps
+constexpr int WS_ACC = 4;                  // accumulators in TMEM
+constexpr int WS_EW = 8;                   // epilogue warps
+constexpr int WS_THREADS = 64 + 32 * WS_EW;
+constexpr int WS_SMAX = 64;                // slices of a cell at most
 constexpr uint32_t WS_WAIT = 1u << 22;     // polls before a wait gives up
+constexpr int WP_T = 256;                  // k_wpool threads
 
 struct WsArgs {
     int cells, T, w, ph;  // ph: half-width of the max pool
+    int S, tps;           // slices per cell, tiles per slice
     float scale2;         // scale * log2(e): logits in base-2 units
     float *votes;         // workspace [cells][T]
+    float2 *stat;         // workspace [cells][S][WS_N]: (reference, sum of 2^(x - reference))
+    int32_t *err;         // workspace [2][cells][S]: a wait of the CTA gave up
     float *scores;        // [cells][T]
     int32_t *status;      // [cells] or null
 };
-
-__device__ __forceinline__ void ws_named_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
 // 2^x by the hardware approximation (ex2.approx.ftz: ~2 ulp, well inside the
 // score's 1e-4 tolerance); the per-(key, query) exponentials are most of the
@@ -54,7 +68,7 @@ __device__ __forceinline__ float ex2a(float x)
     return y;
 }
 
-// combine two (max, sum of 2^(x - max)) pairs
+// combine two (reference, sum of 2^(x - reference)) pairs; -inf: nothing seen
 __device__ __forceinline__ void ms_merge(float &m, float &z, float m2, float z2)
 {
     const float mn = fmaxf(m, m2);
@@ -64,42 +78,55 @@ __device__ __forceinline__ void ms_merge(float &m, float &z, float m2, float z2)
     z = a + b;
 }
 
-template <int D>
+template <int D, int PASS>
 __global__ void __launch_bounds__(WS_THREADS, 2) k_wscore(const __grid_constant__ CUtensorMap tmK,
-                                                       const __grid_constant__ CUtensorMap tmQ, const WsArgs a)
+                                                          const __grid_constant__ CUtensorMap tmQ, const WsArgs a)
 {
     constexpr int NBOX = D / 64;          // 128-byte boxes across d
     constexpr int KBOX = WS_KT * 128;     // bytes of one K box
     constexpr int KSTAGE = NBOX * KBOX;   // bytes of one K tile
     constexpr int QBOX = WS_N * 128;      // bytes of one Q box
+    // warps that read one accumulator: all, or the tile's half of them
+    constexpr int READERS = PASS == 1 ? WS_EW : WS_EW / 2;
     extern __shared__ uint8_t smraw[];
     uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~(uintptr_t)1023);
     uint8_t *sK = sm;                            // [STAGES][NBOX][128 rows x 128 B]
     uint8_t *sQ = sm + WS_STAGES * KSTAGE;       // [NBOX][32 rows x 128 B]
-    __shared__ __align__(8) uint64_t full[WS_STAGES], empty[WS_STAGES], accfull[2], accempty[2], qfull;
+    __shared__ __align__(8) uint64_t full[WS_STAGES], empty[WS_STAGES], accfull[WS_ACC], accempty[WS_ACC], qfull;
     __shared__ uint32_t s_taddr;
     __shared__ int s_err;
-    __shared__ float s_m[4][WS_N], s_z[4][WS_N];
+    __shared__ float2 s_mz[WS_EW / 2][WS_N];     // pass 1: (reference, sum) by lane quarter
+    __shared__ __align__(16) float2 s_st[WS_N];  // pass 2: (max, 1 / sum) of every query
 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int c = blockIdx.x;
+    const int c = blockIdx.x / a.S, sl = blockIdx.x - c * a.S;
     const int T = a.T, w = a.w;
     const int ntiles = (T + WS_KT - 1) / WS_KT;
-    const int total = 2 * ntiles;
+    const int t0 = sl * a.tps, total = min(ntiles, t0 + a.tps) - t0;  // (total >= 1: the launch's slices cover the tiles)
     if (tid == 0) {
         for (int s = 0; s < WS_STAGES; ++s) {
             tc::mbar_init(&full[s], 1);
             tc::mbar_init(&empty[s], 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < WS_ACC; ++b) {
             tc::mbar_init(&accfull[b], 1);
-            tc::mbar_init(&accempty[b], 4);
+            tc::mbar_init(&accempty[b], READERS);
         }
         tc::mbar_init(&qfull, 1);
         tc::mbar_init_fence();
         s_err = 0;
     }
-    if (wid == 1) tc::tmem_alloc(&s_taddr, 64);
+    if (wid == 1) tc::tmem_alloc(&s_taddr, WS_ACC * WS_N);
+    if (PASS == 2 && tid >= 64 && tid < 64 + WS_N) {
+        // the softmax statistics of every query over all keys of the cell
+        const int i = tid - 64;
+        float m = -INFINITY, z = 0.f;
+        for (int s = 0; s < a.S; ++s) {
+            const float2 p = a.stat[((int64_t)c * a.S + s) * WS_N + i];
+            ms_merge(m, z, p.x, p.y);
+        }
+        s_st[i] = make_float2(m, z > 0.f ? 1.f / z : 0.f);
+    }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -120,10 +147,9 @@ __global__ void __launch_bounds__(WS_THREADS, 2) k_wscore(const __grid_constant_
                     ok = false;
                     break;
                 }
-                const int t = it % ntiles;
                 tc::mbar_arrive_expect_tx(&full[s], KSTAGE);
                 for (int h = 0; h < NBOX; ++h)
-                    tc::tma_load_2d(sK + s * KSTAGE + h * KBOX, &tmK, 64 * h, c * T + t * WS_KT, &full[s]);
+                    tc::tma_load_2d(sK + s * KSTAGE + h * KBOX, &tmK, 64 * h, c * T + (t0 + it) * WS_KT, &full[s]);
                 ++issued;
             }
             if (!ok) atomicOr(&s_err, 1);
@@ -142,9 +168,10 @@ __global__ void __launch_bounds__(WS_THREADS, 2) k_wscore(const __grid_constant_
             bool ok = tc::mbar_wait(&qfull, 0, WS_WAIT);
             int last = -1;
             for (int it = 0; ok && it < total; ++it) {
-                const int s = it % WS_STAGES, b = it & 1;
+                const int s = it % WS_STAGES, b = it % WS_ACC;
                 ok = tc::mbar_wait(&full[s], (uint32_t)(it / WS_STAGES) & 1u, WS_WAIT);
-                if (ok && it >= 2) ok = tc::mbar_wait(&accempty[b], (uint32_t)((it >> 1) - 1) & 1u, WS_WAIT);
+                if (ok && it >= WS_ACC)
+                    ok = tc::mbar_wait(&accempty[b], (uint32_t)((it / WS_ACC) - 1) & 1u, WS_WAIT);
                 if (!ok) break;
                 tc::fence_after_sync();
 #pragma unroll
@@ -152,7 +179,7 @@ __global__ void __launch_bounds__(WS_THREADS, 2) k_wscore(const __grid_constant_
                     const int h = ks >> 2, off = (ks & 3) * 32;
                     const uint64_t ad = tc::sdesc_sw128(k0 + s * KSTAGE + h * KBOX + off, 16, 1024);
                     const uint64_t bd = tc::sdesc_sw128(q0 + h * QBOX + off, 16, 1024);
-                    tc::mma_bf16(taddr + (uint32_t)(b * 32), ad, bd, idesc, ks > 0);
+                    tc::mma_bf16(taddr + (uint32_t)(b * WS_N), ad, bd, idesc, ks > 0);
                 }
                 tc::commit(&empty[s]);
                 tc::commit(&accfull[b]);
@@ -160,110 +187,174 @@ __global__ void __launch_bounds__(WS_THREADS, 2) k_wscore(const __grid_constant_
             }
             if (!ok) atomicOr(&s_err, 1);
             // the last MMAs have completed before the TMEM can be freed
-            if (last >= 0 && !tc::mbar_wait(&accfull[last & 1], (uint32_t)(last >> 1) & 1u, WS_WAIT))
+            if (last >= 0 && !tc::mbar_wait(&accfull[last % WS_ACC], (uint32_t)(last / WS_ACC) & 1u, WS_WAIT))
                 atomicOr(&s_err, 1);
         }
         __syncwarp();
     } else {
         // --------------------------------------------------------- epilogue
-        const int q4 = wid & 3;  // the TMEM lane quarter this warp may read
-        const int ew = wid - 2;  // epilogue warp 0..3
+        const int q4 = wid & 3;           // the TMEM lane quarter this warp may read
+        const int half = (wid - 2) >> 2;  // pass 1: its half of the queries; pass 2: its tiles' parity
         const float scale2 = a.scale2;
-        float m[WS_N], z[WS_N];  // pass 1: running max / sum; pass 2: max and 1 / sum
-#pragma unroll
-        for (int i = 0; i < WS_N; ++i) {
-            m[i] = -INFINITY;
-            z[i] = 0.f;
-        }
+        const int lim = T - w;  // query i sees keys j <= lim + i
+        const uint32_t lbase = taddr + ((uint32_t)(q4 * 32) << 16);
         bool ok = true;
-        for (int it = 0; it < total; ++it) {
-            const int b = it & 1, pass = it / ntiles, t = it - pass * ntiles;
-            if (pass == 1 && t == 0) {
-                // the softmax statistics of every query over all keys of the cell
+        if constexpr (PASS == 1) {
+            // Per lane and query a reference r (a logit seen) and z = the sum of
+            // 2^(x - r): one exponential and two adds per element.  The
+            // reference only moves when a logit exceeds it by 2^6 octaves (a
+            // rescale then), so no sum can overflow and what underflows is
+            // below 2^-126 of the largest term.
+            float r[WS_H], z[WS_H];
 #pragma unroll
-                for (int i = 0; i < WS_N; ++i) {
-                    float mi = m[i], zi = z[i];
+            for (int i = 0; i < WS_H; ++i) {
+                r[i] = -INFINITY;
+                z[i] = 0.f;
+            }
+            bool first = true;
+            for (int it = 0; it < total; ++it) {
+                const int b = it % WS_ACC;
+                if (ok) ok = tc::mbar_wait(&accfull[b], (uint32_t)(it / WS_ACC) & 1u, WS_WAIT);
+                float v[WS_H];
+                if (ok) {
+                    tc::fence_after_sync();
+                    tc::ld16(lbase + (uint32_t)(b * WS_N + half * WS_H), v);
+                    tc::fence_before_sync();
+                }
+                __syncwarp();
+                if (ok && lane == 0) tc::mbar_arrive(&accempty[b]);
+                if (!ok) continue;
+                const int j = (t0 + it) * WS_KT + q4 * 32 + lane;
+                // a tile whose keys every query sees (all but the cell's last) skips the masks
+                const bool open = (t0 + it + 1) * WS_KT - 1 <= lim;
+                if (open && !first) {
+                    float top = -INFINITY;
+                    float dx[WS_H];
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1)
-                        ms_merge(mi, zi, __shfl_xor_sync(FW_FULL, mi, o), __shfl_xor_sync(FW_FULL, zi, o));
-                    if (lane == 0) {
-                        s_m[ew][i] = mi;
-                        s_z[ew][i] = zi;
+                    for (int i = 0; i < WS_H; ++i) {
+                        dx[i] = fmaf(v[i], scale2, -r[i]);
+                        top = fmaxf(top, dx[i]);
+                    }
+                    if (top <= 64.f) {
+#pragma unroll
+                        for (int i = 0; i < WS_H; ++i) z[i] += ex2a(dx[i]);
+                        continue;
                     }
                 }
-                ws_named_barrier();
 #pragma unroll
-                for (int i = 0; i < WS_N; ++i) {
-                    float mi = s_m[0][i], zi = s_z[0][i];
-                    for (int e = 1; e < 4; ++e) ms_merge(mi, zi, s_m[e][i], s_z[e][i]);
-                    m[i] = mi;
-                    z[i] = zi > 0.f ? 1.f / zi : 0.f;
-                }
-            }
-            if (ok) ok = tc::mbar_wait(&accfull[b], (uint32_t)(it >> 1) & 1u, WS_WAIT);
-            float v[WS_N];
-            if (ok) {
-                tc::fence_after_sync();
-                tc::ld32(taddr + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(b * 32), v);
-                tc::fence_before_sync();
-            }
-            __syncwarp();
-            if (ok && lane == 0) tc::mbar_arrive(&accempty[b]);
-            if (!ok) continue;
-            const int j = t * WS_KT + q4 * 32 + lane;
-            const int lim = T - w;  // query i sees keys j <= lim + i
-            // a tile whose keys every query sees (all but the cell's last) skips the masks
-            const bool open = t * WS_KT + WS_KT - 1 <= lim && w == WS_N;
-            if (pass == 0) {
-                // running (max, sum) with one exponential per element: when x
-                // raises the max the old sum is scaled by 2^(m - x), else
-                // 2^(x - m) is added
-#pragma unroll
-                for (int i = 0; i < WS_N; ++i) {
-                    if (open || (j < T && i < w && j <= lim + i)) {
+                for (int i = 0; i < WS_H; ++i) {
+                    const int qi = half * WS_H + i;
+                    if (open || (j < T && j <= lim + qi)) {
                         const float x = v[i] * scale2;
-                        const float dx = x - m[i];
-                        const float e = ex2a(-fabsf(dx));
-                        z[i] = dx > 0.f ? fmaf(z[i], e, 1.f) : z[i] + e;
-                        m[i] = fmaxf(m[i], x);
+                        const float d = x - r[i];
+                        if (d <= 64.f) {
+                            z[i] += ex2a(d);
+                        } else {  // (also the first key seen: r = -inf)
+                            z[i] = fmaf(z[i], r[i] == -INFINITY ? 0.f : ex2a(-d), 1.f);
+                            r[i] = x;
+                        }
                     }
                 }
-            } else if (j < T) {
-                float vote = 0.f;
+                // queries past the window read other rows: their references may be anything
+                first = false;
 #pragma unroll
-                for (int i = 0; i < WS_N; ++i)
-                    if (open || (i < w && j <= lim + i)) vote = fmaf(ex2a(fmaf(v[i], scale2, -m[i])), z[i], vote);
-                a.votes[(int64_t)c * T + j] = vote;
+                for (int i = 0; i < WS_H; ++i) first |= r[i] == -INFINITY;
             }
-        }
-        if (!ok) atomicOr(&s_err, 1);
-        // max pooling along the prefix positions (the cell's votes are in global
-        // memory, written by these four warps)
-        __threadfence_block();
-        ws_named_barrier();
-        const float *vc = a.votes + (int64_t)c * T;
-        const int lim = T - w;
-        for (int j = ew * 32 + lane; j < T; j += 128) {
-            float r = vc[j];
-            if (j < lim) {
-                const int lo = j - a.ph < 0 ? 0 : j - a.ph, hi = j + a.ph < lim ? j + a.ph : lim - 1;
-                for (int q = lo; q <= hi; ++q) r = fmaxf(r, vc[q]);
+            if (!ok) atomicOr(&s_err, 1);
+#pragma unroll
+            for (int i = 0; i < WS_H; ++i) {
+                float mi = r[i], zi = z[i];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+                    ms_merge(mi, zi, __shfl_xor_sync(FW_FULL, mi, o), __shfl_xor_sync(FW_FULL, zi, o));
+                if (lane == 0) s_mz[q4][half * WS_H + i] = make_float2(mi, zi);
             }
-            a.scores[(int64_t)c * T + j] = r;
+        } else {
+            for (int it = half; it < total; it += 2) {
+                const int b = it % WS_ACC;
+                if (ok) ok = tc::mbar_wait(&accfull[b], (uint32_t)(it / WS_ACC) & 1u, WS_WAIT);
+                float v[WS_N];
+                if (ok) {
+                    tc::fence_after_sync();
+                    tc::ld32(lbase + (uint32_t)(b * WS_N), v);
+                    tc::fence_before_sync();
+                }
+                __syncwarp();
+                if (ok && lane == 0) tc::mbar_arrive(&accempty[b]);
+                if (!ok) continue;
+                const int j = (t0 + it) * WS_KT + q4 * 32 + lane;
+                const bool open = (t0 + it + 1) * WS_KT - 1 <= lim;
+                if (j < T) {
+                    float vote = 0.f, vote2 = 0.f;
+#pragma unroll
+                    for (int i = 0; i < WS_N; i += 2) {
+                        const float4 st = *reinterpret_cast<const float4 *>(&s_st[i]);
+                        if (i < w && (open || j <= lim + i)) vote = fmaf(ex2a(fmaf(v[i], scale2, -st.x)), st.y, vote);
+                        if (i + 1 < w && (open || j <= lim + i + 1))
+                            vote2 = fmaf(ex2a(fmaf(v[i + 1], scale2, -st.z)), st.w, vote2);
+                    }
+                    a.votes[(int64_t)c * T + j] = vote + vote2;
+                }
+            }
+            if (!ok) atomicOr(&s_err, 1);
         }
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (tid == 0 && a.status) a.status[c] = s_err ? FW_ERR_TIMEOUT : FW_OK;
+    if (PASS == 1 && tid < WS_N) {
+        float m = -INFINITY, z = 0.f;
+        for (int q = 0; q < WS_EW / 2; ++q) ms_merge(m, z, s_mz[q][tid].x, s_mz[q][tid].y);
+        a.stat[(int64_t)blockIdx.x * WS_N + tid] = make_float2(m, z);
+    }
+    if (tid == 0) a.err[(PASS - 1) * a.cells * a.S + blockIdx.x] = s_err;
     if (wid == 1) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(taddr, 64);
+        tc::tmem_dealloc(taddr, WS_ACC * WS_N);
     }
+}
+
+// Max pooling of the votes along the prefix positions (window positions keep
+// their own); the cell's status from its CTAs' flags.
+__global__ void __launch_bounds__(WP_T) k_wpool(const WsArgs a)
+{
+    const int c = blockIdx.y, lim = a.T - a.w;
+    const float *vc = a.votes + (int64_t)c * a.T;
+    for (int j = blockIdx.x * WP_T + threadIdx.x; j < a.T; j += gridDim.x * WP_T) {
+        float r = vc[j];
+        if (j < lim) {
+            const int lo = j - a.ph < 0 ? 0 : j - a.ph, hi = j + a.ph < lim ? j + a.ph : lim - 1;
+            for (int q = lo; q <= hi; ++q) r = fmaxf(r, vc[q]);
+        }
+        a.scores[(int64_t)c * a.T + j] = r;
+    }
+    if (blockIdx.x == 0 && a.status) {
+        int e = 0;
+        for (int s = threadIdx.x; s < 2 * a.S; s += WP_T)
+            e |= a.err[(s >= a.S ? a.cells * a.S : 0) + c * a.S + (s >= a.S ? s - a.S : s)];
+        e = __syncthreads_or(e);
+        if (threadIdx.x == 0) a.status[c] = e ? FW_ERR_TIMEOUT : FW_OK;
+    }
+}
+
+// tiles per slice: enough CTAs for several waves of two per SM, at least four
+// tiles each (a CTA's setup is about one tile's time), at most WS_SMAX slices
+int slice_tiles(int cells, int T)
+{
+    int sms = 0;
+    if (device_sms(&sms) != FW_OK) sms = 152;  // no device: the size query still answers
+    const int ntiles = (T + WS_KT - 1) / WS_KT;
+    const int64_t want = std::max<int64_t>(1, ((int64_t)sms * 2 * 6 + cells - 1) / cells);
+    const int S = (int)std::min<int64_t>({want, (ntiles + 3) / 4, WS_SMAX});
+    return (ntiles + S - 1) / S;
 }
 
 }  // namespace
 
-size_t window_score_workspace(int cells, int T) { return align256((size_t)cells * T * 4); }
+size_t window_score_workspace(int cells, int T)
+{
+    return align256((size_t)cells * T * 4) + align256((size_t)cells * WS_SMAX * WS_N * sizeof(float2)) +
+           align256((size_t)cells * WS_SMAX * 2 * 4);
+}
 
 fw_status window_score(const void *Qw, const void *K, int cells, int T, int d, int w, float scale, int pool,
                        float *scores, void *ws, int32_t *status, cudaStream_t s)
@@ -276,17 +367,38 @@ fw_status window_score(const void *Qw, const void *K, int cells, int T, int d, i
     a.T = T;
     a.w = w;
     a.ph = pool / 2;
+    a.tps = slice_tiles(cells, T);
+    a.S = ((T + WS_KT - 1) / WS_KT + a.tps - 1) / a.tps;
     a.scale2 = scale * 1.4426950408889634f;
-    a.votes = (float *)ws;
+    char *wp = (char *)ws;
+    a.votes = (float *)wp;
+    wp += align256((size_t)cells * T * 4);
+    a.stat = (float2 *)wp;
+    wp += align256((size_t)cells * WS_SMAX * WS_N * sizeof(float2));
+    a.err = (int32_t *)wp;
     a.scores = scores;
     a.status = status;
     auto launch = [&](auto kernel, int nbox) -> fw_status {
         const size_t smem = 1024 + (size_t)WS_STAGES * nbox * WS_KT * 128 + (size_t)nbox * WS_N * 128;
         FW_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        FW_LAUNCH(kernel, (unsigned)cells, WS_THREADS, smem, s, mk, mq, a);
+        FW_LAUNCH(kernel, (unsigned)(cells * a.S), WS_THREADS, smem, s, mk, mq, a);
         return FW_OK;
     };
-    return d == 128 ? launch(k_wscore<128>, 2) : launch(k_wscore<64>, 1);
+    fw_status st = d == 128 ? launch(k_wscore<128, 1>, 2) : launch(k_wscore<64, 1>, 1);
+    if (st != FW_OK) return st;
+    st = d == 128 ? launch(k_wscore<128, 2>, 2) : launch(k_wscore<64, 2>, 1);
+    if (st != FW_OK) return st;
+    for (int c0 = 0; c0 < cells; c0 += 65535) {  // (the grid's y limit)
+        WsArgs b = a;
+        const int nc = std::min(cells - c0, 65535);
+        b.votes += (int64_t)c0 * T;
+        b.scores += (int64_t)c0 * T;
+        b.err += (int64_t)c0 * a.S;
+        if (b.status) b.status += c0;
+        const dim3 grid((unsigned)std::min((T + WP_T - 1) / WP_T, 64), (unsigned)nc);
+        FW_LAUNCH(k_wpool, grid, WP_T, 0, s, b);
+    }
+    return FW_OK;
 }
 
 }  // namespace fw

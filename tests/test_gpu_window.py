@@ -77,3 +77,15 @@ def test_window_scored_contour_full_scale(fw):
     o = oracle.contour_alloc(np_(sc), cb.floor, cb.total_budget, cb.uniform_s)
     np.testing.assert_array_equal(np_(g["counts"]), o["counts"])
     np.testing.assert_array_equal(np_(g["kept_pos"]), o["kept_pos"])
+
+
+@pytest.mark.parametrize("T,w", [(1500, 32), (640, 5), (513, 17)])
+def test_window_score_rising_logits(fw, T, w):
+    # keys that grow along the positions: logits pass a lane's reference by
+    # more than 2^6 octaves again and again (the rescale), over several slices
+    # of a cell, the last of them partial
+    rng = np.random.default_rng(T + w)
+    Q = workloads.f32_to_bf16_bits(rng.normal(size=(2, w, 64)).astype(np.float32))
+    ramp = np.geomspace(0.1, 30.0, T)[None, :, None]
+    K = workloads.f32_to_bf16_bits((rng.normal(size=(2, T, 64)) * ramp).astype(np.float32))
+    check(fw, Q, K)
