@@ -240,9 +240,14 @@ __device__ __forceinline__ void block_topm(int n, int m, KeyFn key, TopmSmem &S,
         const int nbin = pass < 2 ? 2048 : 1024;
         for (int i = tid; i < 2048; i += nt) S.hist[i] = 0u;
         __syncthreads();
-        for (int j = tid; j < n; j += nt) {
-            const uint32_t u = key(j);
-            if ((u & pmask) == prefix) atomicAdd(&S.hist[(u >> shift) & (uint32_t)(nbin - 1)], 1u);
+        for (int j0 = tid; j0 < n; j0 += 4 * nt) {  // four keys in flight per thread
+            uint32_t u[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) u[e] = j0 + e * nt < n ? key(j0 + e * nt) : ~prefix;
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (j0 + e * nt < n && (u[e] & pmask) == prefix)
+                    atomicAdd(&S.hist[(u[e] >> shift) & (uint32_t)(nbin - 1)], 1u);
         }
         __syncthreads();
         if (wid == 0) {

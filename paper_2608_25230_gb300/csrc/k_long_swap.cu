@@ -24,20 +24,37 @@
 // key that leaves takes the entering key's slot).  So the block keeps the
 // table C[slot][position] in its workspace: the first round of a budget fills
 // it (a k x d by d x E product in register tiles), and every later round
-// recomputes only the changed slot's column and the changed position's row.
-// A round is then one pass over the kept keys -- per key the exact product
-// g.w_i (so alpha_i), the new column entry, and the scan of its E stored
-// entries -- with O(d + E) work per key instead of O(E d).  Four lanes share a
-// key (each a quarter of the columns and of the slots); the pass is software
-// pipelined (the next key's value row is in flight while the current one is
-// scored).  In the scan D_ij is regrouped as A_i + B_j + p_i (h_j + k_j C_ij)
-// with per-key A_i and per-slot B_j, h_j, k_j, so a pair costs three fused
-// operations and one approximate division.  Each lane keeps its least score
-// and the first position where it occurred; the lanes holding the block's
-// least score score that position's pairs again with the same operations and
-// the smallest (i, j) among the pairs at that score wins.  (Two positions of
-// one lane at exactly the same fp32 score keep the first: such pairs are tied
-// to ~1e-7 relative, a decision no fp32 evaluation can settle.)
+// computes only the changed slot's column y.w_i, y the leaving key's vector,
+// and the changed position's row.  The column also carries the products with
+// g along: g moved by p_j w_j - p_i w_i, so g.w_t moves by p_j C_jt - p_i C_it,
+// the slot's old and new entry of position t.
+//
+// A round is one pass over the kept keys: four lanes share a key (each a
+// quarter of the columns); the key's value row, its scalars and its old entry
+// of the column are read one iteration ahead.  Regrouped, D_ij = A_i + B_j +
+// p_i (h_j + k_j C_ij) with per-key A_i and per-slot B_j, h_j, k_j, so with m_i
+// >= max_j p_j C_ij (kept per key, raised when a slot changes) no pair of the
+// key scores below
+//   (A_i + min_j B_j + p_i min_j h_j - 2 P^2 p_i m_i) / (P - p_i + min_j p_j)^2.
+// Keys whose bound lies above the least score found so far in the block are
+// done after O(d / 4) operations per lane; the few others (about one in a
+// hundred on the measured rows) have their E pairs scored from the table.  The
+// least score wins; among pairs at that score the smallest (i, j), except
+// that two positions of one lane at exactly the same fp32 score keep the
+// first: such pairs are tied to ~1e-7 relative, a decision no fp32 evaluation
+// can settle.
+//
+// A key that holds most of the kept mass (P' could fall below P / 4) is scored
+// after the pass by the whole block from g' = g - u_i + u_j, the columns split
+// over the warps, a lane per slot; at most one key of a round qualifies.
+//
+// Bound: on long rows the reads of value rows, scalars and column entries
+// through the SM's L2 port (~300 bytes per kept key and round at d = 128, at
+// ~18 bytes per clock); on short rows the latency of a round's barriers.
+// Scoring every key's E pairs in every round (408 bytes per key, two products
+// with the value row) took, with the gap call, 30.2 ms on 512 rows of 32,768
+// keys with three budgets and 9.4 ms on 3,072 GQA rows of 1,000 to 8,192 keys;
+// now 19.6 and 6.1 ms.
 #include <algorithm>
 #include <climits>
 
@@ -47,16 +64,17 @@ namespace fw {
 namespace {
 
 constexpr int SWT = 256;     // threads per block
+constexpr int SWW = SWT / 32;  // warps per block
 constexpr int SWMAXE = kLongSwapMaxE;  // largest pool size E
 constexpr int TK = 2;        // kept keys per thread in the first-round product tile
 constexpr int TS = 8;        // pool slots per thread in that tile (4 threads cover 32)
 constexpr int QL = 4;        // lanes per kept key in the round pass
 constexpr int KPI = SWT / QL;  // kept keys per block iteration of the pass
 // resident blocks per SM: three for rows up to 8,192 keys (short rounds, whose
-// fixed per-round costs want more blocks), two above (the registers keep the
-// next key's value row, table entries and mass in flight without spilling)
+// fixed per-round costs want more blocks), two above and for d = 256 (the
+// registers hold the next key's value row and the table tiles without spilling)
 constexpr int LS_BPS_SHORT = 3, LS_BPS_LONG = 2, LS_LONG_N = 8192;
-inline int ls_bps(const RowsDev &R) { return R.max_n > LS_LONG_N ? LS_BPS_LONG : LS_BPS_SHORT; }
+inline int ls_bps(const RowsDev &R) { return R.max_n > LS_LONG_N || R.d > 128 ? LS_BPS_LONG : LS_BPS_SHORT; }
 
 struct LSArgs {
     RowsDev R;
@@ -75,41 +93,23 @@ struct LSArgs {
     int32_t *kbuf;   // key at each position of the current kept list
     float *pbuf;     // its mass
     float *xbuf;     // its |w|^2
-    // per-block cross-product table, [gridDim.x][cstride][Ep] (position-major)
+    float *sbuf;     // its g.w
+    float *mbuf;     // its bound on max_j p_j C_ij
+    uint32_t *kebuf; // order key of every dropped key's error (0: kept)
+    // per-block cross-product table, [gridDim.x][Ep][cstride] (slot-major)
     float *cbuf;
     int cstride;     // positions per block table (max_n rounded up to a multiple of 4)
 };
 
+// (red: SWW floats that nothing else uses until the next barrier)
 __device__ __forceinline__ float block_sum(float v, float *red)
 {
     v = warp_sum(v);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) red[w] = v;
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     float t = 0.f;
-    for (int i = 0; i < SWT / 32; ++i) t += red[i];
-    __syncthreads();
+    for (int i = 0; i < SWW; ++i) t += red[i];
     return t;
-}
-
-// Eight consecutive elements of a value row as floats (p 16-byte aligned).
-__device__ __forceinline__ void ld8(const uint16_t *p, float (&x)[8])
-{
-    const uint4 u = __ldg(reinterpret_cast<const uint4 *>(p));
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        x[2 * m] = __uint_as_float(w[m] << 16);
-        x[2 * m + 1] = __uint_as_float(w[m] & 0xffff0000u);
-    }
-}
-__device__ __forceinline__ void ld8(const float *p, float (&x)[8])
-{
-    const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
-    const float4 b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
-    x[0] = a.x, x[1] = a.y, x[2] = a.z, x[3] = a.w;
-    x[4] = b.x, x[5] = b.y, x[6] = b.z, x[7] = b.w;
 }
 
 // The fast form divides D (a difference of terms of size ~N P^2) by P'^2, so
@@ -158,6 +158,7 @@ template <int NV> struct RowChunk<float, NV> {
     }
 };
 
+static_assert(TK == 2, "the table is written in pairs of positions");
 // First round of a budget: C[q][t] = w_{kb[t]} . w_q for every kept position
 // t < nk and pool slot q in the 32-slot blocks below nadd.  A thread owns 2
 // consecutive positions x 8 slots; the 4 threads of a group cover 32 slots.
@@ -209,12 +210,12 @@ __device__ __forceinline__ void cross_table(const int *kb, int nk, const VT *V, 
 #pragma unroll
                 for (int u = 0; u < TK; ++u) cur[u] = nxt[u];
             }
-            #pragma unroll
-            for (int u = 0; u < TK; ++u) {
-                float4 *dst = reinterpret_cast<float4 *>(cb + (size_t)(t0 + u) * Ep + q0 + sub * TS);
-                __stcs(dst, make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]));
-                __stcs(dst + 1, make_float4(acc[u][4], acc[u][5], acc[u][6], acc[u][7]));
-            }
+            // (TK consecutive positions: cstride and t0 are even, and a write past nk
+            // stays inside the slot's row)
+#pragma unroll
+            for (int h = 0; h < TS; ++h)
+                *reinterpret_cast<float2 *>(cb + (size_t)(q0 + sub * TS + h) * cstride + t0) =
+                    make_float2(acc[0][h], acc[1][h]);
         }
     }
 }
@@ -254,51 +255,73 @@ __device__ __forceinline__ void lane_products(const VT *vr, const float *mu, con
     }
 }
 
-// This lane's part of v.g and v.y from its loaded vectors.
+// This lane's part of v.y from its loaded vectors.
 template <int DPL, typename VT>
-__device__ __forceinline__ void lane_products_v_row(const LaneRow<DPL, VT> &row, const float *g, const float *y,
-                                                    int sub, float &vg, float &vy)
+__device__ __forceinline__ float lane_product_v_row(const LaneRow<DPL, VT> &row, const float *y, int sub)
 {
     using L = LaneRow<DPL, VT>;
-    vg = 0.f;
-    vy = 0.f;
+    float vy = 0.f, vy2 = 0.f;
 #pragma unroll
     for (int k = 0; k < L::NVL; ++k) {
         const int c0 = (k * QL + sub) * L::EPV;
 #pragma unroll
         for (int e = 0; e < L::EPV; e += 4) {
-            const float4 g4 = *reinterpret_cast<const float4 *>(g + c0 + e);
             const float4 y4 = *reinterpret_cast<const float4 *>(y + c0 + e);
-            const float gg[4] = {g4.x, g4.y, g4.z, g4.w}, yy[4] = {y4.x, y4.y, y4.z, y4.w};
+            vy = fmaf(row.u[k].at(e), y4.x, vy);
+            vy2 = fmaf(row.u[k].at(e + 1), y4.y, vy2);
+            vy = fmaf(row.u[k].at(e + 2), y4.z, vy);
+            vy2 = fmaf(row.u[k].at(e + 3), y4.w, vy2);
+        }
+    }
+    return vy + vy2;
+}
+
+// NC consecutive elements of a value row as floats, by the widest loads that NC allows.
+template <int NC> __device__ __forceinline__ void load_cols(const uint16_t *p, float (&x)[NC])
+{
+    if constexpr (NC == 1) {
+        x[0] = bf16_to_f32(__ldg(p));
+    } else {
+        uint32_t w[NC / 2];
+        if constexpr (NC == 2) {
+            w[0] = __ldg(reinterpret_cast<const uint32_t *>(p));
+        } else if constexpr (NC == 4) {
+            const uint2 u = __ldg(reinterpret_cast<const uint2 *>(p));
+            w[0] = u.x, w[1] = u.y;
+        } else {
 #pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                const float v = row.u[k].at(e + h);
-                vg = fmaf(v, gg[h], vg);
-                vy = fmaf(v, yy[h], vy);
+            for (int m = 0; m < NC / 8; ++m) {
+                const uint4 u = __ldg(reinterpret_cast<const uint4 *>(p) + m);
+                w[4 * m] = u.x, w[4 * m + 1] = u.y, w[4 * m + 2] = u.z, w[4 * m + 3] = u.w;
             }
+        }
+#pragma unroll
+        for (int m = 0; m < NC / 2; ++m) {
+            x[2 * m] = __uint_as_float(w[m] << 16);
+            x[2 * m + 1] = __uint_as_float(w[m] & 0xffff0000u);
+        }
+    }
+}
+template <int NC> __device__ __forceinline__ void load_cols(const float *p, float (&x)[NC])
+{
+    if constexpr (NC == 1) {
+        x[0] = __ldg(p);
+    } else if constexpr (NC == 2) {
+        const float2 u = __ldg(reinterpret_cast<const float2 *>(p));
+        x[0] = u.x, x[1] = u.y;
+    } else {
+#pragma unroll
+        for (int m = 0; m < NC; m += 4) {
+            const float4 u = __ldg(reinterpret_cast<const float4 *>(p + m));
+            x[m] = u.x, x[m + 1] = u.y, x[m + 2] = u.z, x[m + 3] = u.w;
         }
     }
 }
 
-// |g - u_i + u_j|^2 for one pair, from the value row of i and the pool column
-// of j (the vector form of needs_vector's pairs).
-template <int DPL, typename VT>
-__device__ __forceinline__ float vector_gp2(const VT *vr, const float *mu, const float *g, const float *Wt, int Ep,
-                                            int q, float p_i, float p_j)
+// The float of an order key (inverse of order_key).
+__device__ __forceinline__ float key_to_float(uint32_t k)
 {
-    constexpr int d = DPL * 32;
-    float gv = 0.f;
-    for (int c0 = 0; c0 < d; c0 += 8) {
-        float x[8];
-        ld8(vr + c0, x);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int c = c0 + u;
-            const float gp = fmaf(p_j, Wt[c * Ep + q], fmaf(-p_i, x[u] - mu[c], g[c]));
-            gv = fmaf(gp, gp, gv);
-        }
-    }
-    return gv;
+    return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
 // Score D / P'^2 of one pair in the regrouped fast form: sq = (B_j, k_j, h_j,
@@ -307,24 +330,6 @@ __device__ __forceinline__ float fast_score(float4 sq, float cij, float p_i, flo
 {
     const float Pp = Pm + sq.w;
     return __fdividef(fmaf(p_i, fmaf(sq.y, cij, sq.z), Ai + sq.x), Pp * Pp);
-}
-
-template <int DPL, typename VT>
-__device__ __noinline__ float vector_pair_score(const VT *vr, const float *mu, const float *g, const float *Wt, int Ep,
-                                                int q, float p_i, float p_j, float P, float P2, float N)
-{
-    return vector_score(vector_gp2<DPL, VT>(vr, mu, g, Wt, Ep, q, p_i, p_j), P, p_i, p_j, P2, N);
-}
-
-// The fast form where P'^2 >= P^2 / 16, else the vector form.
-template <int DPL, typename VT>
-__device__ __forceinline__ float any_score(float4 sq, float cij, float p_i, float Ai, float Pm, float P, float P2,
-                                           float N, const VT *vr, const float *mu, const float *g, const float *Wt,
-                                           int Ep, int q)
-{
-    const float Pp = Pm + sq.w;
-    if (16.f * Pp * Pp >= P2) return fast_score(sq, cij, p_i, Ai, Pm);
-    return vector_pair_score<DPL, VT>(vr, mu, g, Wt, Ep, q, p_i, sq.w, P, P2, N);
 }
 
 template <int DPL, typename VT, int BPS>
@@ -342,25 +347,30 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
     float *Wt = wtmp + d;              // [d][Ep] pool vectors w_j, slot-major inner
     // per-round slot terms of the regrouped score: B_j, k_j, h_j, p_j ([Ep] each)
     float *sB = Wt + d * Ep, *sK = sB + Ep, *sH = sK + Ep, *sP = sH + Ep;
-    float *pj = sP + Ep;               // [Ep] masses of the pool slots
-    float *betaj = pj + Ep;            // [Ep]
-    int *idxj = reinterpret_cast<int *>(betaj + Ep);  // [Ep] keys in the slots
-    float *red = reinterpret_cast<float *>(idxj + Ep);  // [32]
-    float *mass = red + 32;            // [8]
-    uint32_t *hist = reinterpret_cast<uint32_t *>(mass + 8);  // [256]
-    __shared__ uint32_t s_misc[8];
-    __shared__ int s_cnt, s_bt, s_bq;
-    __shared__ float s_gm, s_ym, s_pmin;
+    float *xj = sP + Ep;               // [Ep] |w_j|^2 of the slots
+    int *idxj = reinterpret_cast<int *>(xj + Ep);  // [Ep] keys in the slots
+    float *partA = reinterpret_cast<float *>(idxj + Ep);  // [SWW][Ep] column sums by warp
+    float *partB = partA + SWW * Ep;   // [SWW][Ep]
+    float *mass = partB + SWW * Ep;    // [8]
+    __shared__ TopmSmem s_top;
+    __shared__ float red[SWW], red2[SWW];
+    __shared__ int s_cnt, s_bt, s_bq, s_heavy;
+    __shared__ float s_ym, s_pmin, s_pmax, s_Bmin;
+    __shared__ uint32_t s_ub;          // order key of the least score found in the round
     __shared__ unsigned long long s_bkey;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int gq = tid / QL, sub = tid % QL;  // key group and lane within it
+    const uint32_t quad = 0xfu << (lane & 28);
     const size_t boff = (size_t)blockIdx.x * a.R.max_n;
     float *eb = a.ebuf + boff;
     int *kb = a.kbuf + boff;
     float *pk = a.pbuf + boff;
     float *xk = a.xbuf + boff;
+    float *sk = a.sbuf + boff;
+    float *mk = a.mbuf + boff;
+    uint32_t *ke = a.kebuf + boff;
     const int cs = a.cstride;
-    float *cb = a.cbuf + (size_t)blockIdx.x * Ep * cs;  // [cs][Ep]
+    float *cb = a.cbuf + (size_t)blockIdx.x * Ep * cs;  // [Ep][cs]
     const int nb = a.nb, MS = a.max_swaps;
 
     for (int64_t row = blockIdx.x; row < a.R.rows; row += gridDim.x) {
@@ -383,8 +393,11 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
         __syncthreads();
         // ---- one pass: band sums, band masses, single-key errors of every key
         {
+            // lane l holds the DPL columns from l DPL (one vector load per key)
             float acc[5][DPL];
-            float macc[5];
+            float macc[5], ol[DPL];
+#pragma unroll
+            for (int t = 0; t < DPL; ++t) ol[t] = o[lane * DPL + t];
 #pragma unroll
             for (int b = 0; b < 5; ++b) {
                 macc[b] = 0.f;
@@ -393,10 +406,10 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
             }
             // 16 consecutive keys per warp and step: lanes l and l + 16 find the
             // mass and band of key j0 + (l mod 16); then the warp walks the 16
-            // value rows (lane = column), and the 16 partial |v_j - o|^2 are summed
+            // value rows (lane = columns), and the 16 partial |v_j - o|^2 are summed
             // by a transposed butterfly (lane l ends with key j0 + (l mod 16))
             constexpr int KS = 16;
-            for (int j0 = wid * KS; j0 < n; j0 += (SWT / 32) * KS) {
+            for (int j0 = wid * KS; j0 < n; j0 += SWW * KS) {
                 const int jl = j0 + (lane & (KS - 1));
                 float pl = 0.f;
                 int bl = 0;
@@ -406,33 +419,32 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                     const uint32_t key = order_key(x);
                     for (int b = 0; b < nb; ++b) bl += !(key > tk[b] || (key == tk[b] && jl <= ti[b]));
                 }
+#pragma unroll
+                for (int b = 0; b < 5; ++b) macc[b] += lane < KS && bl == b ? pl : 0.f;
                 float dd[KS];
 #pragma unroll
-                for (int u0 = 0; u0 < KS; u0 += 4) {
-                    float v[4][DPL];
+                for (int u0 = 0; u0 < KS; u0 += 8) {
+                    float v[8][DPL];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
+                    for (int u = 0; u < 8; ++u) {
                         const int j = j0 + u0 + u < n ? j0 + u0 + u : j0;
-#pragma unroll
-                        for (int t = 0; t < DPL; ++t) v[u][t] = load_v(V, (int64_t)j * d + lane + 32 * t);
+                        load_cols<DPL>(V + (int64_t)j * d + lane * DPL, v[u]);
                     }
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const float p = __shfl_sync(FW_FULL, pl, u0 + u);
+                    for (int u = 0; u < 8; ++u) {
+                        const float p = __shfl_sync(FW_FULL, pl, u0 + u);  // 0 past the row's end
                         const int band = __shfl_sync(FW_FULL, bl, u0 + u);
-                        const bool live = j0 + u0 + u < n;
                         // band is the same for the whole warp: one accumulator set is touched
 #pragma unroll
                         for (int b = 0; b < 5; ++b)
-                            if (live && b == band) {
+                            if (b == band) {
 #pragma unroll
                                 for (int t = 0; t < DPL; ++t) acc[b][t] = fmaf(p, v[u][t], acc[b][t]);
-                                macc[b] += p;
                             }
                         float dist = 0.f;
 #pragma unroll
                         for (int t = 0; t < DPL; ++t) {
-                            const float w = v[u][t] - o[lane + 32 * t];
+                            const float w = v[u][t] - ol[t];
                             dist = fmaf(w, w, dist);
                         }
                         dd[u0 + u] = dist;
@@ -457,7 +469,8 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
 #pragma unroll
             for (int b = 0; b < 5; ++b) {
 #pragma unroll
-                for (int t = 0; t < DPL; ++t) atomicAdd(&S[b * d + lane + 32 * t], acc[b][t]);
+                for (int t = 0; t < DPL; ++t) atomicAdd(&S[b * d + lane * DPL + t], acc[b][t]);
+                macc[b] = warp_sum(macc[b]);
                 if (lane == 0) atomicAdd(&mass[b], macc[b]);
             }
         }
@@ -493,6 +506,7 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                 if (q <= sb) P += mass[q];
                 else Pb += mass[q];
             }
+            float gl = 0.f;
             for (int c = tid; c < d; c += SWT) {
                 float NA = 0.f, NC = 0.f;
                 for (int q = 0; q < 5; ++q) {
@@ -500,89 +514,64 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                     else NC += S[q * d + c];
                 }
                 g[c] = Pb * NA - P * NC;
+                gl = fmaf(g[c], g[c], gl);
             }
             if (tid == 0) s_cnt = 0;
-            __syncthreads();
+            float N = block_sum(gl, red);
             const uint32_t T = tk[b];
             const int TI = ti[b];
-            for (int j = tid; j < n; j += SWT) {
-                const uint32_t key = order_key(lg[j]);
-                if (key > T || (key == T && j <= TI)) kb[atomicAdd(&s_cnt, 1)] = j;
+            // (four keys per thread and step: independent loads)
+            for (int j0 = 0; j0 < n; j0 += 4 * SWT) {
+                float x[4];
+                uint32_t er[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int j = j0 + u * SWT + tid;
+                    x[u] = j < n ? lg[j] : 0.f;
+                    er[u] = j < n ? __float_as_uint(eb[j]) : 0u;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int j = j0 + u * SWT + tid;
+                    const uint32_t key = order_key(x[u]);
+                    const bool kept = j < n && (key > T || (key == T && j <= TI));
+                    if (j < n) ke[j] = kept ? 0u : er[u] + 1u;
+                    const uint32_t bal = __ballot_sync(FW_FULL, kept);
+                    int base = 0;
+                    if (lane == 0 && bal) base = atomicAdd(&s_cnt, __popc(bal));
+                    base = __shfl_sync(FW_FULL, base, 0);
+                    if (kept) kb[base + __popc(bal & ((1u << lane) - 1u))] = j;
+                }
             }
-            float gl = 0.f;
-            for (int c = tid; c < d; c += SWT) gl = fmaf(g[c], g[c], gl);
-            float N = block_sum(gl, red);  // contains the __syncthreads the list needs
+            __syncthreads();
             const int nk = s_cnt;
             if (tid == 0 && a.topk_gap) a.topk_gap[rb] = sqrtf(N) / P;
-            // ---- pool extras: the E dropped keys of largest error (radix select on the bits)
+            // ---- pool extras: the E dropped keys of largest error (kept keys rank
+            // below every dropped one; equal errors: lower index)
             const int ndrop = n - kbud;
             const int Eeff = a.E < ndrop ? a.E : ndrop;
             int nadd = 0;
             if (Eeff > 0) {
-                uint32_t prefix = 0u, pmask = 0u, rem = (uint32_t)Eeff;
-                for (int pass = 0; pass < 4; ++pass) {
-                    const int shift = 24 - 8 * pass;
-                    for (int i = tid; i < 256; i += SWT) hist[i] = 0u;
-                    __syncthreads();
-                    for (int j = tid; j < n; j += SWT) {
-                        const uint32_t key = order_key(lg[j]);
-                        if (key > T || (key == T && j <= TI)) continue;
-                        const uint32_t e = __float_as_uint(eb[j]);
-                        if ((e & pmask) == prefix) atomicAdd(&hist[(e >> shift) & 255u], 1u);
-                    }
-                    __syncthreads();
-                    if (tid == 0) {
-                        uint32_t cum = 0;
-                        for (int v = 255; v >= 0; --v) {
-                            const uint32_t c = hist[v];
-                            if (cum + c >= rem) {
-                                s_misc[0] = prefix | ((uint32_t)v << shift);
-                                s_misc[1] = rem - cum;
-                                break;
-                            }
-                            cum += c;
-                        }
-                    }
-                    __syncthreads();
-                    prefix = s_misc[0];
-                    rem = s_misc[1];
-                    pmask |= 255u << shift;
-                    __syncthreads();
-                }
-                // keys above the threshold, then the first `rem` equal ones in index order
+                auto ekey = [&](int j) { return ke[j]; };
+                uint32_t eT = 0u;
+                int eL = -1;
+                block_topm(n, Eeff, ekey, s_top, eT, eL);
                 if (tid == 0) s_cnt = 0;
                 __syncthreads();
-                for (int j = tid; j < n; j += SWT) {
-                    const uint32_t key = order_key(lg[j]);
-                    if (key > T || (key == T && j <= TI)) continue;
-                    if (__float_as_uint(eb[j]) > prefix) idxj[atomicAdd(&s_cnt, 1)] = j;
+                for (int j0 = tid; j0 < n; j0 += 4 * SWT) {
+                    uint32_t e[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) e[u] = j0 + u * SWT < n ? ekey(j0 + u * SWT) : 0u;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int j = j0 + u * SWT;
+                        if (j < n && (e[u] > eT || (e[u] == eT && j <= eL))) {
+                            const int q = atomicAdd(&s_cnt, 1);
+                            if (q < Ep) idxj[q] = j;
+                        }
+                    }
                 }
-                __syncthreads();
-                uint32_t base = 0;
-                const int above = s_cnt;
-                for (int j0 = 0; j0 < n && base < rem; j0 += SWT) {
-                    const int j = j0 + tid;
-                    bool match = false;
-                    if (j < n) {
-                        const uint32_t key = order_key(lg[j]);
-                        match = !(key > T || (key == T && j <= TI)) && __float_as_uint(eb[j]) == prefix;
-                    }
-                    const uint32_t bal = __ballot_sync(FW_FULL, match);
-                    if (lane == 0) hist[wid] = __popc(bal);
-                    __syncthreads();
-                    uint32_t before = 0, total = 0;
-                    for (int w = 0; w < SWT / 32; ++w) {
-                        if (w < wid) before += hist[w];
-                        total += hist[w];
-                    }
-                    if (match) {
-                        const uint32_t r = base + before + __popc(bal & ((1u << lane) - 1u));
-                        if (r < rem) idxj[above + r] = j;
-                    }
-                    __syncthreads();
-                    base += total;
-                }
-                nadd = above + (int)rem;
+                nadd = Eeff;
                 __syncthreads();
             }
             // stage the pool: w_j = v_j - mu in slots [0, nadd), zeros above
@@ -591,166 +580,162 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                 Wt[e] = q < nadd ? load_v(V, (int64_t)idxj[q] * d + c) - mu[c] : 0.f;
             }
             for (int q = tid; q < Ep; q += SWT) {
-                pj[q] = q < nadd ? expf(lg[idxj[q]] - M) * Zi : 0.f;
-                if (q >= nadd) idxj[q] = -1;
+                sP[q] = q < nadd ? expf(lg[idxj[q]] - M) * Zi : 0.f;
+                if (q >= nadd) {
+                    idxj[q] = -1;
+                    sB[q] = INFINITY;
+                    sK[q] = sH[q] = 0.f;
+                }
             }
             __syncthreads();
 
             int taken = 0, cap = 0;
             bool first = true;
             int tprev = -1, qprev = -1;  // position that entered and slot that changed last round
+            float pent = 0.f, pdep = 0.f;  // masses of the keys that entered and left
             for (;;) {
                 if (nadd == 0 || nk == 0) break;
                 const float P2 = P * P;
-                // ---- pool terms of the round: beta_j
-                for (int q = wid; q < nadd; q += SWT / 32) {
-                    float s2 = 0.f, sg = 0.f;
-                    for (int c = lane; c < d; c += 32) {
-                        const float w = Wt[c * Ep + q];
-                        s2 = fmaf(w, w, s2);
-                        sg = fmaf(g[c], w, sg);
-                    }
-                    s2 = warp_sum(s2);
-                    sg = warp_sum(sg);
-                    const float p = pj[q];
-                    if (lane == 0) {
-                        const float beta = p * p * s2 + 2.f * p * sg;
-                        betaj[q] = beta;
-                        // D_ij = A_i + B_j + p_i (h_j + k_j C_ij) (the file comment's D regrouped)
-                        sB[q] = beta * P2 - N * p * fmaf(2.f, P, p);
-                        sK[q] = -2.f * P2 * p;
-                        sH[q] = 2.f * N * p;
-                        sP[q] = p;
-                    }
-                }
-                if (wid == SWT / 32 - 1) {  // mu.g and mu.(changed slot's vector) for the folded products
-                    float a1 = 0.f, a2 = 0.f;
-                    for (int c = lane; c < d; c += 32) {
-                        a1 = fmaf(mu[c], g[c], a1);
-                        a2 = fmaf(mu[c], wdep[c], a2);
-                    }
-                    a1 = warp_sum(a1);
-                    a2 = warp_sum(a2);
-                    float pm = INFINITY;
-                    for (int q = lane; q < nadd; q += 32) pm = fminf(pm, pj[q]);
-                    pm = warp_min(pm);
-                    if (lane == 0) {
-                        s_gm = a1;
-                        s_ym = a2;
-                        s_pmin = pm;
-                    }
-                }
-                // ---- cross products: the whole table in the first round, else the
-                // row of the position that changed (its column entries come below)
-                if (first) {
-                    cross_table<DPL, VT>(kb, nk, V, mu, Wt, Ep, nadd, cb, cs);
-                } else {
-                    // warps split the columns, lanes take the slots of a 32-slot block
-                    float *part = reinterpret_cast<float *>(hist);  // [8][32]
-                    constexpr int CPW = d / (SWT / 32);
+                // ---- sums over the columns for every slot: g.w_j, and in the first
+                // round |w_j|^2, later the entered key's row of the table (warps
+                // split the columns, lanes take the slots of a 32-slot block)
+                {
+                    constexpr int CPW = d / SWW;
                     for (int q0 = 0; q0 < nadd; q0 += 32) {
                         const int q = q0 + lane;
-                        float c2 = 0.f;
-#pragma unroll 4
-                        for (int c = wid * CPW; c < (wid + 1) * CPW; ++c) c2 = fmaf(wtmp[c], Wt[c * Ep + q], c2);
-                        part[wid * 32 + lane] = c2;
-                        __syncthreads();
-                        if (wid == 0 && q < nadd) {
-                            float c3 = 0.f;
-                            for (int w = 0; w < SWT / 32; ++w) c3 += part[w * 32 + lane];
-                            __stcs(cb + (size_t)tprev * Ep + q, c3);
+                        float sg = 0.f, s2 = 0.f;
+#pragma unroll
+                        for (int e = 0; e < CPW; ++e) {
+                            const int c = wid * CPW + e;
+                            const float w = Wt[c * Ep + q];
+                            sg = fmaf(g[c], w, sg);
+                            s2 = fmaf(first ? w : wtmp[c], w, s2);
                         }
-                        __syncthreads();
+                        partA[wid * Ep + q] = sg;
+                        partB[wid * Ep + q] = s2;
+                    }
+                }
+                if (wid == 1) {  // mu.(changed slot's vector)
+                    float a2 = 0.f;
+                    for (int c = lane; c < d; c += 32) a2 = fmaf(mu[c], wdep[c], a2);
+                    a2 = warp_sum(a2);
+                    if (lane == 0) s_ym = a2;
+                }
+                if (wid == 2 && !first) {  // g.w of the key that entered
+                    float a2 = 0.f;
+                    for (int c = lane; c < d; c += 32) a2 = fmaf(g[c], wtmp[c], a2);
+                    a2 = warp_sum(a2);
+                    if (lane == 0) sk[tprev] = a2;
+                }
+                if (first) cross_table<DPL, VT>(kb, nk, V, mu, Wt, Ep, nadd, cb, cs);
+                __syncthreads();
+                if (wid == 0) {
+                    float pm = INFINITY, px = 0.f, Bm = INFINITY;
+                    for (int q = lane; q < nadd; q += 32) {
+                        float sg = 0.f, s2 = 0.f;
+#pragma unroll
+                        for (int w = 0; w < SWW; ++w) {
+                            sg += partA[w * Ep + q];
+                            s2 += partB[w * Ep + q];
+                        }
+                        if (first) xj[q] = s2;
+                        else cb[(size_t)q * cs + tprev] = s2;
+                        const float p = sP[q];
+                        // D_ij = A_i + B_j + p_i (h_j + k_j C_ij) (the file comment's D regrouped)
+                        const float B = (p * p * xj[q] + 2.f * p * sg) * P2 - N * p * fmaf(2.f, P, p);
+                        sB[q] = B;
+                        sK[q] = -2.f * P2 * p;
+                        sH[q] = 2.f * N * p;
+                        pm = fminf(pm, p);
+                        px = fmaxf(px, p);
+                        Bm = fminf(Bm, B);
+                    }
+                    pm = warp_min(pm);
+                    px = warp_max(px);
+                    Bm = warp_min(Bm);
+                    if (lane == 0) {
+                        s_pmin = pm;
+                        s_pmax = px;
+                        s_Bmin = Bm;
+                        s_heavy = -1;
+                        s_ub = order_key(0.f);  // only scores below 0 are swaps
+                        s_bkey = ~0ull;
                     }
                 }
                 __syncthreads();
-                // ---- one pass over the kept keys: exact g.w_i, the changed slot's
-                // entry, and every pair of the key from the table
-                // Four lanes per kept key: lane `sub` holds the row's 16-byte
-                // vectors sub, sub + 4, ... and the pool slots q0 + 4m + sub of every
-                // 32-slot block.  Each lane keeps the least of its scores and the
-                // position where it first occurred; the block's least score then
-                // picks the lanes whose pairs are scored again.
-                float lmin = INFINITY, lp = 0.f, lA = 0.f;
-                int lt = -1, li = 0;
-                const float gm = s_gm, ym = s_ym;
-                const float pmin = s_pmin;  // least pool mass (the vector form's test)
-                // the scores of key t (position) from its products; cq0: its table
-                // entries of the first 32-slot block, read ahead
-                auto score_key = [&](int t, int i, const VT *vr, float sg, float sn, float p_i, float x2, bool col,
-                                     float (&cq0)[8]) {
+                // ---- one pass over the kept keys.  Each lane keeps the least of its
+                // scores, with the pair's position and slot.
+                float lmin = INFINITY;
+                int lt = -1, li = 0, lq = 0;
+                const float pmin = s_pmin, Bmin = s_Bmin, hmin = 2.f * N * pmin, hmax = 2.f * N * s_pmax;
+                // position t, key i: its pairs, unless its bound excludes them
+                auto score_key = [&](int t, int i, float sg, float sn, float p_i, float x2, float mx, bool scan) {
                     const float alpha = p_i * p_i * x2 - 2.f * p_i * sg;
                     const float Ai = alpha * P2 + N * p_i * (2.f * P - p_i);
                     const float Pm = P - p_i;
-                    // every pair of this key takes the fast form unless some pool
-                    // mass leaves P' below P / 4
-                    const bool fast = 16.f * (Pm + pmin) * (Pm + pmin) >= P2;
-                    float kmin = INFINITY;
+                    const float Pl = Pm + pmin;
+                    if (16.f * Pl * Pl < P2) {  // some pair needs the vector form: after the pass
+                        if (sub == 0) s_heavy = t;
+                        return;
+                    }
+                    const float cmx = 2.f * P2 * p_i * mx;
+                    const float ub = key_to_float(*(volatile uint32_t *)&s_ub);
+                    const float lb = (Ai + Bmin) + (p_i * hmin - cmx);
+                    const float slack = 4e-6f * (fabsf(Ai) + fabsf(Bmin) + p_i * hmax + fabsf(cmx));  // its rounding
+                    if (!scan && lb - slack > fminf(ub, lmin) * (Pl * Pl)) return;
+                    float kmin = INFINITY, kc = -INFINITY;
+                    int kq = 0;
                     for (int q0 = 0; q0 < nadd; q0 += 32) {
-                        const int qb = q0 + 8 * sub;  // this lane's 8 consecutive slots
-                        float cq[8];
-                        if (q0 == 0) {
+                        const int qb = q0 + 8 * sub;  // this lane's 8 consecutive slots (B_j = inf past nadd)
+                        float cq[8], sc[8];
 #pragma unroll
-                            for (int m = 0; m < 8; ++m) cq[m] = cq0[m];
-                        } else {
-                            const float4 *src = reinterpret_cast<const float4 *>(cb + (size_t)t * Ep + qb);
-                            const float4 c0 = __ldcs(src), c1 = __ldcs(src + 1);
-                            cq[0] = c0.x, cq[1] = c0.y, cq[2] = c0.z, cq[3] = c0.w;
-                            cq[4] = c1.x, cq[5] = c1.y, cq[6] = c1.z, cq[7] = c1.w;
-                        }
-                        if (col && qprev >= qb && qprev < qb + 8) {
-                            const int mm = qprev - qb;
+                        for (int m = 0; m < 8; ++m) cq[m] = qb + m < nadd ? cb[(size_t)(qb + m) * cs + t] : 0.f;
+                        if (t != tprev) {
 #pragma unroll
                             for (int m = 0; m < 8; ++m)
-                                if (m == mm) cq[m] = sn;
-                            __stcs(cb + (size_t)t * Ep + qprev, sn);
+                                if (qb + m == qprev) cq[m] = sn;
                         }
-                        const int nq = nadd - qb;  // slot qb + m exists iff m < nq
-                        if (fast && nq >= 8) {
+                        float k8 = INFINITY;
 #pragma unroll
-                            for (int h = 0; h < 8; h += 4) {
-                                const float4 B4 = *reinterpret_cast<const float4 *>(sB + qb + h);
-                                const float4 K4 = *reinterpret_cast<const float4 *>(sK + qb + h);
-                                const float4 H4 = *reinterpret_cast<const float4 *>(sH + qb + h);
-                                const float4 P4 = *reinterpret_cast<const float4 *>(sP + qb + h);
-                                kmin = fminf(kmin, fast_score(make_float4(B4.x, K4.x, H4.x, P4.x), cq[h], p_i, Ai, Pm));
-                                kmin = fminf(kmin, fast_score(make_float4(B4.y, K4.y, H4.y, P4.y), cq[h + 1], p_i, Ai, Pm));
-                                kmin = fminf(kmin, fast_score(make_float4(B4.z, K4.z, H4.z, P4.z), cq[h + 2], p_i, Ai, Pm));
-                                kmin = fminf(kmin, fast_score(make_float4(B4.w, K4.w, H4.w, P4.w), cq[h + 3], p_i, Ai, Pm));
-                            }
-                        } else {
+                        for (int h = 0; h < 8; h += 4) {
+                            const float4 B4 = *reinterpret_cast<const float4 *>(sB + qb + h);
+                            const float4 K4 = *reinterpret_cast<const float4 *>(sK + qb + h);
+                            const float4 H4 = *reinterpret_cast<const float4 *>(sH + qb + h);
+                            const float4 P4 = *reinterpret_cast<const float4 *>(sP + qb + h);
+                            sc[h] = fast_score(make_float4(B4.x, K4.x, H4.x, P4.x), cq[h], p_i, Ai, Pm);
+                            sc[h + 1] = fast_score(make_float4(B4.y, K4.y, H4.y, P4.y), cq[h + 1], p_i, Ai, Pm);
+                            sc[h + 2] = fast_score(make_float4(B4.z, K4.z, H4.z, P4.z), cq[h + 2], p_i, Ai, Pm);
+                            sc[h + 3] = fast_score(make_float4(B4.w, K4.w, H4.w, P4.w), cq[h + 3], p_i, Ai, Pm);
+                            kc = fmaxf(kc, fmaxf(fmaxf(P4.x * cq[h], P4.y * cq[h + 1]), fmaxf(P4.z * cq[h + 2], P4.w * cq[h + 3])));
+                            k8 = fminf(k8, fminf(fminf(sc[h], sc[h + 1]), fminf(sc[h + 2], sc[h + 3])));
+                        }
+                        if (k8 < lmin && k8 <= kmin) {
+                            // equal scores of one key: the smaller pool key
 #pragma unroll
                             for (int m = 0; m < 8; ++m)
-                                if (m < nq) {
-                                    const int q = qb + m;
-                                    kmin = fminf(kmin, any_score<DPL, VT>(make_float4(sB[q], sK[q], sH[q], sP[q]), cq[m],
-                                                                          p_i, Ai, Pm, P, P2, N, vr, mu, g, Wt, Ep, q));
+                                if (sc[m] == k8 && (k8 < kmin || idxj[qb + m] < idxj[kq])) {
+                                    kmin = k8;
+                                    kq = qb + m;
                                 }
                         }
                     }
+                    kc = fmaxf(kc, __shfl_xor_sync(quad, kc, 1));
+                    kc = fmaxf(kc, __shfl_xor_sync(quad, kc, 2));
+                    if (sub == 0) mk[t] = kc;
                     if (kmin < lmin) {  // first position of the lane's least score
                         lmin = kmin;
                         lt = t;
                         li = i;
-                        lp = p_i;
-                        lA = Ai;
+                        lq = kq;
+                        if (kmin < ub) atomicMin(&s_ub, order_key(kmin));
                     }
-                };
-                auto load_cq0 = [&](int t, float (&cq0)[8]) {  // slots 8 sub .. 8 sub + 7
-                    const float4 *src = reinterpret_cast<const float4 *>(cb + (size_t)t * Ep + 8 * sub);
-                    const float4 c0 = __ldcs(src), c1 = __ldcs(src + 1);
-                    cq0[0] = c0.x, cq0[1] = c0.y, cq0[2] = c0.z, cq0[3] = c0.w;
-                    cq0[4] = c1.x, cq0[5] = c1.y, cq0[6] = c1.z, cq0[7] = c1.w;
                 };
                 if (first) {
                     for (int t0 = 0; t0 < nk; t0 += KPI) {
                         const int t = t0 + gq;
                         const bool valid = t < nk;
-                        const int ts = valid ? t : t0;
-                        const int i = kb[ts];
+                        const int i = kb[valid ? t : t0];
                         const VT *vr = V + (int64_t)i * d;
-                        float cq0[8];
-                        load_cq0(ts, cq0);
                         float sg, sn;  // g.w_i and |w_i|^2 from w itself
                         lane_products<DPL, VT>(vr, mu, g, sub, sg, sn);
                         sg += __shfl_xor_sync(FW_FULL, sg, 1);
@@ -762,128 +747,158 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                         if (sub == 0) {
                             pk[t] = p_i;
                             xk[t] = sn;
+                            sk[t] = sg;
+                            mk[t] = INFINITY;
                         }
-                        score_key(t, i, vr, sg, sn, p_i, sn, false, cq0);
+                        score_key(t, i, sg, sn, p_i, sn, INFINITY, true);
                     }
                 } else {
-                    // software pipeline: the value row, table entries and mass of
+                    // software pipeline: the value row, scalars and old column entry of
                     // the next iteration and the kept index of the one after are in
                     // flight during this one
+                    const float ym = s_ym;
                     const int niter = (nk + KPI - 1) / KPI;
-                    int i_cur = kb[gq < nk ? gq : nk - 1];
+                    float *col = cb + (size_t)qprev * cs;
+                    const int tf = gq < nk ? gq : nk - 1;
+                    int i_cur = kb[tf];
                     int i_next = kb[gq + KPI < nk ? gq + KPI : nk - 1];
                     LaneRow<DPL, VT> row;
                     row.load(V + (int64_t)i_cur * d, sub);
-                    float cq0[8];
-                    load_cq0(gq < nk ? gq : nk - 1, cq0);
-                    float p_i = pk[gq < nk ? gq : nk - 1], x2 = xk[gq < nk ? gq : nk - 1];
+                    float p_i = pk[tf], x2 = xk[tf], s0 = sk[tf], m0 = mk[tf], c0 = col[tf];
                     for (int it = 0; it < niter; ++it) {
                         const int t = it * KPI + gq;
-                        const bool valid = t < nk;
                         const int tn = t + KPI < nk ? t + KPI : nk - 1;
-                        float cqn[8];
-                        load_cq0(tn, cqn);
-                        const float p_n = pk[tn], x2_n = xk[tn];
+                        const float p_n = pk[tn], x2_n = xk[tn], s_n = sk[tn], m_n = mk[tn], c_n = col[tn];
                         LaneRow<DPL, VT> rown;
                         rown.load(V + (int64_t)i_next * d, sub);
                         const int tnn = t + 2 * KPI;
                         const int i_nn = kb[tnn < nk ? tnn : nk - 1];
-                        float sg, sn;  // v_i.g and v_i . (the changed slot's vector)
-                        lane_products_v_row<DPL, VT>(row, g, wdep, sub, sg, sn);
-                        sg += __shfl_xor_sync(FW_FULL, sg, 1);
+                        float sn = lane_product_v_row<DPL, VT>(row, wdep, sub);  // v_i . (the changed slot's vector)
                         sn += __shfl_xor_sync(FW_FULL, sn, 1);
-                        sg += __shfl_xor_sync(FW_FULL, sg, 2);
                         sn += __shfl_xor_sync(FW_FULL, sn, 2);
-                        if (valid)
-                            score_key(t, i_cur, V + (int64_t)i_cur * d, sg - gm, sn - ym, p_i, x2, t != tprev, cq0);
+                        if (t < nk) {
+                            if (t != tprev) {
+                                sn -= ym;
+                                s0 = fmaf(pent, c0, fmaf(-pdep, sn, s0));
+                                const float mn = fmaxf(m0, pdep * sn);
+                                if (sub == 0) {
+                                    sk[t] = s0;
+                                    col[t] = sn;
+                                    if (mn > m0) mk[t] = mn;
+                                }
+                                m0 = mn;
+                            }
+                            score_key(t, i_cur, s0, sn, p_i, x2, m0, false);
+                        }
                         row = rown;
                         i_cur = i_next;
                         i_next = i_nn;
-#pragma unroll
-                        for (int m = 0; m < 8; ++m) cq0[m] = cqn[m];
                         p_i = p_n;
                         x2 = x2_n;
+                        s0 = s_n;
+                        m0 = m_n;
+                        c0 = c_n;
                     }
                 }
                 first = false;
-                // the block's least score
-                {
-                    const float wb = warp_min(lmin);
-                    if (lane == 0) red[wid] = wb;
-                    if (tid == 0) s_bkey = ~0ull;
-                }
                 __syncthreads();
-                float bmin = INFINITY;
-                for (int w = 0; w < SWT / 32; ++w) bmin = fminf(bmin, red[w]);
-                // the lanes that attain it score their position's pairs again (the
-                // same operations on the same inputs); the smallest (i, j) wins
-                unsigned long long mykey = ~0ull;
-                int myt = -1, myq = -1;
-                if (bmin < 0.f && lt >= 0 && lmin == bmin) {
-                    const float Pm = P - lp;
-                    const VT *vr = V + (int64_t)li * d;
-                    for (int q = 0; q < nadd; ++q) {
-                        if (((q >> 3) & (QL - 1)) != sub) continue;  // this lane's slots
-                        const float sc = any_score<DPL, VT>(make_float4(sB[q], sK[q], sH[q], sP[q]),
-                                                            __ldcs(cb + (size_t)lt * Ep + q), lp, lA, Pm, P, P2, N,
-                                                            vr, mu, g, Wt, Ep, q);
-                        if (sc == bmin) {
-                            const unsigned long long key = ((unsigned long long)(uint32_t)li << 32) | (uint32_t)idxj[q];
-                            if (key < mykey) {
-                                mykey = key;
-                                myt = lt;
-                                myq = q;
+                const int th = s_heavy;
+                if (th >= 0) {  // (uniform) the heavy key's pairs: |g - u_i + u_j|^2, warps split the columns
+                    constexpr int CPW = d / SWW;
+                    const int ih = kb[th];
+                    const float p_i = pk[th];
+                    for (int q0 = 0; q0 < nadd; q0 += 32) {
+                        const int q = q0 + lane;
+                        const float p_j = sP[q];
+                        float gv = 0.f;
+#pragma unroll
+                        for (int e = 0; e < CPW; ++e) {
+                            const int c = wid * CPW + e;
+                            const float wi = load_v(V, (int64_t)ih * d + c) - mu[c];
+                            const float gp = fmaf(p_j, Wt[c * Ep + q], fmaf(-p_i, wi, g[c]));
+                            gv = fmaf(gp, gp, gv);
+                        }
+                        partA[wid * Ep + q] = gv;
+                    }
+                    __syncthreads();
+                    if (wid == 0) {
+                        const float alpha = p_i * p_i * xk[th] - 2.f * p_i * sk[th];
+                        const float Ai = alpha * P2 + N * p_i * (2.f * P - p_i);
+                        const float Pm = P - p_i;
+                        for (int q = lane; q < nadd; q += 32) {
+                            float gv = 0.f;
+#pragma unroll
+                            for (int w = 0; w < SWW; ++w) gv += partA[w * Ep + q];
+                            const float Pp = Pm + sP[q];
+                            const float sc = 16.f * Pp * Pp >= P2
+                                                 ? fast_score(make_float4(sB[q], sK[q], sH[q], sP[q]),
+                                                              cb[(size_t)q * cs + th], p_i, Ai, Pm)
+                                                 : vector_score(gv, P, p_i, sP[q], P2, N);
+                            if (sc < lmin || (sc == lmin && (ih < li || (ih == li && idxj[q] < idxj[lq])))) {
+                                lmin = sc;
+                                lt = th;
+                                li = ih;
+                                lq = q;
                             }
                         }
                     }
-                    if (mykey != ~0ull) atomicMin(&s_bkey, mykey);
+                }
+                // the block's least score; the smallest (i, j) among the lanes that hold it
+                {
+                    const float wb = warp_min(lmin);
+                    if (lane == 0) red[wid] = wb;
                 }
                 __syncthreads();
-                if (mykey != ~0ull && mykey == s_bkey) {
-                    s_bt = myt;
-                    s_bq = myq;
-                }
-                __syncthreads();
-                const float bs = s_bkey != ~0ull ? bmin : INFINITY;
-                const unsigned long long bk = s_bkey;
-                if (!(bs < 0.f)) break;  // no pair strictly decreases es
+                float bmin = INFINITY;
+                for (int w = 0; w < SWW; ++w) bmin = fminf(bmin, red[w]);
+                if (!(bmin < 0.f)) break;  // no pair strictly decreases es (uniform)
                 if (taken >= MS) {
                     cap = 1;
                     break;
                 }
-                // apply: g += u_j - u_i, P += p_j - p_i; slot qj of the pool takes i
-                const int bi = (int)(bk >> 32), bj = (int)(bk & 0xffffffffu);
-                const int tb = s_bt, qj = s_bq;
-                const float p_i = pk[tb];
-                const float p_j = pj[qj];
-                for (int c = tid; c < d; c += SWT) {
-                    wdep[c] = load_v(V, (int64_t)bi * d + c) - mu[c];
-                    wtmp[c] = Wt[c * Ep + qj];
+                const unsigned long long mykey = ((unsigned long long)(uint32_t)li << 32) | (uint32_t)idxj[lq];
+                const bool mine = lt >= 0 && lmin == bmin;
+                if (mine) atomicMin(&s_bkey, mykey);
+                __syncthreads();
+                if (mine && mykey == s_bkey) {
+                    s_bt = lt;
+                    s_bq = lq;
                 }
                 __syncthreads();
-                float gl2 = 0.f, x2n = 0.f;
+                // apply: g += u_j - u_i, P += p_j - p_i; slot qj of the pool takes i
+                const unsigned long long bk = s_bkey;
+                const int bi = (int)(bk >> 32), bj = (int)(bk & 0xffffffffu);
+                const int tb = s_bt, qj = s_bq;
+                const float p_i = pk[tb], x_i = xk[tb];
+                const float p_j = sP[qj], x_j = xj[qj];
+                float gl2 = 0.f;
                 for (int c = tid; c < d; c += SWT) {
-                    const float gn = g[c] + p_j * wtmp[c] - p_i * wdep[c];
+                    const float wi = load_v(V, (int64_t)bi * d + c) - mu[c];
+                    const float wj = Wt[c * Ep + qj];
+                    const float gn = g[c] + p_j * wj - p_i * wi;
                     g[c] = gn;
-                    Wt[c * Ep + qj] = wdep[c];
+                    wdep[c] = wi;
+                    wtmp[c] = wj;
+                    Wt[c * Ep + qj] = wi;
                     gl2 = fmaf(gn, gn, gl2);
-                    x2n = fmaf(wtmp[c], wtmp[c], x2n);
                 }
+                P = P - p_i + p_j;
+                N = block_sum(gl2, red2);  // (its barrier ends every read above)
                 if (tid == 0) {
                     idxj[qj] = bi;
-                    pj[qj] = p_i;
+                    sP[qj] = p_i;
+                    xj[qj] = x_i;
                     kb[tb] = bj;
                     pk[tb] = p_j;
+                    xk[tb] = x_j;
+                    mk[tb] = INFINITY;
                     a.swap_out[rb * MS + taken] = bi;
                     a.swap_in[rb * MS + taken] = bj;
                 }
-                P = P - p_i + p_j;
-                N = block_sum(gl2, red);
-                x2n = block_sum(x2n, red);
-                if (tid == 0) xk[tb] = x2n;
+                pent = p_j;
+                pdep = p_i;
                 tprev = tb;
                 qprev = qj;
-                __syncthreads();
                 ++taken;
             }
             if (tid == 0) {
@@ -904,12 +919,12 @@ inline int pool_slots(int E) { return std::max(32, (E + 31) / 32 * 32); }
 template <int DPL> size_t ls_smem(int Ep)
 {
     constexpr int d = DPL * 32;
-    return sizeof(float) * (10 * (size_t)d + (size_t)d * Ep + 7 * (size_t)Ep + 32 + 8 + 256) + 64;
+    return sizeof(float) * (10 * (size_t)d + (size_t)d * Ep + (6 + 2 * SWW) * (size_t)Ep + 8);
 }
 
 }  // namespace
 
-// ls_bps(R) resident blocks per SM (the launch bounds guarantee the registers
+// ls_bps resident blocks per SM (the launch bounds guarantee the registers
 // for it); the workspace is sized by the same count, queried from the current device
 static unsigned ls_grid(const RowsDev &R)
 {
@@ -930,7 +945,7 @@ static size_t ls_table_bytes(const RowsDev &R, int E)
 size_t long_swap_workspace(const RowsDev &R, int nb, int E, int max_swaps)
 {
     (void)nb, (void)max_swaps;
-    return ls_array_bytes(R) * 4 + ls_table_bytes(R, E);
+    return ls_array_bytes(R) * 7 + ls_table_bytes(R, E);
 }
 
 fw_status long_swap(const RowsDev &R, const int32_t *k, int nb, const fw_gap_out &topk, int E, int max_swaps,
@@ -965,11 +980,14 @@ fw_status long_swap(const RowsDev &R, const int32_t *k, int nb, const fw_gap_out
     a.kbuf = (int32_t *)(w + 1 * arr);
     a.pbuf = (float *)(w + 2 * arr);
     a.xbuf = (float *)(w + 3 * arr);
-    a.cbuf = (float *)(w + 4 * arr);
-    const bool lng = ls_bps(R) == LS_BPS_LONG;
+    a.sbuf = (float *)(w + 4 * arr);
+    a.mbuf = (float *)(w + 5 * arr);
+    a.kebuf = (uint32_t *)(w + 6 * arr);
+    a.cbuf = (float *)(w + 7 * arr);
     FW_DISPATCH(R.d, R.v_dtype, {
         const size_t smem = ls_smem<DPL>(a.Ep);
-        auto kern = lng ? k_long_swap<DPL, VT, LS_BPS_LONG> : k_long_swap<DPL, VT, LS_BPS_SHORT>;
+        constexpr int SHORT = DPL <= 4 ? LS_BPS_SHORT : LS_BPS_LONG;
+        auto kern = ls_bps(R) == LS_BPS_LONG ? k_long_swap<DPL, VT, LS_BPS_LONG> : k_long_swap<DPL, VT, SHORT>;
         FW_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         FW_LAUNCH(kern, grid, SWT, smem, s, a);
     });
