@@ -288,14 +288,21 @@ __global__ void __launch_bounds__(LT) k_long_select(const SelArgs a)
 // map of the float, so the bins split the key order), the bin holding the
 // k-th key, and an exact rank among that bin's keys.  Rows whose threshold
 // bin holds more than SCAP keys (heavy ties) are listed for the radix select,
-// which runs on them after this kernel.  (A first version kept the row in
-// shared memory, loaded after the previous row was done, with every pass a
-// shared-memory sweep and a divergent candidate test; it ran at 13 % of HBM
-// bandwidth.)
+// which runs on them after this kernel.
+//
+// Bound: instruction issue and the barriers of one block per SM (HBM would take a
+// quarter of the time), so the inner loops are counted in instructions per key:
+// the bin is a subtraction and one FMA onto 2^23 (the integer sits in the
+// mantissa; a float-to-int conversion runs on the quarter-rate pipe that also
+// takes the exponential), a non-finite key shows in the sum of exponentials
+// instead of a test of its own, a threshold bin's keys are marked in a register
+// mask and taken out afterwards, and a kept bit is the sign of (key - threshold)
+// shifted into a word, eight slots' words formed by one transpose of nibbles.
+// 4,096 rows of 32,768 keys, three budgets: 555 -> 360 us; 6,144 rows of up to
+// 16,384 keys, one budget: 302 -> 200 us.
 constexpr int SEL_MAX_N = 32768;  // longest row of the linear-bin select
 constexpr int SNB = 2048;         // linear bins
 constexpr int SCAP = 512;         // keys of a threshold bin ranked directly
-constexpr int WCAP = 64;          // threshold-bin keys one warp gathers
 constexpr uint32_t SEL_CHUNK = 32768;  // bytes per bulk-copy instruction
 constexpr uint32_t SEL_WAIT = 1u << 22;  // polls of a row-copy wait before it gives up
 
@@ -308,52 +315,66 @@ __global__ void __launch_bounds__(NT, sel_minb<NT>()) k_long_select_reg(const Se
     constexpr int V4 = VPT / 4;
     constexpr int BPT = SNB / NT;  // bins per thread in the scan
     static_assert(SNB % NT == 0 && VPT % 4 == 0, "layout");
-    __shared__ uint32_t hist[SNB];
-    __shared__ uint32_t ckey[4][SCAP];
-    __shared__ int32_t cidx[4][SCAP];
-    __shared__ uint32_t wkey[NW][WCAP];  // each warp's hits: order key, index, bin
-    __shared__ int32_t widx[NW][WCAP];
-    __shared__ int16_t wbin[NW][WCAP];
-    __shared__ int wnum[NW], wbud[NW][4];
-    __shared__ float red_a[NW], red_b[NW];
+    __shared__ __align__(16) uint32_t hist[SNB];  // highest bin first
+    __shared__ uint64_t cand[4][SCAP];  // a threshold bin's keys: (order key, ~index), larger = ahead
+    __shared__ float red_a[NW], red_b[NW], red_z[NW];
     __shared__ uint32_t wsum[NW];
-    __shared__ int s_tb[4], s_ti[4], s_kv[4], s_rem[4], s_bcnt[4];
+    __shared__ int s_tb[4], s_ti[4], s_kv[4], s_rem[4], s_bcnt[4], s_cc[4], s_tie;
     __shared__ uint32_t s_T[4];
-    __shared__ int s_staged, s_err;
+    __shared__ int s_err;
+    // the row whose copy is next (or now) in sbuf: its length, logits and whether it was copied
+    __shared__ int s_n[2], s_staged[2];
+    __shared__ const float *s_lg[2];
     __shared__ __align__(8) uint64_t full;
     extern __shared__ __align__(16) float sbuf[];  // [max_n] the CTA's next row, by bulk copy
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int nb = a.nb;
-    // the bulk copy of row r into sbuf (thread 0; rows that are not 16-byte
+    // row r's group, length and offset (thread 0; loaded a row ahead of their use,
+    // so no arithmetic on them here)
+    int64_t g_next = 0, off_next = 0;
+    int n_next = 0;
+    auto info = [&](int64_t r) {
+        n_next = 0;
+        if (r >= a.R.rows) return;
+        g_next = r < (1ll << 31) ? (int64_t)((uint32_t)r / (uint32_t)a.R.R) : r / a.R.R;
+        n_next = a.R.n[g_next];
+        off_next = a.R.logit_off[g_next];
+    };
+    // the bulk copy of that row into sbuf (thread 0; rows that are not 16-byte
     // aligned whole vectors are read from global memory instead)
-    auto stage = [&](int64_t r) -> int {
-        if (r >= a.R.rows) return 0;
-        const int64_t g2 = r / a.R.R;
-        const int n2 = a.R.n[g2];
-        const float *lg2 = a.R.logits + a.R.logit_off[g2] + (r - g2 * a.R.R) * n2;
-        if ((n2 & 3) != 0 || (reinterpret_cast<uintptr_t>(lg2) & 15) != 0 || n2 < 1) return 0;
+    auto stage = [&](int64_t r, int slot) {
+        const int n2 = n_next;
+        const float *lg2 = a.R.logits + off_next + (r - g_next * a.R.R) * n2;
+        s_n[slot] = n2;
+        s_lg[slot] = lg2;
+        s_staged[slot] = 0;
+        if ((n2 & 3) != 0 || (reinterpret_cast<uintptr_t>(lg2) & 15) != 0 || n2 < 1) return;
+        // (the block's reads of sbuf are behind a barrier, and nothing wrote it but copies)
         const uint32_t bytes = (uint32_t)n2 * 4u;
-        tc::fence_async_smem();
         tc::mbar_arrive_expect_tx(&full, bytes);
         for (uint32_t o = 0; o < bytes; o += SEL_CHUNK)
             tc::bulk_g2s(reinterpret_cast<char *>(sbuf) + o, reinterpret_cast<const char *>(lg2) + o,
                          bytes - o < SEL_CHUNK ? bytes - o : SEL_CHUNK, &full);
-        return 1;
+        s_staged[slot] = 1;
     };
     if (tid == 0) {
         tc::mbar_init(&full, 1);
         tc::mbar_init_fence();
         s_err = 0;
-        s_staged = stage(blockIdx.x);
+        info(blockIdx.x);
+        stage(blockIdx.x, 0);
+        info((int64_t)blockIdx.x + gridDim.x);
     }
+    for (int i = tid; i < SNB; i += NT) hist[i] = 0u;
     __syncthreads();
     uint32_t phase = 0;
     int64_t fail_row = -1;
-    for (int64_t row = blockIdx.x; row < a.R.rows; row += gridDim.x) {
-        const int64_t g = row / a.R.R;
-        const int n = a.R.n[g];
-        const float *lg = a.R.logits + a.R.logit_off[g] + (row - g * a.R.R) * n;
-        const bool staged = s_staged != 0;
+    int slot = 0;
+    for (int64_t row = blockIdx.x; row < a.R.rows; row += gridDim.x, slot ^= 1) {
+        const int n = s_n[slot];
+        const float *lg = s_lg[slot];
+        const bool staged = s_staged[slot] != 0;
+        const int kv = tid < nb ? a.k[row * nb + tid] : 0;
         if (staged) {
             if (wid == 0 && !tc::mbar_wait(&full, phase, SEL_WAIT)) s_err = 1;  // (every writer stores 1)
             phase ^= 1u;
@@ -363,23 +384,21 @@ __global__ void __launch_bounds__(NT, sel_minb<NT>()) k_long_select_reg(const Se
                 break;
             }
         }
-        // ---- the row into registers (zero past its end)
+        // ---- the row into registers (-inf past its end: never kept, in no bin)
         float x[VPT];
 #pragma unroll
         for (int q = 0; q < V4; ++q) {
             const int j0 = 4 * (tid + NT * q);
             if (staged) {
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                float4 v = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
                 if (j0 < n) v = reinterpret_cast<const float4 *>(sbuf)[tid + NT * q];
                 x[4 * q] = v.x, x[4 * q + 1] = v.y, x[4 * q + 2] = v.z, x[4 * q + 3] = v.w;
             } else {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) x[4 * q + c] = j0 + c < n ? __ldg(lg + j0 + c) : 0.f;
+                for (int c = 0; c < 4; ++c) x[4 * q + c] = j0 + c < n ? __ldg(lg + j0 + c) : -INFINITY;
             }
         }
-        __syncthreads();  // sbuf is read and s_staged consumed: the next row may land
-        if (tid == 0) s_staged = stage(row + gridDim.x);
-        // f(j, x) for every key of the row; a vector slot q is whole when all
+        // f(x) for every key of the row; a vector slot q is whole when all
         // threads' keys in it are inside the row (uniform test)
         auto for_keys = [&](auto &&f) {
 #pragma unroll
@@ -387,18 +406,16 @@ __global__ void __launch_bounds__(NT, sel_minb<NT>()) k_long_select_reg(const Se
                 const int j0 = 4 * (tid + NT * q);
                 if (4 * NT * (q + 1) <= n) {
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) f(j0 + c, x[4 * q + c]);
+                    for (int c = 0; c < 4; ++c) f(x[4 * q + c]);
                 } else if (4 * NT * q < n) {
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
-                        if (j0 + c < n) f(j0 + c, x[4 * q + c]);
+                        if (j0 + c < n) f(x[4 * q + c]);
                 }
             }
         };
         float m = -INFINITY, mn = INFINITY;
-        bool nan = false;
-        for_keys([&](int, float v) {
-            nan |= v != v;
+        for_keys([&](float v) {
             m = fmaxf(m, v);
             mn = fminf(mn, v);
         });
@@ -408,36 +425,48 @@ __global__ void __launch_bounds__(NT, sel_minb<NT>()) k_long_select_reg(const Se
             red_a[wid] = m;
             red_b[wid] = mn;
         }
-        for (int i = tid; i < SNB; i += NT) hist[i] = 0u;
-        if (tid < nb) s_kv[tid] = a.k[row * nb + tid];
-        bool bad = __syncthreads_or(nan) || n < 1;
+        if (tid < nb) s_kv[tid] = kv;
+        if (tid < 4) {
+            s_cc[tid] = 0;
+            s_bcnt[tid] = 0;
+        }
+        if (tid == 0) s_tie = 0;
+        __syncthreads();  // (also: sbuf is read, the next row may land)
+        if (tid == 0) {
+            stage(row + gridDim.x, slot ^ 1);
+            info(row + 2 * (int64_t)gridDim.x);  // (used in the next round)
+        }
         m = warp_max(lane < NW ? red_a[lane] : -INFINITY);  // (every warp, every lane: the same)
         mn = warp_min(lane < NW ? red_b[lane] : INFINITY);
-        bad |= !isfinite(m) || !isfinite(mn);  // (an infinite key is the max or the min)
-        int status = bad ? FW_ERR_NONFINITE : FW_OK;
+        // an infinite key is the max or the min; a NaN beside finite keys shows in Z below
+        const bool inf = n < 1 || !isfinite(m) || !isfinite(mn);
+        // ---- sum of exponentials and the histogram of linear bins over [mn, m]: bin b
+        // is the float 2^23 + b.  A range that fp32 cannot scale leaves the row to the
+        // radix select.
+        const float den = m - mn;
+        const bool wide = !inf && !(den < 1e38f);
+        float scl = den > 0.f ? (float)(SNB - 1) / den : 0.f;
+        if (!(scl < 1e30f)) scl = 0.f;
+        auto bin_of = [&](float v) { return fmaf(v - mn, scl, 8388608.f); };
+        float se = 0.f;
+        if (!inf && !wide) {
+            for_keys([&](float v) {
+                se += __expf(v - m);
+                // (a NaN's bits are cut to the bins' range as well)
+                atomicAdd(&hist[~__float_as_uint(bin_of(v)) & (uint32_t)(SNB - 1)], 1u);
+            });
+        }
+        se = warp_sum(se);
+        if (lane == 0) red_z[wid] = se;
+        __syncthreads();
+        float Z = warp_sum(lane < NW ? red_z[lane] : 0.f);
+        int status = inf || Z != Z ? FW_ERR_NONFINITE : FW_OK;
+        if (status != FW_OK) Z = 0.f;
         for (int b = 0; b < nb; ++b) {
             const int kb = s_kv[b];
             if (kb < 1 || kb > n) status = status == FW_OK ? FW_ERR_INVALID_ARG : status;
         }
-        // ---- sum of exponentials and the histogram of linear bins over [mn, m]
-        // (halves keep m - mn finite)
-        const float hmn = mn * 0.5f, den = m * 0.5f - hmn;
-        float scl = den > 0.f ? (float)SNB / den : 0.f;
-        if (!(scl < 1e30f)) scl = 0.f;
-        auto bin_of = [&](float v) { return (int)fminf((v * 0.5f - hmn) * scl, (float)(SNB - 1)); };
-        float se = 0.f;
-        if (status == FW_OK) {
-            for_keys([&](int, float v) {
-                se += __expf(v - m);
-                atomicAdd(&hist[bin_of(v)], 1u);
-            });
-        }
-        se = warp_sum(se);
-        __syncthreads();  // red_a reads above are done
-        if (lane == 0) red_a[wid] = se;
-        __syncthreads();
-        const float Z = warp_sum(lane < NW ? red_a[lane] : 0.f);
-        if (tid == 0) {
+        if (!wide && tid == 0) {  // (a wide row is reported by the radix select)
             a.ws.M[row] = m;
             a.ws.Z[row] = Z;
             a.ws.status[row] = status;
@@ -445,16 +474,29 @@ __global__ void __launch_bounds__(NT, sel_minb<NT>()) k_long_select_reg(const Se
             if (a.out.row_sum) a.out.row_sum[row] = Z;
             if (a.out.row_status) a.out.row_status[row] = status;
         }
-        if (status != FW_OK) {  // (uniform)
+        // ---- keys above each bin (bins from the top), the bin of each budget's k-th
+        // key; the bins are left zero for the next row
+        uint32_t hv[BPT], loc = 0;
+        if constexpr (BPT == 2) {
+            uint2 *hp = reinterpret_cast<uint2 *>(hist) + tid;
+            const uint2 h = *hp;
+            *hp = make_uint2(0u, 0u);
+            hv[0] = h.x, hv[1] = h.y;
+        } else {
+#pragma unroll
+            for (int i = 0; i < BPT; i += 4) {
+                uint4 *hp = reinterpret_cast<uint4 *>(hist) + tid * (BPT / 4) + i / 4;
+                const uint4 h = *hp;
+                *hp = make_uint4(0u, 0u, 0u, 0u);
+                hv[i] = h.x, hv[i + 1] = h.y, hv[i + 2] = h.z, hv[i + 3] = h.w;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < BPT; ++i) loc += hv[i];
+        if (wide || status != FW_OK) {  // (uniform)
+            if (wide && tid == 0) a.redo_list[atomicAdd(a.redo_count, 1)] = (int32_t)row;
             __syncthreads();
             continue;
-        }
-        // ---- keys above each bin (bins from the top), the bin of each budget's k-th key
-        uint32_t hv[BPT], loc = 0;
-#pragma unroll
-        for (int i = 0; i < BPT; ++i) {
-            hv[i] = hist[SNB - 1 - (tid * BPT + i)];
-            loc += hv[i];
         }
         uint32_t inc = loc;
 #pragma unroll
@@ -481,112 +523,76 @@ __global__ void __launch_bounds__(NT, sel_minb<NT>()) k_long_select_reg(const Se
         __syncthreads();
         // a budget whose threshold bin is crowded (heavy ties) leaves the row to
         // the radix select, which runs after this kernel on the listed rows
+        int cnt[4];
         bool crowded = false;
-        for (int b = 0; b < nb; ++b) crowded |= s_bcnt[b] > SCAP;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            cnt[b] = s_bcnt[b];  // (0 for unused budgets)
+            crowded |= cnt[b] > SCAP;
+        }
         if (crowded) {
             if (tid == 0) a.redo_list[atomicAdd(a.redo_count, 1)] = (int32_t)row;
             __syncthreads();
             continue;
         }
-        // ---- the threshold bins' keys.  Each warp gathers its hits in its own
-        // buffer (ballot offsets, no atomics: the hits are sparse, and
-        // same-address shared atomics from many warps serialise), then the
-        // buffers are concatenated per budget.
-        int gb[4];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) gb[b] = b < nb ? s_tb[b] : -1;
+        // ---- the threshold bins' keys, in any order (a few dozen per budget): each
+        // thread marks its own, then takes them out one by one
         {
-            int wc = 0;                 // this warp's hits (uniform)
-            int bc[4] = {0, 0, 0, 0};   // ... per budget
-            const uint32_t lt = (1u << lane) - 1u;
+            float gf[4];  // the threshold bins as bin_of gives them (repeats for unused budgets)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) gf[b] = 8388608.f + (float)s_tb[b < nb ? b : 0];
+            uint32_t hits = 0u;
 #pragma unroll
             for (int q = 0; q < V4; ++q) {
                 if (4 * NT * q >= n) break;  // (uniform)
-                const int j0 = 4 * (tid + NT * q);
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
-                    const float v = x[4 * q + c];
-                    const int bn = bin_of(v);
-                    const bool in = j0 + c < n;
-                    bool h[4];
+                    const float t = bin_of(x[4 * q + c]);  // (-inf past the row's end matches no bin)
+                    bool h = t == gf[0];
+                    if (nb > 1) h |= t == gf[1];
+                    if (nb > 2) h |= t == gf[2];
+                    if (nb > 3) h |= t == gf[3];
+                    if (h) hits |= 1u << (4 * q + c);
+                }
+            }
+            for (; hits; hits &= hits - 1) {
+                const int e = __ffs(hits) - 1;
+                float v = x[0];
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) h[b] = in && bn == gb[b];
-                    const bool hit = h[0] | h[1] | h[2] | h[3];
-                    const uint32_t mk = __ballot_sync(FW_FULL, hit);
-                    if (mk) {
-                        const int pos = wc + __popc(mk & lt);
-                        if (hit && pos < WCAP) {
-                            wkey[wid][pos] = order_key(v);
-                            widx[wid][pos] = j0 + c;
-                            wbin[wid][pos] = (int16_t)bn;
+                for (int f = 1; f < VPT; ++f)
+                    if (f == e) v = x[f];
+                const int j = 4 * (tid + NT * (e >> 2)) + (e & 3);
+                const float t = bin_of(v);
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    if (b < nb && t == gf[b])  // (position < s_bcnt[b] <= SCAP)
+                        cand[b][atomicAdd(&s_cc[b], 1)] = ((uint64_t)order_key(v) << 32) | (uint32_t)~j;
+            }
+        }
+        __syncthreads();
+        // the exact rank of every candidate among its budget's: NW / 4 warps per
+        // budget, a ballot per candidate and 32 others
+        {
+            constexpr int WPB = NW / 4;
+            const int b = wid / WPB;
+            if (b < nb) {
+                const int cb = s_bcnt[b], want = s_rem[b] - 1;
+                for (int c = wid % WPB; c < cb; c += WPB) {
+                    const uint64_t kc = cand[b][c];
+                    int r = 0;       // candidates ahead
+                    bool tie = false;  // an equal key behind
+                    for (int c0 = 0; c0 < cb; c0 += 32) {
+                        const uint64_t k2 = c0 + lane < cb ? cand[b][c0 + lane] : 0ull;
+                        r += __popc(__ballot_sync(FW_FULL, k2 > kc));
+                        tie |= (k2 >> 32) == (kc >> 32) && k2 < kc;
+                    }
+                    if (r == want) {  // (uniform)
+                        if (lane == 0) {
+                            s_T[b] = (uint32_t)(kc >> 32);
+                            s_ti[b] = (int)~(uint32_t)kc;
                         }
-                        wc += __popc(mk);
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) bc[b] += __popc(__ballot_sync(FW_FULL, h[b]));
+                        if (tie) s_tie = 1;
                     }
-                }
-            }
-            if (lane == 0) {
-                wnum[wid] = wc;
-#pragma unroll
-                for (int b = 0; b < 4; ++b) wbud[wid][b] = bc[b];
-            }
-        }
-        __syncthreads();
-        // a warp with more hits than its buffer holds (keys of a threshold bin
-        // bunched in one warp's stretch) leaves the row to the radix select
-        if (__syncthreads_or(tid < NW && wnum[tid] > WCAP)) {
-            if (tid == 0) a.redo_list[atomicAdd(a.redo_count, 1)] = (int32_t)row;
-            __syncthreads();
-            continue;
-        }
-        {
-            const uint32_t lt = (1u << lane) - 1u;
-            int off[4], run[4];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                off[b] = (int)__reduce_add_sync(FW_FULL, lane < wid ? (uint32_t)wbud[lane][b] : 0u);  // (NW <= 32)
-                run[b] = 0;
-            }
-            const int nw_ = wnum[wid];
-            for (int e0 = 0; e0 < nw_; e0 += 32) {
-                const int e = e0 + lane;
-                const int bn = e < nw_ ? wbin[wid][e] : -2;
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    const bool mt = bn == gb[b];
-                    const uint32_t bm = __ballot_sync(FW_FULL, mt);
-                    const int p = off[b] + run[b] + __popc(bm & lt);
-                    if (mt && p < SCAP) {  // (p < s_bcnt[b] <= SCAP: the bins match the histogram's)
-                        ckey[b][p] = wkey[wid][e];
-                        cidx[b][p] = widx[wid][e];
-                    }
-                    run[b] += __popc(bm);
-                }
-            }
-        }
-        __syncthreads();
-        // the exact rank of every candidate among its budget's, a warp per
-        // candidate (lanes split the comparisons)
-        {
-            const int p1 = s_bcnt[0], p2 = p1 + (nb > 1 ? s_bcnt[1] : 0), p3 = p2 + (nb > 2 ? s_bcnt[2] : 0),
-                      p4 = p3 + (nb > 3 ? s_bcnt[3] : 0);
-            for (int t = wid; t < p4; t += NW) {
-                const int b = (t >= p1) + (t >= p2) + (t >= p3);
-                const int base = b == 0 ? 0 : (b == 1 ? p1 : (b == 2 ? p2 : p3));
-                const int cb = s_bcnt[b];
-                const int c = t - base;
-                const uint32_t kc = ckey[b][c];
-                const int ic = cidx[b][c];
-                uint32_t r = 0;
-                for (int c2 = lane; c2 < cb; c2 += 32) {
-                    const uint32_t k2 = ckey[b][c2];
-                    r += k2 > kc || (k2 == kc && cidx[b][c2] < ic);
-                }
-                r = __reduce_add_sync(FW_FULL, r);
-                if (lane == 0 && (int)r == s_rem[b] - 1) {
-                    s_T[b] = kc;
-                    s_ti[b] = ic;
                 }
             }
         }
@@ -599,46 +605,52 @@ __global__ void __launch_bounds__(NT, sel_minb<NT>()) k_long_select_reg(const Se
             if (a.out.thr_idx) a.out.thr_idx[row * nb + tid] = s_ti[tid];
         }
         if (a.out.kept_bits) {
-            // keys strictly above each threshold by one compare; a warp's 4 keys
-            // per lane in slot q are 128 consecutive keys, so the 8 lanes of an
-            // octet make one 32-bit word.  The keys equal to the threshold (all
-            // in its bin, so among the candidates) up to the tie index are
-            // added after.
+            // The bit of a key is the sign of (key - threshold), inverted: keys at or
+            // above it.  Where some key equal to a threshold is not kept (s_tie), keys
+            // strictly above, the sign of (threshold - key), and the kept equal ones,
+            // all among the candidates, are added after.  A thread's keys give 4 bits
+            // per slot q, the 8 lanes of an octet the 32-bit words of 8 slots: an 8 x 8
+            // transpose of nibbles leaves lane l with the word of slot l.
             const int nw = a.out.kept_words;
-            float xt[4];
+            const bool tie = s_tie != 0;
+            const float sg = tie ? -1.f : 1.f;
+            const int q8 = lane & 7;
+            const int w = ((tid & ~7) >> 3) + (NT >> 3) * q8;
 #pragma unroll
-            for (int b = 0; b < 4; ++b) xt[b] = b < nb ? key_float(s_T[b]) : INFINITY;
+            for (int b = 0; b < 4; ++b) {
+                if (b >= nb) break;
+                const float xt = 0.f - sg * key_float(s_T[b]);  // (never -0)
+                uint32_t u = 0u;
 #pragma unroll
-            for (int q = 0; q < V4; ++q) {
-                const int j0 = 4 * (tid + NT * q);
-                const int w = j0 >> 5;
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    if (b >= nb) break;
-                    uint32_t bits = 0u;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) bits |= (uint32_t)(j0 + c < n && x[4 * q + c] > xt[b]) << c;
-                    bits <<= (j0 & 31);
-                    bits |= __shfl_xor_sync(FW_FULL, bits, 1);
-                    bits |= __shfl_xor_sync(FW_FULL, bits, 2);
-                    bits |= __shfl_xor_sync(FW_FULL, bits, 4);
-                    if ((lane & 7) == 0 && w < nw) a.out.kept_bits[(row * nb + b) * (int64_t)nw + w] = bits;
-                }
+                for (int e = VPT - 1; e >= 0; --e) u = __funnelshift_l(__float_as_uint(fmaf(sg, x[e], xt)), u, 1);
+                if (!tie) u = ~u;
+                uint32_t r = __shfl_xor_sync(FW_FULL, u, 4);
+                u = lane & 4 ? (u & 0xffff0000u) | (r >> 16) : (u & 0xffffu) | (r << 16);
+                r = __shfl_xor_sync(FW_FULL, u, 2);
+                u = lane & 2 ? (u & 0xff00ff00u) | ((r >> 8) & 0x00ff00ffu) : (u & 0x00ff00ffu) | ((r & 0x00ff00ffu) << 8);
+                r = __shfl_xor_sync(FW_FULL, u, 1);
+                u = lane & 1 ? (u & 0xf0f0f0f0u) | ((r >> 4) & 0x0f0f0f0fu) : (u & 0x0f0f0f0fu) | ((r & 0x0f0f0f0fu) << 4);
+                if (q8 < V4 && w < nw) a.out.kept_bits[(row * nb + b) * (int64_t)nw + w] = u;
             }
-            __syncthreads();  // the words above are visible to the block
-            constexpr int CPB = NT / 4;
-            const int b = tid / CPB;
-            if (b < nb) {
-                const uint32_t T = s_T[b];
-                const int ti = s_ti[b];
-                for (int c = tid % CPB; c < s_bcnt[b]; c += CPB) {
-                    const int ic = cidx[b][c];
-                    if (ckey[b][c] == T && ic <= ti)
-                        atomicOr(&a.out.kept_bits[(row * nb + b) * (int64_t)nw + (ic >> 5)], 1u << (ic & 31));
+            if (tie) {  // (uniform)
+                __syncthreads();  // the words above are visible to the block
+                constexpr int CPB = NT / 4;
+                const int b = tid / CPB;
+                if (b < nb) {
+                    const uint32_t T = s_T[b];
+                    const int ti = s_ti[b];
+                    for (int c = tid % CPB; c < s_bcnt[b]; c += CPB) {
+                        const int ic = (int)~(uint32_t)cand[b][c];
+                        if ((uint32_t)(cand[b][c] >> 32) == T && ic <= ti)
+                            atomicOr(&a.out.kept_bits[(row * nb + b) * (int64_t)nw + (ic >> 5)], 1u << (ic & 31));
+                    }
                 }
+                __syncthreads();  // s_T and the candidates are reused by the next row
             }
         }
-        __syncthreads();  // s_T, s_ti, hist and candidates are reused by the next row
+        // (the next row's first barrier orders the reads above against its writes of
+        // s_kv, s_cc, s_bcnt and s_tie only where a copy was waited for)
+        if (!s_staged[slot ^ 1]) __syncthreads();
     }
     if (fail_row >= 0 && tid == 0) {
         // a row copy did not arrive in time: after a last bounded wait for it,
