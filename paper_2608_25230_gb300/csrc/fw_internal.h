@@ -40,7 +40,7 @@ fw_status best_subset_stats(const RowsDev &R, const void *ws, fw_best_subset_sta
 struct LongWs {
     float *M, *Z;          // [rows]
     uint32_t *tk;          // [rows][nb]
-    int32_t *ti;           // [rows][nb]
+    int32_t *ti;           // [rows][nb] (INT_MAX where every key equal to the threshold is kept)
     int32_t *status;       // [rows]
 };
 bool long_pv_tc_supported(const RowsDev &R, int nb);

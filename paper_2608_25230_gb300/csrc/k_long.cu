@@ -319,7 +319,8 @@ __global__ void __launch_bounds__(NT, sel_minb<NT>()) k_long_select_reg(const Se
     __shared__ uint64_t cand[4][SCAP];  // a threshold bin's keys: (order key, ~index), larger = ahead
     __shared__ float red_a[NW], red_b[NW], red_z[NW];
     __shared__ uint32_t wsum[NW];
-    __shared__ int s_tb[4], s_ti[4], s_kv[4], s_rem[4], s_bcnt[4], s_cc[4], s_tie;
+    __shared__ int s_tb[4], s_ti[4], s_kv[4], s_rem[4], s_bcnt[4], s_cc[4];
+    __shared__ int s_tie;  // bit b: budget b drops a key equal to its threshold
     __shared__ uint32_t s_T[4];
     __shared__ int s_err;
     // the row whose copy is next (or now) in sbuf: its length, logits and whether it was copied
@@ -591,7 +592,7 @@ __global__ void __launch_bounds__(NT, sel_minb<NT>()) k_long_select_reg(const Se
                             s_T[b] = (uint32_t)(kc >> 32);
                             s_ti[b] = (int)~(uint32_t)kc;
                         }
-                        if (tie) s_tie = 1;
+                        if (tie) atomicOr(&s_tie, 1 << b);
                     }
                 }
             }
@@ -600,7 +601,8 @@ __global__ void __launch_bounds__(NT, sel_minb<NT>()) k_long_select_reg(const Se
         // ---- thresholds and kept bits
         if (tid < nb) {
             a.ws.tk[row * nb + tid] = s_T[tid];
-            a.ws.ti[row * nb + tid] = s_ti[tid];
+            // (for the products: no index test where every equal key is kept)
+            a.ws.ti[row * nb + tid] = (s_tie >> tid) & 1 ? s_ti[tid] : 0x7fffffff;
             if (a.out.thr_key) a.out.thr_key[row * nb + tid] = s_T[tid];
             if (a.out.thr_idx) a.out.thr_idx[row * nb + tid] = s_ti[tid];
         }

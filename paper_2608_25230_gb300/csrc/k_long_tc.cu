@@ -477,6 +477,13 @@ __device__ __forceinline__ uint32_t cvt_bf16x2(float hi_elem, float lo_elem)
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi_elem), "f"(lo_elem));
     return r;
 }
+// all ones where a >= b, else 0
+__device__ __forceinline__ uint32_t set_ge(float a, float b)
+{
+    uint32_t r;
+    asm("set.ge.u32.f32 %0, %1, %2;" : "=r"(r) : "f"(a), "f"(b));
+    return r;
+}
 __device__ __forceinline__ void cp_async_mbar_arrive(uint64_t *bar)
 {
     asm volatile("cp.async.mbarrier.arrive.shared.b64 [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
@@ -489,9 +496,11 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
     constexpr int RT = TM / NBB < MAXRT ? TM / NBB : MAXRT;
     constexpr int PW = pvm_pw<D>();
     constexpr int NT = pvm_nt<D>();
-    constexpr int NPROD = PW * 32;
-    constexpr int TPR = NPROD / MAXRT;          // producer threads per row
-    constexpr int KPTH = KS / TPR;              // keys per producer thread and stage (4 or 8)
+    // the producer warps work in sets of 8, each taking every NSET-th stage: 8
+    // threads per row, 8 keys (one 16-byte vector per band row and term) each
+    constexpr int NSET = PW / 8;
+    constexpr int TPR = 8, KPTH = KS / TPR;
+    static_assert(MAXRT * TPR == 256 && KPTH == 8 && NSET <= ASLOTS, "producer layout");
     constexpr int NVBOX = D / 64;               // 64-dim groups of V
     constexpr int NG = NVBOX + 1;               // ... and one group of ones (the band masses)
     constexpr int B_SLOT_BYTES = NG * KS * 128;
@@ -576,10 +585,10 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
         s_err = 0;
         for (int x = 0; x < PVM_BS; ++x) {
             tc::mbar_init(&fullB[x], 1);
-            tc::mbar_init(&freeB[x], PW + 1);
+            tc::mbar_init(&freeB[x], 8 + 1);
         }
         for (int x = 0; x < ASLOTS; ++x) {
-            tc::mbar_init(&fullA[x], PW);
+            tc::mbar_init(&fullA[x], 8);
             tc::mbar_init(&freeA[x], 1);
         }
         for (int x = 0; x < NACC; ++x) tc::mbar_init(&accfree[x], PW);
@@ -712,33 +721,48 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
     } else {
         // --------------------------------------------------------- producers
         const int pw = wid - 2;                  // 0..PW-1
-        const int ptid = tid - 64;               // 0..NPROD-1
+        const int set = pw >> 3;                 // its stages: it % NSET == set
+        const int ptid = (tid - 64) & 255;       // thread of the set
         const int rr = ptid / TPR;               // row of the tile (0..31)
-        const int kq = ptid % TPR;               // this thread's KPTH keys of the stage
-        const int kc = kq * KPTH / 8, hk = (kq * KPTH) % 8;  // 8-key chunk and first key in it
+        const int kc = ptid % TPR;               // this thread's 8-key chunk of the stage
         const int quarter = wid & 3, part = pw >> 2;  // TMEM lanes / columns this warp flushes
         float racc[FCOLS];
 #pragma unroll
         for (int i = 0; i < FCOLS; ++i) racc[i] = 0.f;
         float rmass = 0.f;
         const bool live = rr < nr && rok[rr];
+        // (a dead row's masses are garbage: they reach its own accumulator rows only)
         const float Mr = live ? rowM[rr] : 0.f, Zr = live ? rowZi[rr] : 0.f;
+        // thresholds in descending order (the sets are nested along it): key y is in set
+        // b when y >= xt[b], or where some key equal to xt[b] is not, by its index
         float xt[NB];
         int tix[NB];
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
-            const uint32_t tk = live ? rtk[rr][b] : 0u;
+            const uint32_t tk = vote ? vT[b] : (live ? rtk[rr][b] : 0u);
             xt[b] = __uint_as_float((tk & 0x80000000u) ? (tk & 0x7fffffffu) : ~tk);
-            tix[b] = live ? rti[rr][b] : -1;
+            tix[b] = vote ? vL[b] : (live ? rti[rr][b] : 0x7fffffff);
         }
+#pragma unroll
+        for (int x = 1; x < NB; ++x)
+#pragma unroll
+            for (int y = x; y > 0; --y)
+                if (xt[y] > xt[y - 1] || (xt[y] == xt[y - 1] && tix[y] < tix[y - 1])) {
+                    const float f = xt[y];
+                    xt[y] = xt[y - 1], xt[y - 1] = f;
+                    const int e = tix[y];
+                    tix[y] = tix[y - 1], tix[y - 1] = e;
+                }
+        bool ties = false;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) ties |= tix[b] != 0x7fffffff;
         uint32_t boff[NBB];
 #pragma unroll
         for (int b = 0; b < NBB; ++b) {
             const int m = b * RT + rr;
-            boff[b] = (uint32_t)((m >> 3) * 1024 + (m & 7) * 128 + ((kc ^ (m & 7)) << 4) + 2 * hk);
+            boff[b] = (uint32_t)((m >> 3) * 1024 + (m & 7) * 128 + ((kc ^ (m & 7)) << 4));
         }
         bool ok = true;
-        auto chunk_end = [&](int st) { return st % CH == CH - 1 || st == nst - 1; };
         auto flush = [&](int st) {
             tc::fence_after_sync();
             const int buf = (st / CH) % NACC;
@@ -752,56 +776,55 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&accfree[buf]);
         };
-        for (int it = 0; it < nst; ++it) {
+        int next = 0;  // the next chunk to flush
+        const int nch = (nst + CH - 1) / CH;
+        auto flush_to = [&](int st) {  // the chunks whose last stage is at most st
+            for (; next < nch && min(next * CH + CH - 1, nst - 1) <= st; ++next) flush(next * CH);
+        };
+        for (int it = set; it < nst; it += NSET) {
             const int bs = it % PVM_BS, as = it % ASLOTS, j0 = it * KS;
-            if (ok) ok = tc::mbar_wait(&fullB[bs], (uint32_t)(it / PVM_BS) & 1u, WAIT_POLLS);
-            // the A slot was last read by the MMAs of stage it - ASLOTS (which also
-            // closes chunk it - ASLOTS for the flush below)
+            // the A slot was last read by the MMAs of stage it - ASLOTS.  This wait comes
+            // first: it also means that stage it - PVM_BS, the copy slot's last, is done,
+            // so the parity below can only be this stage's.
             if (ok && it >= ASLOTS) ok = tc::mbar_wait(&freeA[as], (uint32_t)((it / ASLOTS) - 1) & 1u, WAIT_POLLS);
+            if (ok) ok = tc::mbar_wait(&fullB[bs], (uint32_t)(it / PVM_BS) & 1u, WAIT_POLLS);
             if (!ok) break;
             uint8_t *aslot = sA + as * A_SLOT_BYTES;
             if (rr < RT) {
-                const float *lr = sL + (bs * MAXRT + rr) * KS + kq * KPTH;
-                float xs[KPTH];
+                auto load8 = [](const float *src, float (&v)[KPTH]) {
+                    const float4 a4 = *reinterpret_cast<const float4 *>(src), b4 = *reinterpret_cast<const float4 *>(src + 4);
+                    v[0] = a4.x, v[1] = a4.y, v[2] = a4.z, v[3] = a4.w;
+                    v[4] = b4.x, v[5] = b4.y, v[6] = b4.z, v[7] = b4.w;
+                };
+                float y[KPTH], pv[KPTH];
+                load8(sL + (bs * MAXRT + rr) * KS + kc * KPTH, y);
 #pragma unroll
-                for (int q = 0; q < KPTH / 4; ++q) {
-                    const float4 x4 = *reinterpret_cast<const float4 *>(lr + 4 * q);
-                    xs[4 * q] = x4.x, xs[4 * q + 1] = x4.y, xs[4 * q + 2] = x4.z, xs[4 * q + 3] = x4.w;
+                for (int u = 0; u < KPTH; ++u) pv[u] = __expf(y[u] - Mr) * Zr;
+                if (j0 + KS > n) {  // (uniform) keys past the row's end
+#pragma unroll
+                    for (int u = 0; u < KPTH; ++u)
+                        if (j0 + kc * KPTH + u >= n) pv[u] = 0.f;
                 }
-                float pv[KPTH];
-                uint32_t bdp[KPTH / 2];  // bands of keys 2q, 2q + 1 as 2 x 16 bits
-                bool tie = false;
+                if (vote) load8(sG + bs * KS + kc * KPTH, y);
+                // membership as masks, keys 2q and 2q + 1 in the halves of a word
+                uint32_t in[NB][KPTH / 2];
+                {
+                    uint32_t mk[NB][KPTH];
 #pragma unroll
-                for (int u = 0; u < KPTH; ++u) {
-                    const int j = j0 + kq * KPTH + u;
-                    const float x = xs[u];
-                    pv[u] = (live && j < n) ? __expf(x - Mr) * Zr : 0.f;
-                    int bd = 0;
-                    if (vote) {
-                        const uint32_t gk = order_key(sG[bs * KS + kq * KPTH + u]);
+                    for (int b = 0; b < NB; ++b)
 #pragma unroll
-                        for (int b = 0; b < NB; ++b) bd += !(gk > vT[b] || (gk == vT[b] && j <= vL[b]));
-                    } else {
+                        for (int u = 0; u < KPTH; ++u) mk[b][u] = set_ge(y[u], xt[b]);
+                    if (ties) {  // a key equal to a threshold: its index decides
 #pragma unroll
-                        for (int b = 0; b < NB; ++b) {
-                            bd += x < xt[b];
-                            tie |= x == xt[b];
-                        }
+                        for (int b = 0; b < NB; ++b)
+#pragma unroll
+                            for (int u = 0; u < KPTH; ++u)
+                                if (y[u] == xt[b] && j0 + kc * KPTH + u > tix[b]) mk[b][u] = 0u;
                     }
-                    if (u & 1) bdp[u >> 1] |= (uint32_t)bd << 16;
-                    else bdp[u >> 1] = (uint32_t)bd;
-                }
-                if (tie) {  // a key equal to a threshold: its index decides (rare)
 #pragma unroll
-                    for (int u = 0; u < KPTH; ++u) {
-                        const int j = j0 + kq * KPTH + u;
-                        const float x = xs[u];
-                        int bd = 0;
+                    for (int b = 0; b < NB; ++b)
 #pragma unroll
-                        for (int b = 0; b < NB; ++b) bd += (x < xt[b]) | ((x == xt[b]) & (j > tix[b]));
-                        const uint32_t sh = (u & 1) ? 16u : 0u;
-                        bdp[u >> 1] = (bdp[u >> 1] & ~(0xffffu << sh)) | ((uint32_t)bd << sh);
-                    }
+                        for (int q = 0; q < KPTH / 2; ++q) in[b][q] = __byte_perm(mk[b][2 * q], mk[b][2 * q + 1], 0x5410);
                 }
                 // three bf16 terms per mass, two keys per 32-bit word (key 2q low)
                 uint32_t ph[KPTH / 2], pm[KPTH / 2], pl[KPTH / 2];
@@ -814,26 +837,20 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
                     const float f0 = e0 - __uint_as_float(pm[q] << 16), f1 = e1 - __uint_as_float(pm[q] & 0xffff0000u);
                     pl[q] = cvt_bf16x2(f1, f0);
                 }
+                // band b: the keys of set b that are not in set b - 1 (b = NB: in none)
 #pragma unroll
                 for (int b = 0; b < NBB; ++b) {
-                    uint32_t wh[KPTH / 2], wm[KPTH / 2], wl[KPTH / 2];
-#pragma unroll
-                    for (int q = 0; q < KPTH / 2; ++q) {
-                        const uint32_t msk = __vcmpeq2(bdp[q], (uint32_t)b * 0x00010001u);
-                        wh[q] = ph[q] & msk;
-                        wm[q] = pm[q] & msk;
-                        wl[q] = pl[q] & msk;
-                    }
                     uint8_t *dst = aslot + boff[b];
-                    if constexpr (KPTH == 8) {
-                        *reinterpret_cast<uint4 *>(dst) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
-                        *reinterpret_cast<uint4 *>(dst + A_SPLIT_BYTES) = make_uint4(wm[0], wm[1], wm[2], wm[3]);
-                        *reinterpret_cast<uint4 *>(dst + 2 * A_SPLIT_BYTES) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
-                    } else {
-                        *reinterpret_cast<uint2 *>(dst) = make_uint2(wh[0], wh[1]);
-                        *reinterpret_cast<uint2 *>(dst + A_SPLIT_BYTES) = make_uint2(wm[0], wm[1]);
-                        *reinterpret_cast<uint2 *>(dst + 2 * A_SPLIT_BYTES) = make_uint2(wl[0], wl[1]);
-                    }
+                    auto put = [&](const uint32_t (&w)[KPTH / 2], uint8_t *to) {
+                        uint32_t z[KPTH / 2];
+#pragma unroll
+                        for (int q = 0; q < KPTH / 2; ++q)
+                            z[q] = w[q] & (b < NB ? in[b < NB ? b : 0][q] : ~0u) & (b > 0 ? ~in[b > 0 ? b - 1 : 0][q] : ~0u);
+                        *reinterpret_cast<uint4 *>(to) = make_uint4(z[0], z[1], z[2], z[3]);
+                    };
+                    put(ph, dst);
+                    put(pm, dst + A_SPLIT_BYTES);
+                    put(pl, dst + 2 * A_SPLIT_BYTES);
                 }
             }
             tc::fence_async_smem();
@@ -842,12 +859,13 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
                 tc::mbar_arrive(&fullA[as]);
                 tc::mbar_arrive(&freeB[bs]);  // this warp has read the stage's logits
             }
-            if (it >= ASLOTS && chunk_end(it - ASLOTS)) flush(it - ASLOTS);
+            // chunks whose MMAs the wait above has seen complete
+            flush_to(it - ASLOTS);
         }
         // the last chunks: their MMAs complete before they are read
         for (int st = nst - ASLOTS < 0 ? 0 : nst - ASLOTS; st < nst && ok; ++st) {
             ok = tc::mbar_wait(&freeA[st % ASLOTS], (uint32_t)(st / ASLOTS) & 1u, WAIT_POLLS);
-            if (ok && chunk_end(st)) flush(st);
+            if (ok) flush_to(st);
         }
         if (!ok && lane == 0) atomicOr(&s_err, 1);
         const int m = quarter * 32 + lane;

@@ -1,0 +1,40 @@
+"""The TMA-fed P.V kernel at the stage counts where its producer sets and chunk
+flushes end differently (64-key stages, two sets of producer warps, chunks of
+8 stages), for the gap call and the group vote, ties at the thresholds
+included, against the fp64 oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from tests.test_gpu_long import compare, fw  # noqa: F401  (fw is a fixture)
+from tests.test_gpu_small import rows_batch
+from tests.test_gpu_vote import check_vote, group_budgets, run_vote
+
+pytestmark = pytest.mark.gpu
+
+
+def _batch(n, d, R, ks, ties, seed):
+    rng = np.random.default_rng(seed)
+    L = (rng.normal(size=(R, n)) * 1.5).astype(np.float32)
+    L[:, 0] += 5
+    if ties:
+        L = (np.round(L * 8) / 8).astype(np.float32)  # every threshold has equal keys, some dropped
+    V = rng.normal(size=(1, n, d)).astype(np.float32)
+    return rows_batch(L, V, np.tile(np.asarray(ks, np.int32), (R, 1)), v_dtype="bf16", R=R)
+
+
+# stages 1..11 and 16..19: both sets' last stages, with and without a chunk end near them
+@pytest.mark.parametrize("stages", [1, 2, 3, 7, 8, 9, 10, 11, 16, 17, 18, 19])
+@pytest.mark.parametrize("d", [64, 128])
+def test_stage_counts(fw, stages, d):  # noqa: F811
+    for n in (64 * stages, 64 * stages - 31):
+        ks = [max(1, n // 2), max(1, n // 9), n][: 1 + stages % 3]  # not in order
+        compare(fw, _batch(n, d, 34, ks, stages % 2 == 0, n + d))
+
+
+@pytest.mark.parametrize("n", [64 * 3, 64 * 17 - 5])
+def test_vote_stage_counts(fw, n):  # noqa: F811
+    b = _batch(n, 128, 20, [n // 4, n // 16, n // 2], True, n)
+    s = group_budgets(b)
+    _, _, v = run_vote(fw, b, s)
+    check_vote(oracle.HostRows(b), s, v)
