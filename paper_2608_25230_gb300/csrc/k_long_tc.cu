@@ -454,22 +454,37 @@ __global__ void __launch_bounds__(pv_threads<D>(), 1) k_long_pv_tc(const TcArgs 
 }
 
 // ---------------------------------------------------------------------------
-// The same P.V with one copy warp: V tiles arrive by TMA (64 keys x 64 dims
-// boxes, 128-byte swizzle: the MN-major operand layout) and the stage's
-// logits (64 per row) by 16-byte cp.async, half a warp per row, so the
-// producer warps only build A.  (One bulk copy per 256-byte logit row was
-// tried first: 32 small TMA requests per stage kept the stage time near
-// 1.3 us, about three times the MMA time.)  Warp 0 copies, warp 1 issues the
-// MMAs, the other warps produce: a thread takes KPTH consecutive keys of one
-// row (NB budgets known at compile time) and writes one vector per (band row,
-// term).  Stages whose V rows would cross the end of the group's block (the
-// partial last stage, or a block not aligned to whole rows) go through
-// per-thread cp.async with zero fill instead, and logit rows that are not
-// 16-byte aligned (n not a multiple of 4, misaligned base) through 4-byte
-// cp.async; the barrier tracks every kind.
-template <int D> __host__ __device__ constexpr int pvm_pw() { return D == 128 ? 16 : 8; }  // producer warps
-template <int D> __host__ __device__ constexpr int pvm_nt() { return (pvm_pw<D>() + 2) * 32; }
-constexpr int PVM_BS = 3;                      // copy slots (V + ones + logits)
+// The same P.V with V tiles brought by TMA (64 keys x 64 dims boxes, 128-byte
+// swizzle: the MN-major operand layout).  Warp 0 copies V, warp 1 issues the
+// MMAs, the other 16 warps build A in two sets of 8, one set per stage in
+// turn, so a set has two stage times for its stage.  A thread takes KPTH = 8
+// consecutive keys of one row and writes one 16-byte vector per (band row,
+// term); NB, the number of budgets, is known at compile time, the thresholds are
+// sorted, and membership is a mask per key and budget, so a band's vector is
+// two ANDs per word and no key's band number is computed.
+//
+// What bounds it is the instructions of the producers (the tensor pipe is
+// busy about half the time, and 128 of 152 SMs have a tile at 4,096 rows).
+// Each producer warp therefore copies the logits of its own 4 rows, by 16-byte
+// cp.async a set's stage ahead into a ring of its own: no other warp waits for
+// them, and the copy warp is left with one TMA request per V box.  Tried and
+// slower: one bulk copy per 256-byte logit row (1.3 us per stage), all logits
+// copied by the copy warp (its 16 copies per lane and stage set the pace),
+// plain 32-byte loads by each thread (107M L2 sectors against 40M).
+// Measured on 4,096 rows x 32,768 keys, 3 budgets, the whole gap call: one set,
+// logits by the copy warp, band numbers 980 us; two sets and masks 880; logits
+// by the producers 849.  At d = 64: 580, 474 (one set), and 352 us with both.
+//
+// Stages whose V rows would cross the end of the group's block (the partial last
+// stage, or a block not aligned to whole rows) go through per-thread cp.async
+// with zero fill instead, and logit rows that are not 16-byte aligned (n not a
+// multiple of 4, misaligned base) through 4-byte cp.async.
+constexpr int PVM_PW = 16;                     // producer warps
+constexpr int PVM_NT = (PVM_PW + 2) * 32;      // threads
+constexpr int PVM_BS = 3;                      // copy slots (V + ones)
+// logit slots per producer warp: 20 KB a slot over the 16 warps, and at D = 128 the
+// V slots leave room for two
+template <int D> __host__ __device__ constexpr int pvm_ld() { return D == 128 ? 2 : 3; }
 
 __device__ __forceinline__ uint32_t cvt_bf16x2(float hi_elem, float lo_elem)
 {
@@ -490,12 +505,13 @@ __device__ __forceinline__ void cp_async_mbar_arrive(uint64_t *bar)
 }
 
 template <int D, int NB>
-__global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_constant__ CUtensorMap tmV, const TcArgs a)
+__global__ void __launch_bounds__(PVM_NT, 1) k_long_pv_tma(const __grid_constant__ CUtensorMap tmV, const TcArgs a)
 {
     constexpr int NBB = NB + 1;                 // bands
     constexpr int RT = TM / NBB < MAXRT ? TM / NBB : MAXRT;
-    constexpr int PW = pvm_pw<D>();
-    constexpr int NT = pvm_nt<D>();
+    constexpr int PW = PVM_PW;
+    constexpr int PVM_LD = pvm_ld<D>();
+    constexpr int NT = PVM_NT;
     // the producer warps work in sets of 8, each taking every NSET-th stage: 8
     // threads per row, 8 keys (one 16-byte vector per band row and term) each
     constexpr int NSET = PW / 8;
@@ -507,13 +523,13 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
     constexpr int DN = D + 16;                  // MMA N: the value dims, then 16 columns of masses
     constexpr uint32_t TCOLS = NACC * DN <= 256 ? 256u : 512u;
     constexpr int NC = D / 8;
-    constexpr int FCOLS = D / (PW / 4);         // accumulator columns flushed per warp (32)
+    constexpr int FCOLS = D / (PW / 4);         // accumulator columns flushed per warp
     extern __shared__ uint8_t smraw[];
     uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~(uintptr_t)1023);
     uint8_t *sA = sm;                                     // [ASLOTS][NSPLIT][TM x 128 B]
     uint8_t *sB = sA + ASLOTS * A_SLOT_BYTES;             // [PVM_BS][NG][64 keys x 128 B]
-    float *sL = reinterpret_cast<float *>(sB + PVM_BS * B_SLOT_BYTES);  // [PVM_BS][32][64]
-    float *sG = sL + PVM_BS * MAXRT * KS;                 // [PVM_BS][64] the vote's G
+    // [PW][PVM_LD][5][64]: each producer warp's own copies, its 4 rows' logits and the vote's G
+    float *sL = reinterpret_cast<float *>(sB + PVM_BS * B_SLOT_BYTES);
     float *acc = reinterpret_cast<float *>(sA);           // epilogue: [TM][D + 1]
     __shared__ __align__(8) uint64_t fullB[PVM_BS], freeB[PVM_BS], fullA[ASLOTS], freeA[ASLOTS], accfree[NACC];
     __shared__ uint32_t s_taddr;
@@ -585,7 +601,7 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
         s_err = 0;
         for (int x = 0; x < PVM_BS; ++x) {
             tc::mbar_init(&fullB[x], 1);
-            tc::mbar_init(&freeB[x], 8 + 1);
+            tc::mbar_init(&freeB[x], 1);
         }
         for (int x = 0; x < ASLOTS; ++x) {
             tc::mbar_init(&fullA[x], 8);
@@ -614,9 +630,7 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
 
     if (wid == 0) {
         // ---------------------------------------------------------- copies
-        const uint32_t bbase = tc::smem_u32(sB), lbase = tc::smem_u32(sL);
-        const uint32_t livemask = __ballot_sync(FW_FULL, lane < nr && rok[lane]);
-        const int lc = lane & 15, lh = lane >> 4;  // 16-byte chunk of a logit row, row parity
+        const uint32_t bbase = tc::smem_u32(sB);
         int issued = 0;
         bool ok = true;
         for (int it = 0; it < nst; ++it) {
@@ -628,10 +642,9 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
             }
             const int kn = min(KS, n - j0);  // keys of this stage
             const bool vtma = vrows && kn == KS;
-            const bool live_row = (livemask >> lane) & 1u;
-            // (1) the per-thread copies, each lane's tracked by the barrier: its
-            // pending count rises now and falls when they land, so the phase
-            // cannot complete before them whatever the order of what follows
+            // (1) the per-thread copies of a stage that TMA cannot bring, each lane's
+            // tracked by the barrier: its pending count rises now and falls when they
+            // land, so the phase cannot complete before them
             if (!vtma) {  // V rows past the block's end are zero-filled
                 for (int e = lane; e < KS * NC; e += 32) {
                     const int kk = e / NC, nc = e % NC;
@@ -641,24 +654,8 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
                     const bool in = kk < kn;
                     cp_async16(dst, V + (int64_t)(in ? j0 + kk : 0) * D + nc * 8, in ? 16u : 0u);
                 }
+                cp_async_mbar_arrive(&fullB[bs]);
             }
-            if (lbulk) {  // 16-byte copies, half a warp per row (kn is a multiple of 4)
-                const bool cin = lc * 4 < kn;
-                for (int rp = 0; rp < nr; rp += 2) {
-                    const int r = rp + lh;
-                    if ((livemask >> r) & 1u)
-                        cp_async16(lbase + (uint32_t)(((bs * MAXRT + r) * KS + lc * 4) * 4),
-                                   LG + (int64_t)(r0 + r) * n + j0 + (cin ? lc * 4 : 0), cin ? 16u : 0u);
-                }
-            } else if (live_row) {
-                const uint32_t d0 = lbase + (uint32_t)((bs * MAXRT + lane) * KS * 4);
-                const float *lsrc = LG + (int64_t)(r0 + lane) * n + j0;
-                for (int u = 0; u < kn; ++u) cp_async4(d0 + 4 * u, lsrc + u, 4u);
-            }
-            if (vote)  // the stage's summed masses (zero past the row)
-                for (int e = lane; e < KS; e += 32)
-                    cp_async4(tc::smem_u32(sG + bs * KS + e), GB + j0 + (e < kn ? e : 0), e < kn ? 4u : 0u);
-            cp_async_mbar_arrive(&fullB[bs]);
             // (2) the barrier's one expected arrival, with the bytes of the V boxes
             const uint32_t tx = vtma ? (uint32_t)(NVBOX * 64 * 128) : 0u;
             __syncwarp();
@@ -767,8 +764,9 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
             tc::fence_after_sync();
             const int buf = (st / CH) % NACC;
             const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
-            float v[32];
-            tc::ld32(taddr + lanes + (uint32_t)(buf * DN + part * FCOLS), v);
+            float v[FCOLS];
+            if constexpr (FCOLS == 32) tc::ld32(taddr + lanes + (uint32_t)(buf * DN + part * FCOLS), v);
+            else tc::ld16(taddr + lanes + (uint32_t)(buf * DN + part * FCOLS), v);
 #pragma unroll
             for (int i = 0; i < FCOLS; ++i) racc[i] += v[i];
             if (part == 0) rmass += tc::ld1(taddr + lanes + (uint32_t)(buf * DN + D));
@@ -781,31 +779,74 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
         auto flush_to = [&](int st) {  // the chunks whose last stage is at most st
             for (; next < nch && min(next * CH + CH - 1, nst - 1) <= st; ++next) flush(next * CH);
         };
+        // This warp's 4 rows of logits (and the vote's G) for its stages, PVM_LD - 1 of
+        // them ahead, by cp.async into a ring of its own: no barrier beyond the warp's,
+        // and the copies' instructions are spread over all producers.
+        const int wr = (ptid >> 5) * 4;  // the warp's first row
+        float *ring = sL + (size_t)pw * PVM_LD * 5 * KS;
+        const uint32_t wlive = __ballot_sync(FW_FULL, live);  // (8 lanes per row)
+        const bool gvec = vote && (reinterpret_cast<uintptr_t>(GB) & 15) == 0;
+        auto fetch = [&](int it, int slot) {
+            if (it < nst) {
+                const int j0 = it * KS, kn = min(KS, n - j0);
+                const uint32_t d0 = tc::smem_u32(ring + slot * 5 * KS);
+                if (lbulk) {  // 16-byte copies, half a warp per row (kn is a multiple of 4)
+                    const int c = (lane & 15) * 4;
+                    const bool cin = c < kn;
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int r = 2 * e + (lane >> 4);
+                        if ((wlive >> (8 * r)) & 1u)
+                            cp_async16(d0 + (uint32_t)(r * KS + c) * 4, LG + (int64_t)(r0 + wr + r) * n + j0 + (cin ? c : 0),
+                                       cin ? 16u : 0u);
+                    }
+                } else {
+                    for (int e = lane; e < 4 * KS; e += 32) {
+                        const int r = e / KS, c = e % KS;
+                        if (((wlive >> (8 * r)) & 1u) && c < kn)
+                            cp_async4(d0 + (uint32_t)e * 4, LG + (int64_t)(r0 + wr + r) * n + j0 + c, 4u);
+                    }
+                }
+                if (gvec && kn == KS) {
+                    if (lane < 16) cp_async16(d0 + (uint32_t)(4 * KS + lane * 4) * 4, GB + j0 + lane * 4, 16u);
+                } else if (vote) {  // zero past the row
+                    for (int c = lane; c < KS; c += 32)
+                        cp_async4(d0 + (uint32_t)(4 * KS + c) * 4, GB + j0 + (c < kn ? c : 0), c < kn ? 4u : 0u);
+                }
+            }
+            cp_async_commit();
+        };
+        int slot = 0;
+#pragma unroll
+        for (int e = 0; e < PVM_LD - 1; ++e) fetch(set + e * NSET, e);
         for (int it = set; it < nst; it += NSET) {
-            const int bs = it % PVM_BS, as = it % ASLOTS, j0 = it * KS;
-            // the A slot was last read by the MMAs of stage it - ASLOTS.  This wait comes
-            // first: it also means that stage it - PVM_BS, the copy slot's last, is done,
-            // so the parity below can only be this stage's.
+            const int as = it % ASLOTS, j0 = it * KS;
+            fetch(it + (PVM_LD - 1) * NSET, slot == 0 ? PVM_LD - 1 : slot - 1);
+            asm volatile("cp.async.wait_group %0;" ::"n"(PVM_LD - 1) : "memory");
+            __syncwarp();
+            const float *src = ring + slot * 5 * KS;
+            slot = slot == PVM_LD - 1 ? 0 : slot + 1;
+            float y[KPTH], pv[KPTH];
+            auto load8 = [](const float *q, float (&v)[KPTH]) {
+                const float4 a4 = *reinterpret_cast<const float4 *>(q), b4 = *reinterpret_cast<const float4 *>(q + 4);
+                v[0] = a4.x, v[1] = a4.y, v[2] = a4.z, v[3] = a4.w;
+                v[4] = b4.x, v[5] = b4.y, v[6] = b4.z, v[7] = b4.w;
+            };
+            load8(src + (rr - wr) * KS + kc * KPTH, y);
+#pragma unroll
+            for (int u = 0; u < KPTH; ++u) pv[u] = __expf(y[u] - Mr) * Zr;
+            if (j0 + KS > n) {  // (uniform) keys past the row's end
+#pragma unroll
+                for (int u = 0; u < KPTH; ++u)
+                    if (j0 + kc * KPTH + u >= n) pv[u] = 0.f;
+            }
+            if (vote) load8(src + 4 * KS + kc * KPTH, y);
+            __syncwarp();  // the slot is read: the next fetch may fill it
+            // the A slot was last read by the MMAs of stage it - ASLOTS
             if (ok && it >= ASLOTS) ok = tc::mbar_wait(&freeA[as], (uint32_t)((it / ASLOTS) - 1) & 1u, WAIT_POLLS);
-            if (ok) ok = tc::mbar_wait(&fullB[bs], (uint32_t)(it / PVM_BS) & 1u, WAIT_POLLS);
             if (!ok) break;
             uint8_t *aslot = sA + as * A_SLOT_BYTES;
             if (rr < RT) {
-                auto load8 = [](const float *src, float (&v)[KPTH]) {
-                    const float4 a4 = *reinterpret_cast<const float4 *>(src), b4 = *reinterpret_cast<const float4 *>(src + 4);
-                    v[0] = a4.x, v[1] = a4.y, v[2] = a4.z, v[3] = a4.w;
-                    v[4] = b4.x, v[5] = b4.y, v[6] = b4.z, v[7] = b4.w;
-                };
-                float y[KPTH], pv[KPTH];
-                load8(sL + (bs * MAXRT + rr) * KS + kc * KPTH, y);
-#pragma unroll
-                for (int u = 0; u < KPTH; ++u) pv[u] = __expf(y[u] - Mr) * Zr;
-                if (j0 + KS > n) {  // (uniform) keys past the row's end
-#pragma unroll
-                    for (int u = 0; u < KPTH; ++u)
-                        if (j0 + kc * KPTH + u >= n) pv[u] = 0.f;
-                }
-                if (vote) load8(sG + bs * KS + kc * KPTH, y);
                 // membership as masks, keys 2q and 2q + 1 in the halves of a word
                 uint32_t in[NB][KPTH / 2];
                 {
@@ -855,13 +896,11 @@ __global__ void __launch_bounds__(pvm_nt<D>(), 1) k_long_pv_tma(const __grid_con
             }
             tc::fence_async_smem();
             __syncwarp();
-            if (lane == 0) {
-                tc::mbar_arrive(&fullA[as]);
-                tc::mbar_arrive(&freeB[bs]);  // this warp has read the stage's logits
-            }
+            if (lane == 0) tc::mbar_arrive(&fullA[as]);
             // chunks whose MMAs the wait above has seen complete
             flush_to(it - ASLOTS);
         }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
         // the last chunks: their MMAs complete before they are read
         for (int st = nst - ASLOTS < 0 ? 0 : nst - ASLOTS; st < nst && ok; ++st) {
             ok = tc::mbar_wait(&freeA[st % ASLOTS], (uint32_t)(st / ASLOTS) & 1u, WAIT_POLLS);
@@ -1471,7 +1510,7 @@ template <int D, int NB, int RT> size_t pv_tn_smem()
 template <int D> size_t pv_tma_smem()
 {
     return 1024 + (size_t)ASLOTS * A_SLOT_BYTES + (size_t)PVM_BS * (D / 64 + 1) * KS * 128 +
-           (size_t)PVM_BS * MAXRT * KS * 4 + (size_t)PVM_BS * KS * 4;
+           (size_t)PVM_PW * pvm_ld<D>() * 5 * KS * 4;
 }
 
 template <int D> size_t tc_smem(int RT)
@@ -1519,7 +1558,7 @@ fw_status launch_pv_tma(TcArgs a, const CUtensorMap &mv, cudaStream_t s)
     const unsigned grid = (unsigned)(R.num_groups * a.tiles_per_group);
     auto launch = [&](auto kernel, size_t smem) -> fw_status {
         FW_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        FW_LAUNCH(kernel, grid, (R.d == 128 ? pvm_nt<128>() : pvm_nt<64>()), smem, s, mv, a);
+        FW_LAUNCH(kernel, grid, PVM_NT, smem, s, mv, a);
         return FW_OK;
     };
 #define FW_PV_NB(DD, NN) \
