@@ -211,6 +211,102 @@ __device__ __forceinline__ void stage_value_cols(const VT *V, int n, int d, int 
     }
 }
 
+// A warp's staged rows 0 .. n of DC columns: column c of row r.  Every 4 rows are
+// followed by 16 bytes, so that rows 4 apart, which the lanes of gram_chunk read
+// together 16 bytes at a time, lie on different banks.
+template <int DC> __device__ __forceinline__ int staged_at(int r, int c) { return r * DC + (r >> 2) * 4 + c; }
+__host__ __device__ constexpr int staged_floats(int n, int dc) { return (n + 1) * dc + (n / 4 + 1) * 4; }
+// The Gram matrix of rows 0 .. n (n <= 32), whole 4 x 4 tiles
+constexpr int GRAM_LD = 37;
+__host__ __device__ constexpr int gram_floats(int n) { return (n / 4 + 1) * 4 * GRAM_LD; }
+// Columns [c0, c0 + DC) of the n value rows into that layout, fp32, 8 loads in flight.
+template <int DC, typename VT>
+__device__ __forceinline__ void stage_rows(const VT *V, int n, int d, int c0, float *st, int lane)
+{
+    for (int e0 = 0; e0 < n * DC; e0 += 32 * 8) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int e = e0 + lane + 32 * u;
+            v[u] = e < n * DC ? load_v(V, (int64_t)(e / DC) * d + c0 + e % DC) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int e = e0 + lane + 32 * u;
+            if (e < n * DC) st[staged_at<DC>(e / DC, e % DC)] = v[u];
+        }
+    }
+}
+// The staged columns' part of the Gram matrix of rows 0 .. n into G[x * GRAM_LD + y], both
+// triangles (entries past row n: row n's); `first` stores, later chunks add.  A lane
+// takes 4 x 4 products at a time: 8 16-byte reads per 64 products, where products one by
+// one need 2 reads each.  A product is two chains of SUB / 2 terms per SUB columns, SUB
+// such that a chain has at most D / 4 terms (32 from D = 128 on).
+template <int D, int DC>
+__device__ __forceinline__ void gram_chunk(const float *U, float *G, int n, bool first, int lane)
+{
+    constexpr int SUB = D <= 64 ? D / 2 : DC;
+    const int nt = n / 4 + 1, ntiles = nt * (nt + 1) / 2;  // 4-row blocks
+    for (int q = lane; q < ntiles; q += 32) {
+        int bx = 0, by = q;
+        while (by >= nt - bx) by -= nt - bx, ++bx;
+        by += bx;
+        const float *ux[4], *uy[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            ux[e] = U + staged_at<DC>(min(4 * bx + e, n), 0);
+            uy[e] = U + staged_at<DC>(min(4 * by + e, n), 0);
+        }
+        float tot[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) tot[e] = 0.f;
+#pragma unroll 1
+        for (int c0 = 0; c0 < DC; c0 += SUB) {
+            float sp[16][2];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) sp[e][0] = sp[e][1] = 0.f;
+#pragma unroll 1
+            for (int c = c0; c < c0 + SUB; c += 4) {
+                float4 yv[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) yv[e] = *reinterpret_cast<const float4 *>(uy[e] + c);
+#pragma unroll
+                for (int ex = 0; ex < 4; ++ex) {
+                    const float4 xv = *reinterpret_cast<const float4 *>(ux[ex] + c);
+#pragma unroll
+                    for (int ey = 0; ey < 4; ++ey) {
+                        float *s2 = sp[4 * ex + ey];
+                        s2[0] = fmaf(xv.x, yv[ey].x, s2[0]);
+                        s2[1] = fmaf(xv.y, yv[ey].y, s2[1]);
+                        s2[0] = fmaf(xv.z, yv[ey].z, s2[0]);
+                        s2[1] = fmaf(xv.w, yv[ey].w, s2[1]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < 16; ++e) tot[e] += sp[e][0] + sp[e][1];
+        }
+#pragma unroll
+        for (int ex = 0; ex < 4; ++ex)
+#pragma unroll
+            for (int ey = 0; ey < 4; ++ey) {
+                // (a diagonal tile's mirror entries are the same products in the same order)
+                const int x = 4 * bx + ex, y = 4 * by + ey;
+                float v = tot[4 * ex + ey];
+                if (!first) v += G[x * GRAM_LD + y];
+                tot[4 * ex + ey] = v;
+            }
+#pragma unroll
+        for (int ex = 0; ex < 4; ++ex)
+#pragma unroll
+            for (int ey = 0; ey < 4; ++ey) {
+                const int x = 4 * bx + ex, y = 4 * by + ey;
+                G[x * GRAM_LD + y] = tot[4 * ex + ey];
+                G[y * GRAM_LD + x] = tot[4 * ex + ey];
+            }
+    }
+}
+
 // CTA-wide selection of the m largest of n unsigned order keys, equal keys
 // taken in ascending index order: on return (every thread) T is the m-th
 // largest key and L bounds the indices taken among the keys equal to T (the last

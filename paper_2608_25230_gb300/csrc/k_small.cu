@@ -151,28 +151,47 @@ struct SmallSwapArgs {
     int E, max_swaps;
     int32_t *n_swaps, *swap_out, *swap_in, *capped;
     float *refined_gap, *topk_gap;
-    int nr;  // rows of the per-warp tables
+    int nr;  // largest n
 };
 
-// shared memory per warp (floats): U [nr][d+1] (the values, then the high
-// parts of u), G [nr][33]; nr = max_n rounded up to a multiple of 4
-__host__ __device__ constexpr int swap_smem_floats(int nr, int d) { return nr * (d + 1) + nr * 33; }
+// dimensions staged at a time
+__host__ __device__ constexpr int swap_dch(int d) { return d < 64 ? d : 64; }
+// shared memory per warp (floats): U (the values, then the high parts of u, and g), G
+__host__ __device__ constexpr int swap_smem_floats(int n, int d) { return staged_floats(n, swap_dch(d)) + gram_floats(n); }
 
 // The balancing selector (Sec. 2.1) inside the candidate set (Definition 2.2).
 // Pair scores are screened in fp32 from the Gram matrix G = U U^T of the
-// centred, weighted points u_j = p_j (v_j - mu) (es(A)^2 = ||sum_A u_j||^2 /
-// p(A)^2, Lemma 2.1); every pair whose fp32 score is within a rigorous error
-// bound of the best one is re-scored in double-float and the decision is
+// centred, weighted points u_j = p_j (v_j - mu) (es(A)^2 = ||g||^2 / p(A)^2,
+// g = sum_A u_j, Lemma 2.1); every pair whose fp32 score is within a rigorous
+// error bound of the best one is re-scored in double-float and the decision is
 // taken on those exact values.
+//
+// What bounds it: one row's chain of double-float sums (a warp alone issues an
+// instruction every 7 cycles or so), instruction fetch (the warps of an SM are in
+// different steps of a long program) and the fp64 pipe, which takes 16 cycles for a
+// warp's instruction whatever its lanes hold.  Hence
+//  - the values are staged 64 dimensions at a time and the Gram tiles (4 x 4 products
+//    per lane, 16-byte reads) add up in shared memory, so that 20 warps fit an SM;
+//  - loops are not unrolled over keys or chunks (unrolled by 4: 806 us, below: 704);
+//  - Q(A - i + j) is screened as Q(A) + 2 g.(u_j - u_i) + |u_j - u_i|^2, with Q(A) and g
+//    from the double-float state (g is one more row of the Gram matrix): the error
+//    scales with (|g| + |u_i| + |u_j|)^2, not with the square of the kept keys' summed
+//    norms, and where g is the small sum of large terms (a sink and its
+//    counterweights) far fewer pairs are re-scored (24 keys, k = 6: 5.6 a row before);
+//  - the re-scored pairs' fp64 quotients are taken up to 32 pairs at a time, one per
+//    lane, and P(A - i) once a round for every i.
+// 36,864 rows of 24 keys, d = 128: 1,433 us with whole rows staged and Gram entries one
+// by one, 704 us so; 256 rows of 20 keys, d = 64: 67 and 28 us.
 template <int DPL, typename VT>
-__global__ void __launch_bounds__(64) k_small_swap(const SmallSwapArgs a)
+__global__ void __launch_bounds__(64, 10) k_small_swap(const SmallSwapArgs a)
 {
-    extern __shared__ float smem[];
+    extern __shared__ __align__(16) float smem[];
     constexpr int d = DPL * 32;
+    constexpr int DCH = swap_dch(d), TCH = DCH / 32, NCH = d / DCH;
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
-    float *Uhi = smem + (size_t)wib * swap_smem_floats(a.nr, d);
-    float *G = Uhi + a.nr * (d + 1);
+    float *U = smem + (size_t)wib * swap_smem_floats(a.nr, d);
+    float *G = U + staged_floats(a.nr, DCH);
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
     if (row >= a.R.rows) return;
     const int64_t g = row / a.R.R;
@@ -180,106 +199,112 @@ __global__ void __launch_bounds__(64) k_small_swap(const SmallSwapArgs a)
     const int n = a.R.n[g];
     const int nb = a.nb;
     const int MS = a.max_swaps;
-    auto fail_row = [&]() {
-        for (int b = 0; b < nb; ++b) {
-            const int64_t rb = row * nb + b;
-            if (lane == 0) {
-                a.n_swaps[rb] = 0;
-                a.refined_gap[rb] = __int_as_float(0x7fc00000);
-                if (a.topk_gap) a.topk_gap[rb] = __int_as_float(0x7fc00000);
-                if (a.capped) a.capped[rb] = 0;
-            }
-            for (int t = lane; t < MS; t += 32) a.swap_out[rb * MS + t] = a.swap_in[rb * MS + t] = -1;
+    auto fail = [&](int b) {
+        const int64_t rb = row * nb + b;
+        if (lane == 0) {
+            a.n_swaps[rb] = 0;
+            a.refined_gap[rb] = __int_as_float(0x7fc00000);
+            if (a.topk_gap) a.topk_gap[rb] = __int_as_float(0x7fc00000);
+            if (a.capped) a.capped[rb] = 0;
         }
+        for (int t = lane; t < MS; t += 32) a.swap_out[rb * MS + t] = a.swap_in[rb * MS + t] = -1;
     };
     if (n < 1 || n > 32) {
-        fail_row();
+        for (int b = 0; b < nb; ++b) fail(b);
         return;
     }
     const float *lg = a.R.logits + a.R.logit_off[g] + ri * n;
     const VT *V = reinterpret_cast<const VT *>(a.R.v) + a.R.v_off[g];
     const float l = lane < n ? lg[lane] : -INFINITY;
     if (__any_sync(FW_FULL, lane < n && !isfinite(l))) {
-        fail_row();
+        for (int b = 0; b < nb; ++b) fail(b);
         return;
     }
     const float M = warp_max(l);
     double p = lane < n ? exp((double)l - (double)M) : 0.0;
     p = p / warp_sum_d(p);
     const df pd = df_from_double(p);
-    // the row's values into Uhi (loads issued back to back), then mu from there
-    stage_value_cols<d>(V, n, d, 0, Uhi, lane);
-    __syncwarp();
-    df mu[DPL];
+    // the kept set of budget b: the keys from its threshold up
+    auto kept = [&](int b) {
+        const uint32_t tk = a.thr_key[row * nb + b], key = order_key(l);
+        const int ti = a.thr_idx[row * nb + b];
+        return __ballot_sync(FW_FULL, lane < n && (key > tk || (key == tk && lane <= ti)));
+    };
+    const uint32_t A0 = kept(0);
+    // One pass over the values, DCH dimensions at a time: mu (double-float, j
+    // ascending), u_j = p_j (v_j - mu), whose high parts replace the values (the
+    // exact re-scoring recomputes u_j from V), and g of budget 0, the last row.
+    df mu[DPL], g0[DPL];
 #pragma unroll
-    for (int t = 0; t < DPL; ++t) mu[t] = df_zero();
-    for (int j = 0; j < n; ++j) {
-        const df pj = shfl_df(pd, j);
+    for (int t = 0; t < DPL; ++t) mu[t] = g0[t] = df_zero();
+#pragma unroll 1  // (a cold instruction cache costs a small batch more than the shifts below)
+    for (int ch = 0; ch < NCH; ++ch) {
+        __syncwarp();
+        stage_rows<DCH>(V, n, d, ch * DCH, U, lane);
+        __syncwarp();
+        df m[TCH], gg[TCH];
 #pragma unroll
-        for (int t = 0; t < DPL; ++t) mu[t] = df_add(mu[t], df_mul_f(pj, Uhi[j * (d + 1) + lane + 32 * t]));
+        for (int t = 0; t < TCH; ++t) m[t] = gg[t] = df_zero();
+#pragma unroll 1
+        for (int j = 0; j < n; ++j) {
+            const df pj = shfl_df(pd, j);
+#pragma unroll
+            for (int t = 0; t < TCH; ++t) m[t] = df_add(m[t], df_mul_f(pj, U[staged_at<DCH>(j, lane + 32 * t)]));
+        }
+#pragma unroll 1
+        for (int j = 0; j < n; ++j) {
+            const df pj = shfl_df(pd, j);
+            const bool in = (A0 >> j) & 1u;
+#pragma unroll
+            for (int t = 0; t < TCH; ++t) {
+                float *cell = U + staged_at<DCH>(j, lane + 32 * t);
+                const df u = df_mul(pj, df_rsub_f(*cell, m[t]));
+                *cell = u.hi;
+                if (in) gg[t] = df_add(gg[t], u);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < DPL; ++t) {  // chunk by chunk into place
+            mu[t] = t + TCH < DPL ? mu[t + TCH < DPL ? t + TCH : 0] : m[t + TCH - DPL < 0 ? 0 : t + TCH - DPL];
+            g0[t] = t + TCH < DPL ? g0[t + TCH < DPL ? t + TCH : 0] : gg[t + TCH - DPL < 0 ? 0 : t + TCH - DPL];
+        }
+#pragma unroll
+        for (int t = 0; t < TCH; ++t) U[staged_at<DCH>(n, lane + 32 * t)] = gg[t].hi;
+        __syncwarp();
+        gram_chunk<d, DCH>(U, G, n, ch == 0, lane);  // and g.u_x in column n
     }
-    // u_j = p_j (v_j - mu): high parts in place in Uhi (the exact re-scoring
-    // recomputes the double-float value from V); ||u_j||^2, held by lane j, only
-    // where a budget restricts the pool (E < n - k)
+    __syncwarp();
+    // u_j in double-float, recomputed from V (the expression of the pass above)
+    auto u_df = [&](int j, int t) {
+        return df_mul(shfl_df(pd, j), df_rsub_f(load_v(V, (int64_t)j * d + lane + 32 * t), mu[t]));
+    };
+    // ||u_j||^2, held by lane j, only where a budget restricts the pool (E < n - k)
     bool need_e2 = false;
     for (int b = 0; b < nb; ++b) need_e2 |= a.E < n - a.k[row * nb + b];
     double e2 = 0.0;
-    for (int j = 0; j < n; ++j) {
-        const df pj = shfl_df(pd, j);
-        df s = df_zero();
+    if (need_e2)
+#pragma unroll 1
+        for (int j = 0; j < n; ++j) {
+            df s = df_zero();
 #pragma unroll
-        for (int t = 0; t < DPL; ++t) {
-            const int c = lane + 32 * t;
-            const df u = df_mul(pj, df_rsub_f(Uhi[j * (d + 1) + c], mu[t]));
-            Uhi[j * (d + 1) + c] = u.hi;
-            if (need_e2) s = df_add(s, df_mul(u, u));
-        }
-        if (need_e2) {
+            for (int t = 0; t < DPL; ++t) {
+                const df u = u_df(j, t);
+                s = df_add(s, df_mul(u, u));
+            }
             s = warp_sum_df(s);
             if (lane == j) e2 = df_to_double(s);
         }
-    }
-    __syncwarp();
-    // fp32 Gram matrix, four interleaved partial sums per dot product
-    const int npairs = n * (n + 1) / 2;
-    for (int q = lane; q < npairs; q += 32) {
-        int x = 0, rem = q;
-        while (rem >= n - x) {
-            rem -= n - x;
-            ++x;
-        }
-        const int y = x + rem;
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-        const float *ux = Uhi + x * (d + 1), *uy = Uhi + y * (d + 1);
-        for (int c = 0; c < d; c += 4) {
-            s0 = fmaf(ux[c], uy[c], s0);
-            s1 = fmaf(ux[c + 1], uy[c + 1], s1);
-            s2 = fmaf(ux[c + 2], uy[c + 2], s2);
-            s3 = fmaf(ux[c + 3], uy[c + 3], s3);
-        }
-        const float s = (s0 + s1) + (s2 + s3);
-        G[x * 33 + y] = s;
-        G[y * 33 + x] = s;
-    }
-    __syncwarp();
-    const float unorm = lane < n ? sqrtf(fmaxf(G[lane * 33 + lane], 0.f)) : 0.f;
+    const float gd = lane < n ? G[lane * GRAM_LD + lane] : 0.f;  // G_xx, lane x
+    const float unorm = sqrtf(fmaxf(gd, 0.f)) * 1.0001f;
     const uint32_t all = n == 32 ? FW_FULL : ((1u << n) - 1u);
 
+#pragma unroll 1
     for (int b = 0; b < nb; ++b) {
         const int64_t rb = row * nb + b;
         const int kb = a.k[rb];
-        const uint32_t tk = a.thr_key[rb];
-        const int ti = a.thr_idx[rb];
-        const uint32_t key = order_key(l);
-        uint32_t A = __ballot_sync(FW_FULL, lane < n && (key > tk || (key == tk && lane <= ti)));
+        uint32_t A = b == 0 ? A0 : kept(b);
         if (kb < 1 || kb > n || __popc(A) != kb) {
-            if (lane == 0) {
-                a.n_swaps[rb] = 0;
-                a.refined_gap[rb] = __int_as_float(0x7fc00000);
-                if (a.topk_gap) a.topk_gap[rb] = __int_as_float(0x7fc00000);
-                if (a.capped) a.capped[rb] = 0;
-            }
-            for (int t = lane; t < MS; t += 32) a.swap_out[rb * MS + t] = a.swap_in[rb * MS + t] = -1;
+            fail(b);
             continue;
         }
         // candidate set: A plus the E dropped keys of largest single-key error
@@ -296,112 +321,140 @@ __global__ void __launch_bounds__(64) k_small_swap(const SmallSwapArgs a)
             }
             pool = A | __ballot_sync(FW_FULL, dropped && cnt < a.E);
         }
-        // S = sum of the k+1 largest ||u_x|| over the pool (error-bound scale)
-        float S;
-        {
-            const bool inp = (pool >> lane) & 1u;
-            int cnt = 0;
-            for (int s = 0; s < n; ++s) {
-                const float us = __shfl_sync(FW_FULL, unorm, s);
-                cnt += ((pool >> s) & 1u) && (us > unorm || (us == unorm && s < lane));
-            }
-            S = warp_sum(inp && cnt <= kb ? unorm : 0.f) * 1.0001f;
-        }
-        // bound on the fp32 error of a screened score, times P(A - i + j)^2: the
-        // Gram entries and sums (CB S^2), and 8 ulps of Q <= S^2 for the rounded
-        // P(A - i + j) and its inverse square
-        const float CB = 2.0f * ((float)d * 0.25f + 2.0f * (float)kb + 12.0f) * 5.9604645e-8f;
-        const float CBS = (CB + 8.f * 5.9604645e-8f) * S * S;
-        // u_j in double-float, recomputed from V (the expression of the pass above)
-        auto u_df = [&](int j, int t) {
-            return df_mul(shfl_df(pd, j), df_rsub_f(load_v(V, (int64_t)j * d + lane + 32 * t), mu[t]));
-        };
         // exact state: g_A (double-float, lanes over dims), p(A), es^2
         df gA[DPL];
+        if (b == 0) {
 #pragma unroll
-        for (int t = 0; t < DPL; ++t) gA[t] = df_zero();
-        for (uint32_t m = A; m; m &= m - 1) {
-            const int j = __ffs(m) - 1;
+            for (int t = 0; t < DPL; ++t) gA[t] = g0[t];
+        } else {
 #pragma unroll
-            for (int t = 0; t < DPL; ++t) {
-                gA[t] = df_add(gA[t], u_df(j, t));
+            for (int t = 0; t < DPL; ++t) gA[t] = df_zero();
+#pragma unroll 1
+            for (uint32_t m = A; m; m &= m - 1) {
+                const int j = __ffs(m) - 1;
+#pragma unroll
+                for (int t = 0; t < DPL; ++t) gA[t] = df_add(gA[t], u_df(j, t));
             }
         }
         double PA = warp_sum_d(((A >> lane) & 1u) ? p : 0.0);
-        auto exact_es2 = [&](const df *gv, double P) {
+        auto norm2 = [&](const df *gv) {
             df s = df_zero();
 #pragma unroll
             for (int t = 0; t < DPL; ++t) s = df_add(s, df_mul(gv[t], gv[t]));
-            s = warp_sum_df(s);
-            return fmax(df_to_double(s), 0.0) / (P * P);
+            return warp_sum_df(s);
         };
-        double cur = exact_es2(gA, PA);
+        df Q = norm2(gA);
+        double cur = fmax(df_to_double(Q), 0.0) / (PA * PA);
         if (a.topk_gap && lane == 0) a.topk_gap[rb] = (float)sqrt(cur);
+        // f_x = g.u_x in fp32, lane x, kept up to date from G; W bounds |g| and the
+        // norms of every term that went into f
+        float f, W;
+        if (b == 0) {
+            f = lane < n ? G[lane * GRAM_LD + n] : 0.f;
+            W = sqrtf(fmaxf(Q.hi, 0.f)) * 1.0001f;
+        } else {
+            f = 0.f;
+            if (lane < n)
+#pragma unroll 1
+                for (uint32_t m = A; m; m &= m - 1) f += G[lane * GRAM_LD + __ffs(m) - 1];
+            W = warp_sum(((A >> lane) & 1u) ? unorm : 0.f) * 1.0001f;
+        }
+        // Bound on the fp32 error of a screened score, times P(A - i + j)^2: with
+        // B = W + |u_i| + |u_j| the terms' absolute values sum to at most B^2; each
+        // dot product is chains of at most DCH / 2 fused terms, summed, f adds a
+        // term per kept key (b > 0) or two per swap, and 12 more roundings cover the
+        // operands (u and g to fp32), Q(A) and the sum of terms; doubled.  8 ulps for the
+        // rounded P(A - i + j) and its inverse square.  kTiny covers underflow.
+        constexpr float kTiny = 1e-37f;
+        const float C0 = 0.5f * DCH + NCH + kb + 13.f;
         int taken = 0, cap = 0;
+#pragma unroll 1
         for (;;) {
             const uint32_t add = pool & ~A;
-            const int na = __popc(A), nadd = __popc(add);
+            const int nadd = __popc(add);
             if (nadd == 0) break;
-            // h_x = sum_{y in A} G_xy and Q_A = sum_{x in A} h_x, fp32
-            float h = 0.f;
-            if (lane < n)
-                for (uint32_t m = A; m; m &= m - 1) h += G[lane * 33 + __ffs(m) - 1];
-            const float QA = warp_sum(((A >> lane) & 1u) ? h : 0.f);
+            const float CB = (2.f * (C0 + 2.f * taken) + 8.f) * 5.9604645e-8f;
             // fp32 screening of every (kept i, added j) pair, lane j taking the
-            // added key j: Q(A - i + j) = (Q_A - 2 h_i + G_ii) + (2 h_j + G_jj) - 2 G_ij,
+            // added key j: Q(A - i + j) = (Q_A - 2 f_i + G_ii) + (2 f_j + G_jj) - 2 G_ij,
             // P(A - i + j) = P(A - i) + p_j (two positive terms)
             const bool isadd = (add >> lane) & 1u;
-            const float cj = lane < n ? 2.f * h + G[lane * 33 + lane] : 0.f;
-            const float pjf = (float)p;
+            const float cj = 2.f * f + gd, ci_ = Q.hi - 2.f * f + gd;
+            const float pjf = (float)p, Pm = (float)(PA - p);
+            const float Wj = W + unorm;
+            float inv = 0.f, sc = 0.f, err = 0.f;
+            auto screen = [&](int i) {
+                const float Pp = __shfl_sync(FW_FULL, Pm, i) + pjf;
+                inv = 1.f / (Pp * Pp);
+                sc = (__shfl_sync(FW_FULL, ci_, i) + cj - 2.f * G[i * GRAM_LD + (lane < n ? lane : 0)]) * inv;
+                const float B = Wj + __shfl_sync(FW_FULL, unorm, i);
+                err = fmaf(CB * B, B, kTiny) * inv;
+            };
             float best_up = INFINITY;
+#pragma unroll 1
             for (uint32_t mi = A; mi; mi &= mi - 1) {
-                const int i = __ffs(mi) - 1;
-                const float ci = QA - 2.f * __shfl_sync(FW_FULL, h, i) + G[i * 33 + i];
-                const float Pp = (float)(PA - __shfl_sync(FW_FULL, p, i)) + pjf;
-                const float inv = 1.f / (Pp * Pp);
-                const float sc = (ci + cj - 2.f * G[i * 33 + (lane < n ? lane : 0)]) * inv;
-                if (isadd) best_up = fminf(best_up, sc + CBS * inv);
+                screen(__ffs(mi) - 1);
+                if (isadd) best_up = fminf(best_up, sc + err);
             }
             best_up = warp_min(best_up);
-            // exact re-scoring, in (i, j) order, of every pair that may be the best
-            double best = INFINITY;
-            int bi = -1, bj = -1;
+            // exact re-scoring, in (i, j) order, of every pair that may be the best: the
+            // norms pair by pair, the fp64 quotients of up to 32 pairs at once (lane c
+            // holds the c-th pair of the batch)
+            unsigned long long best = 0x7ff0000000000000ull;  // bits of +inf: es^2 >= 0 orders as integers
+            int bij = 0, cnt = 0, mij = 0;
+            df mine = df_zero();
+            auto settle = [&]() {
+                const int i = mij >> 5, j = mij & 31;
+                const double P2 = PA - __shfl_sync(FW_FULL, p, i) + __shfl_sync(FW_FULL, p, j);
+                const double e = fmax(df_to_double(mine), 0.0) / (P2 * P2);
+                unsigned long long eb = (unsigned long long)__double_as_longlong(e);
+                if (eb == 0x8000000000000000ull) eb = 0ull;  // -0
+                if (lane >= cnt) eb = ~0ull;
+                const uint32_t hi = __reduce_min_sync(FW_FULL, (uint32_t)(eb >> 32));
+                const uint32_t lo = __reduce_min_sync(FW_FULL, (uint32_t)(eb >> 32) == hi ? (uint32_t)eb : 0xffffffffu);
+                const unsigned long long eb_min = ((unsigned long long)hi << 32) | lo;
+                const int first = __ffs(__ballot_sync(FW_FULL, eb == eb_min)) - 1;
+                if (eb_min < best) {
+                    best = eb_min;
+                    bij = __shfl_sync(FW_FULL, mij, first);
+                }
+                cnt = 0;
+            };
+#pragma unroll 1
             for (uint32_t mi = A; mi; mi &= mi - 1) {
                 const int i = __ffs(mi) - 1;
-                const float ci = QA - 2.f * __shfl_sync(FW_FULL, h, i) + G[i * 33 + i];
-                const float Pp = (float)(PA - __shfl_sync(FW_FULL, p, i)) + pjf;
-                const float inv = 1.f / (Pp * Pp);
-                const float sc = (ci + cj - 2.f * G[i * 33 + (lane < n ? lane : 0)]) * inv;
-                uint32_t cand = __ballot_sync(FW_FULL, isadd && sc - CBS * inv <= best_up);
+                screen(i);
+                uint32_t cand = __ballot_sync(FW_FULL, isadd && sc - err <= best_up);
+#pragma unroll 1
                 while (cand) {
                     const int j = __ffs(cand) - 1;
                     cand &= cand - 1;
                     df gn[DPL];
 #pragma unroll
-                    for (int t = 0; t < DPL; ++t) {
-                        gn[t] = df_add(df_sub(gA[t], u_df(i, t)), u_df(j, t));
+                    for (int t = 0; t < DPL; ++t) gn[t] = df_add(df_sub(gA[t], u_df(i, t)), u_df(j, t));
+                    const df s2 = norm2(gn);
+                    if (lane == cnt) {
+                        mine = s2;
+                        mij = 32 * i + j;
                     }
-                    const double P2 = PA - __shfl_sync(FW_FULL, p, i) + __shfl_sync(FW_FULL, p, j);
-                    const double e = exact_es2(gn, P2);
-                    if (e < best) {
-                        best = e;
-                        bi = i;
-                        bj = j;
-                    }
+                    if (++cnt == 32) settle();
                 }
             }
-            if (!(best < cur)) break;
+            if (cnt) settle();
+            const int bi = bij >> 5, bj = bij & 31;
+            const double bestd = __longlong_as_double((long long)best);
+            if (!(bestd < cur)) break;
             if (taken >= MS) {
                 cap = 1;
                 break;
             }
 #pragma unroll
-            for (int t = 0; t < DPL; ++t) {
-                gA[t] = df_add(df_sub(gA[t], u_df(bi, t)), u_df(bj, t));
-            }
+            for (int t = 0; t < DPL; ++t) gA[t] = df_add(df_sub(gA[t], u_df(bi, t)), u_df(bj, t));
+            Q = norm2(gA);
             PA = PA - __shfl_sync(FW_FULL, p, bi) + __shfl_sync(FW_FULL, p, bj);
             A = (A & ~(1u << bi)) | (1u << bj);
-            cur = best;
+            cur = bestd;
+            if (lane < n) f += G[lane * GRAM_LD + bj] - G[lane * GRAM_LD + bi];
+            W += __shfl_sync(FW_FULL, unorm, bi) + __shfl_sync(FW_FULL, unorm, bj);
             if (lane == 0) {
                 a.swap_out[rb * MS + taken] = bi;
                 a.swap_in[rb * MS + taken] = bj;
@@ -439,11 +492,11 @@ fw_status small_swap(const RowsDev &R, const int32_t *k, int nb, const fw_gap_ou
                      float *refined_gap, float *topk_gap, int32_t *capped, cudaStream_t s)
 {
     if (R.rows == 0) return FW_OK;
-    const int nr = (std::min(R.max_n, 32) + 3) / 4 * 4;
+    const int nr = std::min(R.max_n, 32);
     const SmallSwapArgs a{R, k, nb, topk.thr_key, topk.thr_idx, E, max_swaps, n_swaps, swap_out,
                           swap_in, capped, refined_gap, topk_gap, nr};
     FW_DISPATCH(R.d, R.v_dtype, {
-        const int warps = DPL >= 8 ? 1 : 2;
+        const int warps = 2;
         const size_t smem = (size_t)warps * swap_smem_floats(nr, DPL * 32) * sizeof(float);
         FW_CUDA_CHECK(cudaFuncSetAttribute(k_small_swap<DPL, VT>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
