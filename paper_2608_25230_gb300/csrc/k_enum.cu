@@ -43,8 +43,6 @@ constexpr int FBS = 64;   // chunks (blocks) per row on the exhaustive path
 constexpr int MAXD = 24;  // depth bound of the phase-2 walk
 constexpr int PERM = 48;  // local index space per row: NS <= EM + 32
 
-__host__ __device__ constexpr int tri(int a, int b, int n) { return a * n - a * (a - 1) / 2 + (b - a); }
-
 struct EnumArgs {
     RowsDev R;
     const int32_t *k;
@@ -497,46 +495,43 @@ __device__ __forceinline__ void put_linear(const SlotGeom &S, int l, float lin, 
 }
 
 // pref[m] = sum of the m smallest of vals[0, E) for m <= need, then
-// pref[need + 1] = sum |vals| (E <= 512).  Each lane holds its entries
-// lane + 32 u in registers; every round the warp takes the smallest unused one
-// (equal values: any of them, the sums do not depend on it).
+// pref[need + 1] = sum |vals| (E <= 512).  Each lane keeps its entries
+// lane + 32 u in registers, ascending; every round takes the smallest head (one
+// warp reduction of the order keys) and shifts that lane's entries down.  Equal
+// values: any of them, the sums do not depend on it.
+template <int CAP>  // entries per lane
 __device__ __forceinline__ void smallest_prefix(const float *vals, int E, int need, float *pref, int lane)
 {
-    float x[16];
+    float x[CAP];
     float ab = 0.f;
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
+    for (int u = 0; u < CAP; ++u) {
         const int e = lane + 32 * u;
-        x[u] = e < E ? vals[e] : INFINITY;
-        ab += e < E ? fabsf(x[u]) : 0.f;
+        const float v = e < E ? vals[e] : INFINITY;
+        x[u] = v < INFINITY ? v : INFINITY;  // (a NaN is not taken)
+        ab += e < E ? fabsf(v) : 0.f;
     }
     ab = warp_sum(ab);
+    // ascending: odd-even transposition
+#pragma unroll
+    for (int s2 = 0; s2 < CAP; ++s2)
+#pragma unroll
+        for (int u = s2 & 1; u + 1 < CAP; u += 2) {
+            const float lo = fminf(x[u], x[u + 1]);
+            x[u + 1] = fmaxf(x[u], x[u + 1]);
+            x[u] = lo;
+        }
     float run = 0.f;
     if (lane == 0) pref[0] = 0.f;
     for (int m = 0; m < need; ++m) {
-        float bv = INFINITY;
-        int bu = 0;
+        const uint32_t key = order_key(x[0]), mk = __reduce_min_sync(FW_FULL, key);
+        const int wl = __ffs(__ballot_sync(FW_FULL, key == mk)) - 1;
+        const float wv = __shfl_sync(FW_FULL, x[0], wl);
+        if (lane == wl) {
 #pragma unroll
-        for (int u = 0; u < 16; ++u)
-            if (x[u] < bv) {
-                bv = x[u];
-                bu = u;
-            }
-        float wv = bv;
-        int wl = lane;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float ov = __shfl_xor_sync(FW_FULL, wv, o);
-            const int ol = __shfl_xor_sync(FW_FULL, wl, o);
-            if (ov < wv || (ov == wv && ol < wl)) {
-                wv = ov;
-                wl = ol;
-            }
+            for (int u = 0; u + 1 < CAP; ++u) x[u] = x[u + 1];
+            x[CAP - 1] = INFINITY;
         }
-        if (lane == wl)
-#pragma unroll
-            for (int u = 0; u < 16; ++u)
-                if (u == bu) x[u] = INFINITY;
         run += wv < INFINITY ? wv : 0.f;
         if (lane == 0) pref[m + 1] = run;
     }
@@ -544,8 +539,6 @@ __device__ __forceinline__ void smallest_prefix(const float *vals, int E, int ne
 }
 
 constexpr int ERW = 16;  // rows per warp (two lanes per row)
-constexpr int MAXT = 3;         // Gram tiles (2 x 4 products) per lane: 33 rows need at most 96
-constexpr int PPL = 8 * MAXT;   // Gram product slots per lane
 
 // ---- the search in three kernels.  k_enum_prep: one warp per row builds the
 // row's walk tables (slot, key order, kappa and |g0|) in shared memory and
@@ -555,31 +548,46 @@ constexpr int PPL = 8 * MAXT;   // Gram product slots per lane
 constexpr int PREP_W = 4;  // warps (rows) per block of k_enum_prep
 constexpr int RS_W = 8;    // warps (rows) per block of k_enum_rescore
 
-// per-warp shared memory of k_enum_prep (floats): slot, staged values, a_x,
-// p (double), key order and its inverse; a multiple of 4
-__host__ __device__ constexpr int prep_floats(int stride, int ust)
+// per-warp shared memory of k_enum_prep (floats): the staged values, whose place the slot
+// and the list of its pair terms take once the Gram matrix is done; the Gram matrix, a_x,
+// p, key order and its inverse; multiples of 4
+constexpr int PREP_E = 512;  // pair terms
+__host__ __device__ constexpr int prep_slot(int stride) { return (stride + 3) / 4 * 4; }
+__host__ __device__ constexpr int prep_region(int stride, int max_n, int dch)
 {
-    return ((stride + 1) / 2 * 2 + ust + 32 + 64 + (PERM + 32) / 4 + 3) / 4 * 4;
+    const int u = staged_floats(max_n, dch), w = prep_slot(stride) + PREP_E;
+    return u > w ? u : w;
+}
+__host__ __device__ constexpr int prep_floats(int stride, int max_n, int dch)
+{
+    return prep_region(stride, max_n, dch) + gram_floats(max_n) + 32 + 32 + (PERM + 32) / 4;
 }
 constexpr int RCB = 8;     // candidates re-scored per pass over the values
 // per-warp shared memory of k_enum_rescore (floats): the staged values
 __host__ __device__ constexpr int rescore_floats(int ust) { return (ust + 3) / 4 * 4; }
 
+// Bounded like k_small_swap by one row's chain, instruction fetch and, for a fifth of
+// its time, the fp64 pipe.  The tables take the staged values' place and the Gram matrix
+// stays in shared memory, so that 20 warps fit an SM; a table row is written by the
+// whole warp (its kind is uniform) instead of scattering products from registers, and a
+// smallest pair term costs one reduction instead of a shuffle tree with 16 compares.
+// 36,864 rows of 24 keys, d = 128: 1,127 us before, 661 us so (loops over keys unrolled
+// by 4: 738); 256 rows of 20 keys, d = 64: 44 and 26 us.
 template <int DPL, typename VT>
-__global__ void __launch_bounds__(32 * PREP_W, 4) k_enum_prep(const EnumArgs a)
+__global__ void __launch_bounds__(32 * PREP_W, 5) k_enum_prep(const EnumArgs a)
 {
-    extern __shared__ float smem[];
+    extern __shared__ __align__(16) float smem[];
     constexpr int d = DPL * 32;
     constexpr int DCH = d < 64 ? d : 64;  // dimensions staged at a time
     constexpr int TCH = DCH / 32;         // per-lane dims in one chunk
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int ust_floats = (((a.R.max_n + 1) * (DCH + 1)) + 1) & ~1;
-    float *slot = smem + (size_t)wib * prep_floats(a.stride, ust_floats);  // [stride]
-    float *Ust = slot + (a.stride + 1) / 2 * 2;                             // [max_n+1][DCH+1]
-    float *aX = Ust + ust_floats;                                            // [32]
-    float *pfl = aX + 32;                                                    // [32] p (rounded)
-    uint8_t *perms = reinterpret_cast<uint8_t *>(aX + 96);                   // [PERM]
-    uint8_t *inv = perms + PERM;                                             // [32]
+    float *Ust = smem + (size_t)wib * prep_floats(a.stride, a.R.max_n, DCH);  // rows 0 .. max_n
+    float *slot = Ust;                                                         // [stride], later
+    float *G = Ust + prep_region(a.stride, a.R.max_n, DCH);                    // Gram matrix
+    float *aX = G + gram_floats(a.R.max_n);                                    // [32]
+    float *pfl = aX + 32;                                                      // [32] p (rounded)
+    uint8_t *perms = reinterpret_cast<uint8_t *>(pfl + 32);                    // [PERM]
+    uint8_t *inv = perms + PERM;                                               // [32]
     const int64_t row = (int64_t)blockIdx.x * PREP_W + wib;
     if (row >= a.R.rows) return;
     const int64_t g = row / a.R.R;
@@ -636,106 +644,50 @@ __global__ void __launch_bounds__(32 * PREP_W, 4) k_enum_prep(const EnumArgs a)
     S.RH = EM + nHp + 2;
     S.offH = OFF_A + k * S.RA;
     const int tot = slot_floats(k, nHp);
-    for (int i = lane; i < tot; i += 32) S.slot[i] = (i >= nL && i < EM) ? INFINITY : 0.f;
-    // Gram entries over the n keys plus g0 (index n), staged DCH dimensions at a
-    // time.  The upper triangle is cut into tiles of 2 rows x 4 columns (lane
-    // takes tiles lane, lane + 32, ...); a tile reads 6 staged values per
-    // dimension for its 8 products, and each product is four interleaved
-    // partial sums per chunk.  Slot i = 8 * tile + 4 * (x - x0) + (y - y0);
-    // px_ = -1 marks slots outside the triangle (and |g0|^2, known exactly).
-    const int R1 = n + 1, nby = (R1 + 3) / 4;
-    int tx0[MAXT], ty0[MAXT];
-    int px_[PPL], py_[PPL];
-    float acc[PPL];
-#pragma unroll
-    for (int tl = 0; tl < MAXT; ++tl) {
-        int tid_ = lane + 32 * tl, bx = 0;
-        bool ok = true;
-        for (;;) {  // rows 2bx, 2bx+1 hold tiles by = bx/2 .. nby-1
-            if (2 * bx >= R1) {
-                ok = false;
-                break;
-            }
-            const int cnt = nby - bx / 2;
-            if (tid_ < cnt) break;
-            tid_ -= cnt;
-            ++bx;
-        }
-        tx0[tl] = ok ? 2 * bx : -1;
-        ty0[tl] = ok ? 4 * (bx / 2 + tid_) : -1;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int x = tx0[tl] + (e >> 2), y = ty0[tl] + (e & 3);
-            const bool in = ok && x <= y && y < R1 && x < n;
-            px_[8 * tl + e] = in ? x : -1;
-            py_[8 * tl + e] = y;
-            acc[8 * tl + e] = 0.f;
-        }
-    }
+    // Gram entries over the n keys plus g0 (row n), staged DCH dimensions at a time
     df g0[DPL];
 #pragma unroll
     for (int t = 0; t < DPL; ++t) g0[t] = df_zero();
-#pragma unroll
+#pragma unroll 1
     for (int ch = 0; ch < DPL / TCH; ++ch) {
         __syncwarp();
         // the chunk's values of all n keys into Ust (loads issued back to back)
-        stage_value_cols<DCH>(V, n, d, ch * DCH, Ust, lane);
+        stage_rows<DCH>(V, n, d, ch * DCH, Ust, lane);
         __syncwarp();
         // mu over the chunk's columns (j ascending, double-float), then
         // u_j = p_j (v_j - mu) in place
-        df mu[TCH];
+        df mu[TCH], gg[TCH];
 #pragma unroll
-        for (int tt = 0; tt < TCH; ++tt) mu[tt] = df_zero();
+        for (int tt = 0; tt < TCH; ++tt) mu[tt] = gg[tt] = df_zero();
+#pragma unroll 1
         for (int j = 0; j < n; ++j) {
             const df pj = shfl_df(pd, j);
 #pragma unroll
             for (int tt = 0; tt < TCH; ++tt)
-                mu[tt] = df_add(mu[tt], df_mul_f(pj, Ust[j * (DCH + 1) + lane + 32 * tt]));
+                mu[tt] = df_add(mu[tt], df_mul_f(pj, Ust[staged_at<DCH>(j, lane + 32 * tt)]));
         }
+#pragma unroll 1
         for (int j = 0; j < n; ++j) {
             const df pj = shfl_df(pd, j);
             const bool in = (A0 >> j) & 1u;
 #pragma unroll
             for (int tt = 0; tt < TCH; ++tt) {
-                const int t = ch * TCH + tt;
-                float *cell = Ust + j * (DCH + 1) + lane + 32 * tt;
+                float *cell = Ust + staged_at<DCH>(j, lane + 32 * tt);
                 const df u = df_mul(pj, df_rsub_f(*cell, mu[tt]));
                 *cell = u.hi;
-                if (in) g0[t] = df_add(g0[t], u);
+                if (in) gg[tt] = df_add(gg[tt], u);
             }
         }
 #pragma unroll
-        for (int tt = 0; tt < TCH; ++tt) Ust[n * (DCH + 1) + lane + 32 * tt] = g0[ch * TCH + tt].hi;
+        for (int t = 0; t < DPL; ++t)  // chunk by chunk into place
+            g0[t] = t + TCH < DPL ? g0[t + TCH < DPL ? t + TCH : 0] : gg[t + TCH - DPL < 0 ? 0 : t + TCH - DPL];
+#pragma unroll
+        for (int tt = 0; tt < TCH; ++tt) Ust[staged_at<DCH>(n, lane + 32 * tt)] = gg[tt].hi;
         __syncwarp();
-#pragma unroll
-        for (int tl = 0; tl < MAXT; ++tl) {
-            if (tx0[tl] < 0) continue;
-            const float *ux[2], *uy[4];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) ux[e] = Ust + min(tx0[tl] + e, n) * (DCH + 1);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) uy[e] = Ust + min(ty0[tl] + e, n) * (DCH + 1);
-            float sp[8][4];
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-#pragma unroll
-                for (int c4 = 0; c4 < 4; ++c4) sp[e][c4] = 0.f;
-            for (int c = 0; c < DCH; c += 4) {
-#pragma unroll
-                for (int c4 = 0; c4 < 4; ++c4) {
-                    const float a0 = ux[0][c + c4], a1 = ux[1][c + c4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float b = uy[e][c + c4];
-                        sp[e][c4] = fmaf(a0, b, sp[e][c4]);
-                        sp[4 + e][c4] = fmaf(a1, b, sp[4 + e][c4]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[8 * tl + e] += (sp[e][0] + sp[e][1]) + (sp[e][2] + sp[e][3]);
-        }
+        gram_chunk<d, DCH>(Ust, G, n, ch == 0, lane);
     }
+    __syncwarp();
+    for (int i = lane; i < tot; i += 32) S.slot[i] = (i >= nL && i < EM) ? INFINITY : 0.f;
     df nrm = df_zero();
 #pragma unroll
     for (int t = 0; t < DPL; ++t) nrm = df_add(nrm, df_mul(g0[t], g0[t]));
@@ -748,33 +700,28 @@ __global__ void __launch_bounds__(32 * PREP_W, 4) k_enum_prep(const EnumArgs a)
     // kappa: 2.2x the per-subset error bound of an fp32 evaluation of either form
     const int Lc = k * (k + 1) / 2 + 2 * n + 16;
     S.kap = (float)(2.2 * ((double)d * 0.25 + Lc + 16) * 5.9604644775390625e-8);
-    S.g0n = (float)sqrt(g0n2) * 1.0001f;
+    S.g0n = (float)(sqt * P0) * 1.0001f;
     // a_x = |u_x| + sqrt(t) p_x (rounded up) from the diagonal entries
-#pragma unroll
-    for (int i = 0; i < PPL; ++i)
-        if (px_[i] >= 0 && px_[i] == py_[i] && px_[i] < n)
-            aX[px_[i]] = sqrtf(fmaxf(acc[i], 0.f)) * 1.0001f + ((float)sqt * pfl[px_[i]]) * 1.0001f;
+    const float pf = (float)p;
+    float ax = 0.f;
+    if (lane < n) {
+        ax = sqrtf(fmaxf(G[lane * GRAM_LD + lane], 0.f)) * 1.0001f + ((float)sqt * pf) * 1.0001f;
+        aX[lane] = ax;
+    }
     __syncwarp();
-    // scatter the folded entries into the walk tables
+    // the folded entries into the walk tables, a table row at a time (lane = the other key);
+    // G' = u.u - t p p^T in fp32 (a few ulps of a_x a_y, inside kappa's slack)
     const float tf = (float)t, P0f = (float)P0;
-#pragma unroll
-    for (int i = 0; i < PPL; ++i) {
-        const int x = px_[i], y = py_[i];
-        if (x < 0 || x == n) continue;
-        // G' = u.u - t p p^T in fp32 (a few ulps of a_x a_y, inside kappa's slack)
-        const float tpx = tf * pfl[x];
-        if (y == n) {
-            const float sx = ((A0 >> x) & 1u) ? -2.f : 2.f;
-            put_linear(S, inv[x], sx * fmaf(-tpx, P0f, acc[i]), aX[x]);
-        } else {
-            const float gp = fmaf(-tpx, pfl[y], acc[i]);
-            if (x == y) {
-                put_diag(S, inv[x], gp, aX[x]);
-            } else {
-                put_entry(S, inv[x], inv[y], gp, aX[x], aX[y]);
-                put_entry(S, inv[y], inv[x], gp, aX[y], aX[x]);
-            }
-        }
+    const int il = lane < n ? inv[lane] : 0;
+    if (lane < n) {
+        const float tpx = tf * pf, sx = inA0 ? -2.f : 2.f;
+        put_linear(S, il, sx * fmaf(-tpx, P0f, G[lane * GRAM_LD + n]), ax);
+        put_diag(S, il, fmaf(-tpx, pf, G[lane * GRAM_LD + lane]), ax);
+    }
+    for (int x = 0; x < n; ++x) {
+        const float px = pfl[x];
+        const float gp = fmaf(-(tf * (x < lane ? px : pf)), x < lane ? pf : px, G[x * GRAM_LD + (lane < n ? lane : 0)]);
+        if (lane < n && lane != x) put_entry(S, inv[x], il, gp, aX[x], ax);
     }
     __syncwarp();
     // Bounds of the walk: the pair terms of the inner set L (G2, x < y) and of
@@ -784,9 +731,9 @@ __global__ void __launch_bounds__(32 * PREP_W, 4) k_enum_prep(const EnumArgs a)
     // The warp takes the smallest remaining term round by round.
     {
         const int nLL = EM * (EM - 1) / 2, nHH = nHp * (nHp - 1) / 2, E = nLL + nHH + EM * nHp;
-        float *vals = Ust;
+        float *vals = slot + prep_slot(a.stride);
         float *PF = S.slot + off_pref(k, nHp), *PR = S.slot + off_prefr(k, nHp);
-        if (E <= ust_floats && E <= 512) {
+        if (E <= PREP_E) {
             for (int e = lane; e < E; e += 32) {
                 float v;
                 if (e < nLL) {
@@ -814,7 +761,9 @@ __global__ void __launch_bounds__(32 * PREP_W, 4) k_enum_prep(const EnumArgs a)
             for (int pass = 0; pass < 2; ++pass) {
                 const int En = pass == 0 ? nLL : E;
                 const int need = (pass == 0 ? npref(k) : nprefr(k)) - 1;
-                smallest_prefix(vals, En, need, pass == 0 ? PF : PR, lane);
+                float *pref = pass == 0 ? PF : PR;
+                if (En <= 32 * 6) smallest_prefix<6>(vals, En, need, pref, lane);
+                else smallest_prefix<16>(vals, En, need, pref, lane);
             }
         } else if (lane == 0) {  // (cannot happen for n <= 32; the bounds then never prune)
             for (int m = 0; m < npref(k); ++m) PF[m] = -INFINITY;
@@ -1352,7 +1301,7 @@ fw_status best_subset(const RowsDev &R, const int32_t *k, uint64_t *best_rank, f
     FW_DISPATCH(R.d, R.v_dtype, {
         constexpr int DCH = DPL * 32 < 64 ? DPL * 32 : 64;
         const int ust = (((R.max_n + 1) * (DCH + 1)) + 1) & ~1;
-        const size_t smem_p = (size_t)PREP_W * prep_floats(a.stride, ust) * sizeof(float);
+        const size_t smem_p = (size_t)PREP_W * prep_floats(a.stride, R.max_n, DCH) * sizeof(float);
         FW_CUDA_CHECK(cudaFuncSetAttribute(k_enum_prep<DPL, VT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem_p));
         FW_LAUNCH((k_enum_prep<DPL, VT>), (unsigned)((R.rows + PREP_W - 1) / PREP_W), 32 * PREP_W, smem_p, s, a);
