@@ -125,7 +125,7 @@ struct Walk {
     const float *slot;
     const uint8_t *perm;  // local index -> original key
     int k, nL, nHp;
-    int half;             // which of the row's two lanes: takes every other R of each size class
+    int part, parts;      // the row's lanes take the R of each size class in turn: part, part + parts, ...
     uint32_t sync_mask;   // lanes that walk rows of identical (n, k); 0 when they differ
     float kappa, g0n;
     uint32_t *cand;
@@ -240,7 +240,7 @@ __device__ __forceinline__ float inner_dispatch(int c, const float (&w)[EM], flo
     }
 }
 
-// The whole walk of one row (one lane).  Compiled once; every kernel
+// The whole walk of one row by one of its lanes.  Compiled once; every kernel
 // instantiation calls it.
 __device__ __noinline__ void walk_row(const Walk W)
 {
@@ -268,8 +268,8 @@ __device__ __noinline__ void walk_row(const Walk W)
     int path[MAXD];
     const uint32_t nR = 1u << k;
     unsigned long long n_inner = 0, n_leaf = 0, n_ops = 0, n_skip = 0;
-    // Removal sets R of A0 by size class; the row's two lanes take alternate
-    // members of the same class at the same time, so they run the same code.
+    // Removal sets R of A0 by size class; the row's lanes take the members of a
+    // class in turn at the same time, so they run the same code.
     for (int r = 0; r <= k; ++r) {
         if (r > nL + nHp) break;  // cannot add back r keys
         uint32_t R = r == 0 ? 0u : (1u << r) - 1u;
@@ -280,10 +280,14 @@ __device__ __noinline__ void walk_row(const Walk W)
             const uint32_t ri = x + lo;
             return (((ri ^ x) >> 2) / lo) | ri;
         };
-        if (W.half) {
+        for (int i = 0; i < W.part && R < nR; ++i) R = next_same_size(R);
+        valid = R < nR;
+        auto advance = [&]() {
             R = next_same_size(R);
+            if (R < nR) R = next_same_size(R);
+            for (int i = 2; i < W.parts && R < nR; ++i) R = next_same_size(R);
             valid = R < nR;
-        }
+        };
         while (valid) {
         // choose the form with the smaller error bound
         float sR = 0.f, sK = 0.f;
@@ -357,9 +361,7 @@ __device__ __noinline__ void walk_row(const Walk W)
         }
         if (skip_r) {
             ++n_skip;
-            R = next_same_size(R);
-            if (R < nR) R = next_same_size(R);
-            valid = R < nR;
+            advance();
             continue;
         }
         // phase 2: depth-first over I subset of H' with |I| <= r
@@ -435,11 +437,9 @@ __device__ __noinline__ void walk_row(const Walk W)
             ++depth;
             ++e;
         }
-        R = next_same_size(R);
-        if (R < nR) R = next_same_size(R);
-        valid = R < nR;
+        advance();
         }
-        // The two halves may differ by one member in this class; meet again
+        // The lanes may differ by one member in this class; meet again
         // before the next one.  Every lane in sync_mask walks the same (n, k),
         // hence runs this loop the same number of times.
         if (W.sync_mask) __syncwarp(W.sync_mask);
@@ -538,11 +538,9 @@ __device__ __forceinline__ void smallest_prefix(const float *vals, int E, int ne
     if (lane == 0) pref[need + 1] = ab;
 }
 
-constexpr int ERW = 16;  // rows per warp (two lanes per row)
-
 // ---- the search in three kernels.  k_enum_prep: one warp per row builds the
 // row's walk tables (slot, key order, kappa and |g0|) in shared memory and
-// writes them out; k_enum_walk: one warp = ERW rows, two lanes per row split
+// writes them out; k_enum_walk: one warp = ERW rows, 32 / ERW lanes per row split
 // its removal sets; k_enum_rescore: one warp per row re-scores the row's
 // candidates exactly and lists the rows left to the exhaustive path.
 constexpr int PREP_W = 4;  // warps (rows) per block of k_enum_prep
@@ -784,6 +782,7 @@ __global__ void __launch_bounds__(32 * PREP_W, 5) k_enum_prep(const EnumArgs a)
     }
 }
 
+template <int ERW>
 __global__ void __launch_bounds__(32, 1) k_enum_walk(const EnumArgs a)
 {
     extern __shared__ float smem[];
@@ -804,6 +803,7 @@ __global__ void __launch_bounds__(32, 1) k_enum_walk(const EnumArgs a)
             reinterpret_cast<uint4 *>(perms)[i] = reinterpret_cast<const uint4 *>(a.perms + row0 * PERM)[i];
     }
     __syncwarp();
+    static_assert(ERW % 4 == 0, "");
     const int rr = lane & (ERW - 1);
     const int64_t row = row0 + rr;
     Walk my;
@@ -815,13 +815,14 @@ __global__ void __launch_bounds__(32, 1) k_enum_walk(const EnumArgs a)
         my.nHp = n - my.k - my.nL;
         my.slot = slots + rr * a.stride;
         my.perm = perms + rr * PERM;
-        my.half = lane / ERW;
+        my.part = lane / ERW;
+        my.parts = 32 / ERW;
+        my.stats = a.stats;
         const float2 kg = a.kg[row];
         my.kappa = kg.x;
         my.g0n = kg.y;
         my.cand = a.cand + row * ECAP;
         my.ccount = a.cand_count + row;
-        my.stats = a.stats;
     }
     {
         const uint32_t wmask = __ballot_sync(FW_FULL, my_walk);
@@ -891,6 +892,7 @@ __global__ void __launch_bounds__(32 * RS_W) k_enum_rescore(const EnumArgs a)
             }
 #pragma unroll
             for (int ci = 0; ci < RCB; ++ci) {
+                if (c0 + ci >= cc) break;
                 df gv[TCH];
 #pragma unroll
                 for (int tt = 0; tt < TCH; ++tt) gv[tt] = df_zero();
@@ -1234,6 +1236,29 @@ __global__ void k_enum_exhaustive_merge(const EnumArgs a)
     }
 }
 
+template <int ERW> fw_status launch_walk_n(const EnumArgs &a, cudaStream_t s)
+{
+    const size_t smem = (size_t)ERW * a.stride * sizeof(float) + ERW * PERM;
+    FW_CUDA_CHECK(cudaFuncSetAttribute(k_enum_walk<ERW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    FW_LAUNCH((k_enum_walk<ERW>), (unsigned)((a.R.rows + ERW - 1) / ERW), 32, smem, s, a);
+    return FW_OK;
+}
+
+// Lanes per row.  A warp (255 registers, 8 to an SM) lasts as long as its slowest row, so
+// few rows are split finer: 8 lanes each while all their warps are resident at once
+// (32 rows an SM), 4 for twice as many; beyond that the SMs are full either way, and lanes
+// that idle at a class's end and their counters' atomics are lost work.  Measured,
+// 2 / 4 / 8 lanes a row, us: 24 keys, k = 6: 2,000 rows 609 / 487 / 378, 4,000: 634 / 493 /
+// 401, 8,000: 696 / 632 / 647, 16,000: 1,036 / 915 / 858; 16 keys, k = 4: 2,000 rows 191 /
+// 158 / 160, 4,000: 190 / 175 / 177, 8,000: 211 / 212 / 293, 16,000: 256 / 310 / 453;
+// 256 rows of 20 keys, k = 5: 130 / 86 / 74.
+fw_status launch_walk(const EnumArgs &a, int sms, cudaStream_t s)
+{
+    if (a.R.rows <= (int64_t)32 * sms) return launch_walk_n<4>(a, s);
+    if (a.R.rows <= (int64_t)64 * sms) return launch_walk_n<8>(a, s);
+    return launch_walk_n<16>(a, s);
+}
+
 }  // namespace
 
 // floats per row slot: the largest table set over every n <= max_n, k <= k_max (odd stride)
@@ -1305,9 +1330,10 @@ fw_status best_subset(const RowsDev &R, const int32_t *k, uint64_t *best_rank, f
         FW_CUDA_CHECK(cudaFuncSetAttribute(k_enum_prep<DPL, VT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem_p));
         FW_LAUNCH((k_enum_prep<DPL, VT>), (unsigned)((R.rows + PREP_W - 1) / PREP_W), 32 * PREP_W, smem_p, s, a);
-        const size_t smem_w = (size_t)ERW * a.stride * sizeof(float) + ERW * PERM;
-        FW_CUDA_CHECK(cudaFuncSetAttribute(k_enum_walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w));
-        FW_LAUNCH(k_enum_walk, (unsigned)((R.rows + ERW - 1) / ERW), 32, smem_w, s, a);
+        {
+            const fw_status st = launch_walk(a, sms, s);
+            if (st != FW_OK) return st;
+        }
         const size_t smem_r = (size_t)RS_W * rescore_floats(ust) * sizeof(float);
         FW_CUDA_CHECK(cudaFuncSetAttribute(k_enum_rescore<DPL, VT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem_r));

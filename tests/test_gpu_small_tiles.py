@@ -36,6 +36,24 @@ def test_best_tiles(fw, n, k, d):  # noqa: F811
     check_best(fw, _rows(n, d, 9, n * d + k, "bf16" if k % 2 else "f32", [k]))
 
 
+@pytest.mark.parametrize("rows", [1, 3, 4864, 4865, 9729])
+def test_best_lanes_per_row(fw, rows):  # noqa: F811
+    # 8, 4 and 2 lanes walk a row (152 SMs: the lines lie at 4,864 and 9,728 rows): the
+    # same few rows, repeated, give the same answers as in a batch of their own
+    import torch
+
+    m = min(rows, 13)
+    b = _rows(14, 32, m, rows, k=[4])
+    rep = np.arange(rows) % m
+    big = rows_batch(np.asarray(b.logits).reshape(m, 14)[rep], np.asarray(b.v).reshape(m, 14, 32)[rep],
+                     np.asarray(b.k)[rep])
+    check_best(fw, b)
+    few, many = (fw.best_subset(fw.rows_from_batch(x), torch.from_numpy(np.ascontiguousarray(x.k[:, 0])).cuda())
+                 for x in (b, big))
+    for key in ("best_rank", "best_gap", "best_idx", "topk_gap"):
+        np.testing.assert_array_equal(many[key].cpu().numpy(), few[key].cpu().numpy()[rep])
+
+
 def test_swap_rescored_in_batches(fw):  # noqa: F811
     # equal logits and nearly equal values: the screen cannot tell the 240 pairs of a
     # row apart, so they are re-scored 32 at a time; the decision is the oracle's
