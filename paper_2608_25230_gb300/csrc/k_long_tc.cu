@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(pv_threads<D>(), 1) k_long_pv_tc(const TcArgs 
 //
 // Stages whose V rows would cross the end of the group's block (the partial last
 // stage, or a block not aligned to whole rows) go through per-thread cp.async
-// with zero fill instead, and logit rows that are not 16-byte aligned (n not a
+// with zero fill instead (the MMA warp fences them into the async proxy), and logit rows that are not 16-byte aligned (n not a
 // multiple of 4, misaligned base) through 4-byte cp.async.
 constexpr int PVM_PW = 16;                     // producer warps
 constexpr int PVM_NT = (PVM_PW + 2) * 32;      // threads
@@ -693,6 +693,9 @@ __global__ void __launch_bounds__(PVM_NT, 1) k_long_pv_tma(const __grid_constant
                 if (ok && it % CH == 0 && ch >= NACC)
                     ok = tc::mbar_wait(&accfree[ch % NACC], (uint32_t)((ch - NACC) / NACC) & 1u, WAIT_POLLS);
                 if (!ok) break;
+                // a stage whose V came by cp.async was written through the generic proxy: the
+                // MMA's reads, through the async proxy, are ordered behind it by this fence
+                if (!(vrows && (it + 1) * KS <= n)) tc::fence_async_smem();
                 tc::fence_after_sync();
                 const uint32_t dacc = taddr + (uint32_t)((ch % NACC) * DN);
                 const bool fresh = it % CH == 0;

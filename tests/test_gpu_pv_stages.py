@@ -2,6 +2,8 @@
 flushes end differently (64-key stages, two sets of producer warps, chunks of
 8 stages), for the gap call and the group vote, ties at the thresholds
 included, against the fp64 oracle."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -38,3 +40,24 @@ def test_vote_stage_counts(fw, n):  # noqa: F811
     s = group_budgets(b)
     _, _, v = run_vote(fw, b, s)
     check_vote(oracle.HostRows(b), s, v)
+
+
+@pytest.mark.parametrize("n", [64 * 2, 64 * 9 + 1, 64 * 21 - 31])
+@pytest.mark.parametrize("d", [64, 128])
+def test_value_blocks_off_whole_rows(fw, n, d):  # noqa: F811
+    # v_off not a multiple of d: no stage's values can come by TMA, every one is
+    # copied by threads (one of the groups stays on whole rows)
+    R, G = 20, 3
+    rng = np.random.default_rng(n + d)
+    L = (rng.normal(size=(G * R, n)) * 1.5).astype(np.float32)
+    V = rng.normal(size=(G, n, d)).astype(np.float32)
+    b = rows_batch(L, V, np.tile(np.array([n // 3, n // 20 + 1], np.int32), (G * R, 1)), v_dtype="bf16", R=R)
+    off = np.array([8, n * d + d - 8, 2 * n * d + 2 * d], np.int64)
+    v = np.zeros(3 * n * d + 3 * d, b.v.dtype)
+    for g in range(G):
+        v[off[g]:off[g] + n * d] = b.v[g * n * d:(g + 1) * n * d]
+    b = dataclasses.replace(b, v=v, v_off=off)
+    compare(fw, b)
+    s = group_budgets(b)
+    _, _, o = run_vote(fw, b, s)
+    check_vote(oracle.HostRows(b), s, o)
