@@ -682,7 +682,10 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                     const float ub = key_to_float(*(volatile uint32_t *)&s_ub);
                     const float lb = (Ai + Bmin) + (p_i * hmin - cmx);
                     const float slack = 4e-6f * (fabsf(Ai) + fabsf(Bmin) + p_i * hmax + fabsf(cmx));  // its rounding
-                    if (!scan && lb - slack > fminf(ub, lmin) * (Pl * Pl)) return;
+                    // (ub differs by the moment each lane read it, lmin by lane: the four lanes
+                    // leave or stay together, as the shuffles below need; one lane's
+                    // exclusion holds for all, its limit is a score already found)
+                    if (!scan && __any_sync(quad, lb - slack > fminf(ub, lmin) * (Pl * Pl))) return;
                     float kmin = INFINITY, kc = -INFINITY;
                     int kq = 0;
                     for (int q0 = 0; q0 < nadd; q0 += 32) {

@@ -1,8 +1,8 @@
 """The long-row swap kernel where its bounds and branches change: extras that do
 not fill a lane's eight slots, several blocks of 32 slots, rows whose sink
 holds nearly all of the kept mass (scored by the whole block from the vector
-form), rows of equal values and of equal logits, rows longer than 8,192 keys
-(the two-blocks-per-SM form)."""
+form), rows of equal values, rows of thousands of kept keys with close scores,
+rows longer than 8,192 keys (the two-blocks-per-SM form)."""
 import numpy as np
 import pytest
 
@@ -40,3 +40,18 @@ def test_swap_equal_values_take_nothing(fw):  # noqa: F811
     torch.cuda.synchronize()
     assert torch.all(sw["refined_gap"] <= sw["topk_gap"] * (1 + 1e-6) + 1e-7)
     assert torch.all(torch.isfinite(sw["refined_gap"]))
+
+
+@pytest.mark.parametrize("n,k,d,E", [(4000, 2000, 64, 32), (3000, 2900, 128, 96), (700, 350, 256, 40)])
+def test_swap_many_kept_keys(fw, n, k, d, E):  # noqa: F811
+    # flat rows: thousands of kept keys whose scores lie close together, so the least
+    # score keeps falling while the warps use it to leave keys out; the chain is the
+    # oracle's whatever moment each warp saw (gaps to the oracle's tolerance: the
+    # band sums are added by atomics, in an order that differs from run to run)
+    rng = np.random.default_rng(n)
+    rows = 4
+    L = (0.2 * rng.normal(size=(rows, n))).astype(np.float32)
+    V = rng.normal(size=(rows, n, d)).astype(np.float32)
+    b = rows_batch(L, V, np.full((rows, 1), k), v_dtype="bf16")
+    for _ in range(2):
+        check_swap_long(fw, b, E=E, max_swaps=24)
