@@ -668,8 +668,10 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                 float lmin = INFINITY;
                 int lt = -1, li = 0, lq = 0;
                 const float pmin = s_pmin, Bmin = s_Bmin, hmin = 2.f * N * pmin, hmax = 2.f * N * s_pmax;
-                // position t, key i: its pairs, unless its bound excludes them
-                auto score_key = [&](int t, int i, float sg, float sn, float p_i, float x2, float mx, bool scan) {
+                // position t, key i: its pairs, unless its bound excludes them.  Every
+                // argument is the same in the key's four lanes, so they leave or stay
+                // together, as the shuffles below need.
+                auto score_key = [&](int t, int i, float sg, float sn, float p_i, float x2, float mx, float ub, bool scan) {
                     const float alpha = p_i * p_i * x2 - 2.f * p_i * sg;
                     const float Ai = alpha * P2 + N * p_i * (2.f * P - p_i);
                     const float Pm = P - p_i;
@@ -679,13 +681,9 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                         return;
                     }
                     const float cmx = 2.f * P2 * p_i * mx;
-                    const float ub = key_to_float(*(volatile uint32_t *)&s_ub);
                     const float lb = (Ai + Bmin) + (p_i * hmin - cmx);
                     const float slack = 4e-6f * (fabsf(Ai) + fabsf(Bmin) + p_i * hmax + fabsf(cmx));  // its rounding
-                    // (ub differs by the moment each lane read it, lmin by lane: the four lanes
-                    // leave or stay together, as the shuffles below need; one lane's
-                    // exclusion holds for all, its limit is a score already found)
-                    if (!scan && __any_sync(quad, lb - slack > fminf(ub, lmin) * (Pl * Pl))) return;
+                    if (!scan && lb - slack > ub * (Pl * Pl)) return;
                     float kmin = INFINITY, kc = -INFINITY;
                     int kq = 0;
                     for (int q0 = 0; q0 < nadd; q0 += 32) {
@@ -753,7 +751,7 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                             sk[t] = sg;
                             mk[t] = INFINITY;
                         }
-                        score_key(t, i, sg, sn, p_i, sn, INFINITY, true);
+                        score_key(t, i, sg, sn, p_i, sn, INFINITY, 0.f, true);
                     }
                 } else {
                     // software pipeline: the value row, scalars and old column entry of
@@ -779,6 +777,9 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                         float sn = lane_product_v_row<DPL, VT>(row, wdep, sub);  // v_i . (the changed slot's vector)
                         sn += __shfl_xor_sync(FW_FULL, sn, 1);
                         sn += __shfl_xor_sync(FW_FULL, sn, 2);
+                        // the least score found so far, as one lane reads it (other warps lower
+                        // it meanwhile; a vote of a key's lanes instead cost 15 to 21 % of the call)
+                        const float ub = __shfl_sync(FW_FULL, key_to_float(*(volatile uint32_t *)&s_ub), 0);
                         if (t < nk) {
                             if (t != tprev) {
                                 sn -= ym;
@@ -791,7 +792,7 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                                 }
                                 m0 = mn;
                             }
-                            score_key(t, i_cur, s0, sn, p_i, x2, m0, false);
+                            score_key(t, i_cur, s0, sn, p_i, x2, m0, ub, false);
                         }
                         row = rown;
                         i_cur = i_next;
