@@ -25,19 +25,20 @@
 // table C[slot][position] in its workspace: the first round of a budget fills
 // it (a k x d by d x E product in register tiles), and every later round
 // computes only the changed slot's column y.w_i, y the leaving key's vector,
-// and the changed position's row.  The column also carries the products with
-// g along: g moved by p_j w_j - p_i w_i, so g.w_t moves by p_j C_jt - p_i C_it,
-// the slot's old and new entry of position t.
+// and the changed position's row.  g.w_i is formed anew from g in every round,
+// beside the column and from the same read of the value row: carried along from
+// the table's entries (g.w_t moves by p_j C_jt - p_i C_it) it would gather their
+// rounding swap by swap, apart from g's own.
 //
 // A round is one pass over the kept keys: four lanes share a key (each a
-// quarter of the columns); the key's value row, its scalars and its old entry
-// of the column are read one iteration ahead.  Regrouped, D_ij = A_i + B_j +
+// quarter of the columns); the key's value row and its scalars are read one
+// iteration ahead.  Regrouped, D_ij = A_i + B_j +
 // p_i (h_j + k_j C_ij) with per-key A_i and per-slot B_j, h_j, k_j, so with m_i
 // >= max_j p_j C_ij (kept per key, raised when a slot changes) no pair of the
 // key scores below
 //   (A_i + min_j B_j + p_i min_j h_j - 2 P^2 p_i m_i) / (P - p_i + min_j p_j)^2.
 // Keys whose bound lies above the least score found so far in the block are
-// done after O(d / 4) operations per lane; the few others (about one in a
+// done after the two products; the few others (about one in a
 // hundred on the measured rows) have their E pairs scored from the table.  The
 // least score wins; among pairs at that score the smallest (i, j), except
 // that two positions of one lane at exactly the same fp32 score keep the
@@ -48,13 +49,13 @@
 // after the pass by the whole block from g' = g - u_i + u_j, the columns split
 // over the warps, a lane per slot; at most one key of a round qualifies.
 //
-// Bound: on long rows the reads of value rows, scalars and column entries
-// through the SM's L2 port (~300 bytes per kept key and round at d = 128, at
-// ~18 bytes per clock); on short rows the latency of a round's barriers.
-// Scoring every key's E pairs in every round (408 bytes per key, two products
-// with the value row) took, with the gap call, 30.2 ms on 512 rows of 32,768
-// keys with three budgets and 9.4 ms on 3,072 GQA rows of 1,000 to 8,192 keys;
-// now 19.6 and 6.1 ms.
+// Bound: on long rows the reads of value rows and scalars through the SM's L2
+// port (~280 bytes per kept key and round at d = 128) and the products' shared
+// reads; on short rows the latency of a round's barriers.  Scoring every key's E
+// pairs in every round (408 bytes per key) took, with the gap call, 30.2 ms on
+// 512 rows of 32,768 keys with three budgets and 9.4 ms on 3,072 GQA rows of
+// 1,000 to 8,192 keys; now 21.3 and 6.1 ms.  (The products by two-float FMAs;
+// one by one 21.5; g.w carried along 19.6 and 6.1.)
 #include <algorithm>
 #include <climits>
 
@@ -72,7 +73,7 @@ constexpr int QL = 4;        // lanes per kept key in the round pass
 constexpr int KPI = SWT / QL;  // kept keys per block iteration of the pass
 // resident blocks per SM: three for rows up to 8,192 keys (short rounds, whose
 // fixed per-round costs want more blocks), two above and for d = 256 (the
-// registers hold the next key's value row and the table tiles without spilling)
+// registers hold the next key's value row and the table tiles)
 constexpr int LS_BPS_SHORT = 3, LS_BPS_LONG = 2, LS_LONG_N = 8192;
 inline int ls_bps(const RowsDev &R) { return R.max_n > LS_LONG_N || R.d > 128 ? LS_BPS_LONG : LS_BPS_SHORT; }
 
@@ -93,7 +94,6 @@ struct LSArgs {
     int32_t *kbuf;   // key at each position of the current kept list
     float *pbuf;     // its mass
     float *xbuf;     // its |w|^2
-    float *sbuf;     // its g.w
     float *mbuf;     // its bound on max_j p_j C_ij
     uint32_t *kebuf; // order key of every dropped key's error (0: kept)
     // per-block cross-product table, [gridDim.x][Ep][cstride] (slot-major)
@@ -255,25 +255,42 @@ __device__ __forceinline__ void lane_products(const VT *vr, const float *mu, con
     }
 }
 
-// This lane's part of v.y from its loaded vectors.
+// a b + c of two floats at once, each rounded once
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(r)
+        : "l"(*reinterpret_cast<const unsigned long long *>(&a)), "l"(*reinterpret_cast<const unsigned long long *>(&b)),
+          "l"(*reinterpret_cast<const unsigned long long *>(&c)));
+    return *reinterpret_cast<float2 *>(&r);
+}
+
+// This lane's part of v.g and v.y from its loaded vectors (even and odd columns in
+// the halves of a two-float sum).
 template <int DPL, typename VT>
-__device__ __forceinline__ float lane_product_v_row(const LaneRow<DPL, VT> &row, const float *y, int sub)
+__device__ __forceinline__ void lane_products_v_row(const LaneRow<DPL, VT> &row, const float *g, const float *y, int sub,
+                                                    float &vg, float &vy)
 {
     using L = LaneRow<DPL, VT>;
-    float vy = 0.f, vy2 = 0.f;
+    float2 sg = make_float2(0.f, 0.f), sy = sg;
 #pragma unroll
     for (int k = 0; k < L::NVL; ++k) {
         const int c0 = (k * QL + sub) * L::EPV;
 #pragma unroll
         for (int e = 0; e < L::EPV; e += 4) {
+            const float4 g4 = *reinterpret_cast<const float4 *>(g + c0 + e);
             const float4 y4 = *reinterpret_cast<const float4 *>(y + c0 + e);
-            vy = fmaf(row.u[k].at(e), y4.x, vy);
-            vy2 = fmaf(row.u[k].at(e + 1), y4.y, vy2);
-            vy = fmaf(row.u[k].at(e + 2), y4.z, vy);
-            vy2 = fmaf(row.u[k].at(e + 3), y4.w, vy2);
+            const float2 va = make_float2(row.u[k].at(e), row.u[k].at(e + 1));
+            const float2 vb = make_float2(row.u[k].at(e + 2), row.u[k].at(e + 3));
+            sg = fma2(va, make_float2(g4.x, g4.y), sg);
+            sy = fma2(va, make_float2(y4.x, y4.y), sy);
+            sg = fma2(vb, make_float2(g4.z, g4.w), sg);
+            sy = fma2(vb, make_float2(y4.z, y4.w), sy);
         }
     }
-    return vy + vy2;
+    vg = sg.x + sg.y;
+    vy = sy.x + sy.y;
 }
 
 // NC consecutive elements of a value row as floats, by the widest loads that NC allows.
@@ -355,7 +372,7 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
     __shared__ TopmSmem s_top;
     __shared__ float red[SWW], red2[SWW];
     __shared__ int s_cnt, s_bt, s_bq, s_heavy;
-    __shared__ float s_ym, s_pmin, s_pmax, s_Bmin;
+    __shared__ float s_gm, s_ym, s_pmin, s_pmax, s_Bmin, s_hsg;
     __shared__ uint32_t s_ub;          // order key of the least score found in the round
     __shared__ unsigned long long s_bkey;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -366,7 +383,6 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
     int *kb = a.kbuf + boff;
     float *pk = a.pbuf + boff;
     float *xk = a.xbuf + boff;
-    float *sk = a.sbuf + boff;
     float *mk = a.mbuf + boff;
     uint32_t *ke = a.kebuf + boff;
     const int cs = a.cstride;
@@ -592,7 +608,7 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
             int taken = 0, cap = 0;
             bool first = true;
             int tprev = -1, qprev = -1;  // position that entered and slot that changed last round
-            float pent = 0.f, pdep = 0.f;  // masses of the keys that entered and left
+            float pdep = 0.f;              // mass of the key that left
             for (;;) {
                 if (nadd == 0 || nk == 0) break;
                 const float P2 = P * P;
@@ -615,17 +631,18 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                         partB[wid * Ep + q] = s2;
                     }
                 }
-                if (wid == 1) {  // mu.(changed slot's vector)
-                    float a2 = 0.f;
-                    for (int c = lane; c < d; c += 32) a2 = fmaf(mu[c], wdep[c], a2);
+                if (wid == 1) {  // mu.g and mu.(changed slot's vector)
+                    float a1 = 0.f, a2 = 0.f;
+                    for (int c = lane; c < d; c += 32) {
+                        a1 = fmaf(mu[c], g[c], a1);
+                        a2 = fmaf(mu[c], wdep[c], a2);
+                    }
+                    a1 = warp_sum(a1);
                     a2 = warp_sum(a2);
-                    if (lane == 0) s_ym = a2;
-                }
-                if (wid == 2 && !first) {  // g.w of the key that entered
-                    float a2 = 0.f;
-                    for (int c = lane; c < d; c += 32) a2 = fmaf(g[c], wtmp[c], a2);
-                    a2 = warp_sum(a2);
-                    if (lane == 0) sk[tprev] = a2;
+                    if (lane == 0) {
+                        s_gm = a1;
+                        s_ym = a2;
+                    }
                 }
                 if (first) cross_table<DPL, VT>(kb, nk, V, mu, Wt, Ep, nadd, cb, cs);
                 __syncthreads();
@@ -677,7 +694,10 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                     const float Pm = P - p_i;
                     const float Pl = Pm + pmin;
                     if (16.f * Pl * Pl < P2) {  // some pair needs the vector form: after the pass
-                        if (sub == 0) s_heavy = t;
+                        if (sub == 0) {
+                            s_heavy = t;
+                            s_hsg = sg;
+                        }
                         return;
                     }
                     const float cmx = 2.f * P2 * p_i * mx;
@@ -748,16 +768,14 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                         if (sub == 0) {
                             pk[t] = p_i;
                             xk[t] = sn;
-                            sk[t] = sg;
                             mk[t] = INFINITY;
                         }
                         score_key(t, i, sg, sn, p_i, sn, INFINITY, 0.f, true);
                     }
                 } else {
-                    // software pipeline: the value row, scalars and old column entry of
-                    // the next iteration and the kept index of the one after are in
-                    // flight during this one
-                    const float ym = s_ym;
+                    // software pipeline: the value row and scalars of the next iteration and
+                    // the kept index of the one after are in flight during this one
+                    const float gm = s_gm, ym = s_ym;
                     const int niter = (nk + KPI - 1) / KPI;
                     float *col = cb + (size_t)qprev * cs;
                     const int tf = gq < nk ? gq : nk - 1;
@@ -765,43 +783,42 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                     int i_next = kb[gq + KPI < nk ? gq + KPI : nk - 1];
                     LaneRow<DPL, VT> row;
                     row.load(V + (int64_t)i_cur * d, sub);
-                    float p_i = pk[tf], x2 = xk[tf], s0 = sk[tf], m0 = mk[tf], c0 = col[tf];
+                    float p_i = pk[tf], x2 = xk[tf], m0 = mk[tf];
                     for (int it = 0; it < niter; ++it) {
                         const int t = it * KPI + gq;
                         const int tn = t + KPI < nk ? t + KPI : nk - 1;
-                        const float p_n = pk[tn], x2_n = xk[tn], s_n = sk[tn], m_n = mk[tn], c_n = col[tn];
+                        const float p_n = pk[tn], x2_n = xk[tn], m_n = mk[tn];
                         LaneRow<DPL, VT> rown;
                         rown.load(V + (int64_t)i_next * d, sub);
                         const int tnn = t + 2 * KPI;
                         const int i_nn = kb[tnn < nk ? tnn : nk - 1];
-                        float sn = lane_product_v_row<DPL, VT>(row, wdep, sub);  // v_i . (the changed slot's vector)
+                        float sg, sn;  // v_i.g and v_i . (the changed slot's vector)
+                        lane_products_v_row<DPL, VT>(row, g, wdep, sub, sg, sn);
+                        sg += __shfl_xor_sync(FW_FULL, sg, 1);
                         sn += __shfl_xor_sync(FW_FULL, sn, 1);
+                        sg += __shfl_xor_sync(FW_FULL, sg, 2);
                         sn += __shfl_xor_sync(FW_FULL, sn, 2);
                         // the least score found so far, as one lane reads it (other warps lower
                         // it meanwhile; a vote of a key's lanes instead cost 15 to 21 % of the call)
                         const float ub = __shfl_sync(FW_FULL, key_to_float(*(volatile uint32_t *)&s_ub), 0);
                         if (t < nk) {
+                            sn -= ym;
                             if (t != tprev) {
-                                sn -= ym;
-                                s0 = fmaf(pent, c0, fmaf(-pdep, sn, s0));
                                 const float mn = fmaxf(m0, pdep * sn);
                                 if (sub == 0) {
-                                    sk[t] = s0;
                                     col[t] = sn;
                                     if (mn > m0) mk[t] = mn;
                                 }
                                 m0 = mn;
                             }
-                            score_key(t, i_cur, s0, sn, p_i, x2, m0, ub, false);
+                            score_key(t, i_cur, sg - gm, sn, p_i, x2, m0, ub, false);
                         }
                         row = rown;
                         i_cur = i_next;
                         i_next = i_nn;
                         p_i = p_n;
                         x2 = x2_n;
-                        s0 = s_n;
                         m0 = m_n;
-                        c0 = c_n;
                     }
                 }
                 first = false;
@@ -826,7 +843,7 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                     }
                     __syncthreads();
                     if (wid == 0) {
-                        const float alpha = p_i * p_i * xk[th] - 2.f * p_i * sk[th];
+                        const float alpha = p_i * p_i * xk[th] - 2.f * p_i * s_hsg;
                         const float Ai = alpha * P2 + N * p_i * (2.f * P - p_i);
                         const float Pm = P - p_i;
                         for (int q = lane; q < nadd; q += 32) {
@@ -899,7 +916,6 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                     a.swap_out[rb * MS + taken] = bi;
                     a.swap_in[rb * MS + taken] = bj;
                 }
-                pent = p_j;
                 pdep = p_i;
                 tprev = tb;
                 qprev = qj;
@@ -949,7 +965,7 @@ static size_t ls_table_bytes(const RowsDev &R, int E)
 size_t long_swap_workspace(const RowsDev &R, int nb, int E, int max_swaps)
 {
     (void)nb, (void)max_swaps;
-    return ls_array_bytes(R) * 7 + ls_table_bytes(R, E);
+    return ls_array_bytes(R) * 6 + ls_table_bytes(R, E);
 }
 
 fw_status long_swap(const RowsDev &R, const int32_t *k, int nb, const fw_gap_out &topk, int E, int max_swaps,
@@ -984,10 +1000,9 @@ fw_status long_swap(const RowsDev &R, const int32_t *k, int nb, const fw_gap_out
     a.kbuf = (int32_t *)(w + 1 * arr);
     a.pbuf = (float *)(w + 2 * arr);
     a.xbuf = (float *)(w + 3 * arr);
-    a.sbuf = (float *)(w + 4 * arr);
-    a.mbuf = (float *)(w + 5 * arr);
-    a.kebuf = (uint32_t *)(w + 6 * arr);
-    a.cbuf = (float *)(w + 7 * arr);
+    a.mbuf = (float *)(w + 4 * arr);
+    a.kebuf = (uint32_t *)(w + 5 * arr);
+    a.cbuf = (float *)(w + 6 * arr);
     FW_DISPATCH(R.d, R.v_dtype, {
         const size_t smem = ls_smem<DPL>(a.Ep);
         constexpr int SHORT = DPL <= 4 ? LS_BPS_SHORT : LS_BPS_LONG;

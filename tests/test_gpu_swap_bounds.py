@@ -6,6 +6,8 @@ rows longer than 8,192 keys (the two-blocks-per-SM form)."""
 import numpy as np
 import pytest
 
+import oracle
+from tests.parity import assert_close, np_, row_onorm
 from tests.test_gpu_long import check_swap_long, fw  # noqa: F401  (fw is a fixture)
 from tests.test_gpu_small import rows_batch
 
@@ -55,3 +57,40 @@ def test_swap_many_kept_keys(fw, n, k, d, E):  # noqa: F811
     b = rows_batch(L, V, np.full((rows, 1), k), v_dtype="bf16")
     for _ in range(2):
         check_swap_long(fw, b, E=E, max_swaps=24)
+
+
+@pytest.mark.parametrize("n,k,d", [(3000, 1000, 256), (2500, 600, 64), (2000, 500, 32)])
+def test_swap_long_chains(fw, n, k, d):  # noqa: F811
+    # 80 to 100 swaps a row, to the end of the chain: the decisions are still good (the
+    # oracle's near-ties may part the two, but every swap lowers the fp64 gap and the
+    # chain ends as low as the oracle's), and the gap is that of the set the swaps name
+    import torch
+
+    rng = np.random.default_rng(n)
+    rows = 3
+    L = (0.5 * rng.normal(size=(rows, n))).astype(np.float32)
+    V = rng.normal(size=(rows, n, d))
+    V += 0.5 * np.sign(L)[:, :, None] * rng.normal(size=(rows, 1, d))  # top-mass values lean to one side
+    V = V.astype(np.float32)
+    b = rows_batch(L, V, np.full((rows, 1), k))
+    r = fw.rows_from_batch(b)
+    kt = torch.as_tensor(np.asarray(b.k)).cuda()
+    sw = fw.swap_refine(r, kt, fw.dense_and_topk_gap(r, kt), E=96, max_swaps=400)
+    o = oracle.swap_refine(b, E=96, max_swaps=400)
+    on = row_onorm(oracle.dense_and_topk_gap(b)["o"])
+    assert_close(np_(sw["refined_gap"]), o["refined_gap"], on, "refined_gap")
+    assert o["n_swaps"].min() >= 60 and not np_(sw["capped"]).any()
+    for row in range(rows):
+        l, v = L[row].astype(np.float64), V[row].astype(np.float64)
+        p = np.exp(l - l.max())
+        p /= p.sum()
+        u = p[:, None] * (v - p @ v)
+        kept = np.zeros(n, bool)
+        kept[np.lexsort((np.arange(n), -l))[:k]] = True
+        es = np.linalg.norm(u[kept].sum(0)) / p[kept].sum()
+        for i, j in np_(torch.stack([sw["swap_out"][row, 0], sw["swap_in"][row, 0]], 1))[:int(sw["n_swaps"][row, 0])]:
+            assert kept[i] and not kept[j]
+            kept[i], kept[j] = False, True
+            last, es = es, np.linalg.norm(u[kept].sum(0)) / p[kept].sum()
+            assert es < last * (1 + 1e-6)  # (fp32 cannot tell smaller steps from none)
+        assert abs(float(sw["refined_gap"][row, 0]) - es) <= 1e-4 * es + 1e-6 * on[row]
