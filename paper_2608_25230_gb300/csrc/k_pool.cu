@@ -20,7 +20,8 @@
 // h = H 1_K,
 //   val(A) = val(K) + sum_R (H_xx - 2 h_x) + sum_D (H_yy + 2 h_y)
 //            + 2 sum_{pairs in R} H + 2 sum_{pairs in D} H - 2 sum_{R x D} H.
-// val(K) and h come from sum_K u, summed in double-float; G is plain fp32.  The
+// val(K) and h come from sum_K u, summed in fp64 (h by double-float products); G is
+// plain fp32.  The
 // rounding of the whole is at most kappa (e^2 + 2 e b + val(K)), b = |sum_K u|
 // + sqrt(t) p(K), e the sum over the exchanged keys of a_x = |u_x| + sqrt(t) p_x
 // -- a bound that leaves out the heavy keys both sets share -- and is a
@@ -28,7 +29,7 @@
 // <= 0" is a necessary condition and costs nothing.  A sweep over the subsets
 // collects those that pass, with their values; value and bound give each an
 // interval for es^2, the few whose lower end does not exceed the least upper
-// end are scored from the value rows in double-float, and the least es wins,
+// end are scored from the value rows in fp64, and the least es wins,
 // exact ties to the smallest colex rank of the members' pool positions.  Where
 // more than GCAP pass -- rows with good subsets that leave out the attention
 // sink, far from the top-mass set, whose values the bound around that set
@@ -355,7 +356,8 @@ struct EnumSm {
     uint32_t rmask[PE_GMAX * PE_CH];
     float rbase[PE_GMAX * PE_CH];
     float o[256];
-    float UKh[256], UKl[256];   // sum over K of u, by column, in double-float
+    double UK[256];             // sum over K of u, by column
+    float UKh[256], UKl[256];   // ... as double-float, for the products below
     float gh[PMAX], gl[PMAX];   // its products with v_x - o
     float pp[PMAX];             // masses
     float ax[PMAX];             // |u_x| + sqrt(t) p_x, scaled
@@ -368,33 +370,29 @@ struct EnumSm {
     int seg_r[PSMAX], seg_g[PSMAX], seg_n[PSMAX], nseg, next_r, next_g;
 };
 
-// columns c + step k (k < NC, below d) of sum over A of p (v - o), in
-// double-float, members ascending; the columns are independent chains
+// columns c + step k (k < NC, below d) of sum over A of p (v - o), in fp64,
+// members ascending; the columns are independent chains
 template <int NC>
 __device__ __forceinline__ void col_sums(const EnumSm &S, const float *v, int d, uint64_t A, int c, int step,
                                          double (&out)[NC])
 {
-    float hi[NC], lo[NC];
+    double o[NC];
 #pragma unroll
-    for (int k = 0; k < NC; ++k) hi[k] = lo[k] = 0.f;
+    for (int k = 0; k < NC; ++k) {
+        out[k] = 0.0;
+        o[k] = c + step * k < d ? (double)S.o[c + step * k] : 0.0;
+    }
     for (uint64_t w = A; w; w &= w - 1) {
         const int x = __ffsll((long long)w) - 1;
-        const float p = S.pp[x];
+        const double p = (double)S.pp[x];
         const float *vx = v + x * (d + 4);
 #pragma unroll
         for (int k = 0; k < NC; ++k) {
             const int ck = c + step * k;
             if (ck >= d) break;
-            const df u = df_two_sum(vx[ck], -S.o[ck]);  // v - o exactly
-            const float q = p * u.hi;
-            const float e = fmaf(p, u.lo, fmaf(p, u.hi, -q));
-            const df t = df_two_sum(hi[k], q);
-            hi[k] = t.hi;
-            lo[k] += t.lo + e;
+            out[k] = fma(p, (double)vx[ck] - o[k], out[k]);
         }
     }
-#pragma unroll
-    for (int k = 0; k < NC; ++k) out[k] = (double)hi[k] + (double)lo[k];
 }
 
 __device__ __forceinline__ double mass_warp(const EnumSm &S, uint64_t A, int lane)
@@ -852,6 +850,7 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
                 double uc[1];
                 col_sums<1>(S, v, d, K, c, 1, uc);
                 const df u = df_from_double(uc[0]);
+                S.UK[c] = uc[0];
                 S.UKh[c] = u.hi;
                 S.UKl[c] = u.lo;
             }
@@ -864,7 +863,7 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
             if (wid == 0) {  // es(K), and the best set so far
                 double q = 0.0;
                 for (int c = lane; c < d; c += 32) {  // (es_warp's order)
-                    const double u = (double)S.UKh[c] + (double)S.UKl[c];
+                    const double u = S.UK[c];
                     q = fma(u, u, q);
                 }
                 q = warp_sum_d(q);

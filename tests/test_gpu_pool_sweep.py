@@ -13,6 +13,7 @@ from tests.test_gpu_pool import check_pool, fw, run_pool  # noqa: F401  (fw is a
 from tests.test_gpu_small import rows_batch
 
 pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
 
 
 def _rows(seed, rows, n, d, sink, tau):
@@ -49,3 +50,19 @@ def test_every_subset_ties(fw):  # noqa: F811
     _, out = run_pool(fw, b, [8])
     assert np.all(np_(out["n_cand"]) == math.comb(14, 6))
     check_pool(fw, b, [8], out=out)
+
+
+def test_sums_that_need_52_bits(fw):  # noqa: F811
+    # equal masses, o = 0.  The best subsets are {4, 5, 6} with key 1 or with key 0: the
+    # first column sums to 1 or to 1 + 2^-24, beside terms of 2^27 that cancel.  Sums
+    # of fewer than 52 bits make it a tie, which key 0 (the smaller rank) would win
+    V = np.zeros((1, 8, 32), np.float32)
+    V[0, :, 0] = [2.0 ** -24, 0, -(2.0 ** -24), 0, 2.0 ** 27, 1, -(2.0 ** 27), -1]
+    V[0, :, 1] = [0, 0, 0, 30, 100, -200, 100, -30]
+    V[0, :, 2] = [0, 0, 50, -50, 0, 0, 0, 0]
+    b = rows_batch(np.zeros((1, 8), np.float32), V, [[4]])
+    rows, out = run_pool(fw, b, [3])
+    top = fw.dense_and_topk_gap(rows, torch.tensor([[4]], dtype=torch.int32).cuda())
+    assert not np_(top["o"]).any()
+    np.testing.assert_array_equal(np_(out["best_idx"])[0, 0, :4], [1, 4, 5, 6])
+    assert float(np_(out["best_gap"])[0, 0]) == 0.25
