@@ -218,7 +218,8 @@ size_t fw_group_vote_workspace(const fw_rows *rows, int32_t nb);
  *   k    : device [rows][nb] budgets, 1 <= s <= min(n, 32, k_max); a slot with
  *          s + min(E[b], n - s) > 64 pool keys, or more than 2^32 subsets on
  *          the pool's smaller side, is refused (row_status FW_ERR_UNSUPPORTED,
- *          its gap NaN); an out-of-range s gives FW_ERR_INVALID_ARG.
+ *          its gap NaN); an out-of-range s gives FW_ERR_INVALID_ARG, a
+ *          non-finite logit or value of the row FW_ERR_NONFINITE (gaps NaN).
  *   E    : HOST [nb] extras per budget slot, >= 0 (the paper's schedule is
  *          24/12/6/4 at s = 4/8/16/32).
  *   topk : a fw_gap_out filled by fw_dense_and_topk_gap for the same rows, k

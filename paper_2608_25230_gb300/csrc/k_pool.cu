@@ -48,12 +48,18 @@
 // (by which rows were drawn) with one warp per item that scored every subset
 // from scratch under an error bound of the whole pool's sum |u| and re-scored
 // what passed in fp64.  16 warps per block (64 registers) rather than 8: 0.71
-// against 0.80 ms, the sweeps wait on shared memory.
+// against 0.80 ms, the sweeps wait on shared memory.  Since then fp64 scores instead
+// of double-float ones cost 1.2 %, the checks of range 2.1 %.
+//
+// Rows with a non-finite logit or value have no es to compare and are reported
+// before any sweep.  Masses are scaled by a power of two where the largest u is
+// far from 1, which changes no es, so that finite rows keep their bounds.
 //
 // Nothing waits on another block; when sweeping around better sets does not
 // bring the hits below GCAP (exact ties by the thousand) the lanes score every
 // hit, so the answer stays exact.
 #include <algorithm>
+#include <cfloat>
 #include <climits>
 
 #include "fw_internal.h"
@@ -80,6 +86,7 @@ constexpr int PE_SWEEPS = 8;         // sweeps before the lanes score every cand
 constexpr uint64_t PE_MAX_SUBSETS = 1ull << 32;
 constexpr int CLD = PMAX + 1;        // table row stride (odd: conflict-free columns)
 constexpr float PE_TINY = 1e-36f;    // slack for subnormal table entries
+constexpr int PE_XMASS = 90;         // largest scale of the masses, as an exponent
 
 // C(a, b) for a <= 64, b <= 32 (all below 2^63), by Pascal's rule at compile time.
 struct Binom64Table {
@@ -109,7 +116,8 @@ struct PoolArgs {
     const int32_t *thr_idx;
     const float *o, *M, *Z;    // [rows][d], [rows], [rows]
     int32_t *pool;             // ws [rows][nb][PMAX] ascending key indices
-    int32_t *pool_n;           // ws [rows][nb] pool size; -1 invalid budget, -2 pool too large
+    int32_t *pool_n;           // ws [rows][nb] pool size; -1 invalid budget, -2 pool too large, -3 a logit
+                               // of the row is not finite
     float *best_gap;           // [rows][nb]
     int32_t *best_idx;         // [rows][nb][k_max]
     int k_max;
@@ -165,6 +173,7 @@ __global__ void __launch_bounds__(PB_T) k_pool_build(PoolArgs a)
             for (int e = 0; e < L::EPV; ++e) so[q * L::EPV + e] = a.o[r * d + (q * PB_Q + sub) * L::EPV + e];
         __syncthreads();  // the previous row's shared arrays are no longer read
         if (tid == 0) s_cnt = 0;
+        bool bad = false;  // a logit is not finite
         // two keys in flight per group of four lanes
         for (int j0 = 0; j0 < n; j0 += 2 * KPI) {
             const int ja = j0 + gq, jb = j0 + KPI + gq;
@@ -172,7 +181,9 @@ __global__ void __launch_bounds__(PB_T) k_pool_build(PoolArgs a)
             ra.load(V + (int64_t)min(ja, n - 1) * d, sub);
             rb.load(V + (int64_t)min(jb, n - 1) * d, sub);
             const int jm = sub & 1 ? jb : ja;  // lanes 0 and 1 finish one key each
-            const float p = sub < 2 ? __expf(__ldg(l + min(jm, n - 1)) - M) * Zi : 0.f;
+            const float lj = __ldg(l + min(jm, n - 1));
+            bad |= !isfinite(lj);
+            const float p = sub < 2 ? __expf(lj - M) * Zi : 0.f;
             float sa = 0.f, sb = 0.f;
 #pragma unroll
             for (int q = 0; q < L::NV; ++q)
@@ -189,6 +200,7 @@ __global__ void __launch_bounds__(PB_T) k_pool_build(PoolArgs a)
             sb += __shfl_xor_sync(FW_FULL, sb, 2);
             if (sub < 2 && jm < n) e2[jm] = p * p * (sub ? sb : sa);
         }
+        const int nonfinite = __syncthreads_or(bad);
         // the budgets: sizes, and the longest prefix of the error order any of them needs
         int m = 0;
         int sb_[4], Eb[4];
@@ -202,11 +214,12 @@ __global__ void __launch_bounds__(PB_T) k_pool_build(PoolArgs a)
             if (b >= a.nb) continue;
             const int64_t rb = r * a.nb + b;
             const int s = a.k[rb];
-            int bad = 0;
-            if (s < 1 || s > n || s > PSMAX || s > a.k_max || a.E[b] < 0) bad = -1;
-            else if (s + min(a.E[b], n - s) > PMAX) bad = -2;
-            if (bad) {
-                if (tid == 0) a.pool_n[rb] = bad;
+            int no = 0;
+            if (s < 1 || s > n || s > PSMAX || s > a.k_max || a.E[b] < 0) no = -1;
+            else if (s + min(a.E[b], n - s) > PMAX) no = -2;
+            else if (nonfinite) no = -3;
+            if (no) {
+                if (tid == 0) a.pool_n[rb] = no;
                 continue;
             }
             sb_[b] = s;
@@ -215,7 +228,6 @@ __global__ void __launch_bounds__(PB_T) k_pool_build(PoolArgs a)
             ti[b] = a.thr_idx[rb];
             m = max(m, s + Eb[b]);
         }
-        __syncthreads();
         if (m == 0) continue;  // (uniform)
         uint32_t T = 0u;
         int Lx = -1;
@@ -341,7 +353,7 @@ __device__ __forceinline__ uint64_t colex_rank64(uint64_t A)
 
 // state of one (row, budget); the value rows v [PMAX][d + 4] follow it
 struct EnumSm {
-    double QK, PK, bes;         // |sum_K u|^2, p(K), the least es known
+    double QK, PK, rPK, bes;    // |sum_K u|^2, p(K) and its inverse, the least es known
     uint64_t K, topK;           // the set exchanged from; kept keys by the thresholds
     uint64_t bmask, brank;      // the best set known, its colex rank
     uint64_t candD[GCAP];       // hits: the big side's keys exchanged ...
@@ -728,13 +740,13 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
         const int P = a.pool_n[it];
         int32_t *bi = a.best_idx + it * a.k_max;
         // refused items: an out-of-range budget (P = -1), a pool over PMAX keys
-        // (P = -2), or more subsets than the enumeration takes
-        int refuse = P == -1 ? FW_ERR_INVALID_ARG : (P < 0 ? FW_ERR_UNSUPPORTED : 0);
-        if (!refuse && P < s) refuse = FW_ERR_INVALID_ARG;  // thresholds that keep fewer than s keys
-        if (!refuse && cb(P, min(s, P - s)) > PE_MAX_SUBSETS) refuse = FW_ERR_UNSUPPORTED;
-        if (refuse) {
+        // (P = -2), a non-finite logit (P = -3), thresholds that keep fewer than s
+        // keys, or more subsets than the enumeration takes
+        int status = P == -2 ? FW_ERR_UNSUPPORTED : (P == -3 ? FW_ERR_NONFINITE : (P < s ? FW_ERR_INVALID_ARG : FW_OK));
+        if (status == FW_OK && cb(P, min(s, P - s)) > PE_MAX_SUBSETS) status = FW_ERR_UNSUPPORTED;
+        if (status != FW_OK) {
             if (tid == 0) {
-                if (a.row_status) atomicMax(a.row_status + r, refuse);
+                if (a.row_status) atomicMax(a.row_status + r, status);
                 a.best_gap[it] = __int_as_float(0x7fc00000);
                 if (a.topk_gap) a.topk_gap[it] = __int_as_float(0x7fc00000);
                 if (a.n_cand) a.n_cand[it] = 0;
@@ -778,38 +790,6 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
             *reinterpret_cast<float4 *>(v + x * ld + c) = u;
         }
         __syncthreads();
-        // ---- G in fp32: 2 x 2 keys per thread and step, four partial sums per entry
-        {
-            const int P2 = (P + 1) / 2, nt = P2 * (P2 + 1) / 2;
-            for (int i = tid; i < nt; i += PE_T) {
-                int x = (int)((sqrtf(8.f * (float)i + 1.f) - 1.f) * 0.5f);
-                while (x * (x + 1) / 2 > i) --x;
-                while ((x + 1) * (x + 2) / 2 <= i) ++x;
-                const int y = i - x * (x + 1) / 2;
-                const float *x0 = v + 2 * x * ld, *y0 = v + 2 * y * ld;
-                float4 s00{}, s01{}, s10{}, s11{};
-                for (int c = 0; c < d; c += 4) {
-                    const float4 o4 = *reinterpret_cast<const float4 *>(S.o + c);
-                    auto diff = [&](const float *q) {
-                        const float4 u = *reinterpret_cast<const float4 *>(q);
-                        return make_float4(u.x - o4.x, u.y - o4.y, u.z - o4.z, u.w - o4.w);
-                    };
-                    const float4 xa = diff(x0 + c), xb = diff(x0 + ld + c), ya = diff(y0 + c), yb = diff(y0 + ld + c);
-                    auto mac = [](float4 &s, const float4 &p, const float4 &q) {
-                        s.x = fmaf(p.x, q.x, s.x), s.y = fmaf(p.y, q.y, s.y);
-                        s.z = fmaf(p.z, q.z, s.z), s.w = fmaf(p.w, q.w, s.w);
-                    };
-                    mac(s00, xa, ya), mac(s01, xa, yb), mac(s10, xb, ya), mac(s11, xb, yb);
-                }
-                auto put = [&](int p, int q, const float4 &s4) {
-                    if (p >= P || q >= P) return;
-                    const float w = ((s4.x + s4.y) + (s4.z + s4.w)) * (S.pp[p] * S.pp[q]);
-                    S.G[p * CLD + q] = S.G[q * CLD + p] = w;
-                };
-                put(2 * x, 2 * y, s00), put(2 * x + 1, 2 * y, s10), put(2 * x + 1, 2 * y + 1, s11);
-                if (x != y) put(2 * x, 2 * y + 1, s01);
-            }
-        }
         const uint64_t topK = S.topK;
         // the set exchanged from: the top-mass set (s keys also where the
         // caller's thresholds keep another count)
@@ -817,7 +797,7 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
         const bool ksmall = s <= P - s;  // the smaller side: K or the keys outside it
         const int ns = ksmall ? s : P - s, nbg = P - ns;
         // roundings: the table sums' chains, and the entries' own (fp32 G)
-        const float kappa = (float)(ns * (ns + 1) / 2 + 2 * ns + 10 + d / 4 + 12) * 1.5f * 5.9604645e-8f;
+        const float kappa = (float)(ns * (ns + 1) / 2 + 2 * ns + 10 + d / 4 + 18) * 1.5f * 5.9604645e-8f;
         int64_t ncand = 1;
         // the block's subset of least value (every thread)
         auto least_of = [&](LaneBest &lb) -> uint64_t {
@@ -844,7 +824,40 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
             return mk;
         };
         // (fp64 runs at 1/60 of fp32's rate here: scalars in fp64 are one thread's work)
+        bool scaled = false;
         for (int round = 0;; ++round) {
+            // ---- G in fp32: 2 x 2 keys per thread and step, four partial sums per entry
+            if (round == 0) {
+                const int P2 = (P + 1) / 2, nt = P2 * (P2 + 1) / 2;
+                for (int i = tid; i < nt; i += PE_T) {
+                    int x = (int)((sqrtf(8.f * (float)i + 1.f) - 1.f) * 0.5f);
+                    while (x * (x + 1) / 2 > i) --x;
+                    while ((x + 1) * (x + 2) / 2 <= i) ++x;
+                    const int y = i - x * (x + 1) / 2;
+                    const float *x0 = v + 2 * x * ld, *y0 = v + 2 * y * ld;
+                    float4 s00{}, s01{}, s10{}, s11{};
+                    for (int c = 0; c < d; c += 4) {
+                        const float4 o4 = *reinterpret_cast<const float4 *>(S.o + c);
+                        auto diff = [&](const float *q) {
+                            const float4 u = *reinterpret_cast<const float4 *>(q);
+                            return make_float4(u.x - o4.x, u.y - o4.y, u.z - o4.z, u.w - o4.w);
+                        };
+                        const float4 xa = diff(x0 + c), xb = diff(x0 + ld + c), ya = diff(y0 + c), yb = diff(y0 + ld + c);
+                        auto mac = [](float4 &s, const float4 &p, const float4 &q) {
+                            s.x = fmaf(p.x, q.x, s.x), s.y = fmaf(p.y, q.y, s.y);
+                            s.z = fmaf(p.z, q.z, s.z), s.w = fmaf(p.w, q.w, s.w);
+                        };
+                        mac(s00, xa, ya), mac(s01, xa, yb), mac(s10, xb, ya), mac(s11, xb, yb);
+                    }
+                    auto put = [&](int p, int q, const float4 &s4) {
+                        if (p >= P || q >= P) return;
+                        const float w = ((s4.x + s4.y) + (s4.z + s4.w)) * S.pp[p] * S.pp[q];
+                        S.G[p * CLD + q] = S.G[q * CLD + p] = w;
+                    };
+                    put(2 * x, 2 * y, s00), put(2 * x + 1, 2 * y, s10), put(2 * x + 1, 2 * y + 1, s11);
+                    if (x != y) put(2 * x, 2 * y + 1, s01);
+                }
+            }
             // ---- sum_K u
             for (int c = tid; c < d; c += PE_T) {
                 double uc[1];
@@ -880,6 +893,7 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
                     }
                     S.QK = q;
                     S.PK = pk;
+                    S.rPK = 1.0 / pk;
                     S.K = K;
                     S.ncand = S.nsurv = 0;
                     if (round == 0 && a.topk_gap && topK == K) a.topk_gap[it] = (float)ek;
@@ -914,18 +928,31 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
                 const double te = es_warp(S, v, d, topK, lane);
                 if (lane == 0) a.topk_gap[it] = (float)te;
             }
-            if (ns == 0) break;
+            if (ns == 0 || !isfinite(S.bes)) break;  // (not finite: a value of the row, hence o, is not)
             // ---- the tables, scaled by a power of two that brings the largest a_x^2 near 1
-            const float tf = (float)S.bes * (float)S.bes;
+            const float te = (float)S.bes;
             float amax = 0.f;
-            for (int x = lane; x < P; x += 32) amax = fmaxf(amax, S.G[x * CLD + x] + tf * S.pp[x] * S.pp[x]);
+            for (int x = lane; x < P; x += 32) amax = fmaxf(amax, fmaxf(sqrtf(S.G[x * CLD + x]), te * S.pp[x]));
             amax = warp_max(amax);
-            // (vectors that are all zero, subnormal or beyond fp32's range: no
-            // value decides anything, every subset is a hit)
-            const bool blind = !(amax > 1e-30f && amax < 1e30f);
+            // es does not change with a factor of the masses: where the products leave the
+            // range whose squares fp32 holds (a sink so heavy that every u is tiny), a power
+            // of two on the masses brings them back, once
+            const bool far = !(amax > 1e-15f && amax < 1e15f);
+            if (far && !scaled && amax > 0.f) {
+                __syncthreads();  // the state above is no longer read
+                if (tid < P) S.pp[tid] = scalbnf(S.pp[tid], amax < INFINITY ? max(-PE_XMASS, min(-ilogbf(amax), PE_XMASS)) : -PE_XMASS);
+                __syncthreads();
+                scaled = true;
+                round = -1;
+                continue;
+            }
+            // (vectors that are all zero, or beyond even that: no value decides anything,
+            // every subset is a hit)
+            const bool blind = far;
+            amax *= amax;
             const float sc = blind ? 1.f : scalbnf(1.f, -ilogbf(amax));
             if (tid < P) {
-                const float st = sqrtf(tf * sc) * 1.00001f;
+                const float st = te * sqrtf(sc) * 1.00001f;
                 S.ax[tid] = sqrtf(S.G[tid * CLD + tid] * sc) * 1.00001f + st * S.pp[tid];
                 // h_x = u_x . sum_K u - t p_x p(K), kept in the slot of the double-float product
                 const double t = S.bes * S.bes;
@@ -933,18 +960,18 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
                 if (tid == 0) {
                     S.red_v[0] = (float)((S.QK - t * S.PK * S.PK) * (double)sc);
                     S.red_v[1] = (sqrtf((float)(S.QK * (double)sc)) + st * (float)S.PK) * 1.00001f;
-                    S.red_v[2] = (float)(t * (double)sc);
+                    S.red_v[2] = te * sqrtf(sc);
                 }
             }
             __syncthreads();
-            const float c0 = S.red_v[0], b0 = S.red_v[1], ts = S.red_v[2];
+            const float c0 = S.red_v[0], b0 = S.red_v[1], rt = S.red_v[2];
             const float base0 = blind ? -1.f : c0 - kappa * fabsf(c0);
             for (int i = wid; i < P; i += PE_NW) {
                 const int x = S.loc[i];
                 const float ax = S.ax[x], px = S.pp[x];
                 for (int j = lane; j <= i; j += 32) {
                     const int y = S.loc[j];
-                    const float H = S.G[x * CLD + y] * sc - ts * px * S.pp[y];
+                    const float H = S.G[x * CLD + y] * sc - (rt * px) * (rt * S.pp[y]);
                     float w;
                     if (i == j) w = H + ((i < ns) == ksmall ? -2.f : 2.f) * S.gh[x] - kappa * ax * (ax + 2.f * b0);
                     else w = ((i < ns) == (j < ns) ? 2.f : -2.f) * H - 2.f * kappa * ax * S.ax[y];
@@ -985,7 +1012,7 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
                 __syncthreads();
                 ncand = 1;
                 for (int w = 0; w < PE_NW; ++w) ncand += S.red_seen[w];
-                if (tid == 0) S.bes = INFINITY;  // (the warps' include it)
+                if (tid == 0) S.bes = DBL_MAX;  // (the warps' include it)
                 break;
             }
             if (S.ncand > GCAP) {  // (uniform)
@@ -997,7 +1024,7 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
                 __syncthreads();  // the state above is no longer read
                 continue;
             }
-            // ---- each hit's interval of es^2 - t: [v, v + 2 bound] / p(A)^2
+            // ---- each hit's interval of es^2 - t, times p(K)^2: [v, v + 2 bound] (p(K) / p(A))^2
             const int seen = S.ncand;
             constexpr int PER = (GCAP + PE_T - 1) / PE_T;
             float up = 0.f;
@@ -1021,7 +1048,7 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
                 }
                 const double pa = S.PK + (ksmall ? pd - pr : pr - pd);
                 // masses that cancel to nothing leave the hit to the exact score
-                const float p2 = !blind && pa > 1e-9 * (pr + pd) ? (float)(pa * pa) : 0.f;
+                const float p2 = !blind && pa > 1e-9 * (pr + pd) ? (float)(pa * S.rPK * (pa * S.rPK)) : 0.f;
                 const float lov = S.candV[i];
                 const float upv = lov + 2.f * kappa * (e * (e + 2.f * b0) + fabsf(c0)) * 1.001f + 2.f * PE_TINY;
                 myl[q] = p2 > 0.f ? (lov - 1e-5f * fabsf(lov)) / p2 : -INFINITY;
@@ -1076,7 +1103,13 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
             break;
         }
         __syncthreads();
-        if (tid == 0) {
+        const bool none = !isfinite(S.bes);  // no subset has an es
+        if (tid == 0 && none) {
+            if (a.row_status) atomicMax(a.row_status + r, (int)FW_ERR_NONFINITE);
+            a.best_gap[it] = __int_as_float(0x7fc00000);
+            if (a.topk_gap) a.topk_gap[it] = __int_as_float(0x7fc00000);
+            if (a.n_cand) a.n_cand[it] = 0;
+        } else if (tid == 0) {
             if (ns > 0)
                 for (int w = 0; w < PE_NW; ++w)
                     if (S.red_es[w] < S.bes || (S.red_es[w] == S.bes && S.red_rank[w] < S.brank)) {
@@ -1088,9 +1121,9 @@ __global__ void __launch_bounds__(PE_T, PE_BPS) k_pool_enum(PoolArgs a)
             if (a.n_cand) a.n_cand[it] = ncand;
         }
         __syncthreads();
-        const uint64_t bmask = S.bmask;
+        const uint64_t bmask = none ? 0 : S.bmask;
         if (tid < P && ((bmask >> tid) & 1ull)) bi[__popcll(bmask & ((1ull << tid) - 1ull))] = S.pidx[tid];
-        for (int q = s + tid; q < a.k_max; q += PE_T) bi[q] = -1;
+        for (int q = (none ? 0 : s) + tid; q < a.k_max; q += PE_T) bi[q] = -1;
     }
 }
 

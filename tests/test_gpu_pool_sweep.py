@@ -1,8 +1,10 @@
 """ES_pool's enumeration at the sizes where its sweeps change shape, against the
 fp64 oracle: one batch or several of the smaller side's subsets, 1 to 9 and
 more exchanged keys (the unrolled and the general member loops), odd and full
-pools, rows whose best subsets leave out the sink (swept again around them)
-and rows of equal values (every subset scored)."""
+pools, rows whose best subsets leave out the sink (swept again around them),
+rows of equal values (every subset scored), non-finite rows and pools whose
+products leave the range fp32 squares hold."""
+import itertools
 import math
 
 import numpy as np
@@ -66,3 +68,43 @@ def test_sums_that_need_52_bits(fw):  # noqa: F811
     assert not np_(top["o"]).any()
     np.testing.assert_array_equal(np_(out["best_idx"])[0, 0, :4], [1, 4, 5, 6])
     assert float(np_(out["best_gap"])[0, 0]) == 0.25
+
+
+def test_rows_without_an_answer(fw):  # noqa: F811
+    # a NaN or infinite logit, or value, leaves no es to compare: the row is reported
+    # and nothing is enumerated (a pool of 1.9e9 subsets a row)
+    L, V = _rows(3, 8, 100, 32, 2.0, 1.0)
+    L[0, 50], L[1, 7], L[2, 8] = np.nan, np.inf, -np.inf
+    V[3, 60, 5], V[4, 0, 31], V[5, 2, 0] = np.nan, np.inf, -np.inf
+    _, out = run_pool(fw, rows_batch(L, V, np.tile(np.array([15, 32], np.int32), (8, 1))), [19, 2])
+    assert list(np_(out["row_status"])) == [fw.FW_ERR_NONFINITE] * 6 + [0, 0]
+    for key in ("best_gap", "topk_gap"):
+        assert np.isnan(np_(out[key])[:6]).all() and np.isfinite(np_(out[key])[6:]).all()
+    assert (np_(out["best_idx"])[:6] == -1).all() and not np_(out["n_cand"])[:6].any()
+
+
+@pytest.mark.parametrize("sink,scale", [(36.0, 1.0), (40.0, 1.0), (5.0, 2.0 ** -55), (5.0, 2.0 ** 55)])
+def test_pools_far_from_unit_scale(fw, sink, scale):  # noqa: F811
+    # masses of 1e-17 beside a sink that the dense output equals, and small and large
+    # values: the sets of fp64, and few of the subsets scored
+    L, V = _rows(17, 6, 60, 64, sink, 1.0)
+    V = (np.round(V * 8) / 8).astype(np.float32) * np.float32(scale)
+    b = rows_batch(L, V, np.full((6, 1), 4))
+    rows, out = run_pool(fw, b, [24])
+    top = fw.dense_and_topk_gap(rows, torch.full((6, 1), 4, dtype=torch.int32).cuda())
+    o, gap, idx = (np_(x).astype(np.float64) for x in (top["o"], out["best_gap"], out["best_idx"]))
+    assert not np_(out["row_status"]).any()
+    for r in range(6):
+        p = np.exp(L[r].astype(np.float64) - L[r].max())
+        u = p[:, None] / p.sum() * (V[r].astype(np.float64) - o[r])  # (the gap call's output, as the pool takes it)
+        e = np.linalg.norm(u, axis=1)
+        kept = np.lexsort((np.arange(60), -L[r].astype(np.float64)))[:4]
+        e[kept] = np.inf
+        pool = np.sort(np.argsort(-e, kind="stable")[:28])
+        sets = np.array(list(itertools.combinations(pool, 4)))
+        es = np.linalg.norm(u[sets].sum(1), axis=1) / (p[sets] / p.sum()).sum(1)
+        best = es.argmin()
+        assert abs(gap[r, 0] - es[best]) <= 1e-5 * es[best]
+        if np.partition(es, 1)[1] > es[best] * (1 + 1e-5):
+            np.testing.assert_array_equal(idx[r, 0, :4], sets[best])
+    assert np_(out["n_cand"]).max() <= 600  # (of 20,475)
