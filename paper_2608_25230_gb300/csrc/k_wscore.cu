@@ -52,11 +52,25 @@ struct WsArgs {
     int S, tps;           // slices per cell, tiles per slice
     float scale2;         // scale * log2(e): logits in base-2 units
     float *votes;         // workspace [cells][T]
-    float2 *stat;         // workspace [cells][S][WS_N]: (reference, sum of 2^(x - reference))
-    int32_t *err;         // workspace [2][cells][S]: a wait of the CTA gave up
     float *scores;        // [cells][T]
     int32_t *status;      // [cells] or null
 };
+
+// A slice's softmax statistics of query i -- a reference logit and the sum of 2^(x -
+// reference), -1 where a wait of the slice's CTA gave up -- sit between the two launches
+// in the cell's part of the scores, which nothing else uses before k_wpool writes them:
+// 2 WS_N floats a slice (slices hold at least 4 tiles where there are several).  A cell
+// of one slice may be shorter than that, so its sums wait among its votes, which its CTA
+// writes after it has read them.
+static_assert((4 * 2 - 4) * WS_KT + 1 >= 2 * 2 * WS_N, "statistics of two slices");
+__device__ __forceinline__ float *stat_ref(const WsArgs &a, int c, int sl)
+{
+    return a.scores + (int64_t)c * a.T + sl * 2 * WS_N;
+}
+__device__ __forceinline__ float *stat_sum(const WsArgs &a, int c, int sl)
+{
+    return a.S == 1 ? a.votes + (int64_t)c * a.T : stat_ref(a, c, sl) + WS_N;
+}
 
 // 2^x by the hardware approximation (ex2.approx.ftz: ~2 ulp, well inside the
 // score's 1e-4 tolerance); the per-(key, query) exponentials are most of the
@@ -117,13 +131,15 @@ __global__ void __launch_bounds__(WS_THREADS, 2) k_wscore(const __grid_constant_
         s_err = 0;
     }
     if (wid == 1) tc::tmem_alloc(&s_taddr, WS_ACC * WS_N);
-    if (PASS == 2 && tid >= 64 && tid < 64 + WS_N) {
+    bool lost = false;
+    if (PASS == 2 && tid >= 64 && tid < 64 + w) {
         // the softmax statistics of every query over all keys of the cell
         const int i = tid - 64;
         float m = -INFINITY, z = 0.f;
         for (int s = 0; s < a.S; ++s) {
-            const float2 p = a.stat[((int64_t)c * a.S + s) * WS_N + i];
-            ms_merge(m, z, p.x, p.y);
+            const float zs = stat_sum(a, c, s)[i];
+            lost |= zs < 0.f;
+            ms_merge(m, z, stat_ref(a, c, s)[i], zs);
         }
         s_st[i] = make_float2(m, z > 0.f ? 1.f / z : 0.f);
     }
@@ -301,12 +317,15 @@ __global__ void __launch_bounds__(WS_THREADS, 2) k_wscore(const __grid_constant_
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (PASS == 1 && tid < WS_N) {
+    if (PASS == 1 && tid < w) {
         float m = -INFINITY, z = 0.f;
         for (int q = 0; q < WS_EW / 2; ++q) ms_merge(m, z, s_mz[q][tid].x, s_mz[q][tid].y);
-        a.stat[(int64_t)blockIdx.x * WS_N + tid] = make_float2(m, z);
+        stat_ref(a, c, sl)[tid] = m;
+        stat_sum(a, c, sl)[tid] = s_err ? -1.f : z;
     }
-    if (tid == 0) a.err[(PASS - 1) * a.cells * a.S + blockIdx.x] = s_err;
+    // the cell's status: OK by the first launch, a failure of either by the second
+    if (PASS == 1 && tid == 0 && sl == 0 && a.status) a.status[c] = FW_OK;
+    if (PASS == 2 && a.status && (lost || (tid == 0 && s_err))) a.status[c] = FW_ERR_TIMEOUT;
     if (wid == 1) {
         tc::fence_after_sync();
         tc::tmem_dealloc(taddr, WS_ACC * WS_N);
@@ -314,7 +333,7 @@ __global__ void __launch_bounds__(WS_THREADS, 2) k_wscore(const __grid_constant_
 }
 
 // Max pooling of the votes along the prefix positions (window positions keep
-// their own); the cell's status from its CTAs' flags.
+// their own).
 __global__ void __launch_bounds__(WP_T) k_wpool(const WsArgs a)
 {
     const int c = blockIdx.y, lim = a.T - a.w;
@@ -326,13 +345,6 @@ __global__ void __launch_bounds__(WP_T) k_wpool(const WsArgs a)
             for (int q = lo; q <= hi; ++q) r = fmaxf(r, vc[q]);
         }
         a.scores[(int64_t)c * a.T + j] = r;
-    }
-    if (blockIdx.x == 0 && a.status) {
-        int e = 0;
-        for (int s = threadIdx.x; s < 2 * a.S; s += WP_T)
-            e |= a.err[(s >= a.S ? a.cells * a.S : 0) + c * a.S + (s >= a.S ? s - a.S : s)];
-        e = __syncthreads_or(e);
-        if (threadIdx.x == 0) a.status[c] = e ? FW_ERR_TIMEOUT : FW_OK;
     }
 }
 
@@ -350,11 +362,7 @@ int slice_tiles(int cells, int T)
 
 }  // namespace
 
-size_t window_score_workspace(int cells, int T)
-{
-    return align256((size_t)cells * T * 4) + align256((size_t)cells * WS_SMAX * WS_N * sizeof(float2)) +
-           align256((size_t)cells * WS_SMAX * 2 * 4);
-}
+size_t window_score_workspace(int cells, int T) { return align256((size_t)cells * T * 4); }
 
 fw_status window_score(const void *Qw, const void *K, int cells, int T, int d, int w, float scale, int pool,
                        float *scores, void *ws, int32_t *status, cudaStream_t s)
@@ -370,12 +378,7 @@ fw_status window_score(const void *Qw, const void *K, int cells, int T, int d, i
     a.tps = slice_tiles(cells, T);
     a.S = ((T + WS_KT - 1) / WS_KT + a.tps - 1) / a.tps;
     a.scale2 = scale * 1.4426950408889634f;
-    char *wp = (char *)ws;
-    a.votes = (float *)wp;
-    wp += align256((size_t)cells * T * 4);
-    a.stat = (float2 *)wp;
-    wp += align256((size_t)cells * WS_SMAX * WS_N * sizeof(float2));
-    a.err = (int32_t *)wp;
+    a.votes = (float *)ws;
     a.scores = scores;
     a.status = status;
     auto launch = [&](auto kernel, int nbox) -> fw_status {
@@ -393,8 +396,6 @@ fw_status window_score(const void *Qw, const void *K, int cells, int T, int d, i
         const int nc = std::min(cells - c0, 65535);
         b.votes += (int64_t)c0 * T;
         b.scores += (int64_t)c0 * T;
-        b.err += (int64_t)c0 * a.S;
-        if (b.status) b.status += c0;
         const dim3 grid((unsigned)std::min((T + WP_T - 1) / WP_T, 64), (unsigned)nc);
         FW_LAUNCH(k_wpool, grid, WP_T, 0, s, b);
     }

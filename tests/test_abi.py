@@ -105,3 +105,10 @@ def test_host_validation_rejects_bad_arguments(lib):
     first = C.c_int64(7)
     assert fw._lib.fw_sync_status(P, -1, C.byref(first), None) == fw.FW_ERR_INVALID_ARG and first.value == -1
     assert fw.launch_count() == before  # nothing was launched
+
+
+@pytest.mark.parametrize("cells,T", [(4096, 64), (1, 1), (256, 32768), (7, 3001)])
+def test_window_score_workspace_is_the_votes(lib, cells, T):
+    # as the header states it: cells x T fp32 (in whole 256-byte units)
+    lib.fw_window_score_workspace.restype = C.c_size_t
+    assert lib.fw_window_score_workspace(cells, T) == (cells * T * 4 + 255) // 256 * 256

@@ -4,6 +4,7 @@ oracle, and ContourKV allocated on that score (Sec. 4's window-scored
 variant).  Scores within 1e-4 relative (1e-6 of the cell's largest score as
 the floor); the allocation on the CUDA scores bit-exact against the oracle's
 allocation of the same scores."""
+import ctypes
 import math
 
 import numpy as np
@@ -89,3 +90,28 @@ def test_window_score_rising_logits(fw, T, w):
     ramp = np.geomspace(0.1, 30.0, T)[None, :, None]
     K = workloads.f32_to_bf16_bits((rng.normal(size=(2, T, 64)) * ramp).astype(np.float32))
     check(fw, Q, K)
+
+
+@pytest.mark.parametrize("cells,T,w,d", [(3, 1, 1, 64), (3, 31, 31, 128), (5, 33, 32, 64), (4, 512, 32, 64),
+                                         (4, 513, 32, 128), (2, 3000, 9, 64), (700, 65, 32, 64)])
+def test_window_score_keeps_to_its_buffers(fw, cells, T, w, d):
+    # cells shorter than a slice's statistics, one and several slices: the answer in
+    # buffers of exactly the documented sizes, nothing written around them
+    rng = np.random.default_rng(cells + T)
+    Q = workloads.f32_to_bf16_bits(rng.normal(size=(cells, w, d)).astype(np.float32))
+    K = workloads.f32_to_bf16_bits(rng.normal(size=(cells, T, d)).astype(np.float32))
+    Qd, Kd = (torch.as_tensor(x.view(np.int16)).cuda() for x in (Q, K))
+    n, pad, need = cells * T, 64, fw.raw().fw_window_score_workspace(cells, T)
+    assert need < n * 4 + 256
+    sc = torch.full((n + 2 * pad,), 7.0, device="cuda")
+    ws = torch.full((need // 4 + 2 * pad,), 7.0, device="cuda")
+    st = torch.full((cells + 2 * pad,), 7, dtype=torch.int32, device="cuda")
+    r = fw.raw().fw_window_score(fw._ptr(Qd), fw._ptr(Kd), cells, T, d, w, ctypes.c_float(d ** -0.5), 7,
+                                 fw._ptr(sc[pad:]), fw._ptr(st[pad:]), fw._ptr(ws[pad:]), need, fw._stream(None))
+    assert r == 0
+    torch.cuda.synchronize()
+    for x, m in ((sc, n), (ws, need // 4), (st, cells)):
+        assert (x[:pad] == 7).all() and (x[pad + m:] == 7).all()
+    assert not st[pad:pad + cells].any()
+    want, _ = oracle.window_score(Q, K, d ** -0.5, 7)
+    assert_close(np_(sc[pad:pad + n]).reshape(cells, T), want, want.max(axis=1), "window score")
