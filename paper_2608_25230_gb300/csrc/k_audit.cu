@@ -45,7 +45,6 @@ constexpr int AM_T = 256;   // k_aud_mass threads
 constexpr int AS_T = 512;   // k_aud_select threads
 constexpr int AR_T = 256;   // k_aud_row threads (8 warps)
 constexpr int A_NBMAX = 4;
-constexpr int AR_MP = 16;      // pages a warp takes by repeated arg-max (above: the block's radix select)
 constexpr int AS_STAGE = 24576;  // candidates whose keys k_aud_select stages (96 KB)
 constexpr size_t AR_SMEM = 196608;  // k_aud_row stages the row where its sets and logits fit this
 constexpr int NSEL = FW_NUM_SELECTORS;
@@ -66,6 +65,14 @@ struct AudArgs {
 
 __device__ __forceinline__ int snap_w(int s) { return max(1, min(32, s / 2)); }
 __host__ __device__ __forceinline__ int quest_p(int q, int s) { return q == 0 ? (s / 4 > 2 ? s / 4 : 2) : 16; }
+// Pages of a row of n keys that a warp takes by repeated arg-max; more are the block's
+// radix select.  The warp reads the row once per page, the block about five times as fast
+// but with barriers that cost as much as 24,000 keys.  Measured on the whole audit, one
+// budget, arg-max / select, us: 256 groups of 4 rows of 4,096 keys, 8 pages 186 / 206, 10
+// pages 213 / 221, 12 pages 237 / 231, 16 pages 289 / 254; 64 x 4 rows of 16,384 keys, 8
+// pages 208 / 182, 16 pages 334 / 212; 128 rows of 32,768 keys, 8 pages 481 / 409, 16 pages
+// 685 / 422; 300 x 4 rows of 1,000 keys, 16 pages 174 / 193.
+__host__ __device__ __forceinline__ int argmax_pages(int n) { return 5 + 24000 / n; }
 
 // ---------------------------------------------------------------- masses
 __global__ void __launch_bounds__(AM_T) k_aud_mass(AudArgs a)
@@ -207,7 +214,7 @@ __global__ void __launch_bounds__(AR_T) k_aud_row(AudArgs a, int stage_n)
         for (int bq = wid; bq < a.nb * 2; bq += AR_T / 32) {
             const int b = bq >> 1, q = bq & 1, s = a.s[b];
             const int P = quest_p(q, s), np = (n + P - 1) / P, mp = s / P;
-            if (!(s >= 1 && s <= n && mp >= 1 && mp <= AR_MP && (q == 0 || s >= 16))) continue;
+            if (!(s >= 1 && s <= n && mp >= 1 && mp <= argmax_pages(n) && (q == 0 || s >= 16))) continue;
             uint32_t *qb = qbits + bq * a.words;
             uint32_t lk = 0xffffffffu;
             int lp = -1;
@@ -236,7 +243,7 @@ __global__ void __launch_bounds__(AR_T) k_aud_row(AudArgs a, int stage_n)
         for (int bq = 0; bq < a.nb * 2; ++bq) {
             const int b = bq >> 1, q = bq & 1, s = a.s[b];
             const int P = quest_p(q, s), np = (n + P - 1) / P, mp = s / P;
-            if (!(s >= 1 && s <= n && mp > AR_MP && (q == 0 || s >= 16))) continue;
+            if (!(s >= 1 && s <= n && mp > argmax_pages(n) && (q == 0 || s >= 16))) continue;
             uint32_t *qb = qbits + bq * a.words;
             __syncthreads();  // pm is free
             for (int p = tid; p < np; p += AR_T) {
@@ -398,8 +405,10 @@ fw_status selector_audit(const RowsDev &R, const int32_t *s, int nb, const fw_ga
     }
     a.pm_floats = 0;
     for (int b = 0; b < nb; ++b)
-        for (int q = 0; q < 2; ++q)  // (pages of at least 2 keys)
-            if (s[b] / quest_p(q, s[b]) > AR_MP) a.pm_floats = (R.max_n + 1) / 2 + 1;
+        for (int q = 0; q < 2; ++q) {
+            const int P = quest_p(q, s[b]);
+            if (s[b] / P > argmax_pages(R.max_n)) a.pm_floats = std::max(a.pm_floats, (R.max_n + P - 1) / P);
+        }
     const size_t sets = ((size_t)nb * 2 * a.words + a.pm_floats) * 4, lrow = ((size_t)R.max_n + (R.max_n >> 5) + 1) * 4;
     const int stage_n = sets + lrow <= AR_SMEM ? R.max_n : 0;
     const size_t smem = sets + (stage_n ? lrow : 0);

@@ -114,3 +114,16 @@ def test_audit_rows_past_the_staging_limits(fw, n):
     L[:, 0] += 8
     V = rng.normal(size=(1, n, d)).astype(np.float32)
     check_audit(fw, rows_batch(L, V, np.ones((R, 1), np.int32), v_dtype="bf16", R=R), [7, 300, 4096])
+
+
+@pytest.mark.parametrize("n", [290, 1999, 8191, 32768])
+def test_audit_quest_pages_by_arg_max_and_select(fw, n):
+    # page counts on both sides of the line between a warp's arg-max and the block's
+    # select, which moves with the row's length; ties among the pages' maxima
+    rng = np.random.default_rng(n)
+    R, d = 2, 32
+    L = (np.round(rng.normal(size=(R, n)) * 8) / 8).astype(np.float32)
+    V = rng.normal(size=(1, n, d)).astype(np.float32)
+    pages = 5 + 24000 // n
+    check_audit(fw, rows_batch(L, V, np.ones((R, 1), np.int32), R=R),
+                sorted({min(n, 16 * p) for p in (pages - 1, pages, pages + 1, 2 * pages)}))
