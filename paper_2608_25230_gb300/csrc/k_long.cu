@@ -633,6 +633,8 @@ __global__ void __launch_bounds__(NT, sel_minb<NT>()) k_long_select_reg(const Se
                 r = __shfl_xor_sync(FW_FULL, u, 1);
                 u = lane & 1 ? (u & 0xf0f0f0f0u) | ((r >> 4) & 0x0f0f0f0fu) : (u & 0x0f0f0f0fu) | ((r & 0x0f0f0f0fu) << 4);
                 if (q8 < V4 && w < nw) a.out.kept_bits[(row * nb + b) * (int64_t)nw + w] = u;
+                // (words past this layout's keys, where the caller asked for more)
+                for (int w2 = NT * VPT / 32 + tid; w2 < nw; w2 += NT) a.out.kept_bits[(row * nb + b) * (int64_t)nw + w2] = 0u;
             }
             if (tie) {  // (uniform)
                 __syncthreads();  // the words above are visible to the block

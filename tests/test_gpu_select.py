@@ -2,6 +2,8 @@
 rows that leave the linear bins: kept bits, thresholds and softmax statistics
 against plain numpy, including NaN and infinite logits and ranges fp32 cannot
 scale."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -76,3 +78,26 @@ def test_select_nonfinite_and_wide_rows(fw):
     assert list(g["row_status"][:3]) == [fw.FW_ERR_NONFINITE] * 3
     for r in (3, 4, 5):
         check(g, r, L[r], [7, 2500])
+
+
+@pytest.mark.parametrize("n,words", [(33, 2), (1000, 40), (1024, 33), (5000, 1500), (20, 9)])
+def test_select_writes_every_word(fw, n, words):
+    # more words than the row has: zero past its keys, on rows that stay in the linear
+    # bins and on one that goes to the radix select
+    rng = np.random.default_rng(n)
+    L = rng.normal(size=(3, n)).astype(np.float32)
+    L[1, :3] = 3e38, -3e38, 0
+    b = rows_batch(L, np.ones((3, n, 32), np.float32), np.tile(np.array([1, n // 2], np.int32), (3, 1)))
+    rows, k = fw.rows_from_batch(b), torch.as_tensor(np.asarray(b.k)).cuda()
+    top = fw.dense_and_topk_gap(rows, k)
+    bits = torch.full((3 * 2 * words + 64,), -1, dtype=torch.int32, device="cuda")
+    c = top["_c"]
+    c.kept_bits, c.kept_words = bits.data_ptr(), words
+    ws = torch.empty(fw.raw().fw_dense_and_topk_gap_workspace(ctypes.byref(rows.c), 2) + 256, dtype=torch.uint8, device="cuda")
+    assert fw.raw().fw_dense_and_topk_gap(ctypes.byref(rows.c), fw._ptr(k), 2, ctypes.byref(c), fw._ptr(ws), ws.numel(),
+                                          fw._stream(None)) == 0
+    torch.cuda.synchronize()
+    assert (bits[-64:] == -1).all()
+    w = np_(bits[:-64]).view(np.uint32).reshape(3, 2, words)
+    for r in range(3):
+        check(dict(row_status=np.zeros(3), kept_bits=w, row_max=L.max(1), row_sum=np_(top["row_sum"])), r, L[r], [1, n // 2])
