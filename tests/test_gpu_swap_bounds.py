@@ -27,21 +27,32 @@ def test_swap_extras_and_sinks(fw, n, d, v_dtype, E, sink):  # noqa: F811
     check_swap_long(fw, rows_batch(L, V, k, v_dtype=v_dtype), E=E, max_swaps=12)
 
 
-def test_swap_equal_values_take_nothing(fw):  # noqa: F811
-    # every set has the same output: no swap strictly lowers es beyond rounding
+@pytest.mark.parametrize("value", [0.0, 1.0])
+def test_swap_equal_values(fw, value):  # noqa: F811
+    # every set has the same output.  Zeros: every score is exactly 0, nothing is taken.
+    # Ones: es is rounding noise and swaps may follow it, but they are swaps of kept
+    # for dropped keys, and the gap of any set is 0 to the oracle's floor
     import torch
 
     rng = np.random.default_rng(1)
     L = rng.normal(size=(2, 100)).astype(np.float32)
-    V = np.ones((2, 100, 64), np.float32)
+    V = np.full((2, 100, 64), value, np.float32)
     b = rows_batch(L, V, np.full((2, 1), 10))
     rows = fw.rows_from_batch(b)
     k = torch.as_tensor(np.asarray(b.k)).cuda()
     top = fw.dense_and_topk_gap(rows, k)
-    sw = fw.swap_refine(rows, k, top, E=32, max_swaps=16)
-    torch.cuda.synchronize()
-    assert torch.all(sw["refined_gap"] <= sw["topk_gap"] * (1 + 1e-6) + 1e-7)
-    assert torch.all(torch.isfinite(sw["refined_gap"]))
+    sw = {x: np_(v) for x, v in fw.swap_refine(rows, k, top, E=32, max_swaps=16).items() if not x.startswith("_")}
+    if value == 0.0:
+        assert not sw["n_swaps"].any() and (sw["swap_out"] == -1).all() and (sw["swap_in"] == -1).all()
+        assert not sw["refined_gap"].any() and not sw["topk_gap"].any()
+    for r in range(2):
+        m = int(sw["n_swaps"][r, 0])
+        assert 0 <= m <= 16 and (sw["swap_out"][r, 0, m:] == -1).all() and (sw["swap_in"][r, 0, m:] == -1).all()
+        kept = set(np.lexsort((np.arange(100), -L[r].astype(np.float64)))[:10].tolist())
+        for i, j in zip(sw["swap_out"][r, 0, :m].tolist(), sw["swap_in"][r, 0, :m].tolist()):
+            assert i in kept and j not in kept and 0 <= j < 100
+            kept = kept - {i} | {j}
+    assert_close(sw["refined_gap"], 0 * sw["refined_gap"], np.full(2, 8.0 * value), "refined_gap")  # ||o|| = 8
 
 
 @pytest.mark.parametrize("n,k,d,E", [(4000, 2000, 64, 32), (3000, 2900, 128, 96), (700, 350, 256, 40)])
