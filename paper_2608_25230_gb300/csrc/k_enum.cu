@@ -131,6 +131,8 @@ struct Walk {
     uint32_t *cand;
     int32_t *ccount;
     unsigned long long *stats;
+    unsigned long long *tot;  // the warp's sums of them, in shared memory
+    int *left;                // lanes of the warp still walking
 };
 
 // Leaves (C(EM, c)) and fp32 add/min operations of one inner<c> enumeration
@@ -444,10 +446,17 @@ __device__ __noinline__ void walk_row(const Walk W)
         // hence runs this loop the same number of times.
         if (W.sync_mask) __syncwarp(W.sync_mask);
     }
-    atomicAdd(W.stats + 0, n_inner);
-    atomicAdd(W.stats + 1, n_leaf);
-    atomicAdd(W.stats + 2, n_ops);
-    atomicAdd(W.stats + 3, n_skip);
+    atomicAdd(W.tot + 0, n_inner);
+    atomicAdd(W.tot + 1, n_leaf);
+    atomicAdd(W.tot + 2, n_ops);
+    atomicAdd(W.tot + 3, n_skip);
+    // The warp's last lane to finish hands its sums on.  (Four global atomics a lane, at
+    // the same four counters, held small walks up: 4,800 rows of 8 keys 213 -> 125 us.
+    // Sums over the warp after the walk cost up to 30 % of it: lanes that had finished
+    // waited for the others.)
+    __threadfence_block();
+    if (atomicAdd(W.left, -1) == 1)
+        for (int q = 0; q < 4; ++q) atomicAdd(W.stats + q, atomicAdd(W.tot + q, 0ull));
 }
 
 // Write one Gram entry (or a_x / l_x) into the walk tables of a row slot.
@@ -789,6 +798,9 @@ __global__ void __launch_bounds__(32, 1) k_enum_walk(const EnumArgs a)
     const int lane = threadIdx.x;
     float *slots = smem;                                                   // [ERW][stride]
     uint8_t *perms = reinterpret_cast<uint8_t *>(smem + ERW * a.stride);   // [ERW][PERM]
+    __shared__ unsigned long long s_tot[4];
+    __shared__ int s_left;
+    if (lane < 4) s_tot[lane] = 0ull;
     const int64_t row0 = (int64_t)blockIdx.x * ERW;
     const int nrow = (int)min((int64_t)ERW, a.R.rows - row0);
     {
@@ -818,6 +830,8 @@ __global__ void __launch_bounds__(32, 1) k_enum_walk(const EnumArgs a)
         my.part = lane / ERW;
         my.parts = 32 / ERW;
         my.stats = a.stats;
+        my.tot = s_tot;
+        my.left = &s_left;
         const float2 kg = a.kg[row];
         my.kappa = kg.x;
         my.g0n = kg.y;
@@ -830,6 +844,8 @@ __global__ void __launch_bounds__(32, 1) k_enum_walk(const EnumArgs a)
         const int key0 = __shfl_sync(FW_FULL, key, wmask ? __ffs(wmask) - 1 : 0);
         const bool same = __all_sync(FW_FULL, !my_walk || key == key0);
         my.sync_mask = same ? wmask : 0u;
+        if (lane == 0) s_left = __popc(wmask);
+        __syncwarp();
     }
     if (my_walk) walk_row(my);
 }
@@ -1236,26 +1252,31 @@ __global__ void k_enum_exhaustive_merge(const EnumArgs a)
     }
 }
 
+template <int ERW> size_t walk_smem(int stride) { return (size_t)ERW * stride * sizeof(float) + ERW * PERM; }
+
 template <int ERW> fw_status launch_walk_n(const EnumArgs &a, cudaStream_t s)
 {
-    const size_t smem = (size_t)ERW * a.stride * sizeof(float) + ERW * PERM;
+    const size_t smem = walk_smem<ERW>(a.stride);
     FW_CUDA_CHECK(cudaFuncSetAttribute(k_enum_walk<ERW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     FW_LAUNCH((k_enum_walk<ERW>), (unsigned)((a.R.rows + ERW - 1) / ERW), 32, smem, s, a);
     return FW_OK;
 }
 
 // Lanes per row.  A warp (255 registers, 8 to an SM) lasts as long as its slowest row, so
-// few rows are split finer: 8 lanes each while all their warps are resident at once
-// (32 rows an SM), 4 for twice as many; beyond that the SMs are full either way, and lanes
-// that idle at a class's end and their counters' atomics are lost work.  Measured,
-// 2 / 4 / 8 lanes a row, us: 24 keys, k = 6: 2,000 rows 609 / 487 / 378, 4,000: 634 / 493 /
-// 401, 8,000: 696 / 632 / 647, 16,000: 1,036 / 915 / 858; 16 keys, k = 4: 2,000 rows 191 /
-// 158 / 160, 4,000: 190 / 175 / 177, 8,000: 211 / 212 / 293, 16,000: 256 / 310 / 453;
-// 256 rows of 20 keys, k = 5: 130 / 86 / 74.
+// few rows are split finer: 8 lanes each while all their warps are resident at once (32
+// rows an SM), then 4.  But the walk works in its stack, which lives in the L1 that
+// shared memory leaves: 4 lanes only where the tables of 8 warps leave 60 KB of it (up to
+// 29 keys at small k), else 2.  Measured, 2 / 4 / 8 lanes a row, whole call, d = 32, us:
+//    8 keys, k = 2:  2,400 rows 89 / 84 / 88, 9,700 182 / 178 / 194, 30,000 404 / 421 / 456
+//   16 keys, k = 4:  338 / 302 / 306, 452 / 425 / 452, 739 / 737 / 803
+//   24 keys, k = 6:  2,485 / 2,217 / 1,787, 3,127 / 2,946 / 2,714, 7,163 / 6,895 / 7,124
+//   28 keys, k = 4:  1,468 / 1,302 / 1,282, 1,904 / 1,489 / 1,758, 3,554 / 3,047 / 4,004
+//   30 keys, k = 3:  493 / 459 / 448, 889 / 1,160 / 1,146, 2,168 / 3,245 / 3,055
+//   32 keys, k = 4:  2,003 / 1,724 / 1,719, 3,186 / 4,063 / 3,648, 8,357 / 11,928 / 10,106
 fw_status launch_walk(const EnumArgs &a, int sms, cudaStream_t s)
 {
     if (a.R.rows <= (int64_t)32 * sms) return launch_walk_n<4>(a, s);
-    if (a.R.rows <= (int64_t)64 * sms) return launch_walk_n<8>(a, s);
+    if (8 * (walk_smem<8>(a.stride) + 1024) <= 196 * 1024) return launch_walk_n<8>(a, s);
     return launch_walk_n<16>(a, s);
 }
 

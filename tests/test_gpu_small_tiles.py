@@ -36,22 +36,24 @@ def test_best_tiles(fw, n, k, d):  # noqa: F811
     check_best(fw, _rows(n, d, 9, n * d + k, "bf16" if k % 2 else "f32", [k]))
 
 
-@pytest.mark.parametrize("rows", [1, 3, 4864, 4865, 9729])
-def test_best_lanes_per_row(fw, rows):  # noqa: F811
-    # 8, 4 and 2 lanes walk a row (152 SMs: the lines lie at 4,864 and 9,728 rows): the
-    # same few rows, repeated, give the same answers as in a batch of their own
+@pytest.mark.parametrize("copies,m,n,k", [(1, 1, 14, 4), (3, 1, 14, 4), (374, 13, 14, 4), (375, 13, 14, 4), (375, 13, 29, 2),
+                                          (375, 13, 30, 2), (375, 13, 32, 3)])
+def test_best_lanes_per_row(fw, copies, m, n, k):  # noqa: F811
+    # 8 lanes walk a row up to 4,864 rows (152 SMs), then 4, or 2 where the walk tables
+    # are large: the same few rows, repeated, give the same answers, and cost the same
+    # search, as in a batch of their own
     import torch
 
-    m = min(rows, 13)
-    b = _rows(14, 32, m, rows, k=[4])
-    rep = np.arange(rows) % m
-    big = rows_batch(np.asarray(b.logits).reshape(m, 14)[rep], np.asarray(b.v).reshape(m, 14, 32)[rep],
-                     np.asarray(b.k)[rep])
+    b = _rows(n, 32, m, 1000 * n + m, k=[k])
+    rep = np.tile(np.arange(m), copies)
+    big = rows_batch(np.asarray(b.logits).reshape(m, n)[rep], np.asarray(b.v).reshape(m, n, 32)[rep], np.asarray(b.k)[rep])
     check_best(fw, b)
-    few, many = (fw.best_subset(fw.rows_from_batch(x), torch.from_numpy(np.ascontiguousarray(x.k[:, 0])).cuda())
-                 for x in (b, big))
+    rows = [fw.rows_from_batch(x) for x in (b, big)]
+    few, many = (fw.best_subset(r, torch.from_numpy(np.ascontiguousarray(x.k[:, 0])).cuda()) for r, x in zip(rows, (b, big)))
     for key in ("best_rank", "best_gap", "best_idx", "topk_gap"):
         np.testing.assert_array_equal(many[key].cpu().numpy(), few[key].cpu().numpy()[rep])
+    one, all_ = (fw.best_subset_stats(r, o) for r, o in zip(rows, (few, many)))
+    assert all_ == {key: copies * v for key, v in one.items()} and one["inner_leaves"] > 0
 
 
 def test_swap_rescored_in_batches(fw):  # noqa: F811
