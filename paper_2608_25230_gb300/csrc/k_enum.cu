@@ -1264,9 +1264,12 @@ template <int ERW> fw_status launch_walk_n(const EnumArgs &a, cudaStream_t s)
 
 // Lanes per row.  A warp (255 registers, 8 to an SM) lasts as long as its slowest row, so
 // few rows are split finer: 8 lanes each while all their warps are resident at once (32
-// rows an SM), then 4.  But the walk works in its stack, which lives in the L1 that
-// shared memory leaves: 4 lanes only where the tables of 8 warps leave 60 KB of it (up to
-// 29 keys at small k), else 2.  Measured, 2 / 4 / 8 lanes a row, whole call, d = 32, us:
+// rows an SM), 4 for twice as many.  But the walk works in its stack, which lives in the
+// L1 that shared memory leaves: 4 lanes only where the tables of 8 warps leave 60 KB of it
+// (up to 29 keys at small k), else 2.  Larger batches take 2: alone most would gain by 4,
+// but where several run on streams of their own the SMs are full either way (168,192 rows
+// of 24 keys in five batches at once: 14.3 ms a step, 14.8 with 4).  Measured, 2 / 4 / 8
+// lanes a row, whole call alone, d = 32, us:
 //    8 keys, k = 2:  2,400 rows 89 / 84 / 88, 9,700 182 / 178 / 194, 30,000 404 / 421 / 456
 //   16 keys, k = 4:  338 / 302 / 306, 452 / 425 / 452, 739 / 737 / 803
 //   24 keys, k = 6:  2,485 / 2,217 / 1,787, 3,127 / 2,946 / 2,714, 7,163 / 6,895 / 7,124
@@ -1276,7 +1279,8 @@ template <int ERW> fw_status launch_walk_n(const EnumArgs &a, cudaStream_t s)
 fw_status launch_walk(const EnumArgs &a, int sms, cudaStream_t s)
 {
     if (a.R.rows <= (int64_t)32 * sms) return launch_walk_n<4>(a, s);
-    if (8 * (walk_smem<8>(a.stride) + 1024) <= 196 * 1024) return launch_walk_n<8>(a, s);
+    const bool l1 = 8 * (walk_smem<8>(a.stride) + 1024) <= 196 * 1024;
+    if (l1 && a.R.rows <= (int64_t)64 * sms) return launch_walk_n<8>(a, s);
     return launch_walk_n<16>(a, s);
 }
 

@@ -36,11 +36,11 @@ def test_best_tiles(fw, n, k, d):  # noqa: F811
     check_best(fw, _rows(n, d, 9, n * d + k, "bf16" if k % 2 else "f32", [k]))
 
 
-@pytest.mark.parametrize("copies,m,n,k", [(1, 1, 14, 4), (3, 1, 14, 4), (374, 13, 14, 4), (375, 13, 14, 4), (375, 13, 29, 2),
-                                          (375, 13, 30, 2), (375, 13, 32, 3)])
+@pytest.mark.parametrize("copies,m,n,k", [(1, 1, 14, 4), (3, 1, 14, 4), (374, 13, 14, 4), (375, 13, 14, 4), (749, 13, 14, 4),
+                                          (375, 13, 29, 2), (375, 13, 30, 2), (375, 13, 32, 3)])
 def test_best_lanes_per_row(fw, copies, m, n, k):  # noqa: F811
-    # 8 lanes walk a row up to 4,864 rows (152 SMs), then 4, or 2 where the walk tables
-    # are large: the same few rows, repeated, give the same answers, and cost the same
+    # 8 lanes walk a row up to 4,864 rows (152 SMs), 4 up to 9,728, or 2 where the walk
+    # tables are large, and 2 beyond: the same few rows, repeated, give the same answers, and cost the same
     # search, as in a batch of their own
     import torch
 
