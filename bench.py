@@ -57,17 +57,17 @@ POOL_SCHED = ((4, 24), (8, 12), (16, 6), (32, 4))  # (s, E): the candidate-set s
 #   group_vote      the same for k_vote_mass + k_vote_select + k_long_pv_tma
 #   contour         64 cells: k_c_* of one allocation + k_compact, per kept row
 #   compact         k_compact alone, per kept row
-#   window_score    k_wscore, per key (it reads K twice)
+#   window_score    k_wscore (both launches, each reads K) and k_wpool, per key
 #   mixed_gap       --mixed-rows-scale 0.1, one gap call per profile, per row
 TRAFFIC_PER_UNIT = {
     # line: (bytes per unit, unit)
-    "fw_best_subset": (40328.0, "row"),
-    "long_gap": (282648.0, "row"),
-    "group_vote": (280709.0, "row"),
+    "fw_best_subset": (40239.0, "row"),
+    "long_gap": (283953.0, "row"),
+    "group_vote": (280731.0, "row"),
     "contour": (1023.2, "kept row"),
     "compact": (830.1, "kept row"),
-    "window_score": (519.4, "key"),
-    "mixed_gap": (322689.0, "row"),
+    "window_score": (520.7, "key"),
+    "mixed_gap": (322793.0, "row"),
 }
 
 
