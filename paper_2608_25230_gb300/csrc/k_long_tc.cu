@@ -27,6 +27,8 @@
 //   p(A) (m_A - mu) = pbar(A) N_A - p(A) N_{A^c}.
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "fw_internal.h"
 #include "tc_sm100.cuh"
 
@@ -685,34 +687,40 @@ __global__ void __launch_bounds__(PVM_NT, 1) k_long_pv_tma(const __grid_constant
             const uint64_t bd0 = tc::sdesc_sw128(tc::smem_u32(sB), KS * 128, 1024);
             bool ok = true;
             int last = -1;
-            for (int it = 0; it < nst && ok; ++it) {
-                const int bs = it % PVM_BS, as = it % ASLOTS;
-                ok = tc::mbar_wait(&fullB[bs], (uint32_t)(it / PVM_BS) & 1u, WAIT_POLLS);
-                if (ok) ok = tc::mbar_wait(&fullA[as], (uint32_t)(it / ASLOTS) & 1u, WAIT_POLLS);
-                const int ch = it / CH;
-                if (ok && it % CH == 0 && ch >= NACC)
-                    ok = tc::mbar_wait(&accfree[ch % NACC], (uint32_t)((ch - NACC) / NACC) & 1u, WAIT_POLLS);
-                if (!ok) break;
-                // a stage whose V came by cp.async was written through the generic proxy: the
-                // MMA's reads, through the async proxy, are ordered behind it by this fence
-                if (!(vrows && (it + 1) * KS <= n)) tc::fence_async_smem();
-                tc::fence_after_sync();
-                const uint32_t dacc = taddr + (uint32_t)((ch % NACC) * DN);
-                const bool fresh = it % CH == 0;
-                const uint64_t abase = ad0 + (uint64_t)((as * A_SLOT_BYTES) >> 4);
-                const uint64_t bbs = bd0 + (uint64_t)((bs * B_SLOT_BYTES) >> 4);
+            // stages [it, end); COPIED: their V came by cp.async
+            auto run = [&](int it, int end, auto copied) {
+                for (; it < end && ok; ++it) {
+                    const int bs = it % PVM_BS, as = it % ASLOTS;
+                    ok = tc::mbar_wait(&fullB[bs], (uint32_t)(it / PVM_BS) & 1u, WAIT_POLLS);
+                    if (ok) ok = tc::mbar_wait(&fullA[as], (uint32_t)(it / ASLOTS) & 1u, WAIT_POLLS);
+                    const int ch = it / CH;
+                    if (ok && it % CH == 0 && ch >= NACC)
+                        ok = tc::mbar_wait(&accfree[ch % NACC], (uint32_t)((ch - NACC) / NACC) & 1u, WAIT_POLLS);
+                    if (!ok) break;
+                    // (written through the generic proxy: the MMA's reads, through the async proxy,
+                    // are ordered behind it by this fence)
+                    if constexpr (decltype(copied)::value) tc::fence_async_smem();
+                    tc::fence_after_sync();
+                    const uint32_t dacc = taddr + (uint32_t)((ch % NACC) * DN);
+                    const bool fresh = it % CH == 0;
+                    const uint64_t abase = ad0 + (uint64_t)((as * A_SLOT_BYTES) >> 4);
+                    const uint64_t bbs = bd0 + (uint64_t)((bs * B_SLOT_BYTES) >> 4);
 #pragma unroll
-                for (int ks = 0; ks < KS / 16; ++ks) {
-                    const uint64_t bd = bbs + (uint64_t)((ks * 2048) >> 4);
+                    for (int ks = 0; ks < KS / 16; ++ks) {
+                        const uint64_t bd = bbs + (uint64_t)((ks * 2048) >> 4);
 #pragma unroll
-                    for (int sp = 0; sp < NSPLIT; ++sp)
-                        tc::mma_bf16(dacc, abase + (uint64_t)((sp * A_SPLIT_BYTES + ks * 32) >> 4), bd, idesc,
-                                     !fresh || ks > 0 || sp > 0);
+                        for (int sp = 0; sp < NSPLIT; ++sp)
+                            tc::mma_bf16(dacc, abase + (uint64_t)((sp * A_SPLIT_BYTES + ks * 32) >> 4), bd, idesc,
+                                         !fresh || ks > 0 || sp > 0);
+                    }
+                    tc::commit(&freeA[as]);
+                    tc::commit(&freeB[bs]);
+                    last = it;
                 }
-                tc::commit(&freeA[as]);
-                tc::commit(&freeB[bs]);
-                last = it;
-            }
+            };
+            const int whole = vrows ? n / KS : 0;  // the first stages come by TMA, the others by cp.async
+            run(0, whole, std::false_type{});
+            run(whole, nst, std::true_type{});
             if (!ok) atomicOr(&s_err, 1);
             if (last >= 0 && !tc::mbar_wait(&freeA[last % ASLOTS], (uint32_t)(last / ASLOTS) & 1u, WAIT_POLLS))
                 atomicOr(&s_err, 1);
