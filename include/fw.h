@@ -150,7 +150,7 @@ fw_status fw_swap_refine(const fw_rows *rows, const int32_t *k, int32_t nb, cons
                          void *workspace, size_t workspace_bytes, void *stream);
 /* Workspace bytes (0 for max_n <= 32): for up to 3 x 152 persistent blocks,
  * per-key arrays of max_n entries and a table of kept x pool cross products
- * (fp32, max_n x round_up(E, 32) entries per block: 1.9 GB for max_n = 32,768
+ * (fp32, max_n x round_up(E, 32) entries per block: 1.6 GB for max_n = 32,768
  * and E = 32). */
 size_t fw_swap_refine_workspace(const fw_rows *rows, int32_t nb, const fw_swap_params *prm);
 

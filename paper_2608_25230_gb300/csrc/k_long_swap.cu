@@ -31,31 +31,34 @@
 // rounding swap by swap, apart from g's own.
 //
 // A round is one pass over the kept keys: four lanes share a key (each a
-// quarter of the columns); the key's value row and its scalars are read one
-// iteration ahead.  Regrouped, D_ij = A_i + B_j +
-// p_i (h_j + k_j C_ij) with per-key A_i and per-slot B_j, h_j, k_j, so with m_i
-// >= max_j p_j C_ij (kept per key, raised when a slot changes) no pair of the
-// key scores below
-//   (A_i + min_j B_j + p_i min_j h_j - 2 P^2 p_i m_i) / (P - p_i + min_j p_j)^2.
-// Keys whose bound lies above the least score found so far in the block are
-// done after the two products; the few others (about one in a
-// hundred on the measured rows) have their E pairs scored from the table.  The
-// least score wins; among pairs at that score the smallest (i, j), except
-// that two positions of one lane at exactly the same fp32 score keep the
-// first: such pairs are tied to ~1e-7 relative, a decision no fp32 evaluation
-// can settle.
+// quarter of the columns, and of every 32 pool slots a class of 8); the key's
+// value row and its scalars are read one iteration ahead.  Regrouped, D_ij =
+// A_i + B_j + p_i (h_j + k_j C_ij) with per-key A_i and per-slot B_j, h_j, k_j,
+// so with m_i >= max_j p_j C_ij over a class (kept per key and class, raised
+// when a slot of it changes) no pair of the key with that class scores below
+//   (A_i + min_j B_j + p_i min_j h_j - 2 P^2 p_i m_i) / (P - p_i + min_j p_j)^2,
+// min_j B_j over the class too.  A lane whose bound lies above the least score
+// that it or the block has found is done after the two products; the few others
+// (one key in a hundred and fewer on the measured rows) score their pairs from
+// the table.  Each lane decides for itself, and nothing in the scoring names
+// another lane.  (One bound over all slots, the key's lanes deciding together:
+// 512 rows of 32,768 keys 20.8 ms, now 20.1, 3,072 GQA rows 6.13 and 5.65: a key
+// of little weight that leaves becomes a slot with a small B_j, and loosens its
+// own class only.)  The least score wins; among pairs at that score the smallest
+// (i, j), except that two positions of one lane at exactly the same fp32 score
+// keep the first: such pairs are tied to ~1e-7 relative, a decision no fp32
+// evaluation can settle.
 //
 // A key that holds most of the kept mass (P' could fall below P / 4) is scored
 // after the pass by the whole block from g' = g - u_i + u_j, the columns split
 // over the warps, a lane per slot; at most one key of a round qualifies.
 //
 // Bound: on long rows the reads of value rows and scalars through the SM's L2
-// port (~280 bytes per kept key and round at d = 128) and the products' shared
+// port (~290 bytes per kept key and round at d = 128) and the products' shared
 // reads; on short rows the latency of a round's barriers.  Scoring every key's E
 // pairs in every round (408 bytes per key) took, with the gap call, 30.2 ms on
 // 512 rows of 32,768 keys with three budgets and 9.4 ms on 3,072 GQA rows of
-// 1,000 to 8,192 keys; now 21.3 and 6.1 ms.  (The products by two-float FMAs;
-// one by one 21.5; g.w carried along 19.6 and 6.1.)
+// 1,000 to 8,192 keys; now 20.1 and 5.65 ms.
 #include <algorithm>
 #include <climits>
 
@@ -94,7 +97,7 @@ struct LSArgs {
     int32_t *kbuf;   // key at each position of the current kept list
     float *pbuf;     // its mass
     float *xbuf;     // its |w|^2
-    float *mbuf;     // its bound on max_j p_j C_ij
+    float *mbuf;     // its bounds on max_j p_j C_ij, by lane class: [4] each
     uint32_t *kebuf; // order key of every dropped key's error (0: kept)
     // per-block cross-product table, [gridDim.x][Ep][cstride] (slot-major)
     float *cbuf;
@@ -372,18 +375,17 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
     __shared__ TopmSmem s_top;
     __shared__ float red[SWW], red2[SWW];
     __shared__ int s_cnt, s_bt, s_bq, s_heavy;
-    __shared__ float s_gm, s_ym, s_pmin, s_pmax, s_Bmin, s_hsg;
+    __shared__ float s_gm, s_ym, s_pmin, s_pmax, s_Bmin[QL], s_hsg;
     __shared__ uint32_t s_ub;          // order key of the least score found in the round
     __shared__ unsigned long long s_bkey;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int gq = tid / QL, sub = tid % QL;  // key group and lane within it
-    const uint32_t quad = 0xfu << (lane & 28);
     const size_t boff = (size_t)blockIdx.x * a.R.max_n;
     float *eb = a.ebuf + boff;
     int *kb = a.kbuf + boff;
     float *pk = a.pbuf + boff;
     float *xk = a.xbuf + boff;
-    float *mk = a.mbuf + boff;
+    float *mk = a.mbuf + boff * QL;
     uint32_t *ke = a.kebuf + boff;
     const int cs = a.cstride;
     float *cb = a.cbuf + (size_t)blockIdx.x * Ep * cs;  // [Ep][cs]
@@ -669,11 +671,13 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                     }
                     pm = warp_min(pm);
                     px = warp_max(px);
-                    Bm = warp_min(Bm);
+                    // (slot q belongs to class (q / 8) % 4, the lane of a key that holds it)
+#pragma unroll
+                    for (int o = 1; o < 8; o <<= 1) Bm = fminf(Bm, __shfl_xor_sync(FW_FULL, Bm, o));
+                    if ((lane & 7) == 0) s_Bmin[lane >> 3] = Bm;
                     if (lane == 0) {
                         s_pmin = pm;
                         s_pmax = px;
-                        s_Bmin = Bm;
                         s_heavy = -1;
                         s_ub = order_key(0.f);  // only scores below 0 are swaps
                         s_bkey = ~0ull;
@@ -684,11 +688,9 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                 // scores, with the pair's position and slot.
                 float lmin = INFINITY;
                 int lt = -1, li = 0, lq = 0;
-                const float pmin = s_pmin, Bmin = s_Bmin, hmin = 2.f * N * pmin, hmax = 2.f * N * s_pmax;
-                // position t, key i: its pairs, unless its bound excludes them.  Every
-                // argument is the same in the key's four lanes, so they leave or stay
-                // together, as the shuffles below need.
-                auto score_key = [&](int t, int i, float sg, float sn, float p_i, float x2, float mx, float ub, bool scan) {
+                const float pmin = s_pmin, Bmin = s_Bmin[sub], hmin = 2.f * N * pmin, hmax = 2.f * N * s_pmax;
+                // position t, key i: this lane's pairs, unless their bound excludes them
+                auto score_key = [&](int t, int i, float sg, float sn, float p_i, float x2, float mx, bool scan) {
                     const float alpha = p_i * p_i * x2 - 2.f * p_i * sg;
                     const float Ai = alpha * P2 + N * p_i * (2.f * P - p_i);
                     const float Pm = P - p_i;
@@ -700,10 +702,12 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                         }
                         return;
                     }
+                    if (8 * sub >= nadd) return;  // no slots
+                    const float ub = key_to_float(*(volatile uint32_t *)&s_ub);
                     const float cmx = 2.f * P2 * p_i * mx;
                     const float lb = (Ai + Bmin) + (p_i * hmin - cmx);
                     const float slack = 4e-6f * (fabsf(Ai) + fabsf(Bmin) + p_i * hmax + fabsf(cmx));  // its rounding
-                    if (!scan && lb - slack > ub * (Pl * Pl)) return;
+                    if (!scan && lb - slack > fminf(ub, lmin) * (Pl * Pl)) return;
                     float kmin = INFINITY, kc = -INFINITY;
                     int kq = 0;
                     for (int q0 = 0; q0 < nadd; q0 += 32) {
@@ -740,9 +744,7 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                                 }
                         }
                     }
-                    kc = fmaxf(kc, __shfl_xor_sync(quad, kc, 1));
-                    kc = fmaxf(kc, __shfl_xor_sync(quad, kc, 2));
-                    if (sub == 0) mk[t] = kc;
+                    mk[QL * t + sub] = kc;
                     if (kmin < lmin) {  // first position of the lane's least score
                         lmin = kmin;
                         lt = t;
@@ -768,9 +770,9 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                         if (sub == 0) {
                             pk[t] = p_i;
                             xk[t] = sn;
-                            mk[t] = INFINITY;
                         }
-                        score_key(t, i, sg, sn, p_i, sn, INFINITY, 0.f, true);
+                        mk[QL * t + sub] = INFINITY;
+                        score_key(t, i, sg, sn, p_i, sn, INFINITY, true);
                     }
                 } else {
                     // software pipeline: the value row and scalars of the next iteration and
@@ -783,11 +785,12 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                     int i_next = kb[gq + KPI < nk ? gq + KPI : nk - 1];
                     LaneRow<DPL, VT> row;
                     row.load(V + (int64_t)i_cur * d, sub);
-                    float p_i = pk[tf], x2 = xk[tf], m0 = mk[tf];
+                    float p_i = pk[tf], x2 = xk[tf], m0 = mk[QL * tf + sub];
+                    const bool mine = (qprev >> 3 & (QL - 1)) == sub;  // the changed slot is of this lane's class
                     for (int it = 0; it < niter; ++it) {
                         const int t = it * KPI + gq;
                         const int tn = t + KPI < nk ? t + KPI : nk - 1;
-                        const float p_n = pk[tn], x2_n = xk[tn], m_n = mk[tn];
+                        const float p_n = pk[tn], x2_n = xk[tn], m_n = mk[QL * tn + sub];
                         LaneRow<DPL, VT> rown;
                         rown.load(V + (int64_t)i_next * d, sub);
                         const int tnn = t + 2 * KPI;
@@ -798,20 +801,16 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                         sn += __shfl_xor_sync(FW_FULL, sn, 1);
                         sg += __shfl_xor_sync(FW_FULL, sg, 2);
                         sn += __shfl_xor_sync(FW_FULL, sn, 2);
-                        // the least score found so far, as one lane reads it (other warps lower
-                        // it meanwhile; a vote of a key's lanes instead cost 15 to 21 % of the call)
-                        const float ub = __shfl_sync(FW_FULL, key_to_float(*(volatile uint32_t *)&s_ub), 0);
                         if (t < nk) {
                             sn -= ym;
                             if (t != tprev) {
-                                const float mn = fmaxf(m0, pdep * sn);
-                                if (sub == 0) {
-                                    col[t] = sn;
-                                    if (mn > m0) mk[t] = mn;
+                                if (sub == 0) col[t] = sn;
+                                if (mine && pdep * sn > m0) {
+                                    m0 = pdep * sn;
+                                    mk[QL * t + sub] = m0;
                                 }
-                                m0 = mn;
                             }
-                            score_key(t, i_cur, sg - gm, sn, p_i, x2, m0, ub, false);
+                            score_key(t, i_cur, sg - gm, sn, p_i, x2, m0, false);
                         }
                         row = rown;
                         i_cur = i_next;
@@ -905,6 +904,7 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                 }
                 P = P - p_i + p_j;
                 N = block_sum(gl2, red2);  // (its barrier ends every read above)
+                if (tid < QL) mk[QL * tb + tid] = INFINITY;
                 if (tid == 0) {
                     idxj[qj] = bi;
                     sP[qj] = p_i;
@@ -912,7 +912,6 @@ __global__ void __launch_bounds__(SWT, BPS) k_long_swap(const LSArgs a)
                     kb[tb] = bj;
                     pk[tb] = p_j;
                     xk[tb] = x_j;
-                    mk[tb] = INFINITY;
                     a.swap_out[rb * MS + taken] = bi;
                     a.swap_in[rb * MS + taken] = bj;
                 }
@@ -965,7 +964,7 @@ static size_t ls_table_bytes(const RowsDev &R, int E)
 size_t long_swap_workspace(const RowsDev &R, int nb, int E, int max_swaps)
 {
     (void)nb, (void)max_swaps;
-    return ls_array_bytes(R) * 6 + ls_table_bytes(R, E);
+    return ls_array_bytes(R) * (5 + QL) + ls_table_bytes(R, E);
 }
 
 fw_status long_swap(const RowsDev &R, const int32_t *k, int nb, const fw_gap_out &topk, int E, int max_swaps,
@@ -1000,9 +999,9 @@ fw_status long_swap(const RowsDev &R, const int32_t *k, int nb, const fw_gap_out
     a.kbuf = (int32_t *)(w + 1 * arr);
     a.pbuf = (float *)(w + 2 * arr);
     a.xbuf = (float *)(w + 3 * arr);
-    a.mbuf = (float *)(w + 4 * arr);
-    a.kebuf = (uint32_t *)(w + 5 * arr);
-    a.cbuf = (float *)(w + 6 * arr);
+    a.kebuf = (uint32_t *)(w + 4 * arr);
+    a.mbuf = (float *)(w + 5 * arr);
+    a.cbuf = (float *)(w + (5 + QL) * arr);
     FW_DISPATCH(R.d, R.v_dtype, {
         const size_t smem = ls_smem<DPL>(a.Ep);
         constexpr int SHORT = DPL <= 4 ? LS_BPS_SHORT : LS_BPS_LONG;
