@@ -182,6 +182,8 @@ __host__ __device__ constexpr int swap_smem_floats(int n, int d) { return staged
 //    lane, and P(A - i) once a round for every i.
 // 36,864 rows of 24 keys, d = 128: 1,433 us with whole rows staged and Gram entries one
 // by one, 704 us so; 256 rows of 20 keys, d = 64: 67 and 28 us.
+// (10 blocks an SM are 96 registers: d = 256 spills 41 of its words, and still takes 763
+// us on 20,000 rows of 24 keys, 2,180 before; with 128 registers 748.)
 template <int DPL, typename VT>
 __global__ void __launch_bounds__(64, 10) k_small_swap(const SmallSwapArgs a)
 {
